@@ -18,6 +18,7 @@
 
 #include "../../include/pgen.h"
 #include "pg_internal.h"
+#include "pg_kron.cuh"
 #include "pg_trace.h"
 
 namespace pgen {
@@ -136,83 +137,23 @@ __device__ __forceinline__ bool ba_link(uint32_t& cur, const BatchJob& J, const 
     return false;
 }
 
-__device__ __forceinline__ void kron_level(uint32_t w, uint32_t base, uint32_t u0, uint32_t u1,
-                                           uint32_t u2, uint64_t& row, uint64_t& col)
-{
-    const uint32_t cell = base + (w > u0) + (w > u1) + (w > u2);
-    row = (row << 1) | (cell >> 1);
-    col = (col << 1) | (cell & 1);
-}
-
-// The same pick for a 2x2 initiator whose four cells are all positive
-// (n_zero = 0, three real thresholds u0 <= u1 <= u2): the row bit is
-// a = (w > u1), the column bit (w > u2) when a is set, else (w > u0).
-__device__ __forceinline__ void kron_level_full(uint32_t w, uint32_t u0, uint32_t u1, uint32_t u2,
-                                                uint64_t& row, uint64_t& col)
-{
-    const uint32_t a = w > u1 ? 1u : 0u;
-    const uint32_t b = w > (a ? u2 : u0) ? 1u : 0u;
-    row = row * 2 + a;
-    col = col * 2 + b;
-}
-
-// The full-initiator 2x2 pick for a job whose ids and edge indices fit 32
-// bits (k <= 32 levels, fewer than 2^32 edges): the same values with 32-bit
-// rows, columns and counters (e, 0, g, 3), the thresholds and k in registers
-// for the whole tile, whole groups of four levels unrolled.
-__device__ __forceinline__ void kron_edge_full32(const Key& key, uint32_t k, uint32_t u0,
-                                                 uint32_t u1, uint32_t u2, uint32_t e,
-                                                 uint32_t& row, uint32_t& col)
-{
-    row = 0;
-    col = 0;
-    uint32_t l = 0;
-    auto level = [&](uint32_t w) {
-        const uint32_t a = w > u1 ? 1u : 0u;
-        const uint32_t b = w > (a ? u2 : u0) ? 1u : 0u;
-        row = row * 2 + a;
-        col = col * 2 + b;
-    };
-    for (uint32_t g = 0; l + 4 <= k; ++g, l += 4) {
-        const uint4 w = philox(make_uint4(e, 0u, g, 3u), key);
-        level(w.x);
-        level(w.y);
-        level(w.z);
-        level(w.w);
-    }
-    if (l < k) {
-        const uint4 w = philox(make_uint4(e, 0u, l >> 2, 3u), key);
-        level(w.x);
-        if (l + 1 < k) level(w.y);
-        if (l + 2 < k) level(w.z);
-    }
-}
-
+// Any initiator, any number of edges: the order-2 thresholds from the job's
+// record, larger ones by binary search in the pool.
 __device__ __forceinline__ void kron_edge(const BatchJob& J, const Key& key,
                                           const uint32_t* pool, uint32_t n_pool, uint64_t e,
                                           uint64_t& row, uint64_t& col)
 {
     row = 0;
     col = 0;
-    if (J.n0 == 2 && J.n_zero == 0 && J.n_u == 3) {
-        uint32_t l = 0;
-        for (uint32_t g = 0; l < J.k; ++g, l += 4) {
-            const uint4 w = philox(make_uint4((uint32_t)e, (uint32_t)(e >> 32), g, 3u), key);
-            kron_level_full(w.x, J.u0, J.u1, J.u2, row, col);
-            if (l + 1 < J.k) kron_level_full(w.y, J.u0, J.u1, J.u2, row, col);
-            if (l + 2 < J.k) kron_level_full(w.z, J.u0, J.u1, J.u2, row, col);
-            if (l + 3 < J.k) kron_level_full(w.w, J.u0, J.u1, J.u2, row, col);
-        }
-        return;
-    }
     if (J.n0 == 2) {
-        uint32_t l = 0;
-        for (uint32_t g = 0; l < J.k; ++g, l += 4) {
-            const uint4 w = philox(make_uint4((uint32_t)e, (uint32_t)(e >> 32), g, 3u), key);
-            kron_level(w.x, J.n_zero, J.u0, J.u1, J.u2, row, col);
-            if (l + 1 < J.k) kron_level(w.y, J.n_zero, J.u0, J.u1, J.u2, row, col);
-            if (l + 2 < J.k) kron_level(w.z, J.n_zero, J.u0, J.u1, J.u2, row, col);
-            if (l + 3 < J.k) kron_level(w.w, J.n_zero, J.u0, J.u1, J.u2, row, col);
+        uint4 w = make_uint4(0, 0, 0, 0);
+        for (uint32_t l = 0; l < J.k; ++l) {
+            if ((l & 3) == 0)
+                w = philox(make_uint4((uint32_t)e, (uint32_t)(e >> 32), l >> 2, 3u), key);
+            const uint32_t x = (l & 3) == 0 ? w.x : (l & 3) == 1 ? w.y : (l & 3) == 2 ? w.z : w.w;
+            const uint32_t cell = J.n_zero + (x > J.u0) + (x > J.u1) + (x > J.u2);
+            row = (row << 1) | (cell >> 1);
+            col = (col << 1) | (cell & 1);
         }
         return;
     }
@@ -232,6 +173,29 @@ __device__ __forceinline__ void kron_edge(const BatchJob& J, const Key& key,
         const uint32_t cell = J.n_zero + lo;
         row = row * J.n0 + cell / J.n0;
         col = col * J.n0 + cell % J.n0;
+    }
+}
+
+// Edges [t0, t0 + n) of an order-2 Kronecker job (indices below 2^32), two per
+// thread, stored from an even arena edge.
+template <typename Id, typename T, bool kFull>
+__device__ __forceinline__ void kron_tile(const BatchJob& J, const Key& key, const uint4* heads,
+                                          Id* arena, uint64_t cap, uint64_t t0, uint32_t n)
+{
+    const uint32_t k = J.k, u0 = J.u0, u1 = J.u1, u2 = J.u2, base = J.n_zero;
+    const uint64_t e_first = J.out_edge + t0;
+    const uint32_t head = (uint32_t)(e_first & 1);
+    // pair i of the tile is its edges 2i - head and 2i + 1 - head; the first
+    // and the last pair may have one edge in the tile only
+    for (uint32_t i = threadIdx.x; 2 * i < n + head; i += blockDim.x) {
+        const uint32_t a = 2 * i - head;   // -1 (as uint32) for the first edge of an odd tile
+        T r0, c0, r1, c1;
+        kron_two_edges<T, kFull>(heads, key, k, u0, u1, u2, base, (uint32_t)t0 + a,
+                                 (uint32_t)t0 + a + 1, r0, c0, r1, c1);
+        const bool one = head == 0 || i > 0, two = a + 1 < n;
+        if (one && two) put_two(arena, cap, e_first + a, r0, c0, r1, c1);
+        else if (one) put_pair(arena, cap, e_first + a, r0, c0);
+        else if (two) put_pair(arena, cap, e_first + (uint32_t)(a + 1), r1, c1);
     }
 }
 
@@ -255,6 +219,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const unsigned cha
     uint32_t* first = reinterpret_cast<uint32_t*>(smem + kMaxTile * sizeof(Id));   // n_jobs + 1
     __shared__ uint32_t s_item, s_job;
     __shared__ BatchJob sJ;
+    __shared__ uint4 heads[kKronMaxGroups];   // of the item's Kronecker job
 
     for (uint32_t t = threadIdx.x; t <= n_jobs; t += blockDim.x) first[t] = first_g[t];
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -326,28 +291,16 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const unsigned cha
                 else
                     put_pair(arena, cap, e_first + t2, s0, (uint64_t)sDst[t2]);
             }
-        } else if (J.n0 == 2 && J.n_zero == 0 && J.n_u == 3 && J.k <= 32 &&
-                   J.n_units <= 0xFFFFFFFFull) {
-            // 32-bit full-initiator descent (the kron2 kernel's arithmetic)
-            const uint32_t k = J.k, u0 = J.u0, u1 = J.u1, u2 = J.u2;
-            const uint64_t e_first = J.out_edge + t0;
-            const uint32_t head = (uint32_t)(e_first & 1) < n ? (uint32_t)(e_first & 1) : n;
-            if (head && threadIdx.x == 0) {
-                uint32_t r, c;
-                kron_edge_full32(key, k, u0, u1, u2, (uint32_t)t0, r, c);
-                put_pair(arena, cap, e_first, r, c);
-            }
-            for (uint32_t t2 = head + 2 * threadIdx.x; t2 < n; t2 += 2 * blockDim.x) {
-                uint32_t r0, c0;
-                kron_edge_full32(key, k, u0, u1, u2, (uint32_t)(t0 + t2), r0, c0);
-                if (t2 + 1 < n) {
-                    uint32_t r1, c1;
-                    kron_edge_full32(key, k, u0, u1, u2, (uint32_t)(t0 + t2 + 1), r1, c1);
-                    put_two(arena, cap, e_first + t2, r0, c0, r1, c1);
-                } else {
-                    put_pair(arena, cap, e_first + t2, r0, c0);
-                }
-            }
+        } else if (J.n0 == 2 && J.n_units <= (1ull << 32)) {
+            // every edge index below 2^32: the single-graph kernel's descent
+            if (threadIdx.x < kKronMaxGroups && 4 * threadIdx.x < J.k)
+                heads[threadIdx.x] = kron_group_head(0u, threadIdx.x, key);
+            __syncthreads();
+            const bool full = J.n_zero == 0 && J.n_u == 3;
+            if (J.k <= 32 && full) kron_tile<Id, uint32_t, true>(J, key, heads, arena, cap, t0, n);
+            else if (J.k <= 32) kron_tile<Id, uint32_t, false>(J, key, heads, arena, cap, t0, n);
+            else if (full) kron_tile<Id, uint64_t, true>(J, key, heads, arena, cap, t0, n);
+            else kron_tile<Id, uint64_t, false>(J, key, heads, arena, cap, t0, n);
         } else {
             const uint64_t e_first = J.out_edge + t0;
             const uint32_t head = (uint32_t)(e_first & 1) < n ? (uint32_t)(e_first & 1) : n;

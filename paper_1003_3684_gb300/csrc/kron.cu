@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "pg_internal.h"
+#include "pg_kron.cuh"
 #include "pg_trace.h"
 
 namespace pgen {
@@ -56,153 +57,39 @@ struct Pair2<uint64_t> {
     }
 };
 
-// ---- stochastic descent, initiator order 2 (branch-free 3-threshold pick) --
+// ---- stochastic descent, initiator order 2 ---------------------------------
+// One launch covers local edges [first, first + 2 * n_pairs) of the call, all
+// of whose indices share their high word e_hi; e_lo is the low word of edge
+// `first`'s index. Pairs are aligned to even local edges (16-byte stores):
+// with skip_head the pair's first edge, and with skip_tail the last pair's
+// second one, belongs to another launch or lies past the end.
 // T is uint32_t when k <= 32 (ids fit 32 bits), else uint64_t.
-template <typename T>
-__device__ __forceinline__ void descend2(uint32_t w, uint32_t u0, uint32_t u1, uint32_t u2,
-                                         uint32_t base, T& row, T& col)
-{
-    const uint32_t cell = base + (w > u0) + (w > u1) + (w > u2);
-    row = (row << 1) | (T)(cell >> 1);
-    col = (col << 1) | (T)(cell & 1);
-}
-
-// The same pick when cell 0 has positive weight and all three thresholds
-// are real (n_zero = 0, n_u = 3): with u0 <= u1 <= u2 the row bit of the
-// cell is a = (w > u1), and its column bit is (w > u2) when a is set (cells
-// 2, 3), else (w > u0) (cells 0, 1): two compares instead of three and a
-// parity. row = 2*row + a runs on the multiply-add pipe, not the ALU pipe.
-template <typename T>
-__device__ __forceinline__ void descend2_full(uint32_t w, uint32_t u0, uint32_t u1, uint32_t u2,
-                                              T& row, T& col)
-{
-    const uint32_t a = w > u1 ? 1u : 0u;
-    const uint32_t b = w > (a ? u2 : u0) ? 1u : 0u;
-    row = row * 2 + (T)a;
-    col = col * 2 + (T)b;
-}
-
-template <typename T>
-__device__ __forceinline__ void kron2_edge_full(const KronParams& p, uint64_t e, uint32_t u0,
-                                                uint32_t u1, uint32_t u2, T& row, T& col)
-{
-    row = 0;
-    col = 0;
-    const uint32_t k = p.k;
-    uint32_t l = 0;
-    for (uint32_t g = 0; l + 4 <= k; ++g, l += 4) {
-        const uint4 w = draw(e, g, 3, p.key);
-        descend2_full(w.x, u0, u1, u2, row, col);
-        descend2_full(w.y, u0, u1, u2, row, col);
-        descend2_full(w.z, u0, u1, u2, row, col);
-        descend2_full(w.w, u0, u1, u2, row, col);
-    }
-    if (l < k) {
-        const uint4 w = draw(e, l >> 2, 3, p.key);
-        descend2_full(w.x, u0, u1, u2, row, col);
-        if (l + 1 < k) descend2_full(w.y, u0, u1, u2, row, col);
-        if (l + 2 < k) descend2_full(w.z, u0, u1, u2, row, col);
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ void kron2_edge(const KronParams& p, uint64_t e, uint32_t u0,
-                                           uint32_t u1, uint32_t u2, T& row, T& col)
-{
-    row = 0;
-    col = 0;
-    const uint32_t k = p.k;
-    uint32_t l = 0;
-    for (uint32_t g = 0; l + 4 <= k; ++g, l += 4) {
-        const uint4 w = draw(e, g, 3, p.key);
-        descend2(w.x, u0, u1, u2, p.n_zero, row, col);
-        descend2(w.y, u0, u1, u2, p.n_zero, row, col);
-        descend2(w.z, u0, u1, u2, p.n_zero, row, col);
-        descend2(w.w, u0, u1, u2, p.n_zero, row, col);
-    }
-    if (l < k) {
-        const uint4 w = draw(e, l >> 2, 3, p.key);
-        descend2(w.x, u0, u1, u2, p.n_zero, row, col);
-        if (l + 1 < k) descend2(w.y, u0, u1, u2, p.n_zero, row, col);
-        if (l + 2 < k) descend2(w.z, u0, u1, u2, p.n_zero, row, col);
-    }
-}
-
 template <typename Id, typename T, bool kFull>
 __global__ void __launch_bounds__(256) kron2_kernel(const __grid_constant__ KronParams p,
-                                                    Id* __restrict__ out, uint64_t e_begin,
-                                                    uint64_t n_edges)
+                                                    Id* __restrict__ out, uint64_t first,
+                                                    uint32_t n_pairs, uint32_t e_lo,
+                                                    uint32_t e_hi, uint32_t skip_head,
+                                                    uint32_t skip_tail, uint64_t n_edges)
 {
+    __shared__ uint4 heads[kKronMaxGroups];
+    for (uint32_t g = threadIdx.x; 4 * g < p.k && g < kKronMaxGroups; g += blockDim.x)
+        heads[g] = kron_group_head(e_hi, g, p.key);
+    __syncthreads();
     const uint32_t u0 = p.u[0], u1 = p.u[1], u2 = p.u[2];   // padded to three
-    const uint64_t n_pairs = (n_edges + 1) >> 1;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    auto edge = [&](uint64_t ee, T& r, T& c) {
-        if constexpr (kFull) kron2_edge_full(p, ee, u0, u1, u2, r, c);
-        else kron2_edge(p, ee, u0, u1, u2, r, c);
-    };
-    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n_pairs; t += stride) {
-        const uint64_t e = 2 * t;
-        T r0, c0;
-        edge(e_begin + e, r0, c0);
-        if (e + 1 < n_edges) {
-            T r1, c1;
-            edge(e_begin + e + 1, r1, c1);
-            if (PG_CHECK_OUT(e + 1, n_edges)) Pair2<Id>::store(out, e, r0, c0, r1, c1);
-        } else {
-            if (PG_CHECK_OUT(e, n_edges)) Pair2<Id>::store1(out, e, r0, c0);
-        }
-    }
-}
-
-// The same descent with 32-bit edge indices, counters (e, 0, g, 3), ids and
-// loop arithmetic, for launches whose edge indices all lie below 2^32 and
-// whose ids fit 32 bits (k <= 32): the same values, less index arithmetic.
-template <bool kFull>
-__device__ __forceinline__ void kron2_edge32(const KronParams& p, uint32_t e, uint32_t u0,
-                                             uint32_t u1, uint32_t u2, uint32_t& row,
-                                             uint32_t& col)
-{
-    row = 0;
-    col = 0;
-    const uint32_t k = p.k;
-    auto level = [&](uint32_t w) {
-        if constexpr (kFull) descend2_full(w, u0, u1, u2, row, col);
-        else descend2(w, u0, u1, u2, p.n_zero, row, col);
-    };
-    uint32_t l = 0;
-    for (uint32_t g = 0; l + 4 <= k; ++g, l += 4) {
-        const uint4 w = philox(make_uint4(e, 0u, g, 3u), p.key);
-        level(w.x);
-        level(w.y);
-        level(w.z);
-        level(w.w);
-    }
-    if (l < k) {
-        const uint4 w = philox(make_uint4(e, 0u, l >> 2, 3u), p.key);
-        level(w.x);
-        if (l + 1 < k) level(w.y);
-        if (l + 2 < k) level(w.z);
-    }
-}
-
-template <typename Id, bool kFull>
-__global__ void __launch_bounds__(256) kron2_kernel32(const __grid_constant__ KronParams p,
-                                                      Id* __restrict__ out, uint32_t e_begin,
-                                                      uint32_t n_edges)
-{
-    const uint32_t u0 = p.u[0], u1 = p.u[1], u2 = p.u[2];   // padded to three
-    const uint32_t n_pairs = (n_edges >> 1) + (n_edges & 1);
     const uint32_t stride = gridDim.x * blockDim.x;
+    out += 2 * first;
     for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < n_pairs; t += stride) {
-        const uint32_t e = 2 * t;
-        uint32_t r0, c0;
-        kron2_edge32<kFull>(p, e_begin + e, u0, u1, u2, r0, c0);
-        if (e + 1 < n_edges) {
-            uint32_t r1, c1;
-            kron2_edge32<kFull>(p, e_begin + e + 1, u0, u1, u2, r1, c1);
-            if (PG_CHECK_OUT(e + 1, n_edges)) Pair2<Id>::store(out, e, r0, c0, r1, c1);
-        } else {
-            if (PG_CHECK_OUT(e, n_edges)) Pair2<Id>::store1(out, e, r0, c0);
+        T r0, c0, r1, c1;
+        kron_two_edges<T, kFull>(heads, p.key, p.k, u0, u1, u2, p.n_zero, e_lo + 2 * t,
+                                 e_lo + 2 * t + 1, r0, c0, r1, c1);
+        const uint64_t e = 2 * (uint64_t)t;
+        const bool one = t != 0 || !skip_head, two = t + 1 != n_pairs || !skip_tail;
+        if (one && two) {
+            if (PG_CHECK_OUT(first + e + 1, n_edges)) Pair2<Id>::store(out, e, r0, c0, r1, c1);
+        } else if (one) {
+            if (PG_CHECK_OUT(first + e, n_edges)) Pair2<Id>::store1(out, e, r0, c0);
+        } else if (two) {
+            if (PG_CHECK_OUT(first + e + 1, n_edges)) Pair2<Id>::store1(out, e + 1, r1, c1);
         }
     }
 }
@@ -476,6 +363,30 @@ int grid_for(K kernel, uint64_t work_items, int threads, size_t smem = 0)
 
 PG_CHECK_UNIT(kron)
 
+namespace {
+
+// One launch per run of edges whose indices share their high word.
+template <typename Id, typename T>
+void launch_kron2(const KronParams& p, Id* out, uint64_t e_begin, uint64_t n_edges, cudaStream_t s)
+{
+    const bool full = p.n_zero == 0 && p.n_u == 3;
+    auto k = full ? kron2_kernel<Id, T, true> : kron2_kernel<Id, T, false>;
+    for (uint64_t a = 0; a < n_edges;) {
+        const uint64_t low = e_begin + a;   // index of the run's first edge
+        const uint64_t left = ((uint64_t)1 << 32) - (low & 0xFFFFFFFFu);
+        const uint64_t b = n_edges - a < left ? n_edges : a + left;
+        const uint64_t first = a & ~(uint64_t)1;
+        const uint32_t pairs = (uint32_t)((b - first + 1) / 2);
+        { k<<<grid_for(k, pairs, 256), 256, 0, s>>>(p, out, first, pairs,
+                                                   (uint32_t)(e_begin + first),
+                                                   (uint32_t)(low >> 32), (uint32_t)(a & 1),
+                                                   (uint32_t)(b & 1), n_edges); note_launch(); }
+        a = b;
+    }
+}
+
+}  // namespace
+
 cudaError_t launch_kron_stochastic(const KronParams& p, int id64, void* d_out, uint64_t e_begin,
                                    uint64_t n_edges, cudaStream_t s)
 {
@@ -483,28 +394,9 @@ cudaError_t launch_kron_stochastic(const KronParams& p, int id64, void* d_out, u
     const uint64_t pairs = (n_edges + 1) / 2;
     TraceScope trace(p.n0 == 2 ? "kron_descent_n0_2" : "kron_descent", s);
     if (p.n0 == 2) {
-        // 32-bit descent state when every id fits (k <= 32)
-        const bool full = p.n_zero == 0 && p.n_u == 3;
-        if (p.k <= 32 && e_begin + n_edges < ((uint64_t)1 << 32)) {
-            // every edge index below 2^32: 32-bit indices and counters
-            const uint32_t b = (uint32_t)e_begin, n = (uint32_t)n_edges;
-            if (id64) {
-                auto k = full ? kron2_kernel32<uint64_t, true> : kron2_kernel32<uint64_t, false>;
-                { k<<<grid_for(k, pairs, 256), 256, 0, s>>>(p, (uint64_t*)d_out, b, n); note_launch(); }
-            } else {
-                auto k = full ? kron2_kernel32<uint32_t, true> : kron2_kernel32<uint32_t, false>;
-                { k<<<grid_for(k, pairs, 256), 256, 0, s>>>(p, (uint32_t*)d_out, b, n); note_launch(); }
-            }
-        } else if (id64 && p.k > 32) {
-            auto k = full ? kron2_kernel<uint64_t, uint64_t, true> : kron2_kernel<uint64_t, uint64_t, false>;
-            { k<<<grid_for(k, pairs, 256), 256, 0, s>>>(p, (uint64_t*)d_out, e_begin, n_edges); note_launch(); }
-        } else if (id64) {
-            auto k = full ? kron2_kernel<uint64_t, uint32_t, true> : kron2_kernel<uint64_t, uint32_t, false>;
-            { k<<<grid_for(k, pairs, 256), 256, 0, s>>>(p, (uint64_t*)d_out, e_begin, n_edges); note_launch(); }
-        } else {
-            auto k = full ? kron2_kernel<uint32_t, uint32_t, true> : kron2_kernel<uint32_t, uint32_t, false>;
-            { k<<<grid_for(k, pairs, 256), 256, 0, s>>>(p, (uint32_t*)d_out, e_begin, n_edges); note_launch(); }
-        }
+        if (id64 && p.k > 32) launch_kron2<uint64_t, uint64_t>(p, (uint64_t*)d_out, e_begin, n_edges, s);
+        else if (id64) launch_kron2<uint64_t, uint32_t>(p, (uint64_t*)d_out, e_begin, n_edges, s);
+        else launch_kron2<uint32_t, uint32_t>(p, (uint32_t*)d_out, e_begin, n_edges, s);
     } else {
         if (id64) {
             auto k = kron_generic_kernel<uint64_t>;
