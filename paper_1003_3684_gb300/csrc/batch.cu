@@ -66,7 +66,9 @@ struct PlanHeader {
     uint32_t n_jobs, n_pool;
     uint64_t n_items, total_edges;
     uint64_t off_jobs, off_first, off_pool;
-    uint64_t off_starts;       // n_jobs + 1 uint64: every job's first edge, then the total
+    uint64_t off_slots;        // n_csr + 1 uint64: each CSR job's first union slot (group 0's
+                               // jobs first, in job order), then the number of slots
+    uint64_t off_slot_jobs;    // n_csr uint32: those jobs
     uint64_t off_rstart[2];    // per CSR group g: csr_jobs[g] + 1 uint64, each CSR job's
                                // first row_ptr entry, then the group's end
     uint64_t off_two;          // n_two TwoPhaseJob records (host only)
@@ -86,7 +88,7 @@ size_t plan_bytes(uint32_t n_jobs, uint32_t n_pool, uint32_t n_two, uint32_t n_c
 {
     return a16(sizeof(PlanHeader)) + a16((size_t)n_jobs * sizeof(BatchJob)) +
            a16((size_t)(n_jobs + 1) * 4) + a16((size_t)n_pool * 4) +
-           a16((size_t)(n_jobs + 1) * 8) + 2 * a16((size_t)(n_csr + 1) * 8) +
+           3 * a16((size_t)(n_csr + 1) * 8) + a16((size_t)(n_csr + 1) * 4) +
            a16((size_t)n_two * sizeof(TwoPhaseJob));
 }
 
@@ -328,9 +330,13 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const unsigned cha
 // (vbase + src, dst) pairs, at the job's csr_edge: the union graph of the
 // group, whose CSR is its jobs' CSRs one after another (rows of job t are
 // vbase_t .. vbase_t + n_vertices_t - 1, and its col entries keep their
-// local ids). One pair per thread, moved as one vector load and store; lane
-// 0 of a warp finds the job of the warp's first edge by a binary search over
-// the job starts, and each lane steps from there to its own.
+// local ids). Bound by memory: 8 bytes read and 8 written per union pair (16
+// and 16 with 64-bit ids), whatever the arena holds besides the CSR jobs
+// (walking the arena instead took 9.17 ms of a 256-graph batch in which the
+// CSR jobs have 1/300 of the edges; by union slot 0.02 ms). A warp takes
+// kUnionRun slots; lane 0 finds the job of the first by a binary search, each
+// lane steps from there to its own, and its four loads are in flight at once.
+constexpr uint32_t kUnionRun = 128;
 template <typename Id>
 __global__ void __launch_bounds__(256) batch_union_kernel(const unsigned char* __restrict__ plan,
                                                           const Id* __restrict__ arena,
@@ -339,37 +345,43 @@ __global__ void __launch_bounds__(256) batch_union_kernel(const unsigned char* _
     using P = typename std::conditional<sizeof(Id) == 4, uint2, ulonglong2>::type;
     const PlanHeader& H = *reinterpret_cast<const PlanHeader*>(plan);
     const BatchJob* jobs = reinterpret_cast<const BatchJob*>(plan + H.off_jobs);
-    const uint64_t* starts = reinterpret_cast<const uint64_t*>(plan + H.off_starts);
-    const uint32_t n_jobs = H.n_jobs;
-    const uint64_t E = H.total_edges;
+    const uint64_t* slots = reinterpret_cast<const uint64_t*>(plan + H.off_slots);
+    const uint32_t* slot_jobs = reinterpret_cast<const uint32_t*>(plan + H.off_slot_jobs);
+    const uint32_t n = (uint32_t)(H.csr_jobs[0] + H.csr_jobs[1]);
+    const uint64_t E = H.csr_edges[0] + H.csr_edges[1];
     const P* in = reinterpret_cast<const P*>(arena);
     P* out = reinterpret_cast<P*>(uni);
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    for (uint64_t base = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < E;
-         base += warps * 32) {
-        uint32_t job = 0;
+    for (uint64_t base = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kUnionRun;
+         base < E; base += warps * kUnionRun) {
+        uint32_t t = 0;
         if (lane == 0) {
-            uint32_t lo = 0, hi = n_jobs;   // the last job starting at or before base
+            uint32_t lo = 0, hi = n;   // the last job starting at or before base
             while (hi - lo > 1) {
                 const uint32_t mid = (lo + hi) >> 1;
-                if (starts[mid] <= base) lo = mid;
+                if (slots[mid] <= base) lo = mid;
                 else hi = mid;
             }
-            job = lo;
+            t = lo;
         }
-        job = __shfl_sync(0xFFFFFFFFu, job, 0);
-        const uint64_t e = base + lane;
-        if (e >= E) continue;
-        while (job + 1 < n_jobs && starts[job + 1] <= e) ++job;
-        const BatchJob& J = jobs[job];
-        const uint64_t local = e - J.out_edge;   // past the job's edges: an alignment gap
-        if (!J.want_csr || local >= J.edges) continue;
-        const uint64_t at = J.csr_edge + local;
-        if (PG_CHECK(at, H.csr_edges[0] + H.csr_edges[1])) {
-            P p = in[e];
-            p.x += (decltype(p.x))J.vbase;
-            out[at] = p;
+        t = __shfl_sync(0xFFFFFFFFu, t, 0);
+        P p[kUnionRun / 32];
+#pragma unroll
+        for (uint32_t u = 0; u < kUnionRun / 32; ++u) {
+            const uint64_t at = base + 32 * u + lane;
+            if (at >= E) break;
+            while (t + 1 < n && slots[t + 1] <= at) ++t;
+            const BatchJob& J = jobs[slot_jobs[t]];
+            const uint64_t local = at - J.csr_edge;
+            if (!PG_CHECK(local, J.edges)) break;
+            p[u] = in[J.out_edge + local];
+            p[u].x += (decltype(p[u].x))J.vbase;
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < kUnionRun / 32; ++u) {
+            const uint64_t at = base + 32 * u + lane;
+            if (at < E) out[at] = p[u];
         }
     }
 }
@@ -484,11 +496,13 @@ pg_status pg_batch_plan(const pg_job* jobs, uint32_t n_jobs, uint32_t tile_edges
     for (uint32_t i = 0; i < n_jobs; ++i)
         if (jobs[i].kind == PG_JOB_KRON && jobs[i].n0 > 2 && jobs[i].n0 <= 16)
             pool_entries += jobs[i].n0 * jobs[i].n0;
-    H.off_starts = H.off_pool + a16((size_t)pool_entries * 4);
-    H.off_rstart[0] = H.off_starts + a16((size_t)(n_jobs + 1) * 8);
+    H.off_slots = H.off_pool + a16((size_t)pool_entries * 4);
+    H.off_slot_jobs = H.off_slots + a16((size_t)(n_csr + 1) * 8);
+    H.off_rstart[0] = H.off_slot_jobs + a16((size_t)(n_csr + 1) * 4);
     H.off_rstart[1] = H.off_rstart[0] + a16((size_t)(n_csr + 1) * 8);
     H.off_two = H.off_rstart[1] + a16((size_t)(n_csr + 1) * 8);
-    uint64_t* starts = (uint64_t*)(base + H.off_starts);
+    uint64_t* slots = (uint64_t*)(base + H.off_slots);
+    uint32_t* slot_jobs = (uint32_t*)(base + H.off_slot_jobs);
     TwoPhaseJob* two = (TwoPhaseJob*)(base + H.off_two);
     uint64_t edges = 0, items = 0;
     uint32_t n_pool = 0;
@@ -565,7 +579,6 @@ pg_status pg_batch_plan(const pg_job* jobs, uint32_t n_jobs, uint32_t tile_edges
             return PG_EINVAL;
         }
         b.out_edge = edges;
-        starts[i] = edges;
         edges += b.edges;
         if (q.want_csr) b.want_csr = 1 + (q.kind == PG_JOB_KRON ? 1u : 0u);
         first[i] = (uint32_t)items;
@@ -574,7 +587,6 @@ pg_status pg_batch_plan(const pg_job* jobs, uint32_t n_jobs, uint32_t tile_edges
         if (h_edge_offsets) h_edge_offsets[i] = b.out_edge;
     }
     first[n_jobs] = (uint32_t)items;
-    starts[n_jobs] = edges;
     // the CSR groups: each job's rows in its group's union graph, then its
     // places in the output arenas (group 0's jobs first, in job order)
     for (uint32_t i = 0; i < n_jobs; ++i) {
@@ -597,12 +609,16 @@ pg_status pg_batch_plan(const pg_job* jobs, uint32_t n_jobs, uint32_t tile_edges
         uint64_t* rstart = (uint64_t*)(base + H.off_rstart[g]);
         J[i].csr_edge = col_base[g] + e_g[g];
         J[i].rbase = row_base[g] + J[i].vbase + t_g[g];
+        const uint64_t t = (g ? H.csr_jobs[0] : 0) + t_g[g];
+        slots[t] = J[i].csr_edge;
+        slot_jobs[t] = i;
         rstart[t_g[g]++] = J[i].rbase;
         e_g[g] += J[i].edges;
     }
     for (uint32_t g = 0; g < 2; ++g)
         ((uint64_t*)(base + H.off_rstart[g]))[H.csr_jobs[g]] =
             row_base[g] + H.csr_vertices[g] + H.csr_jobs[g];
+    slots[n_csr] = H.csr_edges[0] + H.csr_edges[1];
     H.n_items = items;
     H.total_edges = edges;
     H.n_pool = n_pool;
@@ -767,7 +783,7 @@ pg_status gen_batch_csr(const void* h_plan, const void* d_plan, uint32_t n_jobs,
     if (cudaMemsetAsync(wait, 0, 4, s) != cudaSuccess) return PG_ECUDA;
     if (cols > 0) {
         TraceScope trace("batch_csr_union", s);
-        const uint64_t warps = (H.total_edges + 31) / 32;
+        const uint64_t warps = (cols + kUnionRun - 1) / kUnionRun;
         const uint64_t full = (uint64_t)device_sm_count() * 8;
         const int grid = (int)(warps / 8 + 1 < full ? warps / 8 + 1 : full);
         if (w == PG_ID64)

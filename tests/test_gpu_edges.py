@@ -71,3 +71,28 @@ def test_batch_kronecker_tiles_at_odd_arena_edges(id64):
     for i, j in enumerate(jobs):
         assert np.array_equal(host(plan.edges_of(arena, i)),
                               o.kron(j["initiator"], j["k"], j["n_edges"], j["seed"])), i
+
+
+@pytest.mark.parametrize("id64", [False, True])
+def test_batch_csr_of_jobs_around_a_union_run(id64):
+    """CSR jobs of 0, 1 and about 128 edges (a warp's run of union slots),
+    between jobs without CSR."""
+    jobs = []
+    for i, E in enumerate([0, 1, 127, 128, 129, 0, 0, 300, 5, 2, 128]):
+        jobs.append(dict(kind="kron", initiator=W.KRON_INITIATOR, k=3 + i % 5, n_edges=E,
+                         seed=i, want_csr=True))
+        jobs.append(dict(kind="kron", initiator=W.KRON_INITIATOR, k=6, n_edges=777, seed=i + 50))
+        jobs.append(dict(kind="pba", n=E // 3, m=3, n0=4, seed=i, want_csr=i % 2 == 0))
+    plan = pg.BatchPlan(jobs, tile_edges=64, id64=id64)
+    arena = pg.gen_batch(plan)
+    rp, col = pg.gen_batch_csr(plan, arena, check=True)
+    torch.cuda.synchronize()
+    for i, j in enumerate(jobs):
+        if not j.get("want_csr"):
+            continue
+        edges = (o.kron(j["initiator"], j["k"], j["n_edges"], j["seed"]) if j["kind"] == "kron"
+                 else o.ba(j["n"], 3, 4, j["seed"]))
+        ref_rp, ref_col = o.csr(np.asarray(edges).astype(np.uint64), pg._job_vertices(j))
+        got_rp, got_col = plan.csr_of(rp, col, i)
+        assert np.array_equal(host(got_rp), ref_rp), i
+        assert np.array_equal(host(got_col), ref_col), i
