@@ -94,9 +94,8 @@ PbaGeom make_geom(uint64_t n_b, uint64_t N_e, uint32_t m, uint32_t B, uint32_t n
     g.coin_thr = coin_threshold(f);
     g.coin_on = (B > W && g.coin_thr > 0) ? 1 : 0;
     g.key = make_key(seed);
-    g.S = pba_segments(N_e, B, device_sm_count());
-    g.seg_len = pba_segment_length(N_e, g.S);
-    g.P = pba_prefix_len(N_e);
+    pba_set_segments(&g, pba_segment_length(N_e, B, device_sm_count(), false));
+    g.P = pba_prefix_len(N_e, B, device_sm_count());
     g.nb_shift = 0xFFFFFFFFu;
     if (n_b > 0 && (n_b & (n_b - 1)) == 0) {
         g.nb_shift = 0;
@@ -198,7 +197,8 @@ size_t pg_pba_workspace_size(uint64_t n, uint32_t m, uint32_t blocks)
     if (blocks <= 1) return 0;
     const PbaCheck c = check_pba(n, m, blocks, 2, blocks, 0.0, PG_ID64);
     if (c.st != PG_OK) return 0;
-    const uint32_t S = pba_segments(c.N_e, blocks, device_sm_count());
+    const uint32_t S =
+        pba_segments(c.N_e, pba_segment_length(c.N_e, blocks, device_sm_count(), false));
     return pba_workspace_layout((c.N_e + 7) & ~(uint64_t)7, blocks, S).total;
 }
 
@@ -401,9 +401,8 @@ pg_status gen_pba_to_host(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0,
     HostCopy hc = per_dev[dev];
     hc.h_edges = h_edges;
     // about one wave of emit CTAs per chunk
-    const uint64_t ctas_per_block = (g.S + 7) / 8;
-    const uint64_t wave = (uint64_t)device_sm_count() * 4;
-    uint64_t per = (wave + ctas_per_block - 1) / ctas_per_block;
+    const uint64_t wave = (uint64_t)device_sm_count() * 4 * 8;   // warps, one segment each
+    uint64_t per = (wave + g.S - 1) / g.S;
     uint64_t chunks = (blocks + per - 1) / per;
     if (chunks > kMaxCopyChunks) chunks = kMaxCopyChunks;
     if (chunks < 1) chunks = 1;

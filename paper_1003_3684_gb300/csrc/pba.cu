@@ -5,7 +5,8 @@
 // on one GPU, and every message becomes HBM traffic:
 //
 //   pba_prefix   phase 1, first P entries of every block's list A_p, built in
-//                shared memory level by level: entries [L, 2L) copy from
+//                shared memory by one CTA, level by level (the first one
+//                entry per thread): entries [L, 2L) copy from
 //                [0, L) (already final) or follow their own chain inside
 //                [L, 2L). Writes A_p[0, P) and counts it.
 //   pba_pass     phase 1, one level [L, hi) of every block per launch, with
@@ -20,6 +21,7 @@
 //                A_p in L2); a copy with r >= L follows r's own draw. Adds
 //                the counts of each (block, segment) -- the paper's count
 //                message -- into cnt.
+//                Graphs of few entries take fewer, faster-growing levels.
 //   pba_scan     exclusive scan of the counts over (requester, segment) per
 //                target block: R_q (how many endpoints q must produce) and
 //                where each requester segment's slice of q's list starts.
@@ -46,15 +48,24 @@
 namespace pgen {
 namespace {
 
-constexpr uint32_t kGranule = 16384;        // segment lengths are multiples of this
+constexpr uint32_t kGranule = 16384;        // levels of phase 1 start at multiples of this
+constexpr uint32_t kMinSegment = 512;       // shortest segment (two emit runs)
 constexpr uint32_t kPrefixMax = 6 * kGranule;   // phase-1 prefix built in smem (192 KB)
 constexpr int kPrefixThreads = 1024;
-constexpr int kPassThreads = 512;
-constexpr uint32_t kPassRun = 1024;             // entries per warp run in a pass
-constexpr uint32_t kPassChunk = (kPassThreads / 32) * kPassRun;   // 16384 per CTA
+// A pass CTA: 16 warps with runs of 1024 entries for levels that fill the GPU,
+// 8 warps with runs of 256 for shorter ones.
+template <bool kLarge>
+struct PassShape {
+    static constexpr int warps = kLarge ? 16 : 8;
+    static constexpr uint32_t run = kLarge ? 1024 : 256;
+    static constexpr uint32_t chunk = warps * run;   // 16384 or 2048 entries per CTA
+};
+constexpr uint32_t kHistWords = 8192;   // prefix: counters of the segments counted at once
 constexpr int kEmitWarps = 8;
 constexpr int kEmitThreads = kEmitWarps * 32;
 constexpr uint64_t kLevelDiv = 2;   // phase-1 level [L, L + L/kLevelDiv)
+constexpr uint32_t kPrefixFew = 8192;   // the prefix when blocks are few
+constexpr uint64_t kShortWaves = 8;     // see pba_segment_length
 constexpr int kEmitItems = 8;
 constexpr uint32_t kEmitRun = 32 * kEmitItems;                   // 256 entries per warp run
 constexpr uint32_t kMaxBlocks = 1024;
@@ -66,8 +77,10 @@ struct BaShape {   // 32 KB of staging for either id width
     static constexpr uint32_t tile = (kBaThreads / 32) * run;
 };
 
-static_assert(kPassChunk == kGranule, "a pass CTA covers one granule");
-static_assert(kGranule % kEmitRun == 0, "segments hold whole emit runs");
+static_assert(PassShape<true>::chunk == kGranule, "a large pass CTA covers one granule");
+static_assert(kGranule % PassShape<false>::chunk == 0, "small pass CTAs divide a granule");
+static_assert(kMinSegment % kEmitRun == 0, "segments hold whole emit runs");
+static_assert(PassShape<false>::run <= kMinSegment, "a small pass run lies in one segment");
 
 // Inter-faction pick: uniform over the B - W blocks outside [phi, phi + W).
 __device__ __forceinline__ uint32_t fresh_block(uint32_t w3, uint32_t B, uint32_t W,
@@ -130,11 +143,13 @@ __device__ __forceinline__ void flush_counts(const uint32_t* hist, uint32_t* cnt
 
 // ---------------------------------------------------------------------------
 // Phase 1, prefix [0, P) of each block, built in shared memory.
-// grid = B, block = kPrefixThreads, dynamic smem = P*2 (rounded to 16) + B*4.
+// grid = B, block = kPrefixThreads, dynamic smem = P*2 (rounded to 16) + the
+// counters of n_hist segments.
 // ---------------------------------------------------------------------------
 template <bool kTable>
 __global__ void __launch_bounds__(kPrefixThreads) pba_prefix_kernel(
-    const __grid_constant__ PbaGeom g, uint16_t* __restrict__ A, uint32_t* __restrict__ cnt)
+    const __grid_constant__ PbaGeom g, uint32_t n_hist, uint16_t* __restrict__ A,
+    uint32_t* __restrict__ cnt)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     uint16_t* sA = reinterpret_cast<uint16_t*>(smem);
@@ -147,7 +162,10 @@ __global__ void __launch_bounds__(kPrefixThreads) pba_prefix_kernel(
     for (uint32_t t = threadIdx.x; t < s; t += blockDim.x) sA[t] = (uint16_t)F.member(t);
     __syncthreads();
     for (uint32_t L = s; L < P;) {
-        const uint32_t hi = (2 * L < P) ? 2 * L : P;
+        // the first level is one entry per thread, whose chains run down to
+        // the list; each later one doubles the finished part
+        const uint32_t up = 2 * L > kPrefixThreads ? 2 * L : kPrefixThreads;
+        const uint32_t hi = up < P ? up : P;
         for (uint32_t j = L + threadIdx.x; j < hi; j += blockDim.x) {
             uint32_t cur = j, v;
             for (;;) {
@@ -170,36 +188,43 @@ __global__ void __launch_bounds__(kPrefixThreads) pba_prefix_kernel(
     }
     uint16_t* Ap = A + (uint64_t)p * g.A_stride;
     for (uint32_t t = threadIdx.x; t < P; t += blockDim.x) Ap[t] = sA[t];
-    // counts of the prefix, per segment it overlaps
-    for (uint32_t sgm = 0; (uint64_t)sgm * g.seg_len < P; ++sgm) {
-        const uint32_t a = (uint32_t)((uint64_t)sgm * g.seg_len);
-        const uint32_t b = (uint32_t)((a + g.seg_len < P) ? a + g.seg_len : P);
-        for (uint32_t t = threadIdx.x; t < g.B; t += blockDim.x) hist[t] = 0;
+    // counts of the prefix, n_hist of the segments it overlaps at a time
+    const uint32_t segs = (uint32_t)((P + g.seg_len - 1) / g.seg_len);
+    for (uint32_t s0 = 0; s0 < segs; s0 += n_hist) {
+        const uint32_t ns = segs - s0 < n_hist ? segs - s0 : n_hist;
+        const uint32_t a = (uint32_t)(s0 * g.seg_len);
+        const uint64_t b0 = (uint64_t)(s0 + ns) * g.seg_len;
+        const uint32_t b = b0 < P ? (uint32_t)b0 : P;
+        for (uint32_t t = threadIdx.x; t < ns * g.B; t += blockDim.x) hist[t] = 0;
         __syncthreads();
-        for (uint32_t t = a + threadIdx.x; t < b; t += blockDim.x)
-            if (PG_CHECK(sA[t], g.B)) atomicAdd(&hist[sA[t]], 1u);
+        for (uint32_t t = a + threadIdx.x; t < b; t += blockDim.x) {
+            const uint32_t at = g.seg_shift ? ((t - a) >> g.seg_shift) : 0u;
+            if (PG_CHECK(sA[t], g.B)) atomicAdd(&hist[at * g.B + sA[t]], 1u);
+        }
         __syncthreads();
-        flush_counts(hist, cnt, g, p, sgm);
+        for (uint32_t i = 0; i < ns; ++i) flush_counts(hist + i * g.B, cnt, g, p, s0 + i);
         __syncthreads();
     }
 }
 
 // ---------------------------------------------------------------------------
 // Phase 1, one level [L, hi) of every block; grid = (chunks, B),
-// chunk c = [L + c*kPassChunk, ...). dynamic smem = B*4 (histogram) + one
-// staged run of kPassRun entries per warp.
+// chunk c = [L + c*chunk, ...). dynamic smem = a histogram of B counters per
+// segment of the chunk (one when a segment holds the chunk) + one staged run
+// per warp.
 // A copy that lands below L loads A_p[r]; the load is consumed one loop trip
 // later (after the next Philox), so its latency overlaps arithmetic.
 // ---------------------------------------------------------------------------
-template <bool kTable>
-__global__ void __launch_bounds__(kPassThreads) pba_pass_kernel(const __grid_constant__ PbaGeom g,
-                                                                uint32_t L, uint32_t hi,
-                                                                uint16_t* __restrict__ A,
-                                                                uint32_t* __restrict__ cnt)
+template <bool kTable, bool kLarge>
+__global__ void __launch_bounds__(PassShape<kLarge>::warps * 32)
+    pba_pass_kernel(const __grid_constant__ PbaGeom g, uint32_t L, uint32_t hi, uint32_t n_hist,
+                    uint16_t* __restrict__ A, uint32_t* __restrict__ cnt)
 {
+    constexpr uint32_t kPassRun = PassShape<kLarge>::run, kPassChunk = PassShape<kLarge>::chunk;
     extern __shared__ __align__(16) unsigned char smem[];
-    uint32_t* hist = reinterpret_cast<uint32_t*>(smem);                              // B
-    uint16_t* stage = reinterpret_cast<uint16_t*>(smem + (((size_t)g.B * 4 + 15) & ~(size_t)15));
+    uint32_t* hist = reinterpret_cast<uint32_t*>(smem);                       // n_hist * B
+    uint16_t* stage =
+        reinterpret_cast<uint16_t*>(smem + (((size_t)n_hist * g.B * 4 + 15) & ~(size_t)15));
     const uint32_t p = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
@@ -207,8 +232,8 @@ __global__ void __launch_bounds__(kPassThreads) pba_pass_kernel(const __grid_con
     const PhiloxHead ph = philox_head(0u, p, 1u, g.key);   // counters (j, 0, p, 1)
     uint16_t* Ap = A + (uint64_t)p * g.A_stride;
     uint16_t* my = stage + wid * kPassRun;              // this warp's run, staged
-    const uint32_t chunk = L + blockIdx.x * kPassChunk;   // a granule: one segment
-    for (uint32_t t = threadIdx.x; t < g.B; t += blockDim.x) hist[t] = 0;
+    const uint32_t chunk = L + blockIdx.x * kPassChunk;
+    for (uint32_t t = threadIdx.x; t < n_hist * g.B; t += blockDim.x) hist[t] = 0;
     __syncthreads();
 
     const uint32_t run = chunk + wid * kPassRun;
@@ -219,7 +244,6 @@ __global__ void __launch_bounds__(kPassThreads) pba_pass_kernel(const __grid_con
     bool active = item < n_items;
     bool pend = false, pend_load = false;
     uint32_t pend_k = 0, pend_v = 0, lv = 0;
-    uint32_t own = 0;   // entries equal to p (the most frequent value) counted here
     // every lane draws (an idle lane's draw is discarded), so the trip is
     // straight-line code apart from the deferred store. A copy of the
     // finished prefix is loaded into lv and first read one trip later, by
@@ -253,11 +277,22 @@ __global__ void __launch_bounds__(kPassThreads) pba_pass_kernel(const __grid_con
     while (next < n_items) trip();
     while (__any_sync(0xFFFFFFFFu, active || pend)) trip();
     __syncwarp();
-    // counts of the finished run, outside the pooled loop (converged lanes)
-    for (uint32_t t = lane; t < n_items; t += 32) {
-        const uint32_t v = my[t];
-        if (v == p) ++own;
-        else if (PG_CHECK(v, g.B)) atomicAdd(&hist[v], 1u);
+    // counts of the finished run, outside the pooled loop (converged lanes);
+    // entries equal to p, the most frequent value, are counted in a register.
+    // A run of the large shape may hold two segments.
+    const uint32_t part = (kLarge && n_hist > 1 && g.seg_len < kPassRun) ? (uint32_t)g.seg_len
+                                                                        : kPassRun;
+    for (uint32_t t0 = 0; t0 < n_items; t0 += part) {
+        const uint32_t at = n_hist > 1 ? (wid * kPassRun + t0) >> g.seg_shift : 0u;
+        uint32_t* hs = hist + at * g.B;
+        const uint32_t t1 = t0 + part < n_items ? t0 + part : n_items;
+        uint32_t own = 0;
+        for (uint32_t t = t0 + lane; t < t1; t += 32) {
+            const uint32_t v = my[t];
+            if (v == p) ++own;
+            else if (PG_CHECK(v, g.B)) atomicAdd(&hs[v], 1u);
+        }
+        if (own) atomicAdd(&hs[p], own);
     }
     // the run back to A: 16-byte stores when the run is whole (run is a
     // multiple of 8 entries and rows are 16-byte aligned), marked streaming
@@ -270,9 +305,10 @@ __global__ void __launch_bounds__(kPassThreads) pba_pass_kernel(const __grid_con
     } else if (in_row) {
         for (uint32_t t = lane; t < n_items; t += 32) Ap[run + t] = my[t];
     }
-    if (own) atomicAdd(&hist[p], own);
     __syncthreads();
-    flush_counts(hist, cnt, g, p, (uint32_t)(chunk / g.seg_len));
+    const uint32_t s0 = (uint32_t)(chunk / g.seg_len);
+    for (uint32_t i = 0; i < n_hist && s0 + i < g.S; ++i)
+        flush_counts(hist + i * g.B, cnt, g, p, s0 + i);
 }
 
 // ---------------------------------------------------------------------------
@@ -313,8 +349,9 @@ __device__ __forceinline__ uint32_t sigma32(uint32_t x, const QRecip& c)
     return (uint32_t)(t1 >> 32) + x * c.C2;
 }
 
-__global__ void __launch_bounds__(1024) pba_scan_kernel(const uint32_t* __restrict__ cnt,
-                                                        uint64_t* __restrict__ off,
+// `in`: the counts themselves (off: another array), or chunk sums (in place).
+template <typename In>
+__global__ void __launch_bounds__(1024) pba_scan_kernel(const In* in, uint64_t* off,
                                                         uint64_t* __restrict__ R,
                                                         FastDiv* __restrict__ divR,
                                                         QRecip* __restrict__ recip, uint32_t nb,
@@ -327,40 +364,118 @@ __global__ void __launch_bounds__(1024) pba_scan_kernel(const uint32_t* __restri
     if (blockIdx.x == 0)
         for (uint32_t e = threadIdx.x; e < kSeedTab; e += blockDim.x)
             stab[e] = e < e0 ? seed_endpoint(e, 0, n0) | (seed_endpoint(e, 1, n0) << 16) : 0u;
-    __shared__ uint64_t part[32][33];
-    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t q = blockIdx.x * 32 + lane;
-    const uint32_t per = (rows + 31) / 32;
-    const uint32_t r0 = w * per;
+    // places: (row slab, target), consecutive threads on consecutive targets
+    __shared__ uint64_t part[1024];
+    const uint32_t lanes = B < 32 ? B : 32, slabs = blockDim.x / lanes;
+    const uint32_t slab = threadIdx.x / lanes;
+    const uint32_t q = blockIdx.x * lanes + threadIdx.x % lanes;
+    const bool in_use = q < B && slab < slabs;
+    const uint32_t per = (rows + slabs - 1) / slabs;
+    const uint32_t r0 = slab * per < rows ? slab * per : rows;
     const uint32_t r1 = (r0 + per < rows) ? r0 + per : rows;
     uint64_t sum = 0;
-    if (q < B)
-        for (uint32_t r = r0; r < r1; ++r) sum += cnt[(uint64_t)r * B + q];
-    part[w][lane] = sum;
+    if (in_use) {
+#pragma unroll 8
+        for (uint32_t r = r0; r < r1; ++r) sum += in[(uint64_t)r * B + q];
+    }
+    part[threadIdx.x] = sum;
     __syncthreads();
-    if (w == 0) {
-        uint64_t acc = 0;
-        for (int x = 0; x < 32; ++x) {
-            const uint64_t c = part[x][lane];
-            part[x][lane] = acc;
-            acc += c;
+    uint64_t acc = sum;   // inclusive over the slabs
+    for (uint32_t o = 1; o < slabs; o <<= 1) {
+        const uint64_t y = slab >= o ? part[threadIdx.x - o * lanes] : 0;
+        __syncthreads();
+        acc += y;
+        part[threadIdx.x] = acc;
+        __syncthreads();
+    }
+    if (!in_use) return;
+    if (slab + 1 == slabs) {
+        R[q] = acc;
+        divR[q] = make_fastdiv(acc > 0 ? acc : 1);
+        recip[q] = make_recip(acc, nb);
+        if (force_wide || acc + e0 >= ((uint64_t)1 << 32)) atomicOr(wide_flag, 1u);
+    }
+    acc -= sum;
+#pragma unroll 8
+    for (uint32_t r = r0; r < r1; ++r) {
+        const uint64_t c = in[(uint64_t)r * B + q];
+        off[(uint64_t)r * B + q] = acc;
+        acc += c;
+    }
+}
+
+// Many rows (2^30 vertices in 1024 blocks: 40,960 rows of 1024 targets, 0.379
+// -> 0.174 ms): the column scan in three steps, over chunks of kChunkRows rows
+// or more. A CTA owns one chunk; its threads take (row group, target) places,
+// consecutive threads on consecutive targets. Step 1 (kApply false) writes the
+// chunk's column sums, the kernel above scans them, and step 2 (kApply true)
+// turns them into every row's offsets. Bound by memory: 4 bytes read twice
+// and 8 written per (row, target).
+constexpr uint32_t kScanThreads = 256;
+constexpr uint32_t kChunkRows = 32;
+constexpr uint32_t kOneStepRows = 64;    // rows per thread up to which one launch scans them all
+template <bool kApply>
+__global__ void __launch_bounds__(kScanThreads) pba_chunk_kernel(const uint32_t* __restrict__ cnt,
+                                                                 uint64_t* __restrict__ sums,
+                                                                 uint64_t* __restrict__ off,
+                                                                 uint32_t B, uint32_t rows,
+                                                                 uint32_t chunk_rows)
+{
+    __shared__ uint64_t part[kScanThreads];
+    const uint32_t r0 = blockIdx.x * chunk_rows;
+    const uint32_t r1 = rows - r0 < chunk_rows ? rows : r0 + chunk_rows;
+    // row groups: several when there are fewer targets than threads
+    const uint32_t lanes = B < kScanThreads ? B : kScanThreads;
+    const uint32_t groups = kScanThreads / lanes;
+    const uint32_t grp = threadIdx.x / lanes;
+    const uint32_t per = (r1 - r0 + groups - 1) / groups;
+    uint32_t a = r0 + grp * per, b = a + per;
+    if (a > r1 || grp >= groups) a = r1;
+    if (b > r1 || grp >= groups) b = r1;
+    for (uint32_t q0 = 0; q0 < B; q0 += lanes) {
+        const uint32_t q = q0 + threadIdx.x % lanes;
+        const bool in = q < B;
+        uint64_t sum = 0;
+        if (in && (!kApply || groups > 1)) {
+#pragma unroll 8
+            for (uint32_t r = a; r < b; ++r) sum += cnt[(uint64_t)r * B + q];
         }
-        if (q < B) {
-            R[q] = acc;
-            divR[q] = make_fastdiv(acc > 0 ? acc : 1);
-            recip[q] = make_recip(acc, nb);
-            if (force_wide || acc + e0 >= ((uint64_t)1 << 32)) atomicOr(wide_flag, 1u);
+        if (groups > 1) {   // uniform; then one trip covers every target
+            part[threadIdx.x] = sum;
+            __syncthreads();
+            if (!kApply && grp == 0) {
+                for (uint32_t x = 1; x < groups; ++x) sum += part[x * lanes + q];
+            } else if (kApply) {
+                sum = 0;
+                for (uint32_t x = 0; x < grp && x < groups; ++x) sum += part[x * lanes + q];
+            }
+        }
+        if (!in) continue;
+        if (!kApply) {
+            if (grp == 0) sums[(uint64_t)blockIdx.x * B + q] = sum;
+        } else {
+            uint64_t acc = sums[(uint64_t)blockIdx.x * B + q] + sum;
+#pragma unroll 8
+            for (uint32_t r = a; r < b; ++r) {
+                const uint64_t c = cnt[(uint64_t)r * B + q];
+                off[(uint64_t)r * B + q] = acc;
+                acc += c;
+            }
         }
     }
-    __syncthreads();
-    if (q < B) {
-        uint64_t acc = part[w][lane];
-        for (uint32_t r = r0; r < r1; ++r) {
-            const uint64_t c = cnt[(uint64_t)r * B + q];
-            off[(uint64_t)r * B + q] = acc;
-            acc += c;
-        }
-    }
+}
+
+// Whether pba_scan_kernel alone scans the rows: one CTA per 32 targets, a
+// thread taking few enough rows.
+bool scan_in_one_step(uint64_t rows, uint32_t B)
+{
+    return rows <= kOneStepRows * (uint64_t)(1024 / (B < 32 ? B : 32));
+}
+
+uint32_t scan_chunk_rows(uint32_t B)
+{
+    const uint32_t rows = 16384 / B;
+    return rows > kChunkRows ? rows : kChunkRows;
 }
 
 // ---------------------------------------------------------------------------
@@ -597,7 +712,8 @@ __device__ __forceinline__ void emit_run(Id* out, uint64_t cap, uint64_t e_first
 
 // ---------------------------------------------------------------------------
 // Phase 2 + substitution + emission. Every warp owns one segment of one block
-// (grid = (ceil(S / kEmitWarps), B)) and walks it in runs of kEmitRun entries:
+// (warp i of the launch: segment i mod S of block block_off + i div S) and
+// walks it in runs of kEmitRun entries:
 //   rank   entry j gets i = (next unused slot of T_{A[j]} for this segment),
 //          by a warp match over 32 entries and per-warp cursors in smem;
 //   chain  the lanes resolve T_q[i] for the run's entries, pooled;
@@ -625,16 +741,23 @@ __global__ void __launch_bounds__(kEmitThreads) pba_emit_kernel(
     const uint64_t* __restrict__ off, const uint64_t* __restrict__ R,
     const FastDiv* __restrict__ divR, const QRecip* __restrict__ recip,
     const uint32_t* __restrict__ wide_flag, const uint32_t* __restrict__ stab,
-    Id* __restrict__ out, uint32_t block_off, uint32_t out_block0, uint64_t out_cap)
+    Id* __restrict__ out, uint32_t block_off, uint32_t n_blocks, uint32_t out_block0,
+    uint64_t out_cap)
 {
     constexpr bool kFast = kMode != 0;
     using CurT = typename std::conditional<kFast, uint32_t, uint64_t>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if ((*wide_flag == 0) != kFast) return;   // the other variant does the work
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint32_t p = blockIdx.y + block_off;
-    const uint32_t sw = blockIdx.x * kEmitWarps + wid;
-    if (sw >= g.S) return;                   // no block-wide barrier follows
+    // gridDim.y is n_blocks when a block's segments fill whole CTAs (or there
+    // is one block); otherwise the warps of all blocks are numbered through
+    uint32_t sw = blockIdx.x * kEmitWarps + wid, b = blockIdx.y;
+    if (gridDim.y != n_blocks) {
+        b = sw / g.S;
+        sw -= b * g.S;
+    }
+    if (b >= n_blocks || sw >= g.S) return;  // no block-wide barrier follows
+    const uint32_t p = b + block_off;
     EmitWarpSmem<CurT>& ws = reinterpret_cast<EmitWarpSmem<CurT>*>(smem_raw)[wid];
     const uint32_t B = g.B;
     const uint32_t lt = (1u << lane) - 1u;
@@ -870,28 +993,65 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 PG_CHECK_UNIT(pba)
 
-uint32_t pba_prefix_len(uint64_t N_e) { return (uint32_t)(N_e < kPrefixMax ? N_e : kPrefixMax); }
-
-uint32_t pba_segments(uint64_t N_e, uint32_t B, int sm_count)
+// The phase-1 prefix built by one CTA per block. Blocks enough to fill the
+// GPU twice: as much as shared memory holds. Fewer blocks leave SMs idle
+// meanwhile, so the passes take over early: at a sixteenth of the list (two
+// levels growing fourfold), between kSmallChunk and kPrefixFew entries. 2^24
+// vertices in 64 blocks: prefix 0.144 -> 0.023 ms, passes 0.529 -> 0.534 ms;
+// 160,000 in 16 blocks: 0.064 -> 0.019 ms and two passes of 0.021 ms.
+uint32_t pba_prefix_len(uint64_t N_e, uint32_t B, int sm_count)
 {
-    // about eight waves of warps (32 resident per SM), each warp one segment;
-    // a multiple of kEmitWarps segments per block when the entries allow
-    const uint64_t target = 8ull * 32ull * (uint64_t)(sm_count > 0 ? sm_count : 1);
-    uint64_t S = (target + B - 1) / B;
+    constexpr uint64_t kSmallChunk = PassShape<false>::chunk;
+    uint64_t P = kPrefixMax;
+    if (B < 2 * (uint32_t)(sm_count > 0 ? sm_count : 1)) {
+        P = (N_e / 16 + kSmallChunk - 1) / kSmallChunk * kSmallChunk;
+        P = P < kSmallChunk ? kSmallChunk : P > kPrefixFew ? kPrefixFew : P;
+    }
+    return (uint32_t)(N_e < P ? N_e : P);
+}
+
+// Entries per segment (one emit warp each). Large graphs: about eight waves
+// of warps (32 resident per SM), in whole granules. Graphs that would give
+// fewer than kShortWaves waves that way: the power of two that does, at least
+// kMinSegment and 2 B entries (a segment costs a row of B counters and B
+// offsets). `coarse`: whole granules whatever the size, which makes the
+// smallest workspace. Measured (GB300, pba_emit): 160,000 vertices in 16
+// blocks, m = 4, in segments of 512 instead of 16384: 0.423 -> 0.028 ms (48
+// warps before); 2^24 vertices in 64 blocks, m = 5, in segments of 4096:
+// 1.166 -> 0.902 ms (5120 warps, just over one wave, before; with waves for
+// kShortWaves = 2, 4: 1.118, 0.964 ms).
+uint64_t pba_segment_length(uint64_t N_e, uint32_t B, int sm_count, bool coarse)
+{
+    const uint64_t sms = (uint64_t)(sm_count > 0 ? sm_count : 1);
+    const uint64_t short_len = N_e * B / (kShortWaves * 32ull * sms);
+    if (!coarse && short_len < kGranule) {
+        uint64_t len = kMinSegment;
+        while (len < kGranule && (len < 2 * (uint64_t)B || len < short_len)) len *= 2;
+        return len;
+    }
+    uint64_t S = (8ull * 32ull * sms + B - 1) / B;
     S = (S + kEmitWarps - 1) / kEmitWarps * kEmitWarps;
     const uint64_t max_s = (N_e + kGranule - 1) / kGranule;
     if (S > max_s) S = max_s;
     if (S < 1) S = 1;
-    const uint64_t len = pba_segment_length(N_e, (uint32_t)S);
-    const uint64_t used = (N_e + len - 1) / len;
+    const uint64_t per = (N_e + S - 1) / S;
+    const uint64_t len = (per + kGranule - 1) / kGranule * kGranule;
+    return len ? len : kGranule;
+}
+
+uint32_t pba_segments(uint64_t N_e, uint64_t seg_len)
+{
+    const uint64_t used = (N_e + seg_len - 1) / seg_len;
     return (uint32_t)(used > 0 ? used : 1);
 }
 
-uint64_t pba_segment_length(uint64_t N_e, uint32_t S)
+void pba_set_segments(PbaGeom* g, uint64_t seg_len)
 {
-    const uint64_t per = (N_e + S - 1) / (S ? S : 1);
-    uint64_t len = (per + kGranule - 1) / kGranule * kGranule;
-    return len ? len : kGranule;
+    g->seg_len = seg_len;
+    g->S = pba_segments(g->N_e, seg_len);
+    g->seg_shift = 0;
+    if (seg_len < kGranule)
+        while (((uint64_t)1 << g->seg_shift) < seg_len) ++g->seg_shift;
 }
 
 PbaWorkspace pba_workspace_layout(uint64_t A_stride, uint32_t B, uint32_t S)
@@ -914,6 +1074,12 @@ PbaWorkspace pba_workspace_layout(uint64_t A_stride, uint32_t B, uint32_t S)
     o += 256;
     w.off_stab = o;
     o += align256(kSeedTab * 4);
+    w.off_sums = o;
+    const uint64_t rows = (uint64_t)B * S;
+    if (!scan_in_one_step(rows, B)) {
+        const uint32_t per = scan_chunk_rows(B);
+        o += align256((size_t)((rows + per - 1) / per) * B * 8);
+    }
     w.total = o;
     return w;
 }
@@ -964,6 +1130,7 @@ struct PbaBuffers {
     QRecip* recip;
     uint32_t* wide;
     uint32_t* stab;
+    uint64_t* sums;
 };
 
 PbaBuffers pba_buffers(const PbaGeom& g, void* d_ws)
@@ -973,7 +1140,8 @@ PbaBuffers pba_buffers(const PbaGeom& g, void* d_ws)
     return PbaBuffers{(uint16_t*)(ws + L.off_A), (uint32_t*)(ws + L.off_cnt),
                       (uint64_t*)(ws + L.off_off), (uint64_t*)(ws + L.off_R),
                       (FastDiv*)(ws + L.off_magic), (QRecip*)(ws + L.off_recip),
-                      (uint32_t*)(ws + L.off_flag), (uint32_t*)(ws + L.off_stab)};
+                      (uint32_t*)(ws + L.off_flag), (uint32_t*)(ws + L.off_stab),
+                      (uint64_t*)(ws + L.off_sums)};
 }
 
 constexpr size_t kSmemFast = kEmitWarps * sizeof(EmitWarpSmem<uint32_t>);
@@ -992,12 +1160,18 @@ PerDeviceOnce g_pba_attrs;
 cudaError_t set_pba_attributes()
 {
     return g_pba_attrs.run_current([] {
-        const int prefix = (int)(kPrefixMax * 2 + kMaxBlocks * 4);
+        const int prefix = (int)(kPrefixMax * 2 + kHistWords * 4);
+        // a chunk's segments hold 2 B entries or more, so at most 32 KB of counters
+        const int pass = (int)(PassShape<true>::chunk * 4);
         return first_error({
             cudaFuncSetAttribute(pba_prefix_kernel<false>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, prefix),
             cudaFuncSetAttribute(pba_prefix_kernel<true>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, prefix),
+            cudaFuncSetAttribute(pba_pass_kernel<false, true>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, pass),
+            cudaFuncSetAttribute(pba_pass_kernel<true, true>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, pass),
             cudaFuncSetAttribute(pba_emit_kernel<uint32_t, 2>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFast),
             cudaFuncSetAttribute(pba_emit_kernel<uint64_t, 2>,
@@ -1015,6 +1189,29 @@ cudaError_t set_pba_attributes()
 
 }  // namespace
 
+namespace {
+
+template <bool kLarge>
+cudaError_t launch_pass(const PbaGeom& g, uint64_t lvl, uint64_t hi, const PbaBuffers& W,
+                        cudaStream_t s)
+{
+    using Shape = PassShape<kLarge>;
+    // segments in a chunk (seg_shift: shorter than a granule, a power of two)
+    const uint32_t nh = g.seg_shift && g.seg_len < Shape::chunk
+                            ? (uint32_t)(Shape::chunk / g.seg_len) : 1u;
+    const uint32_t chunks = (uint32_t)((hi - lvl + Shape::chunk - 1) / Shape::chunk);
+    const size_t smem = (((size_t)nh * g.B * 4 + 15) & ~(size_t)15) + (size_t)Shape::chunk * 2;
+    if (g.ftab)
+        { pba_pass_kernel<true, kLarge><<<dim3(chunks, g.B), Shape::warps * 32, smem, s>>>(
+            g, (uint32_t)lvl, (uint32_t)hi, nh, W.A, W.cnt); note_launch(); }
+    else
+        { pba_pass_kernel<false, kLarge><<<dim3(chunks, g.B), Shape::warps * 32, smem, s>>>(
+            g, (uint32_t)lvl, (uint32_t)hi, nh, W.A, W.cnt); note_launch(); }
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 // Phase 1, counts and their scan: everything the emission of any block
 // range reads, left in the workspace.
 cudaError_t launch_pba_phase1(const PbaGeom& g, void* d_ws, cudaStream_t s)
@@ -1028,37 +1225,51 @@ cudaError_t launch_pba_phase1(const PbaGeom& g, void* d_ws, cudaStream_t s)
     if (g.N_e > 0) {
         {
             TraceScope trace("pba_prefix", s);
-            const size_t smem = ((size_t)g.P * 2 + 15) / 16 * 16 + (size_t)g.B * 4;
+            const uint32_t segs = (uint32_t)((g.P + g.seg_len - 1) / g.seg_len);
+            uint32_t nh = kHistWords / g.B;
+            if (nh > segs) nh = segs;
+            if (nh < 1 || g.seg_shift == 0) nh = 1;
+            const size_t smem = ((size_t)g.P * 2 + 15) / 16 * 16 + (size_t)nh * g.B * 4;
             if (g.ftab)
-                { pba_prefix_kernel<true><<<g.B, kPrefixThreads, smem, s>>>(g, W.A, W.cnt); note_launch(); }
+                { pba_prefix_kernel<true><<<g.B, kPrefixThreads, smem, s>>>(g, nh, W.A, W.cnt); note_launch(); }
             else
-                { pba_prefix_kernel<false><<<g.B, kPrefixThreads, smem, s>>>(g, W.A, W.cnt); note_launch(); }
+                { pba_prefix_kernel<false><<<g.B, kPrefixThreads, smem, s>>>(g, nh, W.A, W.cnt); note_launch(); }
         }
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         TraceScope trace("pba_phase1", s);
+        // a level that fills the GPU with large CTAs (four fit an SM) takes those
+        const uint64_t wave = (uint64_t)device_sm_count() * 4 * PassShape<true>::chunk;
         for (uint64_t lvl = g.P; lvl < g.N_e;) {
-            // level [lvl, hi): lvl / kLevelDiv more entries, in whole granules
-            const uint64_t grow = (lvl / kLevelDiv + kPassChunk - 1) / kPassChunk * kPassChunk;
-            const uint64_t hi = (lvl + grow < g.N_e) ? lvl + grow : g.N_e;
-            const uint32_t chunks = (uint32_t)((hi - lvl + kPassChunk - 1) / kPassChunk);
-            const size_t smem = (((size_t)g.B * 4 + 15) & ~(size_t)15) +
-                                (size_t)(kPassThreads / 32) * kPassRun * 2;
-            if (g.ftab)
-                { pba_pass_kernel<true><<<dim3(chunks, g.B), kPassThreads, smem, s>>>(
-                    g, (uint32_t)lvl, (uint32_t)hi, W.A, W.cnt); note_launch(); }
-            else
-                { pba_pass_kernel<false><<<dim3(chunks, g.B), kPassThreads, smem, s>>>(
-                    g, (uint32_t)lvl, (uint32_t)hi, W.A, W.cnt); note_launch(); }
-            if ((err = cudaGetLastError()) != cudaSuccess) return err;
+            // level [lvl, hi), in whole granules. While the finished part is
+            // small a launch costs more than longer chains do, so levels grow
+            // fourfold up to a tenth of a wave and twofold up to one, then by
+            // lvl / kLevelDiv; a short rest joins the last level
+            const uint64_t done = lvl * g.B;
+            const uint64_t more = done < wave / 10 ? 3 * lvl : done < wave ? lvl : lvl / kLevelDiv;
+            const uint64_t end = (lvl + more + kGranule - 1) / kGranule * kGranule;
+            const uint64_t hi = (done < wave ? end + end / 4 : end) < g.N_e ? end : g.N_e;
+            const bool large = (hi - lvl) * g.B >= wave && lvl % kGranule == 0;
+            err = large ? launch_pass<true>(g, lvl, hi, W, s) : launch_pass<false>(g, lvl, hi, W, s);
+            if (err != cudaSuccess) return err;
             lvl = hi;
         }
     }
     {
         TraceScope trace("pba_scan", s);
-        { pba_scan_kernel<<<(g.B + 31) / 32, 1024, 0, s>>>(W.cnt, W.off, W.R, W.divR, W.recip,
-                                                          (uint32_t)g.n_b, g.B, g.B * g.S, g.e0,
-                                                          wide_path_forced() ? 1u : 0u, W.wide,
-                                                          g.n0, W.stab); note_launch(); }
+        const uint32_t rows = g.B * g.S, fw = wide_path_forced() ? 1u : 0u;
+        const uint32_t qs = g.B < 32 ? 1 : (g.B + 31) / 32, nb = (uint32_t)g.n_b;
+        if (scan_in_one_step(rows, g.B)) {
+            { pba_scan_kernel<uint32_t><<<qs, 1024, 0, s>>>(W.cnt, W.off, W.R, W.divR, W.recip, nb, g.B,
+                                                           rows, g.e0, fw, W.wide, g.n0, W.stab); note_launch(); }
+        } else {
+            const uint32_t per = scan_chunk_rows(g.B), chunks = (rows + per - 1) / per;
+            { pba_chunk_kernel<false><<<chunks, kScanThreads, 0, s>>>(W.cnt, W.sums, W.off, g.B, rows,
+                                                                     per); note_launch(); }
+            { pba_scan_kernel<uint64_t><<<qs, 1024, 0, s>>>(W.sums, W.sums, W.R, W.divR, W.recip, nb, g.B,
+                                                           chunks, g.e0, fw, W.wide, g.n0, W.stab); note_launch(); }
+            { pba_chunk_kernel<true><<<chunks, kScanThreads, 0, s>>>(W.cnt, W.sums, W.off, g.B, rows,
+                                                                    per); note_launch(); }
+        }
     }
     return cudaGetLastError();
 }
@@ -1084,34 +1295,35 @@ cudaError_t launch_pba_emit(const PbaGeom& g, int id64, void* d_out, const void*
     const size_t pair = id64 ? 16 : 8;
     for (uint32_t b0 = b_begin, c = 0; b0 < b_end; b0 += per, ++c) {
         const uint32_t nb = (b_end - b0 < per) ? b_end - b0 : per;
-        const dim3 grid((g.S + kEmitWarps - 1) / kEmitWarps, nb);
+        const dim3 grid = g.S % kEmitWarps == 0 ? dim3(g.S / kEmitWarps, nb)
+                                                : dim3((nb * g.S + kEmitWarps - 1) / kEmitWarps);
         {
             TraceScope trace("pba_emit", s);
             if (id64) {
                 if (lean)
                     { pba_emit_kernel<uint64_t, 2><<<grid, kEmitThreads, kSmemFast, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint64_t*)d_out, b0, b_begin,
+                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint64_t*)d_out, b0, nb, b_begin,
                         out_cap); note_launch(); }
                 else
                     { pba_emit_kernel<uint64_t, 1><<<grid, kEmitThreads, kSmemFast, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint64_t*)d_out, b0, b_begin,
+                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint64_t*)d_out, b0, nb, b_begin,
                         out_cap); note_launch(); }
                 if (!surely_fast)
                     { pba_emit_kernel<uint64_t, 0><<<grid, kEmitThreads, kSmemWide, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint64_t*)d_out, b0, b_begin,
+                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint64_t*)d_out, b0, nb, b_begin,
                         out_cap); note_launch(); }
             } else {
                 if (lean)
                     { pba_emit_kernel<uint32_t, 2><<<grid, kEmitThreads, kSmemFast, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint32_t*)d_out, b0, b_begin,
+                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint32_t*)d_out, b0, nb, b_begin,
                         out_cap); note_launch(); }
                 else
                     { pba_emit_kernel<uint32_t, 1><<<grid, kEmitThreads, kSmemFast, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint32_t*)d_out, b0, b_begin,
+                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint32_t*)d_out, b0, nb, b_begin,
                         out_cap); note_launch(); }
                 if (!surely_fast)
                     { pba_emit_kernel<uint32_t, 0><<<grid, kEmitThreads, kSmemWide, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint32_t*)d_out, b0, b_begin,
+                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint32_t*)d_out, b0, nb, b_begin,
                         out_cap); note_launch(); }
             }
         }

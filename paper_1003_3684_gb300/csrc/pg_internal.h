@@ -109,7 +109,8 @@ struct PbaGeom {
     uint32_t coin_on, coin_thr;    // inter-faction coin: w2 < coin_thr
     Key key;
     uint32_t S;                    // segments per block (one emit warp each)
-    uint64_t seg_len;              // entries per segment (a multiple of 16384)
+    uint64_t seg_len;              // entries per segment: a multiple of 16384, or 2^seg_shift
+    uint32_t seg_shift;            // log2(seg_len) when that is below 16384, else 0
     uint32_t P;                    // phase-1 prefix kept in shared memory
     uint32_t nb_shift;             // log2(n_b) when n_b is a power of two, else 0xffffffff
     uint64_t lean_add;             // (n_b - 1) + e0 * n_b when n_b is a power of two
@@ -127,12 +128,13 @@ constexpr uint32_t kFacStride = kFacHeader + 2 * kFacSlots;
 
 // Workspace layout for B > 1 (all offsets 256-byte aligned).
 struct PbaWorkspace {
-    size_t off_A, off_cnt, off_off, off_R, off_magic, off_recip, off_flag, off_stab, total;
+    size_t off_A, off_cnt, off_off, off_R, off_magic, off_recip, off_flag, off_stab, off_sums, total;
 };
 PbaWorkspace pba_workspace_layout(uint64_t A_stride, uint32_t B, uint32_t S);
-uint32_t pba_segments(uint64_t N_e, uint32_t B, int sm_count);
-uint32_t pba_prefix_len(uint64_t N_e);
-uint64_t pba_segment_length(uint64_t N_e, uint32_t S);
+uint32_t pba_segments(uint64_t N_e, uint64_t seg_len);
+uint32_t pba_prefix_len(uint64_t N_e, uint32_t B, int sm_count);
+uint64_t pba_segment_length(uint64_t N_e, uint32_t B, int sm_count, bool coarse);
+void pba_set_segments(PbaGeom* g, uint64_t seg_len);
 
 void set_wide_path_forced(bool on);
 bool wide_path_forced();

@@ -96,3 +96,53 @@ def test_batch_csr_of_jobs_around_a_union_run(id64):
         got_rp, got_col = plan.csr_of(rp, col, i)
         assert np.array_equal(host(got_rp), ref_rp), i
         assert np.array_equal(host(got_col), ref_col), i
+
+
+@pytest.mark.parametrize("B,n_b,m,Wf,f,n0,id64", [
+    (2, 512, 1, 1, 0.2, 2, False),         # one segment of 512 entries, exactly
+    (3, 513, 1, 1, 0.2, 3, False),         # a second segment of one entry
+    (7, 2049, 1, 1, 0.1, 2, True),         # one entry past the prefix
+    (5, 8192, 1, 5, 0.0, 2, False),        # every block in one faction, one level
+    (130, 1700, 5, 2, 0.1, 6, False),      # segments longer than 512 (2 B entries)
+    (300, 400, 5, 1, 0.3, 6, False),       # 2000 entries per block, uneven segments
+    (31, 9001, 3, 1, 0.1, 4, False),       # 31 targets: fewer than a warp's lanes
+    (33, 9001, 3, 1, 0.1, 4, True),        # two CTAs of targets in the scan
+    (256, 2**14, 5, 1, 0.1, 6, False),     # short segments under a large pass
+    (320, 20_011, 5, 1, 0.1, 6, False),    # one level past the long prefix
+])
+def test_pba_segments(B, n_b, m, Wf, f, n0, id64):
+    n = B * n_b
+    got = pg.gen_pba(n, m, B, n0, Wf, f, 77, id64=id64)
+    ref = o.pba(n, m, B, n0, Wf, f, 77)[0]
+    assert np.array_equal(host(got), np.asarray(ref).astype(np.uint64))
+
+
+@pytest.mark.parametrize("b_begin,b_end", [(0, 7), (3, 4), (6, 7), (2, 5)])
+def test_pba_block_ranges_with_segments_that_do_not_fill_a_cta(b_begin, b_end):
+    B, n_b, m, n0, seed = 7, 1111, 3, 4, 5
+    ref = np.asarray(o.pba(B * n_b, m, B, n0, 1, 0.1, seed)[0]).astype(np.uint64)
+    ws = pg.pg_pba_prepare(B * n_b, m, B, n0, seed=seed)
+    part = pg.gen_pba_blocks(ws, B * n_b, m, B, b_begin, b_end, n0=n0, seed=seed)
+    per = ref.shape[0] // B
+    assert np.array_equal(host(part), ref[b_begin * per:b_end * per])
+
+
+def test_noalloc_takes_a_graph_whose_smallest_workspace_fits():
+    """The workspace of short segments exceeds the fixed scratch; that of
+    whole granules does not."""
+    import ctypes as C
+    L = pg.lib()
+    L.gen_pba_noalloc.argtypes = [C.c_uint64, C.c_uint32, C.c_uint32, C.c_uint32, C.c_uint32,
+                                  C.c_double, C.c_uint64, C.c_int, C.c_void_p, C.c_uint64,
+                                  C.POINTER(C.c_uint64), C.c_void_p]
+    L.pg_pba_noalloc_scratch_bytes.restype = C.c_size_t
+    B, n_b, m = 16, 193_750, 5
+    n = B * n_b
+    assert pg.pg_pba_workspace_size(n, m, B) > L.pg_pba_noalloc_scratch_bytes()
+    E = pg.pg_pba_edge_count(n, m, B, 6)
+    out = torch.full((E, 2), -1, dtype=torch.int32, device="cuda")
+    cnt = C.c_uint64(0)
+    st = L.gen_pba_noalloc(n, m, B, 6, 1, 0.1, 3, 0, C.c_void_p(out.data_ptr()), E, C.byref(cnt),
+                           C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == pg.PG_OK and cnt.value == E
+    assert torch.equal(out, pg.gen_pba(n, m, B, 6, 1, 0.1, 3))
