@@ -39,6 +39,7 @@ namespace pgen {
 namespace {
 
 constexpr int kSortWarps = 16;
+constexpr int kFly = 2;   // items a warp ranks at a time
 constexpr int kSortThreads = kSortWarps * 32;
 constexpr int kMaxDigitBits = 8;
 constexpr uint32_t kMaxBuckets = 1u << kMaxDigitBits;
@@ -164,7 +165,11 @@ CsrWaitHook csr_wait_hook() { return CsrWaitHook{g_hook_spin.load(), g_hook_with
 // from a ticket, so every earlier tile belongs to a CTA already running or
 // done. It publishes its own counts before it waits on anything, and it sums
 // earlier tiles' counts, kLookWindow at a time, until it meets an inclusive
-// one. The look-back runs after the reorder, when the tile's pairs no longer
+// one. Bound by the shared-memory pipe (about 36 wavefronts per 32 pairs at 70 %
+// of its rate); two items in flight and one table lookup per pair in the
+// reorder took k = 20 (2^24 pairs, 5 passes) from 0.645 to 0.577 ms and
+// k = 26 (2^30 pairs, 7 passes) from 44.3 to 40.3 ms (four items in flight:
+// 0.611, 43.0; peers of some items by match.any: no better). The look-back runs after the reorder, when the tile's pairs no longer
 // occupy registers. Every poll loop is bounded: after spin_limit polls of
 // one word (kSpinLimit unless a test hook shortened it) it sets *err and
 // goes on with the partial sum, which can only be too small, so every write
@@ -212,64 +217,68 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     }
     __syncthreads();
     const uint32_t lt = (1u << lane) - 1u;
-    // item r of every lane, in lane order: the lanes holding equal digits
-    // find each other through a word per digit (each ORs in its lane bit,
-    // then all read the word back and clear it; the word table is the
-    // reorder buffer, unused until the ranks are done, one kMaxBuckets-word
-    // slab per warp); the lowest lane of each group reads and advances the
-    // warp's counter, the group gets the old value by shuffle; the counter
-    // is touched by one thread per group and the syncwarp orders it before
-    // the next item's read
-    uint32_t* pmask = reinterpret_cast<uint32_t*>(buf) + wid * kMaxBuckets;
-    for (uint32_t d = lane; d < nb; d += 32) pmask[d] = 0;
+    // kFly items of every lane at a time, in lane order within an item: the
+    // lanes holding equal digits of an item find each other through a word per
+    // digit (each ORs in its lane bit, then all read the word back and clear
+    // it; every item in flight has its own table of kMaxBuckets words per
+    // warp, in the reorder buffer, unused until the ranks are done). Then, item
+    // by item, the lowest lane of each group adds the group's size to the
+    // warp's counter of the digit (two 16-bit counters per word) and the group
+    // gets the old value by shuffle. A warp's shared-memory operations execute
+    // in order, so the adds of the items in flight need no wait between them.
+    uint32_t* pmask = reinterpret_cast<uint32_t*>(buf) + wid * (kFly * kMaxBuckets);
+    for (uint32_t t = lane; t < kFly * kMaxBuckets / 4; t += 32)
+        reinterpret_cast<uint4*>(pmask)[t] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
+    uint32_t* wc = reinterpret_cast<uint32_t*>(wcnt[wid]);
 #pragma unroll
-    for (int r = 0; r < kItems; ++r) {
-        const uint32_t t = wbase + r * 32 + lane;
-        const bool valid = t < n;
-        const uint32_t d = valid ? digit_of(e[r], field, shift, mask, nd) : 0xFFFFFFFFu;
-        if (valid) atomicOr(&pmask[d], 1u << lane);
-        __syncwarp();
-        const uint32_t peers = valid ? pmask[d] : 0u;
-        __syncwarp();
-        if (valid) pmask[d] = 0;
-        const uint32_t leader = __ffs(peers) - 1;
-        uint32_t prev = 0;
-        if (lane == leader && d != 0xFFFFFFFFu) {
-            prev = wcnt[wid][d];
-            wcnt[wid][d] = (uint16_t)(prev + __popc(peers));
+    for (int r0 = 0; r0 < kItems; r0 += kFly) {
+        uint32_t d[kFly], peers[kFly], prev[kFly];
+#pragma unroll
+        for (int u = 0; u < kFly; ++u) {
+            const uint32_t t = wbase + (r0 + u) * 32 + lane;
+            d[u] = t < n ? digit_of(e[r0 + u], field, shift, mask, nd) : 0xFFFFFFFFu;
+            if (d[u] != 0xFFFFFFFFu) atomicOr(&pmask[u * kMaxBuckets + d[u]], 1u << lane);
         }
-        prev = __shfl_sync(0xFFFFFFFFu, prev, leader);
         __syncwarp();
-        const uint32_t rank = prev + __popc(peers & lt);
-        if (r & 1) rk[r >> 1] |= rank << 16;
-        else rk[r >> 1] = rank;
+#pragma unroll
+        for (int u = 0; u < kFly; ++u)
+            peers[u] = d[u] != 0xFFFFFFFFu ? pmask[u * kMaxBuckets + d[u]] : 0u;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < kFly; ++u) {
+            if (d[u] != 0xFFFFFFFFu) pmask[u * kMaxBuckets + d[u]] = 0;
+            prev[u] = 0;
+            if (peers[u] != 0 && (peers[u] & lt) == 0) {
+                const uint32_t sh = (d[u] & 1) * 16;
+                prev[u] = (atomicAdd(&wc[d[u] >> 1], __popc(peers[u]) << sh) >> sh) & 0xFFFFu;
+            }
+            __syncwarp();
+        }
+#pragma unroll
+        for (int u = 0; u < kFly; ++u) {
+            const uint32_t rank = __shfl_sync(0xFFFFFFFFu, prev[u], __ffs(peers[u]) - 1) +
+                                  __popc(peers[u] & lt);
+            const int r = r0 + u;
+            if (r & 1) rk[r >> 1] |= rank << 16;
+            else rk[r >> 1] = rank;
+        }
     }
     __syncthreads();
-    // per digit: prefix over warps (in wcnt) and the tile total (in loff),
-    // published at once so that later tiles can sum it
+    // per digit (one thread each): the tile total, published at once so that
+    // later tiles can sum it; where the digit's run starts in the sorted tile
+    // (loff), and where each warp's part of the run does (in wcnt)
     const unsigned long long tag = (unsigned long long)(pass + 1) << kPassShift;
     volatile unsigned long long* st = status + (uint64_t)tile * nb;
-    for (uint32_t d = threadIdx.x; d < nb; d += blockDim.x) {
-        uint32_t acc = 0;
-#pragma unroll
-        for (int w = 0; w < kSortWarps; ++w) {
-            const uint32_t c = wcnt[w][d];
-            wcnt[w][d] = (uint16_t)acc;
-            acc += c;
-        }
-        loff[d] = acc;
-        if (tile != withhold) st[d] = tag | (tile == 0 ? kInc : kAgg) | acc;
-    }
-    __syncthreads();
-    // exclusive scan of the tile totals over digits (each thread a run of digits)
     {
-        const uint32_t per = (nb + blockDim.x - 1) / blockDim.x;
-        const uint32_t d0 = threadIdx.x * per;
-        uint32_t sum = 0;
-        for (uint32_t d = d0; d < d0 + per && d < nb; ++d) sum += loff[d];
-        // warp inclusive scan of the run sums, then across warps
-        uint32_t x = sum;
+        const uint32_t d = threadIdx.x;
+        uint32_t acc = 0;
+        if (d < nb) {
+#pragma unroll
+            for (int w = 0; w < kSortWarps; ++w) acc += wcnt[w][d];
+            if (tile != withhold) st[d] = tag | (tile == 0 ? kInc : kAgg) | acc;
+        }
+        uint32_t x = acc;   // inclusive over the warp's digits
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
@@ -277,20 +286,16 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
         }
         if (lane == 31) s_part[wid] = x;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t acc = 0;
+        const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? s_part[lane] : 0u);
+        if (d < nb) {
+            uint32_t at = before + x - acc;
+            loff[d] = at;
+#pragma unroll
             for (int w = 0; w < kSortWarps; ++w) {
-                const uint32_t c = s_part[w];
-                s_part[w] = acc;
-                acc += c;
+                const uint32_t c = wcnt[w][d];
+                wcnt[w][d] = (uint16_t)at;   // below the tile's size
+                at += c;
             }
-        }
-        __syncthreads();
-        uint32_t run = s_part[wid] + x - sum;
-        for (uint32_t d = d0; d < d0 + per && d < nb; ++d) {
-            const uint32_t c = loff[d];
-            loff[d] = run;
-            run += c;
         }
     }
     __syncthreads();
@@ -301,7 +306,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
         if (t < n) {
             const uint32_t d = digit_of(e[r], field, shift, mask, nd);
             const uint32_t rank = (rk[r >> 1] >> ((r & 1) * 16)) & 0xFFFFu;
-            const uint32_t at = loff[d] + wcnt[wid][d] + rank;
+            const uint32_t at = wcnt[wid][d] + rank;
             if (PG_CHECK(at, n)) buf[at] = e[r];
         }
     }
@@ -381,9 +386,13 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     }
 }
 
-static_assert(SortShape<uint32_t>::tile * sizeof(uint2) >= kSortWarps * kMaxBuckets * 4 &&
-                  SortShape<uint64_t>::tile * sizeof(ulonglong2) >= kSortWarps * kMaxBuckets * 4,
+static_assert(SortShape<uint32_t>::tile * sizeof(uint2) >= kFly * kSortWarps * kMaxBuckets * 4 &&
+                  SortShape<uint64_t>::tile * sizeof(ulonglong2) >=
+                      kFly * kSortWarps * kMaxBuckets * 4,
               "the reorder buffer holds every warp's digit words");
+static_assert(kSortThreads >= (int)kMaxBuckets, "one thread per digit");
+static_assert(SortShape<uint32_t>::items % kFly == 0 && SortShape<uint64_t>::items % kFly == 0,
+              "whole groups of items");
 
 template <typename Id>
 size_t scatter_smem_bytes()
