@@ -31,6 +31,7 @@
 // dropped), so a bad list cannot make a kernel write out of bounds.
 #include <atomic>
 #include <cstring>
+#include <type_traits>
 
 #include "pg_internal.h"
 #include "pg_trace.h"
@@ -58,23 +59,51 @@ struct PairOf<uint64_t> {
     using T = ulonglong2;
 };
 
+// What the sort moves (K): pairs of 32-bit ids wherever the ids fit, also of a
+// list with 64-bit ids, else pairs of 64-bit ids. A pass is bound by the
+// shared-memory pipe and moves half the bytes in the narrow form: the CSR of
+// 2 * 10^7 pairs of 64-bit ids, k = 21, went from 1.243 to 0.921 ms. (One
+// 64-bit key (src << nd) | dst per pair instead: 1.001 ms, and 0.662 instead
+// of 0.586 ms for the passes of k = 20, whose digits then take 64-bit shifts.)
+// The first pass reads the call's list itself, reversed pairs of a symmetrised
+// list included.
+//
 // The digit of a pass: field 0 = dst and field 1 = src take `mask` bits at
 // `shift` of that id; field 2 is a digit of the key (src << nd) | dst that
 // starts in dst (shift < nd) and ends in src.
-template <typename P>
-__device__ __forceinline__ uint32_t digit_of(const P& e, int field, int shift, uint32_t mask,
-                                             int nd)
+struct Digit {
+    int field, shift, nd;
+    uint32_t mask;
+};
+template <typename K>
+__device__ __forceinline__ uint32_t digit_of(const K& e, const Digit& g)
 {
-    if (field == 2)
-        return (uint32_t)(((uint64_t)e.y >> shift) | ((uint64_t)e.x << (nd - shift))) & mask;
-    const uint64_t v = field ? (uint64_t)e.x : (uint64_t)e.y;
-    return (uint32_t)(v >> shift) & mask;
+    if (g.field == 2)
+        return (uint32_t)(((uint64_t)e.y >> g.shift) | ((uint64_t)e.x << (g.nd - g.shift))) & g.mask;
+    return (uint32_t)((g.field ? e.x : e.y) >> g.shift) & g.mask;
 }
 
+// The list of a call: its pairs, each twice when sym (the second time
+// reversed), in the width the sort moves.
+template <typename K, typename P>
+struct PairList {
+    const P* p;
+    uint32_t sym;
+    __device__ __forceinline__ K operator[](uint64_t i) const
+    {
+        const P e = p[sym ? i >> 1 : i];
+        const bool back = sym && (i & 1);
+        K k;
+        k.x = (decltype(k.x))(back ? e.y : e.x);
+        k.y = (decltype(k.y))(back ? e.x : e.y);
+        return k;
+    }
+};
+
 // Elements per thread of a sort tile: 16 pairs of 32-bit ids or 8 of 64-bit.
-template <typename Id>
+template <typename K>
 struct SortShape {
-    static constexpr int items = sizeof(Id) == 4 ? 16 : 8;
+    static constexpr int items = sizeof(K) == 8 ? 16 : 8;
     static constexpr uint32_t tile = kSortThreads * items;
 };
 
@@ -87,14 +116,18 @@ struct PassList {
     uint32_t n;
     int nd;   // bits of the dst field
     int field[kMaxPasses], shift[kMaxPasses], bits[kMaxPasses];
+    __host__ __device__ Digit digit(uint32_t k) const
+    {
+        return Digit{field[k], shift[k], nd, (1u << bits[k]) - 1};
+    }
 };
 // Digit totals of every pass in one read of the list: tot[k][d] = number of
 // pairs whose pass-k digit is d. Each CTA counts into shared memory
 // (n passes x kMaxBuckets counters, kHistCopies copies of each) and adds its
 // counts once.
-template <typename Id>
+template <typename K, typename In>
 __global__ void __launch_bounds__(256) radix_hist_all_kernel(
-    const typename PairOf<Id>::T* __restrict__ in, uint64_t M, const __grid_constant__ PassList pl,
+    const In in, uint64_t M, const __grid_constant__ PassList pl,
     unsigned long long* __restrict__ tot, const uint32_t* __restrict__ sort_needed)
 {
     extern __shared__ uint32_t h[];
@@ -109,20 +142,19 @@ __global__ void __launch_bounds__(256) radix_hist_all_kernel(
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     constexpr int kU = 4;
     for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < M; i0 += kU * stride) {
-        typename PairOf<Id>::T e[kU];
+        K e[kU];
 #pragma unroll
         for (int u = 0; u < kU; ++u)
             if (i0 + u * stride < M) e[u] = in[i0 + u * stride];
         // pass by pass, so that each pass's digit rule is read once for the
         // kU elements
         for (uint32_t k = 0; k < pl.n; ++k) {
-            const int field = pl.field[k], shift = pl.shift[k];
-            const uint32_t mask = (1u << pl.bits[k]) - 1;
+            const Digit dg = pl.digit(k);
             uint32_t* hk = h + (k * kMaxBuckets) * kHistCopies + copy;
 #pragma unroll
             for (int u = 0; u < kU; ++u)
                 if (i0 + u * stride < M)
-                    atomicAdd(&hk[digit_of(e[u], field, shift, mask, pl.nd) * kHistCopies], 1u);
+                    atomicAdd(&hk[digit_of(e[u], dg) * kHistCopies], 1u);
         }
     }
     __syncthreads();
@@ -174,29 +206,28 @@ CsrWaitHook csr_wait_hook() { return CsrWaitHook{g_hook_spin.load(), g_hook_with
 // one word (kSpinLimit unless a test hook shortened it) it sets *err and
 // goes on with the partial sum, which can only be too small, so every write
 // stays inside the output.
-template <typename Id>
+template <typename K, typename In, typename Id>
 __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
-    const typename PairOf<Id>::T* __restrict__ in, typename PairOf<Id>::T* __restrict__ out,
-    uint64_t M, int field, int shift, int bits, int nd, unsigned long long* __restrict__ status,
+    const In in, K* __restrict__ out, uint64_t M, const Digit dg,
+    unsigned long long* __restrict__ status,
     uint32_t pass, const uint64_t* __restrict__ dstart, uint32_t* __restrict__ ticket,
     uint32_t* __restrict__ err, const uint32_t* __restrict__ sort_needed, uint32_t spin_limit,
     uint32_t withhold, Id* __restrict__ col_out, uint64_t* __restrict__ row_ptr, uint64_t N)
 {
-    using P = typename PairOf<Id>::T;
-    constexpr int kItems = SortShape<Id>::items;
-    constexpr uint32_t kTile = SortShape<Id>::tile;
+    constexpr int kItems = SortShape<K>::items;
+    constexpr uint32_t kTile = SortShape<K>::tile;
     extern __shared__ __align__(16) unsigned char smem[];
     uint16_t (*wcnt)[kMaxBuckets] = reinterpret_cast<uint16_t (*)[kMaxBuckets]>(smem);   // 8 KB
     uint64_t* tbase = reinterpret_cast<uint64_t*>(smem + kSortWarps * kMaxBuckets * 2);   // 2 KB
     uint32_t* loff = reinterpret_cast<uint32_t*>(tbase + kMaxBuckets);                  // 1 KB
-    P* buf = reinterpret_cast<P*>(loff + kMaxBuckets);                                  // tile
+    K* buf = reinterpret_cast<K*>(loff + kMaxBuckets);                                  // tile
     __shared__ uint32_t s_part[kSortWarps + 1];
     __shared__ uint32_t s_tile;
     // after a wait that gave up in an earlier pass the list this pass reads
     // no longer has the digit totals dstart was made from, so a scatter
     // could leave the output: the remaining passes do nothing
     if (*sort_needed == 0 || *(volatile const uint32_t*)err != 0) return;
-    const uint32_t nb = 1u << bits, mask = nb - 1;
+    const uint32_t nb = dg.mask + 1;
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
     for (uint32_t d = threadIdx.x; d < nb; d += blockDim.x)
@@ -206,7 +237,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     const uint64_t tile0 = (uint64_t)tile * kTile;
     const uint32_t n = (uint32_t)((M - tile0 < kTile) ? M - tile0 : kTile);
     const uint32_t wbase = wid * (32 * kItems);
-    P e[kItems];
+    K e[kItems];
     // ranks within the warp (< 32 * kItems <= 512), two per register; the
     // digits are recomputed from e[] where needed, so no array holds them
     uint32_t rk[kItems / 2];
@@ -237,7 +268,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
 #pragma unroll
         for (int u = 0; u < kFly; ++u) {
             const uint32_t t = wbase + (r0 + u) * 32 + lane;
-            d[u] = t < n ? digit_of(e[r0 + u], field, shift, mask, nd) : 0xFFFFFFFFu;
+            d[u] = t < n ? digit_of(e[r0 + u], dg) : 0xFFFFFFFFu;
             if (d[u] != 0xFFFFFFFFu) atomicOr(&pmask[u * kMaxBuckets + d[u]], 1u << lane);
         }
         __syncwarp();
@@ -304,7 +335,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     for (int r = 0; r < kItems; ++r) {
         const uint32_t t = wbase + r * 32 + lane;
         if (t < n) {
-            const uint32_t d = digit_of(e[r], field, shift, mask, nd);
+            const uint32_t d = digit_of(e[r], dg);
             const uint32_t rank = (rk[r >> 1] >> ((r & 1) * 16)) & 0xFFFFu;
             const uint32_t at = wcnt[wid][d] + rank;
             if (PG_CHECK(at, n)) buf[at] = e[r];
@@ -364,8 +395,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     // write runs: sorted position p goes to tbase[d] + p (one table read per pair)
     if (col_out == nullptr) {
         for (uint32_t p = threadIdx.x; p < n; p += blockDim.x) {
-            const P v = buf[p];
-            const uint32_t d = digit_of(v, field, shift, mask, nd);
+            const K v = buf[p];
+            const uint32_t d = digit_of(v, dg);
             if (PG_CHECK(tbase[d] + p, M)) out[tbase[d] + p] = v;
         }
         return;
@@ -375,8 +406,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     // in the tile raises row_ptr[src + 1] to its end (the source's last pair
     // overall gives the maximum; the prefix maximum fills empty rows)
     for (uint32_t p = threadIdx.x; p < n; p += blockDim.x) {
-        const P v = buf[p];
-        const uint32_t d = digit_of(v, field, shift, mask, nd);
+        const K v = buf[p];
+        const uint32_t d = digit_of(v, dg);
         const uint64_t o = tbase[d] + p;
         if (PG_CHECK_OUT(o, M)) col_out[o] = (Id)v.y;
         const uint64_t src = v.x;
@@ -386,19 +417,19 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     }
 }
 
-static_assert(SortShape<uint32_t>::tile * sizeof(uint2) >= kFly * kSortWarps * kMaxBuckets * 4 &&
-                  SortShape<uint64_t>::tile * sizeof(ulonglong2) >=
+static_assert(SortShape<uint2>::tile * sizeof(uint2) >= kFly * kSortWarps * kMaxBuckets * 4 &&
+                  SortShape<ulonglong2>::tile * sizeof(ulonglong2) >=
                       kFly * kSortWarps * kMaxBuckets * 4,
               "the reorder buffer holds every warp's digit words");
 static_assert(kSortThreads >= (int)kMaxBuckets, "one thread per digit");
-static_assert(SortShape<uint32_t>::items % kFly == 0 && SortShape<uint64_t>::items % kFly == 0,
+static_assert(SortShape<uint2>::items % kFly == 0 && SortShape<ulonglong2>::items % kFly == 0,
               "whole groups of items");
 
-template <typename Id>
+template <typename K>
 size_t scatter_smem_bytes()
 {
     return (size_t)kSortWarps * kMaxBuckets * 2 + kMaxBuckets * 8 + kMaxBuckets * 4 +
-           (size_t)SortShape<Id>::tile * sizeof(typename PairOf<Id>::T);
+           (size_t)SortShape<K>::tile * sizeof(K);
 }
 
 // ---- exclusive scan of uint32 counts into uint64 offsets ------------------
@@ -672,23 +703,6 @@ __global__ void __launch_bounds__(256) csr_finish_kernel(const typename PairOf<I
 // their destinations to col in order and marks row ends for the prefix max.
 constexpr uint32_t kOptSym = 1, kOptDedup = 2, kOptNoLoops = 4, kOptOdd = 8;
 
-template <typename Id>
-__global__ void __launch_bounds__(256) csr_sym_kernel(const typename PairOf<Id>::T* __restrict__ in,
-                                                      uint64_t M,
-                                                      typename PairOf<Id>::T* __restrict__ x)
-{
-    using P = typename PairOf<Id>::T;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += stride) {
-        const P e = in[i];
-        P r;
-        r.x = e.y;
-        r.y = e.x;
-        x[2 * i] = e;
-        x[2 * i + 1] = r;
-    }
-}
-
 template <typename P>
 __device__ __forceinline__ bool same_pair(const P& a, const P& b)
 {
@@ -706,8 +720,8 @@ __device__ __forceinline__ bool pair_less(const P& a, const P& b)
 // found by binary search of the sorted list below. (With ids outside the
 // vertex range the list need not be in lexicographic order there, and the
 // search only stays within [0, i].)
-template <typename P>
-__device__ __forceinline__ uint64_t run_start(const P* s, uint64_t i, const P& e)
+template <typename L, typename P>
+__device__ __forceinline__ uint64_t run_start(const L& s, uint64_t i, const P& e)
 {
     uint64_t j = i;
     for (int t = 0; t < 8 && j > 0 && same_pair(s[j - 1], e); ++t) --j;
@@ -722,10 +736,10 @@ __device__ __forceinline__ uint64_t run_start(const P* s, uint64_t i, const P& e
 }
 
 // Whether sorted position i survives the options.
-template <typename P>
-__device__ __forceinline__ bool keep_at(const P* s, uint64_t M, uint64_t i, uint32_t flags)
+template <typename L>
+__device__ __forceinline__ bool keep_at(const L& s, uint64_t M, uint64_t i, uint32_t flags)
 {
-    const P e = s[i];
+    const auto e = s[i];
     if ((flags & kOptNoLoops) && e.x == e.y) return false;
     if (flags & kOptOdd) {
         // the last pair of each run is kept when the run's length is odd
@@ -736,9 +750,8 @@ __device__ __forceinline__ bool keep_at(const P* s, uint64_t M, uint64_t i, uint
     return true;
 }
 
-template <typename Id>
-__global__ void __launch_bounds__(256) csr_keep_count_kernel(const typename PairOf<Id>::T* __restrict__ s,
-                                                             uint64_t M, uint32_t flags,
+template <typename L>
+__global__ void __launch_bounds__(256) csr_keep_count_kernel(const L s, uint64_t M, uint32_t flags,
                                                              uint64_t* __restrict__ part)
 {
     __shared__ uint64_t s_warp[32];
@@ -757,14 +770,12 @@ __global__ void __launch_bounds__(256) csr_keep_count_kernel(const typename Pair
 // the warps' counts are scanned across the block, and the kept destinations
 // are written in sorted order. The last position of every row writes
 // row_ptr[src + 1] = kept entries up to and including it.
-template <typename Id>
-__global__ void __launch_bounds__(256, 4) csr_keep_apply_kernel(const typename PairOf<Id>::T* __restrict__ s,
-                                                             uint64_t M, uint64_t N, uint32_t flags,
+template <typename Id, typename L>
+__global__ void __launch_bounds__(256, 4) csr_keep_apply_kernel(const L s, uint64_t M, uint64_t N, uint32_t flags,
                                                              const uint64_t* __restrict__ part,
                                                              Id* __restrict__ col,
                                                              uint64_t* __restrict__ row_ptr)
 {
-    using P = typename PairOf<Id>::T;
     __shared__ uint64_t s_warp[32];
     constexpr int kRounds = kScanTile / 256;   // rounds of 32 positions per warp
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -788,7 +799,7 @@ __global__ void __launch_bounds__(256, 4) csr_keep_apply_kernel(const typename P
         const bool keep = (m[r] >> lane) & 1u;
         const uint64_t at = e + __popc(m[r] & lt);   // this position's place if kept
         if (i < M) {
-            const P pv = s[i];
+            const auto pv = s[i];
             if (keep && PG_CHECK_OUT(at, M)) col[at] = (Id)pv.y;
             const uint64_t v = pv.x;
             if (v < N && (i + 1 == M || (uint64_t)s[i + 1].x != v))
@@ -856,13 +867,20 @@ PassList make_passes(uint64_t n_src, uint64_t n_dst)
     return pl;
 }
 
+// Whether the sort moves pairs of 32-bit ids.
+bool ids_narrow(uint64_t n_src, uint64_t n_dst)
+{
+    return n_src <= ((uint64_t)1 << 32) && n_dst <= ((uint64_t)1 << 32);
+}
+
 CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst = 0)
 {
     CsrLayout L;
     const PassList pl = make_passes(N, N_dst ? N_dst : N);
+    if (ids_narrow(N, N_dst ? N_dst : N)) pair_bytes = 8;
     int dbits = 0;
     for (uint32_t k = 0; k < pl.n; ++k) dbits = pl.bits[k] > dbits ? pl.bits[k] : dbits;
-    const uint32_t tile = pair_bytes == 8 ? SortShape<uint32_t>::tile : SortShape<uint64_t>::tile;
+    const uint32_t tile = pair_bytes == 8 ? SortShape<uint2>::tile : SortShape<ulonglong2>::tile;
     L.max_nb = 1u << dbits;
     L.n_tiles = (uint32_t)((M + tile - 1) / tile);
     L.n_status = (uint64_t)L.max_nb * L.n_tiles;
@@ -887,47 +905,62 @@ CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst =
 // The opt-in shared-memory sizes of the sort kernels, set once per device
 // for each id width.
 PerDeviceOnce g_csr_attrs[2];
+template <typename K, typename In, typename Id>
+cudaError_t scatter_attribute()
+{
+    return cudaFuncSetAttribute(radix_scatter_kernel<K, In, Id>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)scatter_smem_bytes<K>());
+}
+template <typename K, typename In>
+cudaError_t hist_attribute()
+{
+    return cudaFuncSetAttribute(radix_hist_all_kernel<K, In>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(kMaxPasses * 4 * kMaxBuckets * kHistCopies));
+}
 template <typename Id>
 cudaError_t set_csr_attributes()
 {
+    using P = typename PairOf<Id>::T;
     return g_csr_attrs[sizeof(Id) == 8].run_current([] {
-        return first_error({
-            cudaFuncSetAttribute(radix_scatter_kernel<Id>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)scatter_smem_bytes<Id>()),
-            cudaFuncSetAttribute(radix_hist_all_kernel<Id>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(kMaxPasses * 4 * kMaxBuckets * kHistCopies))});
+        cudaError_t e = first_error({scatter_attribute<uint2, PairList<uint2, P>, Id>(),
+                                     scatter_attribute<uint2, const uint2*, Id>(),
+                                     hist_attribute<uint2, PairList<uint2, P>>(),
+                                     hist_attribute<uint2, const uint2*>()});
+        if constexpr (sizeof(Id) == 8)
+            if (e == cudaSuccess)
+                e = first_error({scatter_attribute<P, PairList<P, P>, Id>(),
+                                 scatter_attribute<P, const P*, Id>(),
+                                 hist_attribute<P, PairList<P, P>>(),
+                                 hist_attribute<P, const P*>()});
+        return e;
     });
 }
 
-// LSD radix passes over M pairs starting at `in` (the digits of the key
-// (src << nd) | dst from its low end). *sorted receives the sorted list (in
-// itself when there is no digit to sort), *spare a ping-pong buffer the
-// result does not occupy. With col_final set, the last pass writes the CSR
-// directly instead of the sorted pairs: destinations to col_final, row ends
-// raised into row_ptr (zeroed by the caller); *sorted is then not a list.
+// LSD radix passes over the M pairs of `first` (the digits of the key
+// (src << nd) | dst from its low end); K is what the passes move. *sorted
+// receives the sorted list (unset when there is no digit to sort). With
+// col_final set, the last pass writes the CSR directly instead: destinations
+// to col_final, row ends raised into row_ptr (zeroed by the caller).
 int sort_grid(uint64_t work);
 
-template <typename Id>
-cudaError_t radix_passes(const typename PairOf<Id>::T* in, uint64_t M, uint64_t N, uint64_t N_dst,
+template <typename K, typename P, typename Id>
+cudaError_t radix_passes(const PairList<K, P> first, uint64_t M, uint64_t N, const PassList& pl,
                          const CsrLayout& L, unsigned char* ws, const uint32_t* sort_needed,
-                         cudaStream_t s, const typename PairOf<Id>::T** sorted,
-                         typename PairOf<Id>::T** spare, Id* col_final = nullptr,
-                         uint64_t* row_ptr = nullptr)
+                         cudaStream_t s, const K** sorted, Id* col_final, uint64_t* row_ptr)
 {
-    using P = typename PairOf<Id>::T;
-    P* buf[2] = {(P*)(ws + L.off_a), (P*)(ws + L.off_b)};
+    K* buf[2] = {(K*)(ws + L.off_a), (K*)(ws + L.off_b)};
     unsigned long long* status = (unsigned long long*)(ws + L.off_status);
     unsigned long long* tot = (unsigned long long*)(ws + L.off_dig);
     uint64_t* dstart = (uint64_t*)(ws + L.off_dig) + (size_t)kMaxPasses * kMaxBuckets;
     uint32_t* tickets = (uint32_t*)(ws + L.off_flag + 64);
     uint32_t* err = (uint32_t*)(ws + L.off_flag + 128);
-    // the passes: digits of the key (src << nd) | dst, at most kMaxDigitBits each
-    const PassList pl = make_passes(N, N_dst);
-    const P* cur = in;
-    int which = 0;
-    cudaError_t err_c;
+    // a list that is what the passes move already is read as it is
+    const K* plain = nullptr;
+    if constexpr (std::is_same<K, P>::value)
+        if (!first.sym) plain = first.p;
+    const K* cur = plain;
     const CsrWaitHook hk = csr_wait_hook();
     // the tickets and the wait error word start at zero on every call that
     // has edges (a call without edges has nothing to sort and no wait)
@@ -940,8 +973,13 @@ cudaError_t radix_passes(const typename PairOf<Id>::T* in, uint64_t M, uint64_t 
             TraceScope trace("csr_radix_hist", s);
             { zero_status_kernel<<<sort_grid(L.n_status / 2 + 1), 256, 0, s>>>(
                 (uint4*)status, (L.n_status * 8 + 15) / 16, sort_needed); note_launch(); }
-            { radix_hist_all_kernel<Id><<<sort_grid(M), 256, (size_t)pl.n * kMaxBuckets * 4 * kHistCopies, s>>>(
-                cur, M, pl, tot, sort_needed); note_launch(); }
+            const size_t smem = (size_t)pl.n * kMaxBuckets * 4 * kHistCopies;
+            if (plain)
+                { radix_hist_all_kernel<K, const K*><<<sort_grid(M), 256, smem, s>>>(
+                    plain, M, pl, tot, sort_needed); note_launch(); }
+            else
+                { radix_hist_all_kernel<K, PairList<K, P>><<<sort_grid(M), 256, smem, s>>>(
+                    first, M, pl, tot, sort_needed); note_launch(); }
         }
         {
             TraceScope trace("csr_scan", s);
@@ -949,17 +987,22 @@ cudaError_t radix_passes(const typename PairOf<Id>::T* in, uint64_t M, uint64_t 
         }
         for (uint32_t k = 0; k < pl.n; ++k) {
             TraceScope trace("csr_radix_scatter", s);
-            { radix_scatter_kernel<Id><<<L.n_tiles, kSortThreads, scatter_smem_bytes<Id>(), s>>>(
-                cur, buf[which], M, pl.field[k], pl.shift[k], pl.bits[k], pl.nd, status, k,
-                dstart + (size_t)k * kMaxBuckets, tickets + k, err, sort_needed, hk.spin_limit,
-                hk.withhold, k + 1 == pl.n ? col_final : nullptr, row_ptr, N); note_launch(); }
-            if ((err_c = cudaGetLastError()) != cudaSuccess) return err_c;
-            cur = buf[which];
-            which ^= 1;
+            Id* col = k + 1 == pl.n ? col_final : nullptr;
+            const uint64_t* ds = dstart + (size_t)k * kMaxBuckets;
+            if (k == 0 && !plain)
+                { radix_scatter_kernel<K, PairList<K, P>, Id><<<L.n_tiles, kSortThreads, scatter_smem_bytes<K>(), s>>>(
+                    first, buf[k & 1], M, pl.digit(k), status, k, ds, tickets + k, err, sort_needed,
+                    hk.spin_limit, hk.withhold, col, row_ptr, N); note_launch(); }
+            else
+                { radix_scatter_kernel<K, const K*, Id><<<L.n_tiles, kSortThreads, scatter_smem_bytes<K>(), s>>>(
+                    cur, buf[k & 1], M, pl.digit(k), status, k, ds, tickets + k, err, sort_needed,
+                    hk.spin_limit, hk.withhold, col, row_ptr, N); note_launch(); }
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+            cur = buf[k & 1];
         }
     }
     *sorted = cur;
-    *spare = buf[which];
     return cudaSuccess;
 }
 
@@ -1002,28 +1045,34 @@ cudaError_t csr_impl(const void* d_edges, uint64_t M, uint64_t N, uint64_t N_dst
                                                    sort_needed); note_launch(); }
     }
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    const P* cur;
-    P* spare;
     // with at least one digit to sort, the last pass writes col and the row
     // ends itself; a key without digits (one vertex) leaves the list as it is
-    const bool in_sort = M > 0 && make_passes(N, N_dst).n > 0;
-    if ((err = radix_passes<Id>((const P*)d_edges, M, N, N_dst, L, ws, sort_needed, s, &cur,
-                                &spare, in_sort ? (Id*)d_col : nullptr, d_row_ptr)) !=
-        cudaSuccess)
-        return err;
+    const PassList pl = make_passes(N, N_dst);
+    const bool in_sort = M > 0 && pl.n > 0;
+    Id* col = in_sort ? (Id*)d_col : nullptr;
+    if (ids_narrow(N, N_dst)) {
+        const uint2* sorted;
+        err = radix_passes<uint2, P, Id>({(const P*)d_edges, 0}, M, N, pl, L, ws, sort_needed, s,
+                                         &sorted, col, d_row_ptr);
+    } else if constexpr (sizeof(Id) == 8) {   // 32-bit ids are always narrow
+        const P* sorted;
+        err = radix_passes<P, P, Id>({(const P*)d_edges, 0}, M, N, pl, L, ws, sort_needed, s, &sorted,
+                                     col, d_row_ptr);
+    }
+    if (err != cudaSuccess) return err;
     if (!in_sort) {
         TraceScope trace("csr_finish", s);
-        { csr_finish_kernel<Id><<<grid, 256, 0, s>>>(cur, M, N, d_row_ptr, (Id*)d_col, sort_needed); note_launch(); }
+        { csr_finish_kernel<Id><<<grid, 256, 0, s>>>((const P*)d_edges, M, N, d_row_ptr, (Id*)d_col, sort_needed); note_launch(); }
     }
     TraceScope trace("csr_rows", s);   // rows without edges take the previous row's end
     return prefix_max(d_row_ptr, N + 1, (uint64_t*)(ws + L.off_rpart), s);
 }
 
 // Workspace of the options path: the sort's layout for the (possibly
-// doubled) list, then the doubled list, and the parts of two scans.
+// doubled) list, and the parts of the compaction's scan.
 struct OptsLayout {
     CsrLayout L;
-    size_t off_x, off_cpart, total;
+    size_t off_cpart, total;
     uint64_t M2, n_cparts;
 };
 
@@ -1033,13 +1082,30 @@ OptsLayout opts_layout(uint64_t M, uint64_t N, uint32_t flags, size_t pair_bytes
     O.M2 = (flags & kOptSym) ? 2 * M : M;
     O.L = csr_layout(O.M2, N, pair_bytes);
     size_t o = a256(O.L.total);
-    O.off_x = o;
-    if (flags & kOptSym) o += a256(O.M2 * pair_bytes);
     O.n_cparts = (O.M2 + kScanTile - 1) / kScanTile;
     O.off_cpart = o;
     o += a256((O.n_cparts + 1) * 8);
     O.total = o;
     return O;
+}
+
+// The wanted positions of the sorted list into col, and the row pointers.
+template <typename Id, typename List>
+cudaError_t csr_compact(const List& list, uint64_t M2, uint64_t N, uint32_t flags,
+                        const OptsLayout& O, unsigned char* ws, const uint32_t* sort_needed,
+                        uint64_t* d_row_ptr, Id* d_col, cudaStream_t s)
+{
+    cudaError_t err;
+    TraceScope trace("csr_compact", s);
+    if (M2 > 0) {
+        uint64_t* cpart = (uint64_t*)(ws + O.off_cpart);
+        { csr_keep_count_kernel<List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, flags, cpart); note_launch(); }
+        { scan_parts_kernel<<<1, 1024, 0, s>>>(cpart, O.n_cparts, sort_needed); note_launch(); }
+        { csr_keep_apply_kernel<Id, List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, N, flags, cpart,
+                                                                              d_col, d_row_ptr); note_launch(); }
+        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    }
+    return prefix_max(d_row_ptr, N + 1, (uint64_t*)(ws + O.L.off_rpart), s);
 }
 
 template <typename Id>
@@ -1057,26 +1123,31 @@ cudaError_t csr_opts_impl(const void* d_edges, uint64_t M, uint64_t N, uint32_t 
     if (cudaMemsetAsync(sort_needed, 1, 4, s) != cudaSuccess) return cudaErrorUnknown;
     if (cudaMemsetAsync(d_row_ptr, 0, (N + 1) * 8, s) != cudaSuccess) return cudaErrorUnknown;
     const P* in = (const P*)d_edges;
-    if ((flags & kOptSym) && M > 0) {
-        P* x = (P*)(ws + O.off_x);
-        { csr_sym_kernel<Id><<<sort_grid(M), 256, 0, s>>>(in, M, x); note_launch(); }
-        in = x;
+    const uint32_t sym = (flags & kOptSym) ? 1 : 0;
+    const PassList pl = make_passes(N, N);
+    if (pl.n == 0) {
+        // one vertex: the list is sorted as it is (its reverse is the same
+        // again), and there is no sort to clear the wait word
+        if (M2 > 0 && cudaMemsetAsync(ws + O.L.off_flag + 64, 0, 128, s) != cudaSuccess)
+            return cudaErrorUnknown;
+        return csr_compact<Id>(PairList<P, P>{in, sym}, M2, N, flags, O, ws, sort_needed, d_row_ptr,
+                               (Id*)d_col, s);
     }
-    const P* cur;
-    P* spare;
-    if ((err = radix_passes<Id>(in, M2, N, N, O.L, ws, sort_needed, s, &cur, &spare)) !=
-        cudaSuccess)
-        return err;
-    TraceScope trace("csr_compact", s);
-    if (M2 > 0) {
-        uint64_t* cpart = (uint64_t*)(ws + O.off_cpart);
-        { csr_keep_count_kernel<Id><<<(unsigned)O.n_cparts, 256, 0, s>>>(cur, M2, flags, cpart); note_launch(); }
-        { scan_parts_kernel<<<1, 1024, 0, s>>>(cpart, O.n_cparts, sort_needed); note_launch(); }
-        { csr_keep_apply_kernel<Id><<<(unsigned)O.n_cparts, 256, 0, s>>>(cur, M2, N, flags, cpart,
-                                                                        (Id*)d_col, d_row_ptr); note_launch(); }
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    if (ids_narrow(N, N)) {
+        const uint2* sorted;
+        if ((err = radix_passes<uint2, P, Id>({in, sym}, M2, N, pl, O.L, ws, sort_needed, s, &sorted,
+                                              nullptr, nullptr)) != cudaSuccess)
+            return err;
+        return csr_compact<Id>(sorted, M2, N, flags, O, ws, sort_needed, d_row_ptr, (Id*)d_col, s);
     }
-    return prefix_max(d_row_ptr, N + 1, (uint64_t*)(ws + O.L.off_rpart), s);
+    if constexpr (sizeof(Id) == 8) {
+        const P* sorted;
+        if ((err = radix_passes<P, P, Id>({in, sym}, M2, N, pl, O.L, ws, sort_needed, s, &sorted,
+                                          nullptr, nullptr)) != cudaSuccess)
+            return err;
+        return csr_compact<Id>(sorted, M2, N, flags, O, ws, sort_needed, d_row_ptr, (Id*)d_col, s);
+    }
+    return cudaErrorInvalidValue;   // 32-bit ids are always narrow
 }
 
 }  // namespace

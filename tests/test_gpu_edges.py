@@ -146,3 +146,27 @@ def test_noalloc_takes_a_graph_whose_smallest_workspace_fits():
                            C.c_void_p(torch.cuda.current_stream().cuda_stream))
     assert st == pg.PG_OK and cnt.value == E
     assert torch.equal(out, pg.gen_pba(n, m, B, 6, 1, 0.1, 3))
+
+
+@pytest.mark.parametrize("N", [2**32, 2**32 + 1])
+@pytest.mark.parametrize("flags", [0, pg.CSR_SYMMETRIZE | pg.CSR_DEDUP])
+def test_csr_of_64_bit_ids_on_both_sides_of_the_narrow_sort(N, flags):
+    """64-bit ids below 2^32 are sorted as pairs of 32-bit ids, larger ones as
+    they are. The row pointers (34 GB) are checked on the device, at the rows
+    that have edges and right after them."""
+    rng = np.random.default_rng(5 + flags)
+    e = rng.integers(0, N, size=(20_011, 2), dtype=np.uint64)
+    e[:300] = e[300:600]                  # repeated pairs
+    e[1000:1200, 0] = N - 1
+    e[1200:1400, 1] = N - 1
+    t = torch.from_numpy(e.view(np.int64)).cuda()
+    rp, col = pg.edges_to_csr_opts(t, N, flags) if flags else pg.edges_to_csr(t, N, check=True)
+    if flags:
+        e = np.unique(np.concatenate([e, e[:, ::-1]]), axis=0)
+    e = e[np.lexsort((e[:, 1], e[:, 0]))]
+    rows, first, counts = np.unique(e[:, 0], return_index=True, return_counts=True)
+    at = torch.from_numpy(rows.view(np.int64)).cuda()
+    assert np.array_equal(host(rp[at]), first.astype(np.uint64))
+    assert np.array_equal(host(rp[at + 1]), (first + counts).astype(np.uint64))
+    assert int(rp[0]) == 0 and int(rp[-1]) == e.shape[0]
+    assert np.array_equal(host(col)[:e.shape[0]], e[:, 1])
