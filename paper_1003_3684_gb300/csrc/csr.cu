@@ -486,20 +486,31 @@ __global__ void __launch_bounds__(kMaxBuckets) radix_dstart_kernel(
     if (d < nb) dstart[(size_t)k * kMaxBuckets + d] = ex;
 }
 
-// exclusive scan of n_parts sums in place, one CTA looping over chunks
+// exclusive scan of n_parts sums in place, one CTA looping over chunks of
+// eight neighbouring sums per thread
 __global__ void __launch_bounds__(1024) scan_parts_kernel(uint64_t* __restrict__ part,
                                                           uint64_t n_parts,
                                                           const uint32_t* __restrict__ sort_needed)
 {
     __shared__ uint64_t s_warp[32];
     if (*sort_needed == 0) return;
+    constexpr int kPer = 8;
     uint64_t carry = 0;
-    for (uint64_t base = 0; base < n_parts; base += blockDim.x) {
-        const uint64_t i = base + threadIdx.x;
-        const uint64_t v = i < n_parts ? part[i] : 0;
+    for (uint64_t base = 0; base < n_parts; base += kPer * blockDim.x) {
+        const uint64_t i = base + kPer * threadIdx.x;
+        uint64_t v[kPer], sum = 0;
+#pragma unroll
+        for (int t = 0; t < kPer; ++t) {
+            v[t] = i + t < n_parts ? part[i + t] : 0;
+            sum += v[t];
+        }
         uint64_t total;
-        const uint64_t ex = block_exclusive_scan(v, s_warp, total);
-        if (i < n_parts) part[i] = carry + ex;
+        uint64_t at = carry + block_exclusive_scan(sum, s_warp, total);
+#pragma unroll
+        for (int t = 0; t < kPer; ++t) {
+            if (i + t < n_parts) part[i + t] = at;
+            at += v[t];
+        }
         carry += total;
     }
 }
@@ -574,92 +585,105 @@ __global__ void __launch_bounds__(256) csr_grouped_kernel(const typename PairOf<
     }
 }
 
-// In-place inclusive prefix maximum over n uint64 (three kernels, as the sums).
-__device__ __forceinline__ uint64_t block_inclusive_max(uint64_t v, uint64_t* s_warp, uint64_t& total)
+// In-place inclusive prefix maximum over the row pointers. A warp takes
+// kScanTile / 8 neighbouring entries, 32 at a time, so that every access is
+// coalesced (row_ptr is aligned to 8 bytes only); V is uint32_t when the
+// values, which are positions in the list, fit it. Bound by memory: an entry
+// is read twice and written once. 2^26 rows: 0.601 -> 0.259 ms with the
+// zeroing; 2^20: 0.025 -> 0.017 (a thread read 16 neighbouring entries before).
+template <typename V>
+__device__ __forceinline__ V warp_inclusive_max(V x, uint32_t lane)
 {
-    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint32_t nw = blockDim.x >> 5;
-    uint64_t x = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        const V y = __shfl_up_sync(0xFFFFFFFFu, x, o);
         if (lane >= (uint32_t)o && y > x) x = y;
     }
-    if (lane == 31) s_warp[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        uint64_t w = lane < nw ? s_warp[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, w, o);
-            if (lane >= (uint32_t)o && y > w) w = y;
-        }
-        if (lane < nw) s_warp[lane] = w;
-    }
-    __syncthreads();
-    total = s_warp[nw - 1];
-    const uint64_t before = wid ? s_warp[wid - 1] : 0;
-    __syncthreads();
-    return x > before ? x : before;
+    return x;
 }
 
+template <typename V>
 __global__ void __launch_bounds__(256) max_reduce_kernel(const uint64_t* __restrict__ in, uint64_t n,
                                                          uint64_t* __restrict__ part)
 {
-    __shared__ uint64_t s_warp[32];
-    const uint64_t base = (uint64_t)blockIdx.x * kScanTile;
-    uint64_t m = 0;
-    for (uint32_t t = threadIdx.x; t < kScanTile; t += blockDim.x)
-        if (base + t < n && in[base + t] > m) m = in[base + t];
-    uint64_t total;
-    block_inclusive_max(m, s_warp, total);
-    if (threadIdx.x == 0) part[blockIdx.x] = total;
+    __shared__ V s_warp[8];
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint64_t base = (uint64_t)blockIdx.x * kScanTile + threadIdx.x;
+    V m = 0;
+#pragma unroll
+    for (uint32_t t = 0; t < kScanTile; t += 256) {
+        const V a = base + t < n ? (V)in[base + t] : 0;
+        if (a > m) m = a;
+    }
+    m = warp_inclusive_max(m, lane);
+    if (lane == 31) s_warp[wid] = m;
+    __syncthreads();
+    if (wid == 0) {
+        m = warp_inclusive_max<V>(lane < 8 ? s_warp[lane] : 0, lane);
+        if (lane == 31) part[blockIdx.x] = m;
+    }
 }
 
 // exclusive prefix maximum of the tile maxima, one CTA looping over chunks
 __global__ void __launch_bounds__(1024) max_parts_kernel(uint64_t* __restrict__ part, uint64_t n_parts)
 {
     __shared__ uint64_t s_warp[32];
-    __shared__ uint64_t s_inc[1024];
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint64_t carry = 0;
     for (uint64_t base = 0; base < n_parts; base += blockDim.x) {
         const uint64_t i = base + threadIdx.x;
-        const uint64_t v = i < n_parts ? part[i] : 0;
-        uint64_t total;
-        s_inc[threadIdx.x] = block_inclusive_max(v, s_warp, total);
+        const uint64_t x = warp_inclusive_max<uint64_t>(i < n_parts ? part[i] : 0, lane);
+        uint64_t ex = __shfl_up_sync(0xFFFFFFFFu, x, 1);
+        if (lane == 0) ex = 0;
+        if (lane == 31) s_warp[wid] = x;
         __syncthreads();
-        uint64_t ex = threadIdx.x ? s_inc[threadIdx.x - 1] : 0;
-        if (ex < carry) ex = carry;
+        const uint64_t w = warp_inclusive_max<uint64_t>(s_warp[lane], lane);
+        const uint64_t before = wid ? __shfl_sync(0xFFFFFFFFu, w, (wid - 1) & 31) : 0;
+        if (before > ex) ex = before;
+        if (carry > ex) ex = carry;
         if (i < n_parts) part[i] = ex;
+        const uint64_t total = __shfl_sync(0xFFFFFFFFu, w, 31);
         if (total > carry) carry = total;
         __syncthreads();
     }
 }
 
+// part == null: one CTA scans all n entries, a tile after another.
+template <typename V>
 __global__ void __launch_bounds__(256) max_apply_kernel(uint64_t* __restrict__ data, uint64_t n,
                                                         const uint64_t* __restrict__ part)
 {
-    __shared__ uint64_t s_warp[32];
-    __shared__ uint64_t s_inc[256];
-    constexpr int per = kScanTile / 256;
-    const uint64_t base = (uint64_t)blockIdx.x * kScanTile + threadIdx.x * per;
-    uint64_t v[per];
-    uint64_t m = 0;
+    __shared__ V s_warp[8];
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int kRounds = kScanTile / 256;
+    V carry = part ? (V)part[blockIdx.x] : 0;
+    for (uint64_t tile = blockIdx.x; tile * kScanTile < n; tile += gridDim.x) {
+        const uint64_t base = tile * kScanTile + wid * (32 * kRounds) + lane;
+        V a[kRounds];
 #pragma unroll
-    for (int t = 0; t < per; ++t) {
-        v[t] = (base + t < n) ? data[base + t] : 0;
-        if (v[t] > m) m = v[t];
-    }
-    uint64_t total;
-    s_inc[threadIdx.x] = block_inclusive_max(m, s_warp, total);
-    __syncthreads();
-    uint64_t run = threadIdx.x ? s_inc[threadIdx.x - 1] : 0;   // previous threads' runs
-    const uint64_t carry = part[blockIdx.x];                    // previous tiles
-    if (run < carry) run = carry;
+        for (int r = 0; r < kRounds; ++r) a[r] = base + 32 * r < n ? (V)data[base + 32 * r] : 0;
+        V run = 0;   // the warp's maximum up to and including round r
 #pragma unroll
-    for (int t = 0; t < per; ++t) {
-        if (v[t] > run) run = v[t];
-        if (base + t < n) data[base + t] = run;
+        for (int r = 0; r < kRounds; ++r) {
+            a[r] = warp_inclusive_max(a[r], lane);
+            if (run > a[r]) a[r] = run;
+            run = __shfl_sync(0xFFFFFFFFu, a[r], 31);
+        }
+        if (lane == 0) s_warp[wid] = run;
+        __syncthreads();
+        V before = carry, all = carry;
+#pragma unroll
+        for (uint32_t w = 0; w < 8; ++w) {
+            const V x = s_warp[w];
+            if (w < wid && x > before) before = x;
+            if (x > all) all = x;
+        }
+#pragma unroll
+        for (int r = 0; r < kRounds; ++r)
+            if (base + 32 * r < n) data[base + 32 * r] = before > a[r] ? before : a[r];
+        if (part) return;
+        carry = all;
+        __syncthreads();
     }
 }
 
@@ -735,77 +759,153 @@ __device__ __forceinline__ uint64_t run_start(const L& s, uint64_t i, const P& e
     return lo;
 }
 
-// Whether sorted position i survives the options.
+// Which positions of the sorted list survive the options, as one bit per
+// position (keep[i / 32]), and how many do in each tile of kScanTile. A warp
+// takes kScanTile / 8 neighbouring positions, 32 at a time, with the loads of
+// kAhead rounds in flight. The runs of equal pairs come out of one ballot per
+// round (bit i: pair i equals pair i - 1), and the rules are bit arithmetic on
+// those words, the same in every lane:
+//   CSR_DEDUP  the first pair of each run;
+//   CSR_ODD    the last pair of each run of odd length: the one whose distance
+//              from its run's start is even. The starts' parities are filled
+//              forward within the word and carried to the next.
+// Bound by reading the list once (8 or 16 bytes per pair). With the apply kernel
+// and the row pointers, 1.8 * 10^7 pairs under CSR_ODD: 0.333 -> 0.119 ms; 4 *
+// 10^7 under CSR_DEDUP and CSR_NO_LOOPS: 0.439 -> 0.210 ms (every position read
+// its neighbours from memory in both kernels, one load in flight, before).
+constexpr int kKeepRounds = kScanTile / 256;
+constexpr int kAhead = 8;
 template <typename L>
-__device__ __forceinline__ bool keep_at(const L& s, uint64_t M, uint64_t i, uint32_t flags)
+__global__ void __launch_bounds__(256) csr_keep_mask_kernel(const L s, uint64_t M, uint32_t flags,
+                                                            uint32_t* __restrict__ keep,
+                                                            uint64_t* __restrict__ part)
 {
-    const auto e = s[i];
-    if ((flags & kOptNoLoops) && e.x == e.y) return false;
-    if (flags & kOptOdd) {
-        // the last pair of each run is kept when the run's length is odd
-        const bool end = (i + 1 == M) || !same_pair(s[i + 1], e);
-        return end && (((i + 1 - run_start(s, i, e)) & 1) != 0);
+    __shared__ uint32_t s_warp[8];
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint64_t wbase = (uint64_t)blockIdx.x * kScanTile + (uint64_t)wid * (32 * kKeepRounds);
+    uint32_t cnt = 0;
+    if (wbase < M) {   // uniform in the warp
+        uint32_t eq[kKeepRounds], loop[kKeepRounds];   // ballots
+        using P = typename std::decay<decltype(s[0])>::type;
+        P prev = s[wbase > 0 ? wbase - 1 : 0];         // the pair before lane 0's
+#pragma unroll
+        for (int r0 = 0; r0 < kKeepRounds; r0 += kAhead) {
+            P e[kAhead];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const uint64_t i = wbase + (r0 + u) * 32 + lane;
+                e[u] = s[i < M ? i : M - 1];
+            }
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const uint64_t i = wbase + (r0 + u) * 32 + lane;
+                P b;   // the pair before this lane's
+                b.x = __shfl_up_sync(0xFFFFFFFFu, e[u].x, 1);
+                b.y = __shfl_up_sync(0xFFFFFFFFu, e[u].y, 1);
+                if (lane == 0) b = prev;
+                eq[r0 + u] = __ballot_sync(0xFFFFFFFFu, i > 0 && i < M && same_pair(b, e[u]));
+                loop[r0 + u] = __ballot_sync(0xFFFFFFFFu, e[u].x == e[u].y);
+                prev.x = __shfl_sync(0xFFFFFFFFu, e[u].x, 31);
+                prev.y = __shfl_sync(0xFFFFFFFFu, e[u].y, 31);
+            }
+        }
+        const uint64_t wend = wbase + 32 * kKeepRounds;
+        const bool open = wend < M && same_pair(s[wend], prev);   // the last run goes on
+        // parity of the start of the run open before this warp's positions
+        uint32_t odd = 0;
+        if ((flags & kOptOdd) && (eq[0] & 1u)) odd = (uint32_t)run_start(s, wbase, s[wbase]) & 1u;
+        uint32_t mine = 0;
+#pragma unroll
+        for (int r = 0; r < kKeepRounds; ++r) {
+            const uint64_t i0 = wbase + r * 32;
+            const uint32_t live = i0 >= M ? 0u : M - i0 >= 32 ? ~0u : (1u << (uint32_t)(M - i0)) - 1u;
+            uint32_t k = live;
+            if (flags & kOptOdd) {
+                // start parities (position parity is the bit's: i0 is even)
+                uint32_t known = ~eq[r], par = known & 0xAAAAAAAAu;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    par |= (par << o) & ~known;
+                    known |= known << o;
+                }
+                if (odd) par |= ~known;
+                odd = par >> 31;
+                const uint32_t more = r + 1 < kKeepRounds ? eq[r + 1 < kKeepRounds ? r + 1 : r] & 1u
+                                                          : (open ? 1u : 0u);
+                const uint32_t last = ~((eq[r] >> 1) | (more << 31));   // ends of runs
+                k &= last & ~(par ^ 0xAAAAAAAAu);
+            } else if (flags & kOptDedup) {
+                k &= ~eq[r];
+            }
+            if (flags & kOptNoLoops) k &= ~loop[r];
+            cnt += __popc(k);
+            if (lane == (uint32_t)r) mine = k;
+        }
+        if (lane < (uint32_t)kKeepRounds && wbase + 32 * lane < M) keep[wbase / 32 + lane] = mine;
     }
-    if (flags & kOptDedup) return i == 0 || !same_pair(s[i - 1], e);
-    return true;
+    if (lane == 0) s_warp[wid] = cnt;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint64_t all = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) all += s_warp[w];
+        part[blockIdx.x] = all;
+    }
 }
 
-template <typename L>
-__global__ void __launch_bounds__(256) csr_keep_count_kernel(const L s, uint64_t M, uint32_t flags,
-                                                             uint64_t* __restrict__ part)
-{
-    __shared__ uint64_t s_warp[32];
-    const uint64_t base = (uint64_t)blockIdx.x * kScanTile;
-    uint64_t cnt = 0;
-    for (uint32_t t = threadIdx.x; t < kScanTile; t += blockDim.x)
-        if (base + t < M) cnt += keep_at(s, M, base + t, flags) ? 1 : 0;
-    uint64_t total;
-    block_exclusive_scan(cnt, s_warp, total);
-    if (threadIdx.x == 0) part[blockIdx.x] = total;
-}
-
-// Each warp takes kScanTile/8 consecutive positions of its tile, 32 at a
-// time (consecutive lanes on consecutive pairs, so the reads coalesce): one
-// ballot per round gives every kept position its place among the warp's,
-// the warps' counts are scanned across the block, and the kept destinations
-// are written in sorted order. The last position of every row writes
-// row_ptr[src + 1] = kept entries up to and including it.
+// The kept destinations to their places, and the row ends: the last position
+// of every row writes row_ptr[src + 1] = kept entries up to and including it.
+// A warp's positions and loads are those of the mask kernel; a position's
+// place is the tile's start, the counts of the warps and rounds before it and
+// the kept bits below it in its word.
 template <typename Id, typename L>
-__global__ void __launch_bounds__(256, 4) csr_keep_apply_kernel(const L s, uint64_t M, uint64_t N, uint32_t flags,
+__global__ void __launch_bounds__(256) csr_keep_apply_kernel(const L s, uint64_t M, uint64_t N,
+                                                             const uint32_t* __restrict__ keep,
                                                              const uint64_t* __restrict__ part,
                                                              Id* __restrict__ col,
                                                              uint64_t* __restrict__ row_ptr)
 {
-    __shared__ uint64_t s_warp[32];
-    constexpr int kRounds = kScanTile / 256;   // rounds of 32 positions per warp
+    __shared__ uint32_t s_warp[8];
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
-    const uint64_t wbase = (uint64_t)blockIdx.x * kScanTile + (uint64_t)wid * (32 * kRounds);
-    uint32_t m[kRounds];
-    uint32_t cnt = 0;
+    const uint64_t wbase = (uint64_t)blockIdx.x * kScanTile + (uint64_t)wid * (32 * kKeepRounds);
+    // lane r holds round r's word
+    const uint32_t word = lane < (uint32_t)kKeepRounds && wbase + 32 * lane < M
+                              ? keep[wbase / 32 + lane] : 0u;
+    const uint32_t mine = __reduce_add_sync(0xFFFFFFFFu, __popc(word));
+    if (lane == 0) s_warp[wid] = mine;
+    __syncthreads();
+    if (wbase >= M) return;
+    uint64_t at = part[blockIdx.x];
+    for (uint32_t w = 0; w < wid; ++w) at += s_warp[w];
 #pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-        const uint64_t i = wbase + r * 32 + lane;
-        m[r] = __ballot_sync(0xFFFFFFFFu, i < M && keep_at(s, M, i, flags));
-        cnt += __popc(m[r]);
-    }
-    // the warps before this one in the tile, from lane 0's exclusive prefix
-    uint64_t total;
-    const uint64_t ex = block_exclusive_scan(lane == 0 ? (uint64_t)cnt : 0, s_warp, total);
-    uint64_t e = part[blockIdx.x] + __shfl_sync(0xFFFFFFFFu, ex, 0);
+    for (int r0 = 0; r0 < kKeepRounds; r0 += kAhead) {
+        typename std::decay<decltype(s[0])>::type e[kAhead];
 #pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-        const uint64_t i = wbase + r * 32 + lane;
-        const bool keep = (m[r] >> lane) & 1u;
-        const uint64_t at = e + __popc(m[r] & lt);   // this position's place if kept
-        if (i < M) {
-            const auto pv = s[i];
-            if (keep && PG_CHECK_OUT(at, M)) col[at] = (Id)pv.y;
-            const uint64_t v = pv.x;
-            if (v < N && (i + 1 == M || (uint64_t)s[i + 1].x != v))
-                row_ptr[v + 1] = at + (keep ? 1 : 0);
+        for (int u = 0; u < kAhead; ++u) {
+            const uint64_t i = wbase + (r0 + u) * 32 + lane;
+            e[u] = s[i < M ? i : M - 1];
         }
-        e += __popc(m[r]);
+        // the source after the batch's last position
+        const uint64_t inext = wbase + (r0 + kAhead) * 32;
+        const auto after = s[inext < M ? inext : M - 1].x;
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const uint64_t i = wbase + (r0 + u) * 32 + lane;
+            const uint32_t m = __shfl_sync(0xFFFFFFFFu, word, r0 + u);
+            auto nx = __shfl_down_sync(0xFFFFFFFFu, e[u].x, 1);
+            const auto first = u + 1 < kAhead ? __shfl_sync(0xFFFFFFFFu, e[u + 1 < kAhead ? u + 1 : u].x, 0)
+                                              : after;
+            if (lane == 31) nx = first;
+            const uint64_t here = at + __popc(m & lt);
+            const uint32_t kept = (m >> lane) & 1u;
+            if (i < M) {
+                if (kept && PG_CHECK_OUT(here, M)) col[here] = (Id)e[u].y;
+                const uint64_t v = e[u].x;
+                if (v < N && (i + 1 == M || (uint64_t)nx != v)) row_ptr[v + 1] = here + kept;
+            }
+            at += __popc(m);
+        }
     }
 }
 
@@ -1006,15 +1106,28 @@ cudaError_t radix_passes(const PairList<K, P> first, uint64_t M, uint64_t N, con
     return cudaSuccess;
 }
 
-// In-place prefix maximum over n uint64 (three kernels).
-cudaError_t prefix_max(uint64_t* data, uint64_t n, uint64_t* parts, cudaStream_t s)
+// In-place prefix maximum over the n row pointers, whose values are at most M:
+// three kernels, or one CTA alone where the launches would cost more than its
+// pass over a few tiles.
+constexpr uint64_t kMaxAlone = 8;
+template <typename V>
+cudaError_t prefix_max_as(uint64_t* data, uint64_t n, uint64_t* parts, cudaStream_t s)
 {
     const uint64_t n_parts = (n + kScanTile - 1) / kScanTile;
     if (n_parts == 0) return cudaSuccess;
-    { max_reduce_kernel<<<(unsigned)n_parts, 256, 0, s>>>(data, n, parts); note_launch(); }
+    if (n_parts <= kMaxAlone) {
+        { max_apply_kernel<V><<<1, 256, 0, s>>>(data, n, nullptr); note_launch(); }
+        return cudaGetLastError();
+    }
+    { max_reduce_kernel<V><<<(unsigned)n_parts, 256, 0, s>>>(data, n, parts); note_launch(); }
     { max_parts_kernel<<<1, 1024, 0, s>>>(parts, n_parts); note_launch(); }
-    { max_apply_kernel<<<(unsigned)n_parts, 256, 0, s>>>(data, n, parts); note_launch(); }
+    { max_apply_kernel<V><<<(unsigned)n_parts, 256, 0, s>>>(data, n, parts); note_launch(); }
     return cudaGetLastError();
+}
+cudaError_t prefix_max(uint64_t* data, uint64_t n, uint64_t M, uint64_t* parts, cudaStream_t s)
+{
+    return M < ((uint64_t)1 << 32) ? prefix_max_as<uint32_t>(data, n, parts, s)
+                                   : prefix_max_as<uint64_t>(data, n, parts, s);
 }
 
 int sort_grid(uint64_t work)
@@ -1065,14 +1178,14 @@ cudaError_t csr_impl(const void* d_edges, uint64_t M, uint64_t N, uint64_t N_dst
         { csr_finish_kernel<Id><<<grid, 256, 0, s>>>((const P*)d_edges, M, N, d_row_ptr, (Id*)d_col, sort_needed); note_launch(); }
     }
     TraceScope trace("csr_rows", s);   // rows without edges take the previous row's end
-    return prefix_max(d_row_ptr, N + 1, (uint64_t*)(ws + L.off_rpart), s);
+    return prefix_max(d_row_ptr, N + 1, M, (uint64_t*)(ws + L.off_rpart), s);
 }
 
 // Workspace of the options path: the sort's layout for the (possibly
 // doubled) list, and the parts of the compaction's scan.
 struct OptsLayout {
     CsrLayout L;
-    size_t off_cpart, total;
+    size_t off_cpart, off_keep, total;
     uint64_t M2, n_cparts;
 };
 
@@ -1085,6 +1198,8 @@ OptsLayout opts_layout(uint64_t M, uint64_t N, uint32_t flags, size_t pair_bytes
     O.n_cparts = (O.M2 + kScanTile - 1) / kScanTile;
     O.off_cpart = o;
     o += a256((O.n_cparts + 1) * 8);
+    O.off_keep = o;
+    o += a256((O.M2 + 31) / 32 * 4);
     O.total = o;
     return O;
 }
@@ -1099,13 +1214,14 @@ cudaError_t csr_compact(const List& list, uint64_t M2, uint64_t N, uint32_t flag
     TraceScope trace("csr_compact", s);
     if (M2 > 0) {
         uint64_t* cpart = (uint64_t*)(ws + O.off_cpart);
-        { csr_keep_count_kernel<List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, flags, cpart); note_launch(); }
+        uint32_t* keep = (uint32_t*)(ws + O.off_keep);
+        { csr_keep_mask_kernel<List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, flags, keep, cpart); note_launch(); }
         { scan_parts_kernel<<<1, 1024, 0, s>>>(cpart, O.n_cparts, sort_needed); note_launch(); }
-        { csr_keep_apply_kernel<Id, List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, N, flags, cpart,
+        { csr_keep_apply_kernel<Id, List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, N, keep, cpart,
                                                                               d_col, d_row_ptr); note_launch(); }
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
     }
-    return prefix_max(d_row_ptr, N + 1, (uint64_t*)(ws + O.L.off_rpart), s);
+    return prefix_max(d_row_ptr, N + 1, M2, (uint64_t*)(ws + O.L.off_rpart), s);
 }
 
 template <typename Id>

@@ -170,3 +170,38 @@ def test_csr_of_64_bit_ids_on_both_sides_of_the_narrow_sort(N, flags):
     assert np.array_equal(host(rp[at + 1]), (first + counts).astype(np.uint64))
     assert int(rp[0]) == 0 and int(rp[-1]) == e.shape[0]
     assert np.array_equal(host(col)[:e.shape[0]], e[:, 1])
+
+
+@pytest.mark.parametrize("flags", [pg.CSR_ODD, pg.CSR_ODD | pg.CSR_NO_LOOPS, pg.CSR_DEDUP,
+                                   pg.CSR_SYMMETRIZE | pg.CSR_ODD, pg.CSR_NO_LOOPS])
+@pytest.mark.parametrize("run", [1, 2, 3, 31, 32, 33, 64, 511, 513, 4095, 4097])
+def test_csr_options_with_runs_around_words_and_tiles(flags, run):
+    """Runs of equal pairs of odd and even lengths that start at every offset
+    of a 32-position word, cross words, a warp's positions and tiles."""
+    lens = [run, 1, run + 1, 2, run, 3, run + 2, 5, 1, run] + [1 + i % 7 for i in range(400)]
+    n = len(lens)
+    src = np.arange(n) // 9
+    dst = np.where(np.arange(n) % 9 == 4, src, 1000 + np.arange(n) % 9)     # some self-loops
+    e = np.repeat(np.stack([src, dst], 1), lens, axis=0).astype(np.uint32)
+    e = e[np.random.default_rng(run).permutation(e.shape[0])]
+    N = 1100
+    rp, col = pg.edges_to_csr_opts(torch.from_numpy(e.view(np.int32)).cuda(), N, flags)
+    ref_rp, ref_col = o.csr_opts(e.astype(np.uint64), N, flags)
+    assert np.array_equal(host(rp), ref_rp)
+    assert np.array_equal(host(col)[:ref_col.shape[0]], ref_col)
+
+
+@pytest.mark.parametrize("N", [1, 31, 4094, 4095, 4096, 8 * 4096 - 1, 8 * 4096, 8 * 4096 + 1,
+                               9 * 4096 + 17])
+@pytest.mark.parametrize("off", [0, 1])
+def test_csr_rows_without_edges(N, off):
+    """Row pointers over long gaps, into row_ptr buffers that are and are not
+    aligned to 16 bytes, at the sizes where one CTA stops scanning them."""
+    rng = np.random.default_rng(N)
+    e = rng.integers(0, N, size=(7, 2), dtype=np.uint32)
+    buf = torch.full((N + 3,), -7, dtype=torch.int64, device="cuda")
+    rp, col = pg.edges_to_csr(torch.from_numpy(e.view(np.int32)).cuda(), N, row_ptr=buf[off:])
+    ref_rp, ref_col = o.csr(e.astype(np.uint64), N)
+    assert np.array_equal(host(buf[off:off + N + 1]), ref_rp)
+    assert np.array_equal(host(col), ref_col)
+    assert (buf[off + N + 1:] == -7).all() and (off == 0 or int(buf[0]) == -7)
