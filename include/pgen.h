@@ -19,7 +19,7 @@
  *    library).
  *  - `stream` is a cudaStream_t passed as void* (NULL = legacy default
  *    stream). Calls only enqueue work and do not synchronise the stream,
- *    except pg_bfs, which waits once per search level (see there). Outputs
+ *    except pg_bfs, which waits for parts of its search (see there). Outputs
  *    written through h_* pointers are computed from the arguments on the
  *    host before any launch and are valid on return.
  *  - Arguments are validated on the host before anything is launched; an
@@ -428,7 +428,9 @@ pg_status gen_random_cells(uint64_t n_vertices, uint64_t n_edges, uint64_t seed,
  *   d_dist[v] (n_vertices uint32) = hops from source, 0xFFFFFFFF where
  *   unreached. n_vertices < 2^32 - 1. Workspace: pg_bfs_workspace_size()
  *   bytes, 256-byte aligned. Unlike the generators, this call waits for the
- *   stream once per BFS level (to read the next frontier's size);
+ *   stream: after each stretch of top-down levels (one cooperative launch)
+ *   and after each bottom-up level, to read the next frontier's size.
+ *   PG_ETIMEOUT: a bounded wait between levels gave up (d_dist unspecified);
  *   *levels_out (host) = number of levels run (the source's eccentricity + 1
  *   within its component), *scanned_out (host) = the sum of the reached
  *   vertices' row lengths (the adjacency entries a top-down search reads).

@@ -490,7 +490,7 @@ def bfs(row_ptr, col, source: int, dist=None, workspace=None, stream=None,
         undirected: bool = False):
     """BFS hop distances from source (int32 view of uint32; -1 = unreached).
 
-    Returns (dist, levels, scanned). Waits for the stream once per level.
+    Returns (dist, levels, scanned). Waits for the stream during the search (pgen.h).
     undirected=True declares the CSR symmetric, so that wide levels may run
     bottom-up (same results)."""
     import torch

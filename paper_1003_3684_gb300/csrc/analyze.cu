@@ -5,7 +5,9 @@
 // Every result is exact integer work. Degrees and histogram counts are sums
 // (atomic order does not change them); BFS distances are unique even though
 // the order in which a level's vertices are found depends on the schedule.
+#include <cstddef>
 #include <cstring>
+#include <utility>
 
 #include "../../include/pgen.h"
 #include "pg_internal.h"
@@ -17,16 +19,37 @@ namespace {
 constexpr uint32_t kBfsWarps = 8;          // warps per CTA of the BFS level kernel
 constexpr uint32_t kHistSmem = 8192;   // histograms up to this many buckets count in smem
 
+// Bound by the L2's atomics. A generated list often names one source on
+// several edges in a row, so a warp counts equal neighbouring sources first
+// and the first lane of each run adds the run's length.
 template <typename Id>
 __global__ void __launch_bounds__(256) degree_kernel(const Id* __restrict__ e, uint64_t M,
                                                      uint64_t N, int which,
                                                      unsigned long long* __restrict__ deg)
 {
+    const uint32_t lane = threadIdx.x & 31;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += stride) {
-        const uint64_t s = e[2 * i], d = e[2 * i + 1];
-        if (which != PG_DEG_IN && s < N) atomicAdd(&deg[s], 1ull);
-        if (which != PG_DEG_OUT && d < N) atomicAdd(&deg[d], 1ull);
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < M;
+         i0 += stride) {
+        const uint64_t i = i0 + lane;
+        const bool in = i < M;
+        uint64_t s = 0, d = 0;
+        if (in) {
+            s = e[2 * i];
+            d = e[2 * i + 1];
+        }
+        if (which != PG_DEG_IN) {
+            const uint64_t before = __shfl_up_sync(0xFFFFFFFFu, s, 1);
+            const uint32_t live = __ballot_sync(0xFFFFFFFFu, in);
+            const uint32_t first = __ballot_sync(0xFFFFFFFFu, in && (lane == 0 || before != s));
+            if (((first >> lane) & 1u) && s < N) {
+                // up to the next run's first lane, or the last live one
+                const uint32_t above = lane == 31 ? 0u : first >> (lane + 1);
+                const uint32_t len = above ? (uint32_t)__ffs(above) : __popc(live >> lane);
+                atomicAdd(&deg[s], (unsigned long long)len);
+            }
+        }
+        if (which != PG_DEG_OUT && in && d < N) atomicAdd(&deg[d], 1ull);
     }
 }
 
@@ -42,12 +65,19 @@ __global__ void __launch_bounds__(256) histogram_kernel(const uint64_t* __restri
         for (uint32_t t = threadIdx.x; t < nb; t += blockDim.x) h[t] = 0;
         __syncthreads();
     }
+    constexpr int kU = 4;   // degrees in flight per thread
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += stride) {
-        const uint64_t d = deg[v];
-        const uint32_t b = d <= max_deg ? (uint32_t)d : max_deg + 1;
-        if (in_smem) atomicAdd(&h[b], 1u);
-        else atomicAdd(&hist[b], 1ull);
+    for (uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v0 < N; v0 += kU * stride) {
+        uint64_t d[kU];
+#pragma unroll
+        for (int t = 0; t < kU; ++t) d[t] = v0 + t * stride < N ? deg[v0 + t * stride] : 0;
+#pragma unroll
+        for (int t = 0; t < kU; ++t) {
+            if (v0 + t * stride >= N) break;
+            const uint32_t b = d[t] <= max_deg ? (uint32_t)d[t] : max_deg + 1;
+            if (in_smem) atomicAdd(&h[b], 1u);
+            else atomicAdd(&hist[b], 1ull);
+        }
     }
     if (in_smem) {
         __syncthreads();
@@ -126,58 +156,116 @@ struct BfsQueue {
     }
 };
 
-// Rows of kLongRow or more entries leave the level kernel for the slice
-// kernel, which cuts them into slices of kSlice entries spread over all warps.
+// Rows of kLongRow or more entries are cut into slices spread over all warps.
 constexpr uint64_t kLongRow = 64;
-constexpr uint32_t kSlice = 512;
-
-// One BFS level, short rows. Each warp takes 32 frontier vertices at a time
-// and walks their short rows as one concatenated range, 32 adjacency entries
-// per step: lane k of a step finds the vertex owning entry base + k by a
-// binary search over the 32 rows' starts (a warp scan of their degrees, kept
-// in shared memory), so short rows (most rows of a power-law graph) do not
-// leave lanes idle. A long row is appended to the long-row list instead:
-// one 64-bit atomic on long_ctr adds 1 to the row count (high word) and its
-// slice count to the slice total (low word), so the slice bases of the list
-// ascend with its index. scanned += the short rows' lengths.
-template <typename Id>
-__global__ void __launch_bounds__(kBfsWarps * 32) bfs_level_kernel(const uint64_t* __restrict__ row_ptr,
-                                                        const Id* __restrict__ col,
-                                                        const uint32_t* __restrict__ frontier,
-                                                        uint32_t fsize, uint32_t* __restrict__ next,
-                                                        uint32_t* __restrict__ nsize,
-                                                        uint32_t* __restrict__ dist,
-                                                        uint32_t* __restrict__ vis, uint32_t level,
-                                                        uint64_t N,
-                                                        unsigned long long* __restrict__ long_ctr,
-                                                        uint32_t* __restrict__ long_v,
-                                                        uint32_t* __restrict__ long_base)
+// Slices, and frontier vertices per warp, are short while the frontier is: a
+// level is a chain of dependent loads per step of a warp, and few vertices
+// must not become many steps of few warps. (2^24 vertices: levels of 7, 96 and
+// 3630 frontier vertices took 14, 76 and 96 us with 32 vertices per warp and
+// slices of 512 entries.)
+constexpr uint32_t kWideFrontier = 1u << 15;
+__device__ __forceinline__ uint32_t slice_of(uint32_t fsize)
 {
-    __shared__ uint32_t wbuf[kBfsWarps][64];
-    __shared__ uint64_t wstart[kBfsWarps][32];   // the 32 rows' starts in the concatenation
-    __shared__ uint64_t wrow[kBfsWarps][32];     // and in col
-    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    return fsize < kWideFrontier ? 64u : 512u;
+}
+
+// Counters of a search, in its workspace. Sizes and long-row counts have a
+// slot per level mod 4: a slot is cleared a level before its use, three levels
+// after its last reader passed a barrier.
+struct BfsState {
+    uint32_t size[4];              // next frontier's vertices
+    unsigned long long longs[4];   // long rows << 32 | their slices
+    unsigned long long scanned;
+    uint32_t arrived, error;       // grid barrier: arrivals so far, a wait that gave up
+    uint32_t level, fsize, cur, pad;
+    unsigned long long visited;
+};
+static_assert(sizeof(BfsState) <= 256, "the counters' region of the workspace");
+
+// Barrier over a cooperative grid. Each wait is bounded; one that gives up
+// sets the error word and its CTA leaves the kernel, so the others give up too.
+constexpr uint32_t kBarrierPolls = 1u << 24;   // some ten seconds
+__device__ __forceinline__ bool grid_barrier(BfsState* st, uint32_t& epoch)
+{
+    __shared__ uint32_t s_ok;
+    __syncthreads();
+    ++epoch;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(&st->arrived, 1u);
+        const uint32_t want = epoch * gridDim.x;
+        uint32_t polls = 0, ok = 1;
+        // (the count may wrap; it is never far from what is waited for)
+        while ((int32_t)(*(volatile uint32_t*)&st->arrived - want) < 0) {
+            if (++polls > kBarrierPolls || *(volatile uint32_t*)&st->error) {
+                atomicOr(&st->error, 1u);
+                ok = 0;
+                break;
+            }
+            __nanosleep(32);
+        }
+        __threadfence();
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// One step of two adjacency entries per lane, both loads in flight.
+template <typename F>
+__device__ __forceinline__ void bfs_claim_two(BfsQueue& Q, uint64_t N, uint32_t lane, uint32_t lt,
+                                              F&& entry)
+{
+    uint64_t u[2];
+    bool have[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) have[t] = entry(t, u[t]) && u[t] < N;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) Q.step(have[t], (uint32_t)u[t], lane, lt);
+}
+
+// A top-down level's short rows. Each warp takes `chunk` (1 to 32) frontier
+// vertices at a time and walks their rows as one concatenated range, 64
+// adjacency entries per step: a lane finds the vertex owning an entry by a
+// binary search over the rows' starts (a warp scan of their degrees, kept in
+// shared memory), so short rows (most rows of a power-law graph) do not leave
+// lanes idle. A long row is appended to the long-row list instead: one 64-bit
+// atomic on long_ctr adds 1 to the row count (high word) and its slice count
+// to the slice total (low word), so the slice bases of the list ascend with
+// its index. Lists written in this launch are read past the L1 (ldcg).
+template <typename Id>
+__device__ __forceinline__ void bfs_short_rows(const uint64_t* __restrict__ row_ptr,
+                                               const Id* __restrict__ col,
+                                               const uint32_t* frontier, uint32_t fsize,
+                                               BfsQueue& Q, uint64_t* st, uint64_t* rw,
+                                               unsigned long long* long_ctr, uint32_t* long_v,
+                                               uint32_t* long_base)
+{
+    const uint64_t N = Q.N;
+    const uint32_t lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
-    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    BfsQueue Q{wbuf[wid], 0, next, nsize, dist, vis, level, N};
-    uint64_t* st = wstart[wid];
-    uint64_t* rw = wrow[wid];
-    const uint64_t first = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32;
-    for (uint64_t c = first; c < fsize; c += warps * 32) {
+    const uint64_t warps = (uint64_t)gridDim.x * kBfsWarps;
+    const uint64_t warp = (uint64_t)blockIdx.x * kBfsWarps + (threadIdx.x >> 5);
+    const uint32_t slice = slice_of(fsize);
+    uint64_t chunk = (fsize + warps - 1) / warps;
+    if (chunk > 32) chunk = 32;
+    for (uint64_t c = warp * chunk; c < fsize; c += warps * chunk) {
         uint64_t a = 0, d = 0;
-        if (c + lane < fsize && PG_CHECK(frontier[c + lane], N)) {
-            const uint32_t v = frontier[c + lane];
-            a = row_ptr[v];
-            d = row_ptr[v + 1] - a;
-            if (d >= kLongRow) {
-                const uint64_t ns = (d + kSlice - 1) / kSlice;
-                const unsigned long long old = atomicAdd(long_ctr, (1ull << 32) | ns);
-                const uint32_t r = (uint32_t)(old >> 32);
-                if (PG_CHECK(r, N)) {
-                    long_v[r] = v;
-                    long_base[r] = (uint32_t)old;
+        if (lane < chunk && c + lane < fsize) {
+            const uint32_t v = __ldcg(frontier + c + lane);
+            if (PG_CHECK(v, N)) {
+                a = row_ptr[v];
+                d = row_ptr[v + 1] - a;
+                if (d >= kLongRow) {
+                    const uint64_t ns = (d + slice - 1) / slice;
+                    const unsigned long long old = atomicAdd(long_ctr, (1ull << 32) | ns);
+                    const uint32_t r = (uint32_t)(old >> 32);
+                    if (PG_CHECK(r, N)) {
+                        long_v[r] = v;
+                        long_base[r] = (uint32_t)old;
+                    }
+                    d = 0;
                 }
-                d = 0;
             }
         }
         // inclusive scan of the short rows' lengths over the warp
@@ -191,125 +279,238 @@ __global__ void __launch_bounds__(kBfsWarps * 32) bfs_level_kernel(const uint64_
         st[lane] = incl - d;
         rw[lane] = a;
         __syncwarp();
-        for (uint64_t base = 0; base < total; base += 32) {
-            const uint64_t k = base + lane;
-            bool have = false;
-            uint32_t u = 0;
-            if (k < total) {
+        for (uint64_t base = 0; base < total; base += 64)
+            bfs_claim_two(Q, N, lane, lt, [&](int t, uint64_t& u) {
+                const uint64_t k = base + 32 * t + lane;
+                if (k >= total) return false;
                 // the last row whose start is at or below k owns entry k (an
                 // empty row starts where the next one does)
                 uint32_t o = 0;
 #pragma unroll
                 for (uint32_t step = 16; step > 0; step >>= 1)
                     if (st[o + step] <= k) o += step;
-                const uint64_t u64 = load_streaming(col + rw[o] + (k - st[o]));
-                have = u64 < N;
-                u = (uint32_t)u64;
-            }
-            Q.step(have, u, lane, lt);
-        }
+                u = load_streaming(col + rw[o] + (k - st[o]));
+                return true;
+            });
         __syncwarp();   // the next chunk rewrites the row tables
     }
-    Q.flush(lane);
 }
 
-// One BFS level, long rows: slice t of the level's long rows is entries
-// [t - long_base[r]) * kSlice, ...) of row r, the last row whose base is at
-// or below t. Warps take slices t = warp, warp + warps, ...; a warp finds r
-// by a 32-way search (each round the lanes test 32 evenly spaced bases and
-// a ballot keeps the interval below the first base above t), then walks the
-// slice 32 entries per step with the same claims as the level kernel.
+// A top-down level's long rows: slice t of them is entries [t - long_base[r])
+// * slice, ...) of row r, the last row whose base is at or below t. Warps take
+// slices t = warp, warp + warps, ...; a warp finds r by a 32-way search (each
+// round the lanes test 32 evenly spaced bases and a ballot keeps the interval
+// below the first base above t), then walks the slice.
 template <typename Id>
-__global__ void __launch_bounds__(kBfsWarps * 32) bfs_long_kernel(const uint64_t* __restrict__ row_ptr,
-                                                       const Id* __restrict__ col,
-                                                       uint32_t* __restrict__ next,
-                                                       uint32_t* __restrict__ nsize,
-                                                       uint32_t* __restrict__ dist,
-                                                       uint32_t* __restrict__ vis, uint32_t level,
-                                                       uint64_t N,
-                                                       const unsigned long long* __restrict__ long_ctr,
-                                                       const uint32_t* __restrict__ long_v,
-                                                       const uint32_t* __restrict__ long_base)
+__device__ __forceinline__ void bfs_long_rows(const uint64_t* __restrict__ row_ptr,
+                                              const Id* __restrict__ col, BfsQueue& Q,
+                                              unsigned long long ctr, uint32_t slice,
+                                              const uint32_t* long_v, const uint32_t* long_base)
 {
-    __shared__ uint32_t wbuf[kBfsWarps][64];
-    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint64_t N = Q.N;
+    const uint32_t lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
-    const unsigned long long ctr = *long_ctr;   // written by the level kernel before
     const uint32_t rows = (uint32_t)(ctr >> 32), slices = (uint32_t)ctr;
-    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
-    BfsQueue Q{wbuf[wid], 0, next, nsize, dist, vis, level, N};
-    for (uint32_t t = blockIdx.x * (blockDim.x >> 5) + wid; t < slices; t += warps) {
+    const uint32_t warps = gridDim.x * kBfsWarps;
+    for (uint32_t t = blockIdx.x * kBfsWarps + (threadIdx.x >> 5); t < slices; t += warps) {
         uint32_t lo = 0, n = rows;   // r lies in [lo, lo + n); long_base[lo] <= t
         while (n > 1) {
             const uint32_t step = (n + 31) / 32;
             const uint32_t off = lane * step;
-            const bool le = off < n && PG_CHECK(lo + off, rows) && long_base[lo + off] <= t;
+            const bool le = off < n && PG_CHECK(lo + off, rows) && __ldcg(long_base + lo + off) <= t;
             const uint32_t m = __ballot_sync(0xFFFFFFFFu, le);   // lane 0 always set
             const uint32_t k = 31 - __clz(m);
             lo += k * step;
             n = (n - k * step < step) ? n - k * step : step;
         }
         uint64_t e0 = 0, e1 = 0;
-        if (PG_CHECK(lo, rows) && PG_CHECK(long_v[lo], N)) {
-            const uint32_t v = long_v[lo];
-            const uint64_t a = row_ptr[v], end = row_ptr[v + 1];
-            e0 = a + (uint64_t)(t - long_base[lo]) * kSlice;
-            e1 = (e0 + kSlice < end) ? e0 + kSlice : end;
-            if (e0 > e1) e0 = e1;
-        }
-        for (uint64_t e = e0; e < e1; e += 32) {
-            bool have = false;
-            uint32_t u = 0;
-            if (e + lane < e1) {
-                const uint64_t u64 = load_streaming(col + e + lane);
-                have = u64 < N;
-                u = (uint32_t)u64;
+        if (PG_CHECK(lo, rows)) {
+            const uint32_t v = __ldcg(long_v + lo);
+            if (PG_CHECK(v, N)) {
+                const uint64_t a = row_ptr[v], end = row_ptr[v + 1];
+                e0 = a + (uint64_t)(t - __ldcg(long_base + lo)) * slice;
+                e1 = (e0 + slice < end) ? e0 + slice : end;
+                if (e0 > e1) e0 = e1;
             }
-            Q.step(have, u, lane, lt);
         }
+        for (uint64_t e = e0; e < e1; e += 64)
+            bfs_claim_two(Q, N, lane, lt, [&](int k, uint64_t& u) {
+                if (e + 32 * k + lane >= e1) return false;
+                u = load_streaming(col + e + 32 * k + lane);
+                return true;
+            });
     }
-    Q.flush(lane);
+}
+
+// Top-down levels from (level, fsize) on, in one cooperative launch with a
+// grid barrier between levels instead of a launch and a host round trip (a
+// level of a small frontier is a few microseconds of latency): until the
+// frontier is empty, or until bottom-up would be chosen on an undirected
+// graph (never for the first level). Leaves where it stopped in the state.
+template <typename Id>
+__global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_top_down_kernel(
+    const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, uint32_t* f0, uint32_t* f1,
+    uint32_t cur, uint32_t fsize, uint64_t visited, uint32_t level, uint32_t undirected,
+    uint32_t* dist, uint32_t* vis, uint64_t N, uint32_t* long_v, uint32_t* long_base,
+    BfsState* state)
+{
+    __shared__ uint32_t wbuf[kBfsWarps][64];
+    __shared__ uint64_t wstart[kBfsWarps][32];   // the rows' starts in the concatenation
+    __shared__ uint64_t wrow[kBfsWarps][32];     // and in col
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t epoch = 0;
+    for (bool first = true; fsize > 0; first = false) {
+        if (visited >= N) {   // nothing left to find: the last level is empty
+            fsize = 0;
+            ++level;
+            break;
+        }
+        if (!first && undirected && (uint64_t)fsize * 30 > N - visited) break;
+        uint32_t* frontier = cur ? f1 : f0;
+        uint32_t* next = cur ? f0 : f1;
+        const uint32_t slot = level & 3, after = (level + 1) & 3;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            state->size[after] = 0;
+            state->longs[after] = 0;
+        }
+        BfsQueue Q{wbuf[wid], 0, next, &state->size[slot], dist, vis, level, N};
+        bfs_short_rows(row_ptr, col, frontier, fsize, Q, wstart[wid], wrow[wid],
+                       &state->longs[slot], long_v, long_base);
+        Q.flush(lane);
+        if (!grid_barrier(state, epoch)) return;
+        const unsigned long long ctr = __ldcg(&state->longs[slot]);
+        if (ctr) {   // the same in every CTA
+            Q.held = 0;
+            bfs_long_rows(row_ptr, col, Q, ctr, slice_of(fsize), long_v, long_base);
+            Q.flush(lane);
+            if (!grid_barrier(state, epoch)) return;
+        }
+        fsize = __ldcg(&state->size[slot]);
+        visited += fsize;
+        cur ^= 1;
+        ++level;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        state->level = level;
+        state->fsize = fsize;
+        state->cur = cur;
+        state->visited = visited;
+    }
+}
+
+// The frontier of `level` as a bitmap, from the distances.
+__global__ void __launch_bounds__(256) bfs_bitmap_kernel(const uint32_t* __restrict__ dist,
+                                                         uint32_t level, uint64_t N,
+                                                         uint32_t* __restrict__ bits)
+{
+    constexpr int kU = 8;   // words in flight per warp
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    for (uint64_t b = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32 * kU); b < N;
+         b += warps * (32 * kU)) {
+        uint32_t d[kU], mine = 0;
+#pragma unroll
+        for (int t = 0; t < kU; ++t) {
+            const uint64_t v = b + 32 * t + lane;
+            d[t] = v < N ? dist[v] : 0xFFFFFFFFu;
+        }
+#pragma unroll
+        for (int t = 0; t < kU; ++t) {
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, d[t] == level);
+            if (lane == (uint32_t)t) mine = m;
+        }
+        if (lane < kU && b + 32 * lane < N) bits[(b >> 5) + lane] = mine;
+    }
+}
+
+// The vertices of a bitmap as a list (in any order), *count of them.
+__global__ void __launch_bounds__(256) bfs_list_kernel(const uint32_t* __restrict__ bits, uint64_t N,
+                                                       uint32_t* __restrict__ list,
+                                                       uint32_t* __restrict__ count)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t words = (N + 31) / 32, stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t w0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); w0 < words;
+         w0 += stride) {
+        const uint64_t w = w0 + lane;
+        uint32_t m = w < words ? bits[w] : 0u;
+        uint32_t incl = __popc(m);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= (uint32_t)o) incl += y;
+        }
+        uint32_t at = 0;
+        if (lane == 31 && incl) at = atomicAdd(count, incl);
+        at = __shfl_sync(0xFFFFFFFFu, at, 31) + incl - __popc(m);
+        for (; m; m &= m - 1, ++at)
+            if (PG_CHECK(at, N)) list[at] = (uint32_t)(w * 32 + __ffs(m) - 1);
+    }
 }
 
 // One BFS level bottom-up (Beamer, Asanovic and Patterson, "Direction-
 // Optimizing Breadth-First Search", SC'12), for a symmetric CSR: every vertex
-// not yet visited looks through its row for a neighbour at distance `level`
-// and, at the first one, takes distance level + 1. A warp owns 32 consecutive
-// vertices, one visited word, and sets their new bits with one plain store:
-// no other warp writes that word during the level. A neighbour claimed in
-// the same level already reads level + 1, so it is never taken for a parent.
+// not yet visited looks through its row for a neighbour in the frontier and,
+// at the first one, takes distance level + 1. The frontier is a bitmap (2 MB
+// for 2^24 vertices, in L2, where the distances, 64 MB, miss: the widest level
+// of 2^24 vertices took 0.64-0.87 ms with those, 0.33-0.56 now, bound by the
+// L2's sectors). A warp owns the 32 vertices of a word: one visited word and
+// one word of the next frontier's bitmap, written with plain stores, as no
+// other warp writes them during the level. It looks at eight words at once, so
+// that late levels, whose words are full, cost no wait per word; the words are
+// a grid stride apart, since neighbouring ids share hubs (eight neighbouring
+// words: 0.95 ms).
 template <typename Id>
 __global__ void __launch_bounds__(kBfsWarps * 32) bfs_bottom_up_kernel(
-    const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, uint32_t* __restrict__ next,
-    uint32_t* __restrict__ nsize, uint32_t* __restrict__ dist, uint32_t* __restrict__ vis,
-    uint32_t level, uint64_t N)
+    const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col,
+    const uint32_t* __restrict__ front, uint32_t* __restrict__ next, uint32_t* __restrict__ nsize,
+    uint32_t* __restrict__ dist, uint32_t* __restrict__ vis, uint32_t level, uint64_t N)
 {
-    __shared__ uint32_t wbuf[kBfsWarps][64];
-    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
+    constexpr uint32_t kWords = 8;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t words = (N + 31) / 32;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    BfsQueue Q{wbuf[wid], 0, next, nsize, dist, vis, level, N};
-    for (uint64_t base = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < N;
-         base += warps * 32) {
-        const uint64_t v = base + lane;
-        const uint32_t word = vis[base >> 5];
-        bool found = false;
-        if (v < N && ((word >> lane) & 1u) == 0) {
-            const uint64_t b = row_ptr[v + 1];
-            for (uint64_t e = row_ptr[v]; e < b; ++e) {
-                const uint64_t u = load_streaming(col + e);
-                if (u < N && dist[u] == level) {
-                    found = true;
-                    break;
+    uint32_t found_all = 0;
+    for (uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w0 < words;
+         w0 += warps * kWords) {
+        // lane t < kWords keeps word w0 + t * warps (neighbouring vertices, hubs
+        // among them, go to different warps); past the last vertex every bit
+        // is set
+        const uint64_t my_w = w0 + lane * warps;
+        const bool has = lane < kWords && my_w < words;
+        uint32_t mine = 0xFFFFFFFFu, out = 0;
+        if (has) {
+            mine = vis[my_w];
+            const uint64_t left = N - my_w * 32;
+            if (left < 32) mine |= ~0u << left;
+        }
+        uint32_t todo = __ballot_sync(0xFFFFFFFFu, mine != 0xFFFFFFFFu);
+        for (; todo; todo &= todo - 1) {
+            const uint32_t t = __ffs(todo) - 1;
+            const uint32_t word = __shfl_sync(0xFFFFFFFFu, mine, t);
+            const uint64_t v = (w0 + t * warps) * 32 + lane;
+            bool found = false;
+            if (((word >> lane) & 1u) == 0) {
+                const uint64_t b = row_ptr[v + 1];
+                for (uint64_t e = row_ptr[v]; e < b; ++e) {
+                    const uint64_t u = __ldg(col + e);
+                    if (u < N && ((front[u >> 5] >> (u & 31)) & 1u)) {
+                        found = true;
+                        break;
+                    }
                 }
             }
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, found);
+            if (found) dist[v] = level + 1;
+            if (lane == t) out = m;
+            found_all += __popc(m);
         }
-        const uint32_t m = __ballot_sync(0xFFFFFFFFu, found);
-        if (found) dist[v] = level + 1;
-        if (lane == 0 && m) vis[base >> 5] = word | m;
-        Q.push(found, (uint32_t)v, lane, lt);
+        if (has) {
+            next[my_w] = out;
+            if (out) vis[my_w] = mine | out;
+        }
     }
-    Q.flush(lane);
+    if (lane == 0 && found_all) atomicAdd(nsize, found_all);
 }
 
 // scanned = the sum of the reached vertices' row lengths (what a top-down
@@ -319,10 +520,23 @@ __global__ void __launch_bounds__(256) bfs_reach_kernel(const uint64_t* __restri
                                                         uint64_t N,
                                                         unsigned long long* __restrict__ scanned)
 {
+    constexpr int kU = 4;   // vertices in flight per thread
     unsigned long long sum = 0;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += stride)
-        if (dist[v] != 0xFFFFFFFFu) sum += row_ptr[v + 1] - row_ptr[v];
+    for (uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v0 < N; v0 += kU * stride) {
+        uint64_t a[kU], b[kU];
+        uint32_t d[kU];
+#pragma unroll
+        for (int t = 0; t < kU; ++t) {
+            const uint64_t v = v0 + t * stride < N ? v0 + t * stride : N - 1;
+            d[t] = v0 + t * stride < N ? dist[v] : 0xFFFFFFFFu;
+            a[t] = row_ptr[v];
+            b[t] = row_ptr[v + 1];
+        }
+#pragma unroll
+        for (int t = 0; t < kU; ++t)
+            if (d[t] != 0xFFFFFFFFu) sum += b[t] - a[t];
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xFFFFFFFFu, sum, o);
     if ((threadIdx.x & 31) == 0 && sum) atomicAdd(scanned, sum);
@@ -342,6 +556,39 @@ int grid_cap(uint64_t items)
     const uint64_t full = (uint64_t)device_sm_count() * 8;
     const uint64_t need = (items + 255) / 256;
     return (int)(need < 1 ? 1 : (need < full ? need : full));
+}
+
+// Top-down levels from the host's state h on, in one cooperative launch: every
+// CTA resident, and no more of them than the graph can use.
+template <typename Id>
+cudaError_t launch_top_down(const uint64_t* row_ptr, const Id* col, uint32_t* const* fr,
+                            const BfsState& h, uint32_t undirected, uint32_t* dist, uint32_t* vis,
+                            uint64_t N, uint32_t* long_v, uint32_t* long_base, BfsState* state,
+                            cudaStream_t s)
+{
+    int per_sm = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bfs_top_down_kernel<Id>,
+                                                                  kBfsWarps * 32, 0);
+    if (e != cudaSuccess) return e;
+    // four CTAs per SM where levels are short (a barrier of 608 CTAs instead of
+    // 1216: 2^20 vertices 0.350 -> 0.237 ms per search); all that fit where wide
+    // levels run top-down (2^24 vertices, directed: 3.26 -> 3.08 ms)
+    if (per_sm > 4 && (undirected || N <= (1u << 22))) per_sm = 4;
+    const uint64_t full = (uint64_t)device_sm_count() * (per_sm > 0 ? per_sm : 1);
+    const uint64_t want = (N + 63) / 64;
+    const unsigned grid = (unsigned)(want < full ? want : full);
+    // the counters and the barrier start at zero; scanned and error are kept
+    e = cudaMemsetAsync(state, 0, offsetof(BfsState, scanned), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(&state->arrived, 0, 4, s);
+    if (e != cudaSuccess) return e;
+    uint32_t *f0 = fr[0], *f1 = fr[1], cur = h.cur, fsize = h.fsize, level = h.level;
+    unsigned long long visited = h.visited;
+    void* args[] = {&row_ptr, &col,  &f0,  &f1, &cur,    &fsize,     &visited, &level,
+                    &undirected, &dist, &vis, &N,  &long_v, &long_base, &state};
+    e = cudaLaunchCooperativeKernel((const void*)bfs_top_down_kernel<Id>, dim3(grid),
+                                    dim3(kBfsWarps * 32), args, 0, s);
+    note_launch();
+    return e;
 }
 
 }  // namespace
@@ -409,80 +656,87 @@ pg_status pg_bfs(const uint64_t* d_row_ptr, const void* d_col, uint64_t n_vertic
     const size_t fbytes = ((size_t)n_vertices * 4 + 255) & ~(size_t)255;
     unsigned char* ws = (unsigned char*)d_ws;
     uint32_t* fr[2] = {(uint32_t*)ws, (uint32_t*)(ws + fbytes)};
-    // counters: the next frontier's size and the long-row list's counts,
-    // zeroed every level, then the scanned total
-    uint32_t* nsize = (uint32_t*)(ws + 2 * fbytes);
-    unsigned long long* long_ctr = (unsigned long long*)(ws + 2 * fbytes + 8);
-    unsigned long long* scanned = (unsigned long long*)(ws + 2 * fbytes + 16);
+    BfsState* state = (BfsState*)(ws + 2 * fbytes);
     uint32_t* vis = (uint32_t*)(ws + 2 * fbytes + 256);
     const size_t vbytes = ((size_t)n_vertices + 31) / 32 * 4;
     unsigned char* lists = ws + 2 * fbytes + 256 + ((vbytes + 255) & ~(size_t)255);
+    // the long-row list of top-down levels; bottom-up ones keep the frontier's
+    // and the next frontier's bitmaps there
     uint32_t* long_v = (uint32_t*)lists;
     uint32_t* long_base = (uint32_t*)(lists + fbytes);
     if (cudaMemsetAsync(d_dist, 0xFF, n_vertices * 4, s) != cudaSuccess) return PG_ECUDA;
     if (cudaMemsetAsync(ws + 2 * fbytes, 0, 256, s) != cudaSuccess) return PG_ECUDA;
     if (cudaMemsetAsync(vis, 0, vbytes, s) != cudaSuccess) return PG_ECUDA;
     { bfs_seed_kernel<<<1, 1, 0, s>>>(d_dist, vis, fr[0], (uint32_t)source); note_launch(); }
-    uint32_t fsize = 1, level = 0, cur = 0;
-    uint64_t visited = 1;
-    bool bottom_up = false;
     TraceScope trace("bfs", s);
-    // the slice kernel's grid: every warp of a full wave takes slices
-    const int long_grid = device_sm_count() * 8;
-    const bool undirected = (flags & PG_BFS_UNDIRECTED) != 0;
-    while (fsize > 0) {
-        // direction of this level (Beamer et al.'s rule with vertex counts
-        // standing in for edge counts): bottom-up once the frontier is more
-        // than 1/30 of the vertices not yet visited, top-down again once it
-        // is under 1/24 of all vertices
-        if (undirected) {
-            if (!bottom_up && (uint64_t)fsize * 30 > n_vertices - visited) bottom_up = true;
-            else if (bottom_up && (uint64_t)fsize * 24 < n_vertices) bottom_up = false;
+    const uint32_t undirected = (flags & PG_BFS_UNDIRECTED) ? 1 : 0;
+    BfsState h;   // the search's state on the host
+    std::memset(&h, 0, sizeof(h));
+    h.fsize = 1;
+    h.visited = 1;
+    auto fetch = [&] {
+        return cudaMemcpyAsync(&h, state, sizeof(h), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
+               cudaStreamSynchronize(s) == cudaSuccess;
+    };
+    // direction of a level (Beamer et al.'s rule with vertex counts standing in
+    // for edge counts): bottom-up once the frontier is more than 1/30 of the
+    // vertices not yet visited, top-down again once it is under 1/24 of all
+    bool bottom_up = undirected && (uint64_t)h.fsize * 30 > n_vertices - h.visited;
+    const uint32_t grid_all = (uint32_t)grid_cap(n_vertices);
+    while (h.fsize > 0) {
+        if (!bottom_up) {
+            const cudaError_t e =
+                w == PG_ID64
+                    ? launch_top_down(d_row_ptr, (const uint64_t*)d_col, fr, h, undirected, d_dist, vis,
+                                      n_vertices, long_v, long_base, state, s)
+                    : launch_top_down(d_row_ptr, (const uint32_t*)d_col, fr, h, undirected, d_dist, vis,
+                                      n_vertices, long_v, long_base, state, s);
+            if (e != cudaSuccess || !fetch()) return PG_ECUDA;
+            if (h.error) return PG_ETIMEOUT;
+            bottom_up = true;   // or the search is over
+            continue;
         }
-        if (cudaMemsetAsync(nsize, 0, 16, s) != cudaSuccess) return PG_ECUDA;
-        if (bottom_up) {
-            TraceScope bu_trace("bfs_bottom_up", s);
-            const int grid = grid_cap(n_vertices);
+        TraceScope bu_trace("bfs_bottom_up", s);
+        uint32_t *front = long_v, *next = long_base;
+        { bfs_bitmap_kernel<<<grid_all, 256, 0, s>>>(d_dist, h.level, n_vertices, front); note_launch(); }
+        do {
+            if (cudaMemsetAsync(&state->size[0], 0, 4, s) != cudaSuccess) return PG_ECUDA;
             if (w == PG_ID64)
-                { bfs_bottom_up_kernel<uint64_t><<<grid, kBfsWarps * 32, 0, s>>>(
-                    d_row_ptr, (const uint64_t*)d_col, fr[cur ^ 1], nsize, d_dist, vis, level,
+                { bfs_bottom_up_kernel<uint64_t><<<grid_all, kBfsWarps * 32, 0, s>>>(
+                    d_row_ptr, (const uint64_t*)d_col, front, next, &state->size[0], d_dist, vis, h.level,
                     n_vertices); note_launch(); }
             else
-                { bfs_bottom_up_kernel<uint32_t><<<grid, kBfsWarps * 32, 0, s>>>(
-                    d_row_ptr, (const uint32_t*)d_col, fr[cur ^ 1], nsize, d_dist, vis, level,
+                { bfs_bottom_up_kernel<uint32_t><<<grid_all, kBfsWarps * 32, 0, s>>>(
+                    d_row_ptr, (const uint32_t*)d_col, front, next, &state->size[0], d_dist, vis, h.level,
                     n_vertices); note_launch(); }
-        } else {
-            const int grid = grid_cap(fsize);
-            if (w == PG_ID64) {
-                { bfs_level_kernel<uint64_t><<<grid, kBfsWarps * 32, 0, s>>>(
-                    d_row_ptr, (const uint64_t*)d_col, fr[cur], fsize, fr[cur ^ 1], nsize, d_dist,
-                    vis, level, n_vertices, long_ctr, long_v, long_base); note_launch(); }
-                { bfs_long_kernel<uint64_t><<<long_grid, kBfsWarps * 32, 0, s>>>(
-                    d_row_ptr, (const uint64_t*)d_col, fr[cur ^ 1], nsize, d_dist, vis, level,
-                    n_vertices, long_ctr, long_v, long_base); note_launch(); }
-            } else {
-                { bfs_level_kernel<uint32_t><<<grid, kBfsWarps * 32, 0, s>>>(
-                    d_row_ptr, (const uint32_t*)d_col, fr[cur], fsize, fr[cur ^ 1], nsize, d_dist,
-                    vis, level, n_vertices, long_ctr, long_v, long_base); note_launch(); }
-                { bfs_long_kernel<uint32_t><<<long_grid, kBfsWarps * 32, 0, s>>>(
-                    d_row_ptr, (const uint32_t*)d_col, fr[cur ^ 1], nsize, d_dist, vis, level,
-                    n_vertices, long_ctr, long_v, long_base); note_launch(); }
+            if (cudaGetLastError() != cudaSuccess) return PG_ECUDA;
+            // the next frontier's size decides whether and how another level runs
+            if (cudaMemcpyAsync(&h.fsize, &state->size[0], 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                cudaStreamSynchronize(s) != cudaSuccess)
+                return PG_ECUDA;
+            h.visited += h.fsize;
+            ++h.level;
+            std::swap(front, next);
+            if (h.fsize > 0 && h.visited >= n_vertices) {   // the last level finds nothing
+                h.fsize = 0;
+                ++h.level;
             }
+        } while (h.fsize > 0 && (uint64_t)h.fsize * 24 >= n_vertices);
+        bottom_up = false;
+        if (h.fsize > 0) {
+            // top-down again: the bitmap's vertices as a list
+            if (cudaMemsetAsync(&state->size[0], 0, 4, s) != cudaSuccess) return PG_ECUDA;
+            { bfs_list_kernel<<<grid_cap((n_vertices + 31) / 32), 256, 0, s>>>(front, n_vertices, fr[0],
+                                                                              &state->size[0]); note_launch(); }
+            h.cur = 0;
         }
-        if (cudaGetLastError() != cudaSuccess) return PG_ECUDA;
-        // the next frontier's size decides whether another level runs
-        if (cudaMemcpyAsync(&fsize, nsize, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess)
-            return PG_ECUDA;
-        visited += fsize;
-        cur ^= 1;
-        ++level;
     }
-    { bfs_reach_kernel<<<grid_cap(n_vertices), 256, 0, s>>>(d_row_ptr, d_dist, n_vertices, scanned); note_launch(); }
+    { bfs_reach_kernel<<<grid_all, 256, 0, s>>>(d_row_ptr, d_dist, n_vertices, &state->scanned); note_launch(); }
     uint64_t sc = 0;
-    if (cudaMemcpyAsync(&sc, scanned, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    if (cudaMemcpyAsync(&sc, &state->scanned, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return PG_ECUDA;
+    const uint32_t level = h.level;
     if (levels_out) *levels_out = level;
     if (scanned_out) *scanned_out = sc;
     return PG_OK;

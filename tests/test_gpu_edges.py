@@ -205,3 +205,41 @@ def test_csr_rows_without_edges(N, off):
     assert np.array_equal(host(buf[off:off + N + 1]), ref_rp)
     assert np.array_equal(host(col), ref_col)
     assert (buf[off + N + 1:] == -7).all() and (off == 0 or int(buf[0]) == -7)
+
+
+@pytest.mark.parametrize("N", [1, 2, 31, 32, 33, 255, 256, 257, 2500, 70_001])
+@pytest.mark.parametrize("id64", [False, True])
+def test_bfs_around_words_and_switches(N, id64):
+    """Random graphs whose searches switch direction both ways, at vertex
+    counts around a bitmap word and a warp's words; a hub with more slices of
+    a narrow and of a wide level than one row may have; unreached vertices."""
+    rng = np.random.default_rng(N)
+    e = rng.integers(0, max(N - N // 7, 1), size=(3 * N, 2), dtype=np.uint64)
+    chain = np.arange(N - N // 7, N - 1, dtype=np.uint64)      # a long tail of narrow levels
+    e = np.concatenate([e, np.stack([chain[::2], chain[::2] + 1], 1)]) if N > 60 else e
+    hub = np.stack([np.full(N // 3, N // 2), rng.integers(0, N, N // 3)], 1).astype(np.uint64)
+    e = np.concatenate([e, hub])
+    for flags in (0, o.CSR_SYMMETRIZE):
+        rp_h, col_h = o.csr_opts(e, N, flags)
+        rp = torch.from_numpy(rp_h.view(np.int64)).cuda()
+        col = torch.from_numpy(col_h.astype(np.uint64 if id64 else np.uint32)
+                               .view(np.int64 if id64 else np.int32)).cuda()
+        for s in {0, N // 2, N - 1}:
+            ref = o.bfs(rp_h, col_h, s)
+            for undirected in ([False, True] if flags else [False]):
+                dist, levels, scanned = pg.bfs(rp, col, s, undirected=undirected)
+                assert np.array_equal(dist.cpu().numpy().view(np.uint32), ref[0]), (s, flags)
+                assert (levels, scanned) == ref[1:], (s, flags, undirected)
+
+
+@pytest.mark.parametrize("which", [pg.DEG_OUT, pg.DEG_IN, pg.DEG_TOTAL])
+@pytest.mark.parametrize("M", [1, 31, 32, 33, 1000])
+def test_degrees_of_grouped_sources(which, M):
+    """Runs of one source inside a warp, across warps and at the list's end;
+    sources past the vertex count."""
+    rng = np.random.default_rng(M)
+    src = np.repeat(np.arange(M), 1 + np.arange(M) % 40)[:M]
+    e = np.stack([src, rng.integers(0, 12, M)], 1).astype(np.uint32)
+    N = max(int(src.max()), 1)                                  # the last source is outside
+    deg = pg.degrees(torch.from_numpy(e.view(np.int32)).cuda(), N, which)
+    assert np.array_equal(host(deg), o.degrees(e.astype(np.uint64), N, which))
