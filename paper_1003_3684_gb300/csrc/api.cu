@@ -104,6 +104,8 @@ PbaGeom make_geom(uint64_t n_b, uint64_t N_e, uint32_t m, uint32_t B, uint32_t n
     }
     g.div_m = make_fastdiv(m);
     g.div_m32 = make_fastdiv32(m);
+    if (m > 1 && (u128)N_e * m <= ((u128)1 << 32))
+        g.mul_m = (uint32_t)((((uint64_t)1 << 32) + m - 1) / m);
     g.div_nb = make_fastdiv(n_b > 0 ? n_b : 1);
     return g;
 }

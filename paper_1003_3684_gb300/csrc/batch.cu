@@ -51,7 +51,8 @@ struct BatchJob {              // 256 bytes, one per job
     uint64_t csr_edge;         // want_csr: first col entry of the job (and its union slot)
     uint64_t rbase;            // want_csr: first row_ptr entry of the job
     uint64_t edges;            // the job's edges: [out_edge, out_edge + edges) of the arena
-    uint8_t reserved[256 - 80 - 88 - 40];
+    uint32_t mul_m;            // BA: ceil(2^32 / m) when j div m is its product's high word, else 0
+    uint8_t reserved[256 - 80 - 88 - 40 - 4];
 };
 static_assert(sizeof(BatchJob) == 256, "job record is 256 bytes");
 
@@ -116,27 +117,31 @@ __device__ __forceinline__ void put_two(Id* out, uint64_t cap, uint64_t e, uint6
     }
 }
 
-// One serial-BA link with 32-bit indices (as in the single-graph kernel).
-__device__ __forceinline__ bool ba_link(uint32_t& cur, const BatchJob& J, const Key& key,
-                                        const PhiloxHead& ph, uint32_t& v)
+// One serial-BA link with 32-bit indices, sigma(cur) = cur div m carried from
+// link to link (as in the single-graph kernel). The job's numbers are the
+// caller's registers.
+struct BaJob {
+    uint32_t e0, m, n0, mul_m;
+    FastDiv32 div_m;
+    __device__ __forceinline__ uint32_t div(uint32_t j) const
+    {
+        return mul_m ? __umulhi(j, mul_m) : fdiv32(j, div_m);
+    }
+};
+__device__ __forceinline__ bool ba_link(uint32_t& cur, uint32_t& sig, const BaJob& J,
+                                        const Key& key, const PhiloxHead& ph, uint32_t& v)
 {
-    const uint32_t sig = fdiv32(cur, J.div_m);
     const uint4 w = philox_headed(cur, ph, key);   // counter (cur, 0, 0, 2)
-    const uint32_t X = (uint32_t)J.e0 + sig * J.m;
+    const uint32_t X = J.e0 + sig * J.m;
     const uint64_t s = (uint64_t)w.y * X + (((uint64_t)w.x * X) >> 32);
     const uint32_t e = (uint32_t)(s >> 32);
     const uint32_t side = ((uint32_t)s) >> 31;
-    if (e < (uint32_t)J.e0) {
-        v = seed_endpoint(e, side, J.n0);
-        return true;
-    }
-    const uint32_t e2 = e - (uint32_t)J.e0;
-    if (side == 0) {
-        v = J.n0 + fdiv32(e2, J.div_m);
-        return true;
-    }
-    cur = e2;
-    return false;
+    const bool seed = e < J.e0;
+    cur = e - J.e0;
+    sig = J.div(cur);
+    v = J.n0 + sig;
+    if (seed) v = seed_endpoint(e, side, J.n0);
+    return seed || side == 0;
 }
 
 // Any initiator, any number of edges: the order-2 thresholds from the job's
@@ -261,35 +266,37 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(const unsigned cha
             const uint32_t r0 = wid * per < n ? wid * per : n;
             const uint32_t r1 = r0 + per < n ? r0 + per : n;
             const uint32_t n_items_w = r1 - r0;
+            const BaJob B{(uint32_t)J.e0, J.m, J.n0, J.mul_m, J.div_m};
+            const uint32_t first = (uint32_t)t0 + r0;
             uint32_t next = 32, item = lane;
-            uint32_t cur = (uint32_t)(t0 + r0 + item);
+            uint32_t cur = first + item, sig = B.div(cur);
             bool active = item < n_items_w;
             const PhiloxHead ph = philox_head(0u, 0u, 2u, key);
-            while (__any_sync(0xFFFFFFFFu, active)) {
-                bool done = false;
-                if (active) {
-                    uint32_t v;
-                    done = ba_link(cur, J, key, ph, v);
-                    if (done && PG_CHECK(r0 + item, kMaxTile)) sDst[r0 + item] = (Id)v;
-                }
+            auto trip = [&] {
+                uint32_t v;
+                const bool done = ba_link(cur, sig, B, key, ph, v) && active;
+                if (done && PG_CHECK(r0 + item, kMaxTile)) sDst[r0 + item] = (Id)v;
                 const uint32_t dm = __ballot_sync(0xFFFFFFFFu, done);
                 if (done) {
                     item = next + __popc(dm & lt);
-                    cur = (uint32_t)(t0 + r0 + item);
+                    cur = first + item;
+                    sig = B.div(cur);
                     active = item < n_items_w;
                 }
                 next += __popc(dm);
-            }
+            };
+            while (next < n_items_w) trip();
+            while (__any_sync(0xFFFFFFFFu, active)) trip();
             __syncthreads();
             const uint64_t e_first = J.out_edge + J.e0 + t0;
             const uint32_t head = (uint32_t)(e_first & 1) < n ? (uint32_t)(e_first & 1) : n;
             if (head && threadIdx.x == 0)
-                put_pair(arena, cap, e_first, J.n0 + fdiv32((uint32_t)t0, J.div_m), (uint64_t)sDst[0]);
+                put_pair(arena, cap, e_first, J.n0 + B.div((uint32_t)t0), (uint64_t)sDst[0]);
             for (uint32_t t2 = head + 2 * threadIdx.x; t2 < n; t2 += 2 * blockDim.x) {
-                const uint64_t s0 = J.n0 + fdiv32((uint32_t)(t0 + t2), J.div_m);
+                const uint64_t s0 = J.n0 + B.div((uint32_t)(t0 + t2));
                 if (t2 + 1 < n)
                     put_two(arena, cap, e_first + t2, s0, (uint64_t)sDst[t2],
-                            J.n0 + fdiv32((uint32_t)(t0 + t2 + 1), J.div_m), (uint64_t)sDst[t2 + 1]);
+                            J.n0 + B.div((uint32_t)(t0 + t2 + 1)), (uint64_t)sDst[t2 + 1]);
                 else
                     put_pair(arena, cap, e_first + t2, s0, (uint64_t)sDst[t2]);
             }
@@ -542,6 +549,8 @@ pg_status pg_batch_plan(const pg_job* jobs, uint32_t n_jobs, uint32_t tile_edges
             b.n0 = q.n0;
             b.n_units = (uint64_t)ne;
             b.div_m = make_fastdiv32(q.m);
+            if (q.m > 1 && ne * q.m <= ((unsigned __int128)1 << 32))
+                b.mul_m = (uint32_t)((((uint64_t)1 << 32) + q.m - 1) / q.m);
             b.edges = b.e0 + b.n_units;
             b.n_vertices = (uint64_t)q.n0 + q.n;
             job_items = (b.n_units + tile_edges - 1) / tile_edges;

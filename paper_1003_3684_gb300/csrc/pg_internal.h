@@ -116,6 +116,7 @@ struct PbaGeom {
     uint64_t lean_add;             // (n_b - 1) + e0 * n_b when n_b is a power of two
     FastDiv div_m, div_nb;
     FastDiv32 div_m32;             // j div m for j < 2^32
+    uint32_t mul_m, pad;           // ceil(2^32 / m) when j div m is its product's high word, else 0
     const uint16_t* ftab;          // faction table (device), or null: aligned width-W factions
 };
 
