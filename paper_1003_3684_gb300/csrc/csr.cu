@@ -9,7 +9,7 @@
 // marks each row's end in row_ptr.
 //
 // Any other list: least-significant-digit radix sort of the (src, dst) keys,
-// from the low bits of dst to the high bits of src, up to 8 bits per pass:
+// from the low bits of dst to the high bits of src, up to 8 bits per pass (9 for short lists):
 //   radix_hist_all one read of the list counts the digits of every pass
 //                  (the totals do not depend on the order a pass leaves);
 //   radix_dstart   per pass, where each digit's run starts in the output;
@@ -42,8 +42,6 @@ namespace {
 constexpr int kSortWarps = 16;
 constexpr int kFly = 2;   // items a warp ranks at a time
 constexpr int kSortThreads = kSortWarps * 32;
-constexpr int kMaxDigitBits = 8;
-constexpr uint32_t kMaxBuckets = 1u << kMaxDigitBits;
 constexpr uint32_t kScanTile = 4096;
 constexpr uint32_t kGroupedMaxRow = 32;
 constexpr uint32_t kHistCopies = 8;   // copies of each digit counter in the histogram kernel
@@ -100,12 +98,20 @@ struct PairList {
     }
 };
 
-// Elements per thread of a sort tile: 16 pairs of 32-bit ids or 8 of 64-bit.
-template <typename K>
+// A sort tile and the widest digit. Long lists: 16 pairs of 32-bit ids (8 of
+// 64-bit) per thread and digits of at most 8 bits. Short lists, up to
+// kShortList pairs, are fewer tiles than the GPU has places, so a pass takes a
+// tile's latency: tiles of half the size, and digits of 9 bits for fewer
+// passes (100,003 pairs, k = 13: 0.088 -> 0.071 ms, 2^19 pairs: 0.114 -> 0.108;
+// 2^20 pairs lose, 0.120 -> 0.135).
+template <typename K, bool kShort>
 struct SortShape {
-    static constexpr int items = sizeof(K) == 8 ? 16 : 8;
+    static constexpr int items = (sizeof(K) == 8 ? 16 : 8) / (kShort ? 2 : 1);
     static constexpr uint32_t tile = kSortThreads * items;
+    static constexpr uint32_t buckets = kShort ? 512 : 256;
 };
+constexpr uint32_t kMaxBuckets = 512;
+constexpr uint64_t kShortList = 3u << 18;
 
 // The digits of every LSD pass, from the host: pass k sorts by `bits[k]`
 // bits of the destination (field 0) or source (field 1) at `shift[k]`, or
@@ -114,7 +120,8 @@ struct SortShape {
 constexpr int kMaxPasses = 16;   // 64-bit ids: 128 key bits in digits of 8
 struct PassList {
     uint32_t n;
-    int nd;   // bits of the dst field
+    uint32_t buckets;   // of the widest digit: stride of the passes' tables
+    int nd;             // bits of the dst field
     int field[kMaxPasses], shift[kMaxPasses], bits[kMaxPasses];
     __host__ __device__ Digit digit(uint32_t k) const
     {
@@ -123,7 +130,7 @@ struct PassList {
 };
 // Digit totals of every pass in one read of the list: tot[k][d] = number of
 // pairs whose pass-k digit is d. Each CTA counts into shared memory
-// (n passes x kMaxBuckets counters, kHistCopies copies of each) and adds its
+// (n passes x pl.buckets counters, kHistCopies copies of each) and adds its
 // counts once.
 template <typename K, typename In>
 __global__ void __launch_bounds__(256) radix_hist_all_kernel(
@@ -135,7 +142,7 @@ __global__ void __launch_bounds__(256) radix_hist_all_kernel(
     // kHistCopies copies of every counter, interleaved, lane l adding to copy
     // l mod kHistCopies: lanes whose digits agree (the skewed digits of a
     // power-law graph) mostly hit different words
-    const uint32_t cells = pl.n * kMaxBuckets;
+    const uint32_t cells = pl.n * pl.buckets;
     for (uint32_t t = threadIdx.x; t < cells * kHistCopies; t += blockDim.x) h[t] = 0;
     __syncthreads();
     const uint32_t copy = threadIdx.x & (kHistCopies - 1);
@@ -150,7 +157,7 @@ __global__ void __launch_bounds__(256) radix_hist_all_kernel(
         // kU elements
         for (uint32_t k = 0; k < pl.n; ++k) {
             const Digit dg = pl.digit(k);
-            uint32_t* hk = h + (k * kMaxBuckets) * kHistCopies + copy;
+            uint32_t* hk = h + (k * pl.buckets) * kHistCopies + copy;
 #pragma unroll
             for (int u = 0; u < kU; ++u)
                 if (i0 + u * stride < M)
@@ -206,7 +213,7 @@ CsrWaitHook csr_wait_hook() { return CsrWaitHook{g_hook_spin.load(), g_hook_with
 // one word (kSpinLimit unless a test hook shortened it) it sets *err and
 // goes on with the partial sum, which can only be too small, so every write
 // stays inside the output.
-template <typename K, typename In, typename Id>
+template <typename K, typename In, typename Id, bool kShort>
 __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     const In in, K* __restrict__ out, uint64_t M, const Digit dg,
     unsigned long long* __restrict__ status,
@@ -214,13 +221,14 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     uint32_t* __restrict__ err, const uint32_t* __restrict__ sort_needed, uint32_t spin_limit,
     uint32_t withhold, Id* __restrict__ col_out, uint64_t* __restrict__ row_ptr, uint64_t N)
 {
-    constexpr int kItems = SortShape<K>::items;
-    constexpr uint32_t kTile = SortShape<K>::tile;
+    constexpr int kItems = SortShape<K, kShort>::items;
+    constexpr uint32_t kTile = SortShape<K, kShort>::tile;
+    constexpr uint32_t kBuckets = SortShape<K, kShort>::buckets;
     extern __shared__ __align__(16) unsigned char smem[];
-    uint16_t (*wcnt)[kMaxBuckets] = reinterpret_cast<uint16_t (*)[kMaxBuckets]>(smem);   // 8 KB
-    uint64_t* tbase = reinterpret_cast<uint64_t*>(smem + kSortWarps * kMaxBuckets * 2);   // 2 KB
-    uint32_t* loff = reinterpret_cast<uint32_t*>(tbase + kMaxBuckets);                  // 1 KB
-    K* buf = reinterpret_cast<K*>(loff + kMaxBuckets);                                  // tile
+    uint16_t (*wcnt)[kBuckets] = reinterpret_cast<uint16_t (*)[kBuckets]>(smem);
+    uint64_t* tbase = reinterpret_cast<uint64_t*>(smem + kSortWarps * kBuckets * 2);
+    uint32_t* loff = reinterpret_cast<uint32_t*>(tbase + kBuckets);
+    K* buf = reinterpret_cast<K*>(loff + kBuckets);                                  // tile
     __shared__ uint32_t s_part[kSortWarps + 1];
     __shared__ uint32_t s_tile;
     // after a wait that gave up in an earlier pass the list this pass reads
@@ -251,14 +259,14 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     // kFly items of every lane at a time, in lane order within an item: the
     // lanes holding equal digits of an item find each other through a word per
     // digit (each ORs in its lane bit, then all read the word back and clear
-    // it; every item in flight has its own table of kMaxBuckets words per
+    // it; every item in flight has its own table of kBuckets words per
     // warp, in the reorder buffer, unused until the ranks are done). Then, item
     // by item, the lowest lane of each group adds the group's size to the
     // warp's counter of the digit (two 16-bit counters per word) and the group
     // gets the old value by shuffle. A warp's shared-memory operations execute
     // in order, so the adds of the items in flight need no wait between them.
-    uint32_t* pmask = reinterpret_cast<uint32_t*>(buf) + wid * (kFly * kMaxBuckets);
-    for (uint32_t t = lane; t < kFly * kMaxBuckets / 4; t += 32)
+    uint32_t* pmask = reinterpret_cast<uint32_t*>(buf) + wid * (kFly * kBuckets);
+    for (uint32_t t = lane; t < kFly * kBuckets / 4; t += 32)
         reinterpret_cast<uint4*>(pmask)[t] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
     uint32_t* wc = reinterpret_cast<uint32_t*>(wcnt[wid]);
@@ -269,16 +277,16 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
         for (int u = 0; u < kFly; ++u) {
             const uint32_t t = wbase + (r0 + u) * 32 + lane;
             d[u] = t < n ? digit_of(e[r0 + u], dg) : 0xFFFFFFFFu;
-            if (d[u] != 0xFFFFFFFFu) atomicOr(&pmask[u * kMaxBuckets + d[u]], 1u << lane);
+            if (d[u] != 0xFFFFFFFFu) atomicOr(&pmask[u * kBuckets + d[u]], 1u << lane);
         }
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < kFly; ++u)
-            peers[u] = d[u] != 0xFFFFFFFFu ? pmask[u * kMaxBuckets + d[u]] : 0u;
+            peers[u] = d[u] != 0xFFFFFFFFu ? pmask[u * kBuckets + d[u]] : 0u;
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < kFly; ++u) {
-            if (d[u] != 0xFFFFFFFFu) pmask[u * kMaxBuckets + d[u]] = 0;
+            if (d[u] != 0xFFFFFFFFu) pmask[u * kBuckets + d[u]] = 0;
             prev[u] = 0;
             if (peers[u] != 0 && (peers[u] & lt) == 0) {
                 const uint32_t sh = (d[u] & 1) * 16;
@@ -417,19 +425,20 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     }
 }
 
-static_assert(SortShape<uint2>::tile * sizeof(uint2) >= kFly * kSortWarps * kMaxBuckets * 4 &&
-                  SortShape<ulonglong2>::tile * sizeof(ulonglong2) >=
-                      kFly * kSortWarps * kMaxBuckets * 4,
-              "the reorder buffer holds every warp's digit words");
 static_assert(kSortThreads >= (int)kMaxBuckets, "one thread per digit");
-static_assert(SortShape<uint2>::items % kFly == 0 && SortShape<ulonglong2>::items % kFly == 0,
+static_assert(SortShape<uint2, true>::items % kFly == 0 &&
+                  SortShape<ulonglong2, false>::items % kFly == 0,
               "whole groups of items");
 
-template <typename K>
+template <typename K, bool kShort>
 size_t scatter_smem_bytes()
 {
-    return (size_t)kSortWarps * kMaxBuckets * 2 + kMaxBuckets * 8 + kMaxBuckets * 4 +
-           (size_t)SortShape<K>::tile * sizeof(K);
+    using Shape = SortShape<K, kShort>;
+    // the reorder buffer, in which the digit words of the items in flight lie too
+    const size_t tile = (size_t)Shape::tile * sizeof(K);
+    const size_t words = (size_t)kFly * kSortWarps * Shape::buckets * 4;
+    return (size_t)kSortWarps * Shape::buckets * 2 + Shape::buckets * 12 +
+           (tile > words ? tile : words);
 }
 
 // ---- exclusive scan of uint32 counts into uint64 offsets ------------------
@@ -472,7 +481,7 @@ __global__ void __launch_bounds__(256) zero_status_kernel(uint4* __restrict__ p,
         p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 // Where each digit's run starts in pass k's output: the exclusive scan of
-// that pass's digit totals. grid = passes, block = kMaxBuckets threads.
+// that pass's digit totals. grid = passes, block = pl.buckets threads.
 __global__ void __launch_bounds__(kMaxBuckets) radix_dstart_kernel(
     const unsigned long long* __restrict__ tot, const __grid_constant__ PassList pl,
     uint64_t* __restrict__ dstart, const uint32_t* __restrict__ sort_needed)
@@ -480,10 +489,10 @@ __global__ void __launch_bounds__(kMaxBuckets) radix_dstart_kernel(
     __shared__ uint64_t s_warp[32];
     if (*sort_needed == 0) return;
     const uint32_t k = blockIdx.x, nb = 1u << pl.bits[k], d = threadIdx.x;
-    const uint64_t c = d < nb ? tot[(size_t)k * kMaxBuckets + d] : 0;
+    const uint64_t c = d < nb ? tot[(size_t)k * pl.buckets + d] : 0;
     uint64_t total;
     const uint64_t ex = block_exclusive_scan(c, s_warp, total);
-    if (d < nb) dstart[(size_t)k * kMaxBuckets + d] = ex;
+    if (d < nb) dstart[(size_t)k * pl.buckets + d] = ex;
 }
 
 // exclusive scan of n_parts sums in place, one CTA looping over chunks of
@@ -933,19 +942,33 @@ struct CsrLayout {
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Whether the sort moves pairs of 32-bit ids.
+bool ids_narrow(uint64_t n_src, uint64_t n_dst)
+{
+    return n_src <= ((uint64_t)1 << 32) && n_dst <= ((uint64_t)1 << 32);
+}
+
+// Whether the sort of M pairs takes the short-list shape.
+bool short_list(uint64_t M, uint64_t n_src, uint64_t n_dst)
+{
+    return M <= kShortList && ids_narrow(n_src, n_dst);
+}
+
 // The LSD passes that sort pairs by (src, dst): the key (src << nd) | dst,
 // nd = the bits of n_dst - 1 and ns those of n_src - 1, cut from its low end
-// into ceil((nd + ns) / kMaxDigitBits) digits whose widths differ by at most
+// into ceil((nd + ns) / digit_bits) digits whose widths differ by at most
 // one (the wider ones first). A digit inside one id reads that id alone; the
 // one that contains the boundary reads both.
-PassList make_passes(uint64_t n_src, uint64_t n_dst)
+PassList make_passes(uint64_t n_src, uint64_t n_dst, uint64_t M)
 {
     PassList pl;
     std::memset(&pl, 0, sizeof(pl));
     const int nd = bit_length(n_dst > 0 ? n_dst - 1 : 0);
     const int ns = bit_length(n_src > 0 ? n_src - 1 : 0);
     const int total = nd + ns;
-    const int n = (total + kMaxDigitBits - 1) / kMaxDigitBits;
+    const int digit_bits = short_list(M, n_src, n_dst) ? 9 : 8;
+    const int n = (total + digit_bits - 1) / digit_bits;
+    pl.buckets = 1u << digit_bits;
     pl.nd = nd;
     int shift = 0;
     for (int k = 0; k < n; ++k) {
@@ -967,20 +990,17 @@ PassList make_passes(uint64_t n_src, uint64_t n_dst)
     return pl;
 }
 
-// Whether the sort moves pairs of 32-bit ids.
-bool ids_narrow(uint64_t n_src, uint64_t n_dst)
-{
-    return n_src <= ((uint64_t)1 << 32) && n_dst <= ((uint64_t)1 << 32);
-}
-
 CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst = 0)
 {
     CsrLayout L;
-    const PassList pl = make_passes(N, N_dst ? N_dst : N);
-    if (ids_narrow(N, N_dst ? N_dst : N)) pair_bytes = 8;
+    const uint64_t nd = N_dst ? N_dst : N;
+    const PassList pl = make_passes(N, nd, M);
+    if (ids_narrow(N, nd)) pair_bytes = 8;
     int dbits = 0;
     for (uint32_t k = 0; k < pl.n; ++k) dbits = pl.bits[k] > dbits ? pl.bits[k] : dbits;
-    const uint32_t tile = pair_bytes == 8 ? SortShape<uint2>::tile : SortShape<ulonglong2>::tile;
+    const uint32_t tile = pair_bytes != 8 ? SortShape<ulonglong2, false>::tile
+                          : short_list(M, N, nd) ? SortShape<uint2, true>::tile
+                                                 : SortShape<uint2, false>::tile;
     L.max_nb = 1u << dbits;
     L.n_tiles = (uint32_t)((M + tile - 1) / tile);
     L.n_status = (uint64_t)L.max_nb * L.n_tiles;
@@ -1005,33 +1025,35 @@ CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst =
 // The opt-in shared-memory sizes of the sort kernels, set once per device
 // for each id width.
 PerDeviceOnce g_csr_attrs[2];
-template <typename K, typename In, typename Id>
+template <typename K, typename In, typename Id, bool kShort>
 cudaError_t scatter_attribute()
 {
-    return cudaFuncSetAttribute(radix_scatter_kernel<K, In, Id>,
+    return cudaFuncSetAttribute(radix_scatter_kernel<K, In, Id, kShort>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)scatter_smem_bytes<K>());
+                                (int)scatter_smem_bytes<K, kShort>());
 }
 template <typename K, typename In>
 cudaError_t hist_attribute()
 {
     return cudaFuncSetAttribute(radix_hist_all_kernel<K, In>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(kMaxPasses * 4 * kMaxBuckets * kHistCopies));
+                                (int)(kMaxPasses * 4 * 256 * kHistCopies));   // of 256, or 8 of 512
 }
 template <typename Id>
 cudaError_t set_csr_attributes()
 {
     using P = typename PairOf<Id>::T;
     return g_csr_attrs[sizeof(Id) == 8].run_current([] {
-        cudaError_t e = first_error({scatter_attribute<uint2, PairList<uint2, P>, Id>(),
-                                     scatter_attribute<uint2, const uint2*, Id>(),
+        cudaError_t e = first_error({scatter_attribute<uint2, PairList<uint2, P>, Id, false>(),
+                                     scatter_attribute<uint2, const uint2*, Id, false>(),
+                                     scatter_attribute<uint2, PairList<uint2, P>, Id, true>(),
+                                     scatter_attribute<uint2, const uint2*, Id, true>(),
                                      hist_attribute<uint2, PairList<uint2, P>>(),
                                      hist_attribute<uint2, const uint2*>()});
         if constexpr (sizeof(Id) == 8)
             if (e == cudaSuccess)
-                e = first_error({scatter_attribute<P, PairList<P, P>, Id>(),
-                                 scatter_attribute<P, const P*, Id>(),
+                e = first_error({scatter_attribute<P, PairList<P, P>, Id, false>(),
+                                 scatter_attribute<P, const P*, Id, false>(),
                                  hist_attribute<P, PairList<P, P>>(),
                                  hist_attribute<P, const P*>()});
         return e;
@@ -1067,13 +1089,13 @@ cudaError_t radix_passes(const PairList<K, P> first, uint64_t M, uint64_t N, con
     if (M > 0 && cudaMemsetAsync(ws + L.off_flag + 64, 0, 128, s) != cudaSuccess)
         return cudaErrorUnknown;
     if (M > 0 && pl.n > 0) {
-        if (cudaMemsetAsync(tot, 0, (size_t)pl.n * kMaxBuckets * 8, s) != cudaSuccess)
+        if (cudaMemsetAsync(tot, 0, (size_t)pl.n * pl.buckets * 8, s) != cudaSuccess)
             return cudaErrorUnknown;
         {
             TraceScope trace("csr_radix_hist", s);
             { zero_status_kernel<<<sort_grid(L.n_status / 2 + 1), 256, 0, s>>>(
                 (uint4*)status, (L.n_status * 8 + 15) / 16, sort_needed); note_launch(); }
-            const size_t smem = (size_t)pl.n * kMaxBuckets * 4 * kHistCopies;
+            const size_t smem = (size_t)pl.n * pl.buckets * 4 * kHistCopies;
             if (plain)
                 { radix_hist_all_kernel<K, const K*><<<sort_grid(M), 256, smem, s>>>(
                     plain, M, pl, tot, sort_needed); note_launch(); }
@@ -1083,20 +1105,27 @@ cudaError_t radix_passes(const PairList<K, P> first, uint64_t M, uint64_t N, con
         }
         {
             TraceScope trace("csr_scan", s);
-            { radix_dstart_kernel<<<pl.n, kMaxBuckets, 0, s>>>(tot, pl, dstart, sort_needed); note_launch(); }
+            { radix_dstart_kernel<<<pl.n, pl.buckets, 0, s>>>(tot, pl, dstart, sort_needed); note_launch(); }
         }
         for (uint32_t k = 0; k < pl.n; ++k) {
             TraceScope trace("csr_radix_scatter", s);
             Id* col = k + 1 == pl.n ? col_final : nullptr;
-            const uint64_t* ds = dstart + (size_t)k * kMaxBuckets;
-            if (k == 0 && !plain)
-                { radix_scatter_kernel<K, PairList<K, P>, Id><<<L.n_tiles, kSortThreads, scatter_smem_bytes<K>(), s>>>(
-                    first, buf[k & 1], M, pl.digit(k), status, k, ds, tickets + k, err, sort_needed,
-                    hk.spin_limit, hk.withhold, col, row_ptr, N); note_launch(); }
-            else
-                { radix_scatter_kernel<K, const K*, Id><<<L.n_tiles, kSortThreads, scatter_smem_bytes<K>(), s>>>(
-                    cur, buf[k & 1], M, pl.digit(k), status, k, ds, tickets + k, err, sort_needed,
-                    hk.spin_limit, hk.withhold, col, row_ptr, N); note_launch(); }
+            const uint64_t* ds = dstart + (size_t)k * pl.buckets;
+            auto launch = [&](auto in, auto is_short) {
+                constexpr bool kShort = decltype(is_short)::value;
+                { radix_scatter_kernel<K, decltype(in), Id, kShort>
+                    <<<L.n_tiles, kSortThreads, scatter_smem_bytes<K, kShort>(), s>>>(
+                        in, buf[k & 1], M, pl.digit(k), status, k, ds, tickets + k, err, sort_needed,
+                        hk.spin_limit, hk.withhold, col, row_ptr, N); note_launch(); }
+            };
+            auto shaped = [&](auto in) {
+                if constexpr (sizeof(K) == 8)
+                    if (pl.buckets == SortShape<K, true>::buckets)
+                        return launch(in, std::true_type());
+                launch(in, std::false_type());
+            };
+            if (k == 0 && !plain) shaped(first);
+            else shaped(cur);
             const cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
             cur = buf[k & 1];
@@ -1160,7 +1189,7 @@ cudaError_t csr_impl(const void* d_edges, uint64_t M, uint64_t N, uint64_t N_dst
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     // with at least one digit to sort, the last pass writes col and the row
     // ends itself; a key without digits (one vertex) leaves the list as it is
-    const PassList pl = make_passes(N, N_dst);
+    const PassList pl = make_passes(N, N_dst, M);
     const bool in_sort = M > 0 && pl.n > 0;
     Id* col = in_sort ? (Id*)d_col : nullptr;
     if (ids_narrow(N, N_dst)) {
@@ -1240,7 +1269,7 @@ cudaError_t csr_opts_impl(const void* d_edges, uint64_t M, uint64_t N, uint32_t 
     if (cudaMemsetAsync(d_row_ptr, 0, (N + 1) * 8, s) != cudaSuccess) return cudaErrorUnknown;
     const P* in = (const P*)d_edges;
     const uint32_t sym = (flags & kOptSym) ? 1 : 0;
-    const PassList pl = make_passes(N, N);
+    const PassList pl = make_passes(N, N, M2);
     if (pl.n == 0) {
         // one vertex: the list is sorted as it is (its reverse is the same
         // again), and there is no sort to clear the wait word
