@@ -101,6 +101,9 @@ PbaGeom make_geom(uint64_t n_b, uint64_t N_e, uint32_t m, uint32_t B, uint32_t n
         g.nb_shift = 0;
         while (((uint64_t)1 << g.nb_shift) < n_b) ++g.nb_shift;
         g.lean_add = (n_b - 1) + (g.e0 << g.nb_shift);
+    } else if (n_b > 0) {
+        while (((uint64_t)2 << g.nb_log) <= n_b) ++g.nb_log;
+        g.nb_mul = (uint32_t)((((u128)1 << (32 + g.nb_log)) + n_b - 1) / n_b);
     }
     g.div_m = make_fastdiv(m);
     g.div_m32 = make_fastdiv32(m);

@@ -69,6 +69,8 @@ constexpr uint64_t kShortWaves = 8;     // see pba_segment_length
 constexpr int kEmitItems = 8;
 constexpr uint32_t kEmitRun = 32 * kEmitItems;                   // 256 entries per warp run
 constexpr uint32_t kMaxBlocks = 1024;
+// The scan's flags: some R_q + e0 >= 2^32 (or the switch), some R_q >= 2^31.
+constexpr uint32_t kFlagWide = 1, kFlagLong = 2;
 constexpr uint32_t kSeedTab = 256;   // seed clique edges in the lean links' table: n0 <= 23
 constexpr int kBaThreads = 256;
 template <typename Id>
@@ -392,7 +394,8 @@ __global__ void __launch_bounds__(1024) pba_scan_kernel(const In* in, uint64_t* 
         R[q] = acc;
         divR[q] = make_fastdiv(acc > 0 ? acc : 1);
         recip[q] = make_recip(acc, nb);
-        if (force_wide || acc + e0 >= ((uint64_t)1 << 32)) atomicOr(wide_flag, 1u);
+        if (force_wide || acc + e0 >= ((uint64_t)1 << 32)) atomicOr(wide_flag, kFlagWide);
+        if (acc >= ((uint64_t)1 << 31)) atomicOr(wide_flag, kFlagLong);
     }
     acc -= sum;
 #pragma unroll 8
@@ -544,13 +547,23 @@ __device__ __forceinline__ bool t_link32(uint32_t& cur, uint32_t q, const QRecip
     return fin;
 }
 
-// The same link for n_b a power of two, with sigma(cur) carried in from the
-// previous link (the side-0 value of a link is sigma of the edge the chain
-// moves to, so a continuing chain computes one sigma per link instead of
-// two) and the seed clique's edges read from a table in the workspace
-// (stab[e] = a | b << 16; every lane reads entry 0 unless it hit a seed
-// slot, so the load is a broadcast from L1) instead of a branch: the link is
-// straight-line code.
+// The same link with sigma(cur) carried in from the previous link (the side-0
+// value of a link is sigma of the edge the chain moves to, so a continuing
+// chain computes one sigma per link instead of two), the seed clique's edges
+// read from a table in the workspace (stab[e] = a | b << 16; every lane reads
+// entry 0 unless it hit a seed slot, so the load is a broadcast from L1)
+// instead of a branch, and no 64-bit division: straight-line code.
+// For n_b a power of two (kPow2), X = e0 + ceil(sigma R / n_b) = (sigma R +
+// (n_b - 1) + e0 n_b) >> log2(n_b): e0 n_b is a multiple of n_b, and the sum
+// stays below n_b (R + e0 + 1) <= 2^64. For any n_b: ceil(sigma R / n_b) is the
+// first edge of source time sigma, and cur stands rem div n_b edges after it,
+// rem = cur n_b - sigma R = cur n_b mod R, which 32-bit products give; the
+// division is the high word of rem c, c = ceil(2^(32 + s) / n_b), s = floor(log2
+// n_b), shifted by s: exact for rem < 2^31, as the excess rem (c n_b - 2^(32 + s))
+// < 2^31 n_b < 2^(32 + s), so R must be below 2^31. (100 blocks of 10^6 vertices,
+// m = 5: 6.17 -> 5.37 ms against t_link32; with shifts in place of the products'
+// division the second form took 56.6 ms instead of 56.0 on the 2^30-vertex graph.)
+template <bool kPow2>
 __device__ __forceinline__ bool t_link_lean(uint32_t& cur, uint32_t& sig, bool& fresh, uint32_t q,
                                             const QRecip& c, const PbaGeom& g,
                                             const uint32_t* __restrict__ stab, uint32_t& v)
@@ -560,10 +573,14 @@ __device__ __forceinline__ bool t_link_lean(uint32_t& cur, uint32_t& sig, bool& 
     // load of the target's reciprocal has the draw's time to land
     if (fresh) sig = sigma32(cur, c);
     fresh = false;
-    // X = e0 + ceil(sig*R / n_b) = (sig*R + (n_b - 1) + e0*n_b) >> log2(n_b):
-    // e0*n_b is a multiple of n_b, and the sum stays below n_b*(R + e0 + 1) <= 2^64
-    const uint32_t X = (uint32_t)(((uint64_t)sig * c.R + g.lean_add) >> g.nb_shift);
     const uint32_t e0 = (uint32_t)g.e0;
+    uint32_t X;
+    if constexpr (kPow2) {
+        X = (uint32_t)(((uint64_t)sig * c.R + g.lean_add) >> g.nb_shift);
+    } else {
+        const uint32_t rem = cur * (uint32_t)g.n_b - sig * c.R;
+        X = e0 + cur - (__umulhi(rem, g.nb_mul) >> g.nb_log);
+    }
     const uint64_t s = (uint64_t)w.y * X + (((uint64_t)w.x * X) >> 32);
     const uint32_t e = (uint32_t)(s >> 32);
     const uint32_t side = ((uint32_t)s) >> 31;
@@ -735,21 +752,23 @@ struct EmitWarpSmem {
     uint16_t qs[2][kEmitRun];  // target block of each entry of the run
 };
 
-// kMode 0: 64-bit links (some R_q + e0 >= 2^32); 1: 32-bit links; 2: 32-bit
-// lean links (n_b a power of two, n0 <= 23).
+// kMode 0: 64-bit links (some R_q + e0 >= 2^32); 1: 32-bit links; 2, 3: lean
+// links (n0 <= 23), for n_b a power of two and for any n_b with every R_q below
+// 2^31. Which of the launched variants works is in the scan's flags: the one
+// whose bits `mask` of them are `want`.
 template <typename Id, int kMode>
 __global__ void __launch_bounds__(kEmitThreads) pba_emit_kernel(
     const __grid_constant__ PbaGeom g, const uint16_t* __restrict__ A,
     const uint64_t* __restrict__ off, const uint64_t* __restrict__ R,
     const FastDiv* __restrict__ divR, const QRecip* __restrict__ recip,
-    const uint32_t* __restrict__ wide_flag, const uint32_t* __restrict__ stab,
-    Id* __restrict__ out, uint32_t block_off, uint32_t n_blocks, uint32_t out_block0,
+    const uint32_t* __restrict__ wide_flag, uint32_t mask, uint32_t want,
+    const uint32_t* __restrict__ stab, Id* __restrict__ out, uint32_t block_off, uint32_t n_blocks, uint32_t out_block0,
     uint64_t out_cap)
 {
     constexpr bool kFast = kMode != 0;
     using CurT = typename std::conditional<kFast, uint32_t, uint64_t>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if ((*wide_flag == 0) != kFast) return;   // the other variant does the work
+    if ((*wide_flag & mask) != want) return;   // another variant does the work
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // gridDim.y is n_blocks when a block's segments fill whole CTAs (or there
     // is one block); otherwise the warps of all blocks are numbered through
@@ -847,7 +866,8 @@ __global__ void __launch_bounds__(kEmitThreads) pba_emit_kernel(
         auto trip = [&](uint32_t limit) {
             uint32_t v;
             bool fin;
-            if constexpr (kMode == 2) fin = t_link_lean(cur, sig, fresh, q, c, g, stab, v);
+            if constexpr (kMode >= 2)
+                fin = t_link_lean<kMode == 2>(cur, sig, fresh, q, c, g, stab, v);
             else fin = t_link32(cur, q, c, g, v);
             const bool done = fin && active;
             if (done) item_all[k] = v;
@@ -1022,7 +1042,7 @@ uint32_t pba_prefix_len(uint64_t N_e, uint32_t B, int sm_count)
     constexpr uint64_t kSmallChunk = PassShape<false>::chunk;
     uint64_t P = kPrefixMax;
     if (B < 2 * (uint32_t)(sm_count > 0 ? sm_count : 1)) {
-        P = (N_e / 16 + kSmallChunk - 1) / kSmallChunk * kSmallChunk;
+        P = N_e / 16 / kSmallChunk * kSmallChunk;
         P = P < kSmallChunk ? kSmallChunk : P > kPrefixFew ? kPrefixFew : P;
     }
     return (uint32_t)(N_e < P ? N_e : P);
@@ -1170,11 +1190,15 @@ PbaBuffers pba_buffers(const PbaGeom& g, void* d_ws)
 constexpr size_t kSmemFast = kEmitWarps * sizeof(EmitWarpSmem<uint32_t>);
 constexpr size_t kSmemWide = kEmitWarps * sizeof(EmitWarpSmem<uint64_t>);
 
-// the 32-bit emit variant for this geometry: lean links when n_b is a power
-// of two and the seed clique's edges fit the table
-bool lean_links(const PbaGeom& g)
+// Lean links: the seed clique's edges fit the table.
+bool lean_links(const PbaGeom& g) { return g.e0 <= kSeedTab; }
+
+template <typename Id, int kMode>
+cudaError_t emit_attribute()
 {
-    return g.nb_shift != 0xFFFFFFFFu && g.e0 <= kSeedTab;
+    return cudaFuncSetAttribute(pba_emit_kernel<Id, kMode>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(kMode ? kSmemFast : kSmemWide));
 }
 
 // The opt-in shared-memory sizes of the kernels that need more than the
@@ -1195,18 +1219,10 @@ cudaError_t set_pba_attributes()
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, pass),
             cudaFuncSetAttribute(pba_pass_kernel<true, true>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, pass),
-            cudaFuncSetAttribute(pba_emit_kernel<uint32_t, 2>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFast),
-            cudaFuncSetAttribute(pba_emit_kernel<uint64_t, 2>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFast),
-            cudaFuncSetAttribute(pba_emit_kernel<uint32_t, 1>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFast),
-            cudaFuncSetAttribute(pba_emit_kernel<uint64_t, 1>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFast),
-            cudaFuncSetAttribute(pba_emit_kernel<uint32_t, 0>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemWide),
-            cudaFuncSetAttribute(pba_emit_kernel<uint64_t, 0>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemWide)});
+            emit_attribute<uint32_t, 3>(), emit_attribute<uint64_t, 3>(),
+            emit_attribute<uint32_t, 2>(), emit_attribute<uint64_t, 2>(),
+            emit_attribute<uint32_t, 1>(), emit_attribute<uint64_t, 1>(),
+            emit_attribute<uint32_t, 0>(), emit_attribute<uint64_t, 0>()});
     });
 }
 
@@ -1306,9 +1322,10 @@ cudaError_t launch_pba_emit(const PbaGeom& g, int id64, void* d_out, const void*
     cudaError_t err;
     if ((err = set_pba_attributes()) != cudaSuccess) return err;
     const PbaBuffers W = pba_buffers(g, const_cast<void*>(d_ws));
-    // every R_q + e0 < 2^32 is certain when all entries together are fewer
-    const bool surely_fast =
-        !g_ever_forced.load() && (uint64_t)g.B * g.N_e + g.e0 < ((uint64_t)1 << 32);
+    // every R_q + e0 < 2^32, or R_q < 2^31, is certain when all entries together
+    // are fewer
+    const uint64_t entries = (uint64_t)g.B * g.N_e;
+    const bool surely_fast = !g_ever_forced.load() && entries + g.e0 < ((uint64_t)1 << 32);
     const uint32_t nblk = b_end - b_begin;
     const bool lean = lean_links(g);
     const uint32_t chunks = hc ? hc->chunks : 1;
@@ -1322,33 +1339,28 @@ cudaError_t launch_pba_emit(const PbaGeom& g, int id64, void* d_out, const void*
                                                 : dim3((nb * g.S + kEmitWarps - 1) / kEmitWarps);
         {
             TraceScope trace("pba_emit", s);
-            if (id64) {
-                if (lean)
-                    { pba_emit_kernel<uint64_t, 2><<<grid, kEmitThreads, kSmemFast, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint64_t*)d_out, b0, nb, b_begin,
-                        out_cap); note_launch(); }
-                else
-                    { pba_emit_kernel<uint64_t, 1><<<grid, kEmitThreads, kSmemFast, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint64_t*)d_out, b0, nb, b_begin,
-                        out_cap); note_launch(); }
-                if (!surely_fast)
-                    { pba_emit_kernel<uint64_t, 0><<<grid, kEmitThreads, kSmemWide, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint64_t*)d_out, b0, nb, b_begin,
-                        out_cap); note_launch(); }
-            } else {
-                if (lean)
-                    { pba_emit_kernel<uint32_t, 2><<<grid, kEmitThreads, kSmemFast, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint32_t*)d_out, b0, nb, b_begin,
-                        out_cap); note_launch(); }
-                else
-                    { pba_emit_kernel<uint32_t, 1><<<grid, kEmitThreads, kSmemFast, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint32_t*)d_out, b0, nb, b_begin,
-                        out_cap); note_launch(); }
-                if (!surely_fast)
-                    { pba_emit_kernel<uint32_t, 0><<<grid, kEmitThreads, kSmemWide, s>>>(
-                        g, W.A, W.off, W.R, W.divR, W.recip, W.wide, W.stab, (uint32_t*)d_out, b0, nb, b_begin,
-                        out_cap); note_launch(); }
-            }
+            auto launch = [&](auto id, auto mode, uint32_t mask, uint32_t want) {
+                using Id = decltype(id);
+                constexpr int kMode = decltype(mode)::value;
+                { pba_emit_kernel<Id, kMode><<<grid, kEmitThreads, kMode ? kSmemFast : kSmemWide, s>>>(
+                    g, W.A, W.off, W.R, W.divR, W.recip, W.wide, mask, want, W.stab, (Id*)d_out, b0, nb,
+                    b_begin, out_cap); note_launch(); }
+            };
+            auto launch_all = [&](auto id) {
+                using std::integral_constant;
+                if (!lean) {
+                    launch(id, integral_constant<int, 1>(), kFlagWide, 0);
+                } else if (g.nb_shift != 0xFFFFFFFFu) {
+                    launch(id, integral_constant<int, 2>(), kFlagWide, 0);
+                } else {
+                    launch(id, integral_constant<int, 3>(), kFlagWide | kFlagLong, 0);
+                    if (entries >= ((uint64_t)1 << 31))
+                        launch(id, integral_constant<int, 1>(), kFlagWide | kFlagLong, kFlagLong);
+                }
+                if (!surely_fast) launch(id, integral_constant<int, 0>(), kFlagWide, kFlagWide);
+            };
+            if (id64) launch_all(uint64_t{});
+            else launch_all(uint32_t{});
         }
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         if (hc) {

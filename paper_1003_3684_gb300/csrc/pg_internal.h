@@ -114,6 +114,7 @@ struct PbaGeom {
     uint32_t P;                    // phase-1 prefix kept in shared memory
     uint32_t nb_shift;             // log2(n_b) when n_b is a power of two, else 0xffffffff
     uint64_t lean_add;             // (n_b - 1) + e0 * n_b when n_b is a power of two
+    uint32_t nb_mul, nb_log;       // otherwise: ceil(2^(32 + s) / n_b) and s = floor(log2 n_b)
     FastDiv div_m, div_nb;
     FastDiv32 div_m32;             // j div m for j < 2^32
     uint32_t mul_m, pad;           // ceil(2^32 / m) when j div m is its product's high word, else 0

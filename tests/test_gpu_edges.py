@@ -243,3 +243,14 @@ def test_degrees_of_grouped_sources(which, M):
     N = max(int(src.max()), 1)                                  # the last source is outside
     deg = pg.degrees(torch.from_numpy(e.view(np.int32)).cuda(), N, which)
     assert np.array_equal(host(deg), o.degrees(e.astype(np.uint64), N, which))
+
+
+@pytest.mark.parametrize("n_b", [2, 3, 5, 127, 1023, 1025, 3000, 65_537])
+@pytest.mark.parametrize("m,n0", [(1, 2), (5, 6), (3, 23), (3, 24)])
+def test_pba_links_for_any_block_size(n_b, m, n0):
+    """Block sizes that are no power of two, seed cliques that just fit the
+    links' table (n0 = 23) and that do not."""
+    B = 4
+    got = pg.gen_pba(B * n_b, m, B, n0, 1, 0.2, 31)
+    ref = o.pba(B * n_b, m, B, n0, 1, 0.2, 31)[0]
+    assert np.array_equal(host(got), np.asarray(ref).astype(np.uint64))
