@@ -52,11 +52,12 @@ KERNEL_WORK = {
 
 # Sorting kernels of the CSR step: HBM-bound; unit = one edge per launch, bytes
 # = what one launch must move at least (a radix pass reads and writes every
-# pair; the histogram pass and the sortedness check read every pair once).
+# pair; the histogram pass reads every pair once, and the pass for grouped
+# lists also writes every destination).
 CSR_WORK = {
     "csr_radix_scatter": dict(ops=0, bytes=16),
     "csr_radix_hist": dict(ops=0, bytes=8),
-    "csr_check": dict(ops=0, bytes=8),
+    "csr_grouped": dict(ops=0, bytes=12),
     "csr_finish": dict(ops=0, bytes=12),
 }
 

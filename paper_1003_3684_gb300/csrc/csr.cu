@@ -4,9 +4,9 @@
 // result is unique for a given multiset of edges.
 //
 // Grouped lists (non-decreasing src, as gen_pba and serial BA write them,
-// rows of at most kGroupedMaxRow edges): csr_check finds the list grouped and
-// csr_grouped places each destination at its rank within its own row and
-// marks each row's end in row_ptr.
+// rows of at most kGroupedMaxRow edges): csr_grouped finds the list grouped as
+// it goes, places each destination at its rank within its own row and marks
+// each row's end in row_ptr.
 //
 // Any other list: least-significant-digit radix sort of the (src, dst) keys,
 // from the low bits of dst to the high bits of src, up to 8 bits per pass (9 for short lists):
@@ -23,9 +23,9 @@
 // (a hub with 10^5 edges) costs no more than any other key. The last pass
 // writes the destinations to col itself and raises row_ptr[src + 1] at the
 // last pair of each source in each tile. Both paths then take a parallel
-// prefix maximum over row_ptr, which fills the rows without edges. The sort kernels
-// read the sortedness flag and return at once when the grouped path applied,
-// so no host round trip decides the path.
+// prefix maximum over row_ptr, which fills the rows without edges. The sort
+// kernels read the flag that csr_grouped sets and return at once when the
+// grouped path applied, so no host round trip decides the path.
 //
 // Ids at or above n_vertices are never used as an index (such edges are
 // dropped), so a bad list cannot make a kernel write out of bounds.
@@ -86,11 +86,11 @@ __device__ __forceinline__ uint32_t digit_of(const K& e, const Digit& g)
 template <typename K, typename P>
 struct PairList {
     const P* p;
-    uint32_t sym;
+    uint32_t sym;   // 0 or 1
     __device__ __forceinline__ K operator[](uint64_t i) const
     {
-        const P e = p[sym ? i >> 1 : i];
-        const bool back = sym && (i & 1);
+        const P e = p[i >> sym];
+        const bool back = (uint32_t)i & sym;
         K k;
         k.x = (decltype(k.x))(back ? e.y : e.x);
         k.y = (decltype(k.y))(back ? e.x : e.y);
@@ -237,191 +237,196 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     if (*sort_needed == 0 || *(volatile const uint32_t*)err != 0) return;
     const uint32_t nb = dg.mask + 1;
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
-    for (uint32_t d = threadIdx.x; d < nb; d += blockDim.x)
-        for (int w = 0; w < kSortWarps; ++w) wcnt[w][d] = 0;
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    const uint64_t tile0 = (uint64_t)tile * kTile;
-    const uint32_t n = (uint32_t)((M - tile0 < kTile) ? M - tile0 : kTile);
-    const uint32_t wbase = wid * (32 * kItems);
-    K e[kItems];
-    // ranks within the warp (< 32 * kItems <= 512), two per register; the
-    // digits are recomputed from e[] where needed, so no array holds them
-    uint32_t rk[kItems / 2];
+    for (;;) {
+        if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+        for (uint32_t d = threadIdx.x; d < nb; d += blockDim.x)
+            for (int w = 0; w < kSortWarps; ++w) wcnt[w][d] = 0;
+        __syncthreads();
+        const uint32_t tile = s_tile;
+        if ((uint64_t)tile * kTile >= M) return;   // uniform: no tile left
+        const uint64_t tile0 = (uint64_t)tile * kTile;
+        const uint32_t n = (uint32_t)((M - tile0 < kTile) ? M - tile0 : kTile);
+        const uint32_t wbase = wid * (32 * kItems);
+        K e[kItems];
+        // ranks within the warp (< 32 * kItems <= 512), two per register; the
+        // digits are recomputed from e[] where needed, so no array holds them
+        uint32_t rk[kItems / 2];
 #pragma unroll
-    for (int r = 0; r < kItems; ++r) {
-        const uint32_t t = wbase + r * 32 + lane;
-        if (t < n) e[r] = in[tile0 + t];
-    }
-    __syncthreads();
-    const uint32_t lt = (1u << lane) - 1u;
-    // kFly items of every lane at a time, in lane order within an item: the
-    // lanes holding equal digits of an item find each other through a word per
-    // digit (each ORs in its lane bit, then all read the word back and clear
-    // it; every item in flight has its own table of kBuckets words per
-    // warp, in the reorder buffer, unused until the ranks are done). Then, item
-    // by item, the lowest lane of each group adds the group's size to the
-    // warp's counter of the digit (two 16-bit counters per word) and the group
-    // gets the old value by shuffle. A warp's shared-memory operations execute
-    // in order, so the adds of the items in flight need no wait between them.
-    uint32_t* pmask = reinterpret_cast<uint32_t*>(buf) + wid * (kFly * kBuckets);
-    for (uint32_t t = lane; t < kFly * kBuckets / 4; t += 32)
-        reinterpret_cast<uint4*>(pmask)[t] = make_uint4(0u, 0u, 0u, 0u);
-    __syncwarp();
-    uint32_t* wc = reinterpret_cast<uint32_t*>(wcnt[wid]);
-#pragma unroll
-    for (int r0 = 0; r0 < kItems; r0 += kFly) {
-        uint32_t d[kFly], peers[kFly], prev[kFly];
-#pragma unroll
-        for (int u = 0; u < kFly; ++u) {
-            const uint32_t t = wbase + (r0 + u) * 32 + lane;
-            d[u] = t < n ? digit_of(e[r0 + u], dg) : 0xFFFFFFFFu;
-            if (d[u] != 0xFFFFFFFFu) atomicOr(&pmask[u * kBuckets + d[u]], 1u << lane);
+        for (int r = 0; r < kItems; ++r) {
+            const uint32_t t = wbase + r * 32 + lane;
+            if (t < n) e[r] = in[tile0 + t];
         }
+        __syncthreads();
+        const uint32_t lt = (1u << lane) - 1u;
+        // kFly items of every lane at a time, in lane order within an item: the
+        // lanes holding equal digits of an item find each other through a word per
+        // digit (each ORs in its lane bit, then all read the word back and clear
+        // it; every item in flight has its own table of kBuckets words per
+        // warp, in the reorder buffer, unused until the ranks are done). Then, item
+        // by item, the lowest lane of each group adds the group's size to the
+        // warp's counter of the digit (two 16-bit counters per word) and the group
+        // gets the old value by shuffle. A warp's shared-memory operations execute
+        // in order, so the adds of the items in flight need no wait between them.
+        uint32_t* pmask = reinterpret_cast<uint32_t*>(buf) + wid * (kFly * kBuckets);
+        for (uint32_t t = lane; t < kFly * kBuckets / 4; t += 32)
+            reinterpret_cast<uint4*>(pmask)[t] = make_uint4(0u, 0u, 0u, 0u);
         __syncwarp();
+        uint32_t* wc = reinterpret_cast<uint32_t*>(wcnt[wid]);
 #pragma unroll
-        for (int u = 0; u < kFly; ++u)
-            peers[u] = d[u] != 0xFFFFFFFFu ? pmask[u * kBuckets + d[u]] : 0u;
-        __syncwarp();
+        for (int r0 = 0; r0 < kItems; r0 += kFly) {
+            uint32_t d[kFly], peers[kFly], prev[kFly];
 #pragma unroll
-        for (int u = 0; u < kFly; ++u) {
-            if (d[u] != 0xFFFFFFFFu) pmask[u * kBuckets + d[u]] = 0;
-            prev[u] = 0;
-            if (peers[u] != 0 && (peers[u] & lt) == 0) {
-                const uint32_t sh = (d[u] & 1) * 16;
-                prev[u] = (atomicAdd(&wc[d[u] >> 1], __popc(peers[u]) << sh) >> sh) & 0xFFFFu;
+            for (int u = 0; u < kFly; ++u) {
+                const uint32_t t = wbase + (r0 + u) * 32 + lane;
+                d[u] = t < n ? digit_of(e[r0 + u], dg) : 0xFFFFFFFFu;
+                if (d[u] != 0xFFFFFFFFu) atomicOr(&pmask[u * kBuckets + d[u]], 1u << lane);
             }
             __syncwarp();
-        }
 #pragma unroll
-        for (int u = 0; u < kFly; ++u) {
-            const uint32_t rank = __shfl_sync(0xFFFFFFFFu, prev[u], __ffs(peers[u]) - 1) +
-                                  __popc(peers[u] & lt);
-            const int r = r0 + u;
-            if (r & 1) rk[r >> 1] |= rank << 16;
-            else rk[r >> 1] = rank;
-        }
-    }
-    __syncthreads();
-    // per digit (one thread each): the tile total, published at once so that
-    // later tiles can sum it; where the digit's run starts in the sorted tile
-    // (loff), and where each warp's part of the run does (in wcnt)
-    const unsigned long long tag = (unsigned long long)(pass + 1) << kPassShift;
-    volatile unsigned long long* st = status + (uint64_t)tile * nb;
-    {
-        const uint32_t d = threadIdx.x;
-        uint32_t acc = 0;
-        if (d < nb) {
+            for (int u = 0; u < kFly; ++u)
+                peers[u] = d[u] != 0xFFFFFFFFu ? pmask[u * kBuckets + d[u]] : 0u;
+            __syncwarp();
 #pragma unroll
-            for (int w = 0; w < kSortWarps; ++w) acc += wcnt[w][d];
-            if (tile != withhold) st[d] = tag | (tile == 0 ? kInc : kAgg) | acc;
-        }
-        uint32_t x = acc;   // inclusive over the warp's digits
+            for (int u = 0; u < kFly; ++u) {
+                if (d[u] != 0xFFFFFFFFu) pmask[u * kBuckets + d[u]] = 0;
+                prev[u] = 0;
+                if (peers[u] != 0 && (peers[u] & lt) == 0) {
+                    const uint32_t sh = (d[u] & 1) * 16;
+                    prev[u] = (atomicAdd(&wc[d[u] >> 1], __popc(peers[u]) << sh) >> sh) & 0xFFFFu;
+                }
+                __syncwarp();
+            }
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-            if (lane >= (uint32_t)o) x += y;
+            for (int u = 0; u < kFly; ++u) {
+                const uint32_t rank = __shfl_sync(0xFFFFFFFFu, prev[u], __ffs(peers[u]) - 1) +
+                                      __popc(peers[u] & lt);
+                const int r = r0 + u;
+                if (r & 1) rk[r >> 1] |= rank << 16;
+                else rk[r >> 1] = rank;
+            }
         }
-        if (lane == 31) s_part[wid] = x;
         __syncthreads();
-        const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? s_part[lane] : 0u);
-        if (d < nb) {
-            uint32_t at = before + x - acc;
-            loff[d] = at;
+        // per digit (one thread each): the tile total, published at once so that
+        // later tiles can sum it; where the digit's run starts in the sorted tile
+        // (loff), and where each warp's part of the run does (in wcnt)
+        const unsigned long long tag = (unsigned long long)(pass + 1) << kPassShift;
+        volatile unsigned long long* st = status + (uint64_t)tile * nb;
+        {
+            const uint32_t d = threadIdx.x;
+            uint32_t acc = 0;
+            if (d < nb) {
 #pragma unroll
-            for (int w = 0; w < kSortWarps; ++w) {
-                const uint32_t c = wcnt[w][d];
-                wcnt[w][d] = (uint16_t)at;   // below the tile's size
-                at += c;
+                for (int w = 0; w < kSortWarps; ++w) acc += wcnt[w][d];
+                if (tile != withhold) st[d] = tag | (tile == 0 ? kInc : kAgg) | acc;
             }
-        }
-    }
-    __syncthreads();
-    // reorder the tile by digit in shared memory
+            uint32_t x = acc;   // inclusive over the warp's digits
 #pragma unroll
-    for (int r = 0; r < kItems; ++r) {
-        const uint32_t t = wbase + r * 32 + lane;
-        if (t < n) {
-            const uint32_t d = digit_of(e[r], dg);
-            const uint32_t rank = (rk[r >> 1] >> ((r & 1) * 16)) & 0xFFFFu;
-            const uint32_t at = wcnt[wid][d] + rank;
-            if (PG_CHECK(at, n)) buf[at] = e[r];
-        }
-    }
-    // look back through up to kLookWindow earlier tiles per round trip
-    for (uint32_t d = threadIdx.x; d < nb; d += blockDim.x) {
-        unsigned long long excl = 0;
-        if (tile > 0) {
-            uint32_t next = tile - 1;   // nearest tile not yet summed (tile 0 is inclusive)
-            uint32_t polls = 0;
-            bool found = false;
-            while (!found) {
-                unsigned long long w[kLookWindow];
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+                if (lane >= (uint32_t)o) x += y;
+            }
+            if (lane == 31) s_part[wid] = x;
+            __syncthreads();
+            const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? s_part[lane] : 0u);
+            if (d < nb) {
+                uint32_t at = before + x - acc;
+                loff[d] = at;
 #pragma unroll
-                for (int u = 0; u < kLookWindow; ++u)
-                    w[u] = (next >= (uint32_t)u)
-                               ? *((volatile const unsigned long long*)status +
-                                   (uint64_t)(next - u) * nb + d)
-                               : 0ull;
-                int used = 0;
-                bool stalled = false;
-#pragma unroll
-                for (int u = 0; u < kLookWindow; ++u) {
-                    if (found || stalled) continue;
-                    const unsigned long long flag =
-                        (w[u] >> kPassShift) == pass + 1 ? w[u] & (3ull << 57) : 0;
-                    if (flag == 0) {
-                        stalled = true;
-                        continue;
-                    }
-                    excl += w[u] & kCountMask;
-                    ++used;
-                    if (flag == kInc) found = true;
-                }
-                if (found) break;
-                next -= used;
-                if (stalled) {
-                    if (++polls > spin_limit) {
-                        atomicOr(err, 1u);
-                        break;
-                    }
-                    __nanosleep(32);
-                } else {
-                    polls = 0;
+                for (int w = 0; w < kSortWarps; ++w) {
+                    const uint32_t c = wcnt[w][d];
+                    wcnt[w][d] = (uint16_t)at;   // below the tile's size
+                    at += c;
                 }
             }
-            const uint32_t cnt_d = (d + 1 < nb ? loff[d + 1] : n) - loff[d];
-            if (tile != withhold) st[d] = tag | kInc | (excl + cnt_d);
         }
-        // where the tile's run of d starts in the output, less its start in
-        // the sorted tile (never negative: the tile's counts of the lower
-        // digits, loff[d], are at most their totals, which dstart[d] sums)
-        tbase[d] = dstart[d] + excl - loff[d];
-    }
-    __syncthreads();
-    // write runs: sorted position p goes to tbase[d] + p (one table read per pair)
-    if (col_out == nullptr) {
-        for (uint32_t p = threadIdx.x; p < n; p += blockDim.x) {
-            const K v = buf[p];
-            const uint32_t d = digit_of(v, dg);
-            if (PG_CHECK(tbase[d] + p, M)) out[tbase[d] + p] = v;
+        __syncthreads();
+        // reorder the tile by digit in shared memory
+#pragma unroll
+        for (int r = 0; r < kItems; ++r) {
+            const uint32_t t = wbase + r * 32 + lane;
+            if (t < n) {
+                const uint32_t d = digit_of(e[r], dg);
+                const uint32_t rank = (rk[r >> 1] >> ((r & 1) * 16)) & 0xFFFFu;
+                const uint32_t at = wcnt[wid][d] + rank;
+                if (PG_CHECK(at, n)) buf[at] = e[r];
+            }
         }
-        return;
-    }
-    // the last pass of a CSR: the tile is in (src, dst) order, so each
-    // destination goes straight to col, and the last pair of each source
-    // in the tile raises row_ptr[src + 1] to its end (the source's last pair
-    // overall gives the maximum; the prefix maximum fills empty rows)
-    for (uint32_t p = threadIdx.x; p < n; p += blockDim.x) {
-        const K v = buf[p];
-        const uint32_t d = digit_of(v, dg);
-        const uint64_t o = tbase[d] + p;
-        if (PG_CHECK_OUT(o, M)) col_out[o] = (Id)v.y;
-        const uint64_t src = v.x;
-        if (src < N && (p + 1 == n || (uint64_t)buf[p + 1].x != src))
-            atomicMax(reinterpret_cast<unsigned long long*>(row_ptr) + src + 1,
-                      (unsigned long long)(o + 1));
+        // look back through up to kLookWindow earlier tiles per round trip
+        for (uint32_t d = threadIdx.x; d < nb; d += blockDim.x) {
+            unsigned long long excl = 0;
+            if (tile > 0) {
+                uint32_t next = tile - 1;   // nearest tile not yet summed (tile 0 is inclusive)
+                uint32_t polls = 0;
+                bool found = false;
+                while (!found) {
+                    unsigned long long w[kLookWindow];
+#pragma unroll
+                    for (int u = 0; u < kLookWindow; ++u)
+                        w[u] = (next >= (uint32_t)u)
+                                   ? *((volatile const unsigned long long*)status +
+                                       (uint64_t)(next - u) * nb + d)
+                                   : 0ull;
+                    int used = 0;
+                    bool stalled = false;
+#pragma unroll
+                    for (int u = 0; u < kLookWindow; ++u) {
+                        if (found || stalled) continue;
+                        const unsigned long long flag =
+                            (w[u] >> kPassShift) == pass + 1 ? w[u] & (3ull << 57) : 0;
+                        if (flag == 0) {
+                            stalled = true;
+                            continue;
+                        }
+                        excl += w[u] & kCountMask;
+                        ++used;
+                        if (flag == kInc) found = true;
+                    }
+                    if (found) break;
+                    next -= used;
+                    if (stalled) {
+                        if (++polls > spin_limit) {
+                            atomicOr(err, 1u);
+                            break;
+                        }
+                        __nanosleep(32);
+                    } else {
+                        polls = 0;
+                    }
+                }
+                const uint32_t cnt_d = (d + 1 < nb ? loff[d + 1] : n) - loff[d];
+                if (tile != withhold) st[d] = tag | kInc | (excl + cnt_d);
+            }
+            // where the tile's run of d starts in the output, less its start in
+            // the sorted tile (never negative: the tile's counts of the lower
+            // digits, loff[d], are at most their totals, which dstart[d] sums)
+            tbase[d] = dstart[d] + excl - loff[d];
+        }
+        __syncthreads();
+        // write runs: sorted position p goes to tbase[d] + p (one table read per pair)
+        if (col_out == nullptr) {
+            for (uint32_t p = threadIdx.x; p < n; p += blockDim.x) {
+                const K v = buf[p];
+                const uint32_t d = digit_of(v, dg);
+                if (PG_CHECK(tbase[d] + p, M)) out[tbase[d] + p] = v;
+            }
+        } else {
+            // the last pass of a CSR: the tile is in (src, dst) order, so each
+            // destination goes straight to col, and the last pair of each source
+            // in the tile raises row_ptr[src + 1] to its end (the source's last pair
+            // overall gives the maximum; the prefix maximum fills empty rows)
+            for (uint32_t p = threadIdx.x; p < n; p += blockDim.x) {
+                const K v = buf[p];
+                const uint32_t d = digit_of(v, dg);
+                const uint64_t o = tbase[d] + p;
+                if (PG_CHECK_OUT(o, M)) col_out[o] = (Id)v.y;
+                const uint64_t src = v.x;
+                if (src < N && (p + 1 == n || (uint64_t)buf[p + 1].x != src))
+                    atomicMax(reinterpret_cast<unsigned long long*>(row_ptr) + src + 1,
+                              (unsigned long long)(o + 1));
+            }
+        }
+        if constexpr (!std::is_pointer_v<In>) return;   // one tile per CTA (see the launch)
+        __syncthreads();   // the next tile reuses the tables
     }
 }
 
@@ -471,14 +476,17 @@ __device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t v, uint64_t* s
     return before + x - v;
 }
 
-// Zeroes the tile status words once per call (nothing when no sort runs).
-__global__ void __launch_bounds__(256) zero_status_kernel(uint4* __restrict__ p, uint64_t n16,
-                                                          const uint32_t* __restrict__ sort_needed)
+// Zeroes the tile status words, and the row pointers a grouped list's tiles may
+// have written (n_rows of them), before a sort (nothing when no sort runs).
+__global__ void __launch_bounds__(256) sort_init_kernel(uint4* __restrict__ p, uint64_t n16,
+                                                        uint64_t* __restrict__ row_ptr, uint64_t n_rows,
+                                                        const uint32_t* __restrict__ sort_needed)
 {
     if (*sort_needed == 0) return;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += stride)
-        p[i] = make_uint4(0u, 0u, 0u, 0u);
+    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (uint64_t i = t; i < n16; i += stride) p[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint64_t i = t; i < n_rows; i += stride) row_ptr[i] = 0;
 }
 // Where each digit's run starts in pass k's output: the exclusive scan of
 // that pass's digit totals. grid = passes, block = pl.buckets threads.
@@ -524,73 +532,119 @@ __global__ void __launch_bounds__(1024) scan_parts_kernel(uint64_t* __restrict__
     }
 }
 
-// ---- final pass: col and row_ptr from the sorted pairs ---------------------
-// Flags (sort_needed = 1) a list that is not grouped by source, or that has
-// a row longer than kGroupedMaxRow.
+// ---- lists grouped by source ------------------------------------------------
+// One pass over the list, as if it were grouped: every destination goes to its
+// row's start + its rank among the row's destinations (ties by position, so
+// equal values keep their multiplicity), and the last edge i of row v writes
+// row_ptr[v + 1] = i + 1. A tile that finds the list not grouped, or a row of
+// more than kGroupedMaxRow edges, sets sort_needed instead; the sort then
+// overwrites col, and row_ptr is cleared again. CTAs look at the flag before
+// each tile, so an unsorted list costs about one round of tiles.
+//
+// Bound by instruction issue (0.52 of HBM at m = 5; a row of r edges takes r
+// compares per edge), so the work per position is kept small: a tile and 32
+// neighbours on each side are staged in shared memory, row starts are one
+// ballot per 32 positions, a row's bounds bit searches in three of these
+// words, and a rank reads the row once, the lanes of a row the same word.
+// Tiles inside the list test no bounds. 2^24 vertices, m = 5: 1.185 -> 0.327 ms
+// (64-bit ids 0.48); m = 2: 0.126; 2^22 vertices, m = 30: 6.22 -> 1.12 (each edge
+// searched and ranked its row in global memory before, after a pass of its
+// own that looked for violations). Six CTAs per SM: five 0.344, eight (spills) 0.37.
+constexpr uint32_t kGroupTile = 2048;
 template <typename Id>
-__global__ void __launch_bounds__(256) csr_check_kernel(const typename PairOf<Id>::T* __restrict__ s,
-                                                        uint64_t M, uint32_t* __restrict__ sort_needed)
+constexpr int kGroupPlaces = sizeof(Id) == 4 ? 6 : 4;   // CTAs per SM
+template <typename Id>
+__global__ void __launch_bounds__(256, kGroupPlaces<Id>)
+    csr_grouped_kernel(const typename PairOf<Id>::T* __restrict__ s, uint64_t M, uint64_t N,
+                       Id* __restrict__ col, uint64_t* __restrict__ row_ptr,
+                       uint32_t* __restrict__ sort_needed)
 {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    // A warp that finds a violation sets the flag (one atomic per warp) and
-    // stops; every few rounds the warps also read the flag and stop once any
-    // warp has set it, so an unsorted list costs about one round, not a full
-    // read. The trip count is uniform across the warp (i0 steps by the grid).
-    const volatile uint32_t* flag = sort_needed;
-    const uint32_t lane = threadIdx.x & 31;
-    uint32_t round = 0;
-    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < M;
-         i0 += stride, ++round) {
-        const uint64_t i = i0 + lane;
-        bool bad = false;
-        if (i < M) {
-            const uint64_t src = s[i].x;
-            const bool starts = (i == 0) || s[i - 1].x != src;
-            bad = i > 0 && (uint64_t)s[i - 1].x > src;
-            bad |= starts && i + kGroupedMaxRow < M && (uint64_t)s[i + kGroupedMaxRow].x == src;
+    static_assert(kGroupedMaxRow == 32, "a row spans at most two neighbouring words");
+    constexpr uint32_t kSpan = kGroupTile + 64;
+    __shared__ Id src[kSpan], dst[kSpan];   // edge base + t at 32 + t
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr uint32_t kWords = kGroupTile / 256;   // 32-position words per warp
+    // `inner`: every position of the span is an edge of the list
+    auto place = [&](uint64_t base, auto inner) -> bool {
+        constexpr bool kInner = decltype(inner)::value;
+        const uint32_t first = kInner || base ? 0 : 32;
+        const uint32_t last = kInner || M - base > kSpan - 32 ? kSpan : (uint32_t)(M - base) + 32;
+        const auto* __restrict__ in = s + base - 32;
+#pragma unroll
+        for (uint32_t t = 0; t < kSpan; t += 256) {
+            const uint32_t k = t + threadIdx.x;
+            if ((t + 256 <= kSpan || k < kSpan) && (kInner || (k >= first && k < last))) {
+                const auto e = in[k];
+                src[k] = e.x;
+                dst[k] = e.y;
+            }
         }
-        if (__any_sync(0xFFFFFFFFu, bad)) {
-            if (lane == 0) atomicOr(sort_needed, 1u);
+        __syncthreads();
+        // bit l of starts[u]: a row starts at position 32 (w0 + u - 1) + l (the
+        // end of the list counts as one, and so does the start)
+        const uint32_t w0 = 1 + wid * kWords;
+        uint32_t starts[kWords + 2];
+        bool bad = false;
+#pragma unroll
+        for (uint32_t u = 0; u < kWords + 2; ++u) {
+            const uint32_t k = 32 * (w0 - 1 + u) + lane;
+            bool st;
+            if (kInner) {
+                const Id x = src[k], y = src[k > 0 ? k - 1 : 0];
+                st = x != y;
+                bad |= y > x;
+                if (u <= kWords) bad |= src[k + 32] == x;
+            } else {
+                st = k == first || k == last;
+                if (k > first && k < last) {
+                    st = src[k - 1] != src[k];
+                    bad |= src[k - 1] > src[k];
+                }
+                if (k >= first && k + kGroupedMaxRow < last) bad |= src[k + kGroupedMaxRow] == src[k];
+            }
+            starts[u] = __ballot_sync(0xFFFFFFFFu, st);
+        }
+        if (__syncthreads_or(bad)) return false;
+        Id* __restrict__ out = col + base - 32;
+#pragma unroll
+        for (uint32_t u = 0; u < kWords; ++u) {
+            const uint32_t k0 = 32 * (w0 + u), k = k0 + lane;
+            const uint32_t before = starts[u], here = starts[u + 1], after = starts[u + 2];
+            if (kInner || k < last) {
+                // the last start at or before the lane, the first one after it
+                const uint32_t lo = here & (0xFFFFFFFFu >> (31 - lane));
+                const uint32_t hi = (here >> lane) >> 1;
+                const uint32_t a = lo ? k0 + 31 - __clz(lo) : k0 - 1 - __clz(before);
+                const uint32_t b = hi ? k + __ffs(hi) : k0 + 31 + __ffs(after);
+                const Id d = dst[k];
+                uint32_t at = a;
+                // smaller destinations of the row, or equal ones before
+#pragma unroll 4
+                for (uint32_t j = a; j < b; ++j) {
+                    const Id o = dst[j];
+                    if constexpr (sizeof(Id) == 4)
+                        at += ((uint64_t)o << 32 | j) < ((uint64_t)d << 32 | k) ? 1u : 0u;
+                    else
+                        at += o < d || (o == d && j < k) ? 1u : 0u;
+                }
+                if (PG_CHECK_OUT(base + at - 32, M)) out[at] = d;
+                if (b == k + 1) {
+                    const uint64_t v = src[k];
+                    if (v < N) row_ptr[v + 1] = base + (k - 31);
+                }
+            }
+        }
+        return true;
+    };
+    for (uint64_t base = (uint64_t)blockIdx.x * kGroupTile; base < M;
+         base += (uint64_t)gridDim.x * kGroupTile) {
+        // (a barrier, too: the last tile's readers are done)
+        if (__syncthreads_or(threadIdx.x == 0 && *(volatile const uint32_t*)sort_needed != 0)) return;
+        const bool inner = base > 0 && M - base >= kGroupTile + 32;
+        if (inner ? !place(base, std::true_type{}) : !place(base, std::false_type{})) {
+            if (threadIdx.x == 0) atomicOr(sort_needed, 1u);
             return;
         }
-        if ((round & 7) == 7 && *flag != 0) return;
-    }
-}
-
-// Row ends of a list sorted (or grouped) by source: the last edge i of row v
-// writes row_ptr[v + 1] = i + 1. A prefix maximum over row_ptr then fills the
-// rows without edges (row_ptr starts zeroed).
-template <typename P>
-__device__ __forceinline__ void mark_row_end(const P* s, uint64_t M, uint64_t N, uint64_t i,
-                                             uint64_t* row_ptr)
-{
-    const uint64_t v = s[i].x;
-    if (v < N && (i + 1 == M || s[i + 1].x != s[i].x)) row_ptr[v + 1] = i + 1;
-}
-
-// Grouped list: destination of edge i goes to its row start + its rank among
-// the row's destinations (ties broken by position, so equal values keep
-// their multiplicity).
-template <typename Id>
-__global__ void __launch_bounds__(256) csr_grouped_kernel(const typename PairOf<Id>::T* __restrict__ s,
-                                                          uint64_t M, uint64_t N, Id* __restrict__ col,
-                                                          uint64_t* __restrict__ row_ptr,
-                                                          const uint32_t* __restrict__ sort_needed)
-{
-    if (*sort_needed != 0) return;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += stride) {
-        const uint64_t src = s[i].x, d = s[i].y;
-        uint64_t a = i, b = i + 1;
-        while (a > 0 && (uint64_t)s[a - 1].x == src) --a;
-        while (b < M && (uint64_t)s[b].x == src) ++b;
-        uint64_t rank = 0;
-        for (uint64_t j = a; j < b; ++j) {
-            const uint64_t dj = s[j].y;
-            rank += (dj < d) || (dj == d && j < i);
-        }
-        if (PG_CHECK_OUT(a + rank, M)) col[a + rank] = (Id)d;
-        mark_row_end(s, M, N, i, row_ptr);
     }
 }
 
@@ -1093,8 +1147,10 @@ cudaError_t radix_passes(const PairList<K, P> first, uint64_t M, uint64_t N, con
             return cudaErrorUnknown;
         {
             TraceScope trace("csr_radix_hist", s);
-            { zero_status_kernel<<<sort_grid(L.n_status / 2 + 1), 256, 0, s>>>(
-                (uint4*)status, (L.n_status * 8 + 15) / 16, sort_needed); note_launch(); }
+            const uint64_t n_rows = col_final ? N + 1 : 0;   // else no grouped pass ran
+            const uint64_t work = L.n_status / 2 > n_rows ? L.n_status / 2 : n_rows;
+            { sort_init_kernel<<<sort_grid(work + 1), 256, 0, s>>>(
+                (uint4*)status, (L.n_status * 8 + 15) / 16, row_ptr, n_rows, sort_needed); note_launch(); }
             const size_t smem = (size_t)pl.n * pl.buckets * 4 * kHistCopies;
             if (plain)
                 { radix_hist_all_kernel<K, const K*><<<sort_grid(M), 256, smem, s>>>(
@@ -1111,10 +1167,20 @@ cudaError_t radix_passes(const PairList<K, P> first, uint64_t M, uint64_t N, con
             TraceScope trace("csr_radix_scatter", s);
             Id* col = k + 1 == pl.n ? col_final : nullptr;
             const uint64_t* ds = dstart + (size_t)k * pl.buckets;
+            // Two CTAs per SM, what its shared memory holds, take tiles until none
+            // is left: as fast as a CTA per tile (2^26 pairs 2.30 -> 2.26 ms, 2^30
+            // 40.5 -> 40.2), but a list that turned out grouped pays a launch per
+            // pass and not a CTA per tile (five passes over 2^24 x 5 edges:
+            // 0.089 -> 0.039 ms). A pass that converts its list keeps a CTA per
+            // tile: in a loop its loads cost more registers than there are
+            // (2^26 pairs of 64-bit ids 0.264 -> 0.325 ms).
+            const unsigned places = 2 * (unsigned)device_sm_count();
             auto launch = [&](auto in, auto is_short) {
                 constexpr bool kShort = decltype(is_short)::value;
+                const bool loops = std::is_pointer_v<decltype(in)> && L.n_tiles > places;
+                const unsigned grid = loops ? places : L.n_tiles;
                 { radix_scatter_kernel<K, decltype(in), Id, kShort>
-                    <<<L.n_tiles, kSortThreads, scatter_smem_bytes<K, kShort>(), s>>>(
+                    <<<grid, kSortThreads, scatter_smem_bytes<K, kShort>(), s>>>(
                         in, buf[k & 1], M, pl.digit(k), status, k, ds, tickets + k, err, sort_needed,
                         hk.spin_limit, hk.withhold, col, row_ptr, N); note_launch(); }
             };
@@ -1181,10 +1247,12 @@ cudaError_t csr_impl(const void* d_edges, uint64_t M, uint64_t N, uint64_t N_dst
     if (cudaMemsetAsync(sort_needed, 0, 4, s) != cudaSuccess) return cudaErrorUnknown;
     if (cudaMemsetAsync(d_row_ptr, 0, (N + 1) * 8, s) != cudaSuccess) return cudaErrorUnknown;
     {
-        TraceScope trace("csr_check", s);
-        { csr_check_kernel<Id><<<grid, 256, 0, s>>>((const P*)d_edges, M, sort_needed); note_launch(); }
-        { csr_grouped_kernel<Id><<<grid, 256, 0, s>>>((const P*)d_edges, M, N, (Id*)d_col, d_row_ptr,
-                                                   sort_needed); note_launch(); }
+        TraceScope trace("csr_grouped", s);
+        const uint64_t tiles = (M + kGroupTile - 1) / kGroupTile;
+        const uint64_t full = (uint64_t)device_sm_count() * kGroupPlaces<Id>;
+        const unsigned places = (unsigned)(tiles < full ? (tiles ? tiles : 1) : full);
+        { csr_grouped_kernel<Id><<<places, 256, 0, s>>>((const P*)d_edges, M, N, (Id*)d_col, d_row_ptr,
+                                                     sort_needed); note_launch(); }
     }
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     // with at least one digit to sort, the last pass writes col and the row

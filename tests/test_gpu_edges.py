@@ -254,3 +254,32 @@ def test_pba_links_for_any_block_size(n_b, m, n0):
     got = pg.gen_pba(B * n_b, m, B, n0, 1, 0.2, 31)
     ref = o.pba(B * n_b, m, B, n0, 1, 0.2, 31)[0]
     assert np.array_equal(host(got), np.asarray(ref).astype(np.uint64))
+
+
+@pytest.mark.parametrize("row", [1, 2, 5, 31, 32, 33])
+@pytest.mark.parametrize("M", [1, 33, 2047, 2048, 2049, 4127, 4128, 4129, 70_000])
+@pytest.mark.parametrize("id64", [False, True])
+def test_csr_grouped_rows_across_tiles(row, M, id64):
+    """Rows of one length cross every tile boundary at every offset; then one
+    edge at a tile's first or last position breaks the order (or, rows of 32,
+    makes a row too long), so that a list partly placed is sorted after all."""
+    rng = np.random.default_rng(M * row)
+    src = (np.arange(M) + rng.integers(0, row)) // row
+    N = 3 * int(src.max()) + 4
+    e = np.stack([3 * src + 1, rng.integers(0, min(N, 50), M)], 1).astype(np.int64)
+
+    def check(e):
+        t = torch.from_numpy(e if id64 else e.astype(np.uint32).view(np.int32)).cuda()
+        rp, col = pg.edges_to_csr(t, N, check=True)
+        ref_rp, ref_col = o.csr(e.astype(np.uint64), N)
+        np.testing.assert_array_equal(host(rp), ref_rp)
+        np.testing.assert_array_equal(host(col), ref_col)
+
+    check(e)
+    for at in {1, min(2048, M - 1), M - 1} & set(range(1, M)):
+        bad = e.copy()
+        if row == 32:
+            bad[max(at - 32, 0):at + 1, 0] = bad[at, 0]
+        else:
+            bad[at, 0] = 0
+        check(bad)
