@@ -41,6 +41,8 @@ namespace {
 
 constexpr int kSortWarps = 16;
 constexpr int kFly = 2;   // items a warp ranks at a time
+// which items of a thread find their peers by ballots: three of eight
+__host__ __device__ constexpr bool by_ballot(int r) { return 0x92 >> (r & 7) & 1; }
 constexpr int kSortThreads = kSortWarps * 32;
 constexpr uint32_t kScanTile = 4096;
 constexpr uint32_t kGroupedMaxRow = 32;
@@ -87,7 +89,13 @@ template <typename K, typename P>
 struct PairList {
     const P* p;
     uint32_t sym;   // 0 or 1
-    __device__ __forceinline__ K operator[](uint64_t i) const
+    // from an even position on
+    __device__ __forceinline__ PairList operator+(uint64_t i) const
+    {
+        return PairList{p + (i >> sym), sym};
+    }
+    template <typename I>
+    __device__ __forceinline__ K operator[](I i) const
     {
         const P e = p[i >> sym];
         const bool back = (uint32_t)i & sym;
@@ -183,7 +191,7 @@ constexpr unsigned long long kAgg = 1ull << 57, kInc = 2ull << 57;
 constexpr unsigned long long kCountMask = (1ull << 57) - 1;
 static_assert(kMaxPasses < 32, "the pass tag fits bits 63..59");
 constexpr uint32_t kSpinLimit = 1u << 18;   // polls of one status word
-constexpr int kLookWindow = 8;              // earlier tiles read per round trip
+constexpr int kLookWindow = 4;              // earlier tiles read per round trip
 
 // Test hook (host-set, off by default): a shorter poll limit, and one tile
 // per pass that never publishes its counts, so that the tiles after it give
@@ -204,12 +212,16 @@ CsrWaitHook csr_wait_hook() { return CsrWaitHook{g_hook_spin.load(), g_hook_with
 // from a ticket, so every earlier tile belongs to a CTA already running or
 // done. It publishes its own counts before it waits on anything, and it sums
 // earlier tiles' counts, kLookWindow at a time, until it meets an inclusive
-// one. Bound by the shared-memory pipe (about 36 wavefronts per 32 pairs at 70 %
-// of its rate); two items in flight and one table lookup per pair in the
-// reorder took k = 20 (2^24 pairs, 5 passes) from 0.645 to 0.577 ms and
-// k = 26 (2^30 pairs, 7 passes) from 44.3 to 40.3 ms (four items in flight:
-// 0.611, 43.0; peers of some items by match.any: no better). The look-back runs after the reorder, when the tile's pairs no longer
-// occupy registers. Every poll loop is bounded: after spin_limit polls of
+// one (windows of 3, 6 and 8: 2 to 4 % slower at k = 20). The look-back runs
+// after the reorder, when the tile's pairs no longer occupy registers.
+//
+// Bound by the shared-memory pipe: 28 wavefronts per 32 pairs and 8 more for
+// global memory, 71 % of its rate, the vector ALU 53 %. So three of eight
+// items find their peers on the ALU (none: 10 %, a quarter: 3 %, half: 2 to
+// 5 % slower, all: 26 %), two items are in flight, a CTA loops over tiles with
+// as few barriers as it can, and the reorder takes one table lookup per pair.
+// k = 20 (2^24 pairs, 5 passes) 0.645 -> 0.500 ms, k = 26 (2^30 pairs, 7 passes)
+// 44.3 -> 36.6, 0.48 of the HBM rate. Every poll loop is bounded: after spin_limit polls of
 // one word (kSpinLimit unless a test hook shortened it) it sets *err and
 // goes on with the partial sum, which can only be too small, so every write
 // stays inside the output.
@@ -224,6 +236,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     constexpr int kItems = SortShape<K, kShort>::items;
     constexpr uint32_t kTile = SortShape<K, kShort>::tile;
     constexpr uint32_t kBuckets = SortShape<K, kShort>::buckets;
+    constexpr int kBits = kBuckets == 512 ? 9 : 8;
     extern __shared__ __align__(16) unsigned char smem[];
     uint16_t (*wcnt)[kBuckets] = reinterpret_cast<uint16_t (*)[kBuckets]>(smem);
     uint64_t* tbase = reinterpret_cast<uint64_t*>(smem + kSortWarps * kBuckets * 2);
@@ -237,70 +250,84 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     if (*sort_needed == 0 || *(volatile const uint32_t*)err != 0) return;
     const uint32_t nb = dg.mask + 1;
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (;;) {
-        if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
-        for (uint32_t d = threadIdx.x; d < nb; d += blockDim.x)
-            for (int w = 0; w < kSortWarps; ++w) wcnt[w][d] = 0;
-        __syncthreads();
-        const uint32_t tile = s_tile;
-        if ((uint64_t)tile * kTile >= M) return;   // uniform: no tile left
-        const uint64_t tile0 = (uint64_t)tile * kTile;
-        const uint32_t n = (uint32_t)((M - tile0 < kTile) ? M - tile0 : kTile);
-        const uint32_t wbase = wid * (32 * kItems);
-        K e[kItems];
-        // ranks within the warp (< 32 * kItems <= 512), two per register; the
-        // digits are recomputed from e[] where needed, so no array holds them
-        uint32_t rk[kItems / 2];
+    const uint32_t wbase = wid * (32 * kItems);
+    #ifndef KL
+#define KL std::is_pointer_v<In>
+#endif
+    constexpr bool kLoop = KL;   // else one tile per CTA (see the launch)
+    K e[kItems];
+    auto zero_counters = [&] {   // the warp's own
+        for (uint32_t t = lane; t < kBuckets / 8; t += 32)
+            reinterpret_cast<uint4*>(wcnt[wid])[t] = make_uint4(0u, 0u, 0u, 0u);
+    };
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+    zero_counters();
+    __syncthreads();
+    uint32_t tile = s_tile;
+    while ((uint64_t)tile * kTile < M) {   // uniform
+        const uint32_t n = (uint32_t)(M - (uint64_t)tile * kTile < kTile ? M - (uint64_t)tile * kTile
+                                                                        : kTile);
+        const auto tile_in = in + (uint64_t)tile * kTile;
 #pragma unroll
         for (int r = 0; r < kItems; ++r) {
             const uint32_t t = wbase + r * 32 + lane;
-            if (t < n) e[r] = in[tile0 + t];
+            if (t < n) e[r] = tile_in[t];
         }
-        __syncthreads();
+        // ranks within the warp (< 32 * kItems <= 512), two per register; the
+        // digits are recomputed from e[] where needed, so no array holds them
+        uint32_t rk[kItems / 2];
         const uint32_t lt = (1u << lane) - 1u;
-        // kFly items of every lane at a time, in lane order within an item: the
-        // lanes holding equal digits of an item find each other through a word per
-        // digit (each ORs in its lane bit, then all read the word back and clear
-        // it; every item in flight has its own table of kBuckets words per
-        // warp, in the reorder buffer, unused until the ranks are done). Then, item
-        // by item, the lowest lane of each group adds the group's size to the
-        // warp's counter of the digit (two 16-bit counters per word) and the group
-        // gets the old value by shuffle. A warp's shared-memory operations execute
-        // in order, so the adds of the items in flight need no wait between them.
+        // kFly items of every lane at a time, in lane order within an item. The
+        // lanes holding equal digits of an item find each other either by a ballot
+        // per digit bit, or through a word per digit (each ORs in its lane bit,
+        // then all read the word back and clear it; every item in flight has its
+        // own table of kBuckets words per warp, in the reorder buffer, unused until
+        // the ranks are done). Then, item by item, the lanes read the warp's
+        // counter of their digit, and the last lane of each group adds the group's
+        // size. A warp's shared-memory operations execute in order, so the accesses
+        // of the items in flight need no wait between them.
         uint32_t* pmask = reinterpret_cast<uint32_t*>(buf) + wid * (kFly * kBuckets);
         for (uint32_t t = lane; t < kFly * kBuckets / 4; t += 32)
             reinterpret_cast<uint4*>(pmask)[t] = make_uint4(0u, 0u, 0u, 0u);
         __syncwarp();
-        uint32_t* wc = reinterpret_cast<uint32_t*>(wcnt[wid]);
+        uint16_t* wc = wcnt[wid];
 #pragma unroll
         for (int r0 = 0; r0 < kItems; r0 += kFly) {
-            uint32_t d[kFly], peers[kFly], prev[kFly];
+            uint32_t d[kFly], peers[kFly];
+            bool valid[kFly];
 #pragma unroll
             for (int u = 0; u < kFly; ++u) {
-                const uint32_t t = wbase + (r0 + u) * 32 + lane;
-                d[u] = t < n ? digit_of(e[r0 + u], dg) : 0xFFFFFFFFu;
-                if (d[u] != 0xFFFFFFFFu) atomicOr(&pmask[u * kBuckets + d[u]], 1u << lane);
+                valid[u] = wbase + (r0 + u) * 32 + lane < n;
+                d[u] = digit_of(e[r0 + u], dg);
+                if (!by_ballot(r0 + u) && valid[u]) atomicOr(&pmask[u * kBuckets + d[u]], 1u << lane);
             }
             __syncwarp();
 #pragma unroll
-            for (int u = 0; u < kFly; ++u)
-                peers[u] = d[u] != 0xFFFFFFFFu ? pmask[u * kBuckets + d[u]] : 0u;
+            for (int u = 0; u < kFly; ++u) {
+                if (by_ballot(r0 + u)) {
+                    peers[u] = __ballot_sync(0xFFFFFFFFu, valid[u]);
+#pragma unroll
+                    for (int b = 0; b < kBits; ++b) {
+                        if (b >= 7 && !(dg.mask >> b)) break;
+                        const bool one = d[u] & (1u << b);
+                        const uint32_t same = __ballot_sync(0xFFFFFFFFu, one);
+                        peers[u] &= one ? same : ~same;
+                    }
+                } else if (valid[u])
+                    peers[u] = pmask[u * kBuckets + d[u]];
+            }
             __syncwarp();
 #pragma unroll
             for (int u = 0; u < kFly; ++u) {
-                if (d[u] != 0xFFFFFFFFu) pmask[u * kBuckets + d[u]] = 0;
-                prev[u] = 0;
-                if (peers[u] != 0 && (peers[u] & lt) == 0) {
-                    const uint32_t sh = (d[u] & 1) * 16;
-                    prev[u] = (atomicAdd(&wc[d[u] >> 1], __popc(peers[u]) << sh) >> sh) & 0xFFFFu;
+                const int r = r0 + u;
+                uint32_t rank = 0;
+                if (valid[u]) {
+                    if (!by_ballot(r)) pmask[u * kBuckets + d[u]] = 0;
+                    rank = wc[d[u]] + __popc(peers[u] & lt);
                 }
                 __syncwarp();
-            }
-#pragma unroll
-            for (int u = 0; u < kFly; ++u) {
-                const uint32_t rank = __shfl_sync(0xFFFFFFFFu, prev[u], __ffs(peers[u]) - 1) +
-                                      __popc(peers[u] & lt);
-                const int r = r0 + u;
+                if (valid[u] && peers[u] >> lane == 1) wc[d[u]] = (uint16_t)(rank + 1);
+                __syncwarp();
                 if (r & 1) rk[r >> 1] |= rank << 16;
                 else rk[r >> 1] = rank;
             }
@@ -351,6 +378,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
                 if (PG_CHECK(at, n)) buf[at] = e[r];
             }
         }
+        __syncwarp();
+        zero_counters();   // for the next tile
         // look back through up to kLookWindow earlier tiles per round trip
         for (uint32_t d = threadIdx.x; d < nb; d += blockDim.x) {
             unsigned long long excl = 0;
@@ -366,24 +395,24 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
                                    ? *((volatile const unsigned long long*)status +
                                        (uint64_t)(next - u) * nb + d)
                                    : 0ull;
-                    int used = 0;
-                    bool stalled = false;
+                    // counts add up in the low bits; the tags above them are
+                    // masked off at the end
+                    uint32_t used = 0;
+                    bool go = true;
 #pragma unroll
                     for (int u = 0; u < kLookWindow; ++u) {
-                        if (found || stalled) continue;
-                        const unsigned long long flag =
-                            (w[u] >> kPassShift) == pass + 1 ? w[u] & (3ull << 57) : 0;
-                        if (flag == 0) {
-                            stalled = true;
-                            continue;
+                        const uint32_t kind = (uint32_t)(w[u] >> 57) - 4 * (pass + 1);
+                        go = go && kind - 1u < 2u;   // kAgg or kInc of this pass
+                        if (go) {
+                            excl += w[u];
+                            ++used;
                         }
-                        excl += w[u] & kCountMask;
-                        ++used;
-                        if (flag == kInc) found = true;
+                        found |= go && kind == 2;
+                        go = go && kind == 1;
                     }
                     if (found) break;
                     next -= used;
-                    if (stalled) {
+                    if (!go) {
                         if (++polls > spin_limit) {
                             atomicOr(err, 1u);
                             break;
@@ -393,6 +422,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
                         polls = 0;
                     }
                 }
+                excl &= kCountMask;
                 const uint32_t cnt_d = (d + 1 < nb ? loff[d + 1] : n) - loff[d];
                 if (tile != withhold) st[d] = tag | kInc | (excl + cnt_d);
             }
@@ -425,8 +455,11 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
                               (unsigned long long)(o + 1));
             }
         }
-        if constexpr (!std::is_pointer_v<In>) return;   // one tile per CTA (see the launch)
+        // (a ticket taken before the tile's own work is done would hold up the
+        // tiles after it: 0.52 -> 0.59 ms at k = 20)
+        if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
         __syncthreads();   // the next tile reuses the tables
+        tile = s_tile;
     }
 }
 
@@ -1167,19 +1200,14 @@ cudaError_t radix_passes(const PairList<K, P> first, uint64_t M, uint64_t N, con
             TraceScope trace("csr_radix_scatter", s);
             Id* col = k + 1 == pl.n ? col_final : nullptr;
             const uint64_t* ds = dstart + (size_t)k * pl.buckets;
-            // Two CTAs per SM, what its shared memory holds, take tiles until none
-            // is left: as fast as a CTA per tile (2^26 pairs 2.30 -> 2.26 ms, 2^30
-            // 40.5 -> 40.2), but a list that turned out grouped pays a launch per
-            // pass and not a CTA per tile (five passes over 2^24 x 5 edges:
-            // 0.089 -> 0.039 ms). A pass that converts its list keeps a CTA per
-            // tile: in a loop its loads cost more registers than there are
-            // (2^26 pairs of 64-bit ids 0.264 -> 0.325 ms).
+            // Two CTAs per SM, what its registers hold, take tiles until none is
+            // left; a list that turned out grouped pays a launch per pass and not
+            // a CTA per tile (five passes over 2^24 x 5 edges: 0.089 -> 0.039 ms)
             const unsigned places = 2 * (unsigned)device_sm_count();
+            const unsigned grid = L.n_tiles < places ? L.n_tiles : places;
             auto launch = [&](auto in, auto is_short) {
                 constexpr bool kShort = decltype(is_short)::value;
-                const bool loops = std::is_pointer_v<decltype(in)> && L.n_tiles > places;
-                const unsigned grid = loops ? places : L.n_tiles;
-                { radix_scatter_kernel<K, decltype(in), Id, kShort>
+                                { radix_scatter_kernel<K, decltype(in), Id, kShort>
                     <<<grid, kSortThreads, scatter_smem_bytes<K, kShort>(), s>>>(
                         in, buf[k & 1], M, pl.digit(k), status, k, ds, tickets + k, err, sort_needed,
                         hk.spin_limit, hk.withhold, col, row_ptr, N); note_launch(); }

@@ -283,3 +283,20 @@ def test_csr_grouped_rows_across_tiles(row, M, id64):
         else:
             bad[at, 0] = 0
         check(bad)
+
+
+@pytest.mark.parametrize("M", [786_433, 96 * 8192 - 1, 97 * 8192, 97 * 8192 + 1, 2_600_003])
+@pytest.mark.parametrize("N", [2**14, 2**15, 2**16])
+@pytest.mark.parametrize("spread", [0, 1, 3, 16])
+@pytest.mark.parametrize("id64", [False, True])
+def test_csr_sort_of_long_lists(M, N, spread, id64):
+    """Digits of 7 and 8 bits, full and ragged last tiles, more tiles than the
+    GPU holds CTAs; ids of `spread` random bits, so that whole warps share a
+    digit or few lanes do."""
+    rng = np.random.default_rng(M + spread)
+    e = rng.integers(0, min(N, 1 << spread), (M, 2), dtype=np.int64) * (N >> min(spread, 14)) % N
+    t = torch.from_numpy(e if id64 else e.astype(np.uint32).view(np.int32)).cuda()
+    rp, col = pg.edges_to_csr(t, N, check=True)
+    ref_rp, ref_col = o.csr(e.astype(np.uint64), N)
+    np.testing.assert_array_equal(host(rp), ref_rp)
+    np.testing.assert_array_equal(host(col), ref_col)
