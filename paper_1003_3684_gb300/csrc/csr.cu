@@ -254,7 +254,6 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
     #ifndef KL
 #define KL std::is_pointer_v<In>
 #endif
-    constexpr bool kLoop = KL;   // else one tile per CTA (see the launch)
     K e[kItems];
     auto zero_counters = [&] {   // the warp's own
         for (uint32_t t = lane; t < kBuckets / 8; t += 32)
@@ -1207,7 +1206,7 @@ cudaError_t radix_passes(const PairList<K, P> first, uint64_t M, uint64_t N, con
             const unsigned grid = L.n_tiles < places ? L.n_tiles : places;
             auto launch = [&](auto in, auto is_short) {
                 constexpr bool kShort = decltype(is_short)::value;
-                                { radix_scatter_kernel<K, decltype(in), Id, kShort>
+                { radix_scatter_kernel<K, decltype(in), Id, kShort>
                     <<<grid, kSortThreads, scatter_smem_bytes<K, kShort>(), s>>>(
                         in, buf[k & 1], M, pl.digit(k), status, k, ds, tickets + k, err, sort_needed,
                         hk.spin_limit, hk.withhold, col, row_ptr, N); note_launch(); }
