@@ -182,35 +182,6 @@ struct BfsState {
 };
 static_assert(sizeof(BfsState) <= 256, "the counters' region of the workspace");
 
-// Barrier over a cooperative grid. Each wait is bounded; one that gives up
-// sets the error word and its CTA leaves the kernel, so the others give up too.
-constexpr uint32_t kBarrierPolls = 1u << 24;   // some ten seconds
-__device__ __forceinline__ bool grid_barrier(BfsState* st, uint32_t& epoch)
-{
-    __shared__ uint32_t s_ok;
-    __syncthreads();
-    ++epoch;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&st->arrived, 1u);
-        const uint32_t want = epoch * gridDim.x;
-        uint32_t polls = 0, ok = 1;
-        // (the count may wrap; it is never far from what is waited for)
-        while ((int32_t)(*(volatile uint32_t*)&st->arrived - want) < 0) {
-            if (++polls > kBarrierPolls || *(volatile uint32_t*)&st->error) {
-                atomicOr(&st->error, 1u);
-                ok = 0;
-                break;
-            }
-            __nanosleep(32);
-        }
-        __threadfence();
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
 // One step of two adjacency entries per lane, both loads in flight.
 template <typename F>
 __device__ __forceinline__ void bfs_claim_two(BfsQueue& Q, uint64_t N, uint32_t lane, uint32_t lt,
@@ -377,13 +348,13 @@ __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_top_down_kernel(
         bfs_short_rows(row_ptr, col, frontier, fsize, Q, wstart[wid], wrow[wid],
                        &state->longs[slot], long_v, long_base);
         Q.flush(lane);
-        if (!grid_barrier(state, epoch)) return;
+        if (!grid_barrier(&state->arrived, &state->error, epoch)) return;
         const unsigned long long ctr = __ldcg(&state->longs[slot]);
         if (ctr) {   // the same in every CTA
             Q.held = 0;
             bfs_long_rows(row_ptr, col, Q, ctr, slice_of(fsize), long_v, long_base);
             Q.flush(lane);
-            if (!grid_barrier(state, epoch)) return;
+            if (!grid_barrier(&state->arrived, &state->error, epoch)) return;
         }
         fsize = __ldcg(&state->size[slot]);
         visited += fsize;

@@ -10,7 +10,7 @@
 //
 // Any other list: least-significant-digit radix sort of the (src, dst) keys,
 // from the low bits of dst to the high bits of src, up to 8 bits per pass (9 for short lists):
-//   radix_hist_all one read of the list counts the digits of every pass
+//   radix_hist     one read of the list counts the digits of every pass
 //                  (the totals do not depend on the order a pass leaves);
 //   radix_dstart   per pass, where each digit's run starts in the output;
 //   radix_scatter  per pass: stable rank of each element within its tile
@@ -18,6 +18,7 @@
 //                  counters + cross-warp scan), a reorder in shared memory, the tile's
 //                  start in each digit's run by decoupled look-back over the
 //                  earlier tiles' published counts, and coalesced writes.
+// A short list does the three in one launch, radix_sort.
 // Ranks come from counts in entry order, never from atomics racing for a
 // slot, so the result does not depend on the schedule, and a power-law row
 // (a hub with 10^5 edges) costs no more than any other key. The last pass
@@ -46,7 +47,7 @@ __host__ __device__ constexpr bool by_ballot(int r) { return 0x92 >> (r & 7) & 1
 constexpr int kSortThreads = kSortWarps * 32;
 constexpr uint32_t kScanTile = 4096;
 constexpr uint32_t kGroupedMaxRow = 32;
-constexpr uint32_t kHistCopies = 8;   // copies of each digit counter in the histogram kernel
+constexpr uint32_t kHistCopies = 8;   // copies of each digit counter, half as many in the short-list kernel
 
 template <typename Id>
 struct PairOf;
@@ -110,8 +111,8 @@ struct PairList {
 // 64-bit) per thread and digits of at most 8 bits. Short lists, up to
 // kShortList pairs, are fewer tiles than the GPU has places, so a pass takes a
 // tile's latency: tiles of half the size, and digits of 9 bits for fewer
-// passes (100,003 pairs, k = 13: 0.088 -> 0.071 ms, 2^19 pairs: 0.114 -> 0.108;
-// 2^20 pairs lose, 0.120 -> 0.135).
+// passes (100,003 pairs, k = 13: 0.088 -> 0.071 ms, 2^19 pairs: 0.114 -> 0.108, both
+// with a launch per pass; 2^20 pairs lose, 0.120 -> 0.135).
 template <typename K, bool kShort>
 struct SortShape {
     static constexpr int items = (sizeof(K) == 8 ? 16 : 8) / (kShort ? 2 : 1);
@@ -136,24 +137,24 @@ struct PassList {
         return Digit{field[k], shift[k], nd, (1u << bits[k]) - 1};
     }
 };
-// Digit totals of every pass in one read of the list: tot[k][d] = number of
+// Digit totals of every pass in one read of the list: tot[k][d] += number of
 // pairs whose pass-k digit is d. Each CTA counts into shared memory
-// (n passes x pl.buckets counters, kHistCopies copies of each) and adds its
-// counts once.
-template <typename K, typename In>
-__global__ void __launch_bounds__(256) radix_hist_all_kernel(
-    const In in, uint64_t M, const __grid_constant__ PassList pl,
-    unsigned long long* __restrict__ tot, const uint32_t* __restrict__ sort_needed)
+// (n passes x pl.buckets counters, kCopies copies of each) and adds its
+// counts once. Bound by the shared-memory atomics, one per pair and pass (2^30
+// pairs, 7 passes: 3.7 ms, of which reading the list takes 1.3).
+template <typename K, uint32_t kCopies, typename In>
+__device__ __forceinline__ void count_digits(const In in, uint64_t M, const PassList& pl,
+                                             unsigned long long* tot)
 {
-    extern __shared__ uint32_t h[];
-    if (*sort_needed == 0) return;
-    // kHistCopies copies of every counter, interleaved, lane l adding to copy
-    // l mod kHistCopies: lanes whose digits agree (the skewed digits of a
-    // power-law graph) mostly hit different words
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint32_t* h = reinterpret_cast<uint32_t*>(smem);
+    // the copies of a counter are interleaved, lane l adding to copy l mod
+    // kCopies: lanes whose digits agree (the skewed digits of a power-law
+    // graph) mostly hit different words
     const uint32_t cells = pl.n * pl.buckets;
-    for (uint32_t t = threadIdx.x; t < cells * kHistCopies; t += blockDim.x) h[t] = 0;
+    for (uint32_t t = threadIdx.x; t < cells * kCopies; t += blockDim.x) h[t] = 0;
     __syncthreads();
-    const uint32_t copy = threadIdx.x & (kHistCopies - 1);
+    const uint32_t copy = threadIdx.x & (kCopies - 1);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     constexpr int kU = 4;
     for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < M; i0 += kU * stride) {
@@ -163,20 +164,19 @@ __global__ void __launch_bounds__(256) radix_hist_all_kernel(
             if (i0 + u * stride < M) e[u] = in[i0 + u * stride];
         // pass by pass, so that each pass's digit rule is read once for the
         // kU elements
+#pragma unroll 2
         for (uint32_t k = 0; k < pl.n; ++k) {
             const Digit dg = pl.digit(k);
-            uint32_t* hk = h + (k * pl.buckets) * kHistCopies + copy;
+            uint32_t* hk = h + (k * pl.buckets) * kCopies + copy;
 #pragma unroll
             for (int u = 0; u < kU; ++u)
-                if (i0 + u * stride < M)
-                    atomicAdd(&hk[digit_of(e[u], dg) * kHistCopies], 1u);
+                if (i0 + u * stride < M) atomicAdd(&hk[digit_of(e[u], dg) * kCopies], 1u);
         }
     }
     __syncthreads();
     for (uint32_t t = threadIdx.x; t < cells; t += blockDim.x) {
         uint32_t c = 0;
-#pragma unroll
-        for (uint32_t r = 0; r < kHistCopies; ++r) c += h[t * kHistCopies + r];
+        for (uint32_t r = 0; r < kCopies; ++r) c += h[t * kCopies + r];
         if (c) atomicAdd(&tot[t], (unsigned long long)c);
     }
 }
@@ -203,6 +203,55 @@ std::atomic<uint32_t> g_hook_spin{kSpinLimit};
 std::atomic<uint32_t> g_hook_withhold{0xFFFFFFFFu};
 CsrWaitHook csr_wait_hook() { return CsrWaitHook{g_hook_spin.load(), g_hook_withhold.load()}; }
 
+// Exclusive scan of the CTA's values, and their sum.
+__device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t v, uint64_t* s_warp,
+                                                         uint64_t& total)
+{
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t nw = blockDim.x >> 5;
+    uint64_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= (uint32_t)o) x += y;
+    }
+    if (lane == 31) s_warp[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        uint64_t w = lane < nw ? s_warp[lane] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, w, o);
+            if (lane >= (uint32_t)o) w += y;
+        }
+        if (lane < nw) s_warp[lane] = w;   // inclusive warp totals
+    }
+    __syncthreads();
+    total = s_warp[nw - 1];
+    const uint64_t before = wid ? s_warp[wid - 1] : 0;
+    __syncthreads();
+    return before + x - v;
+}
+
+// What a sort works on. The words are the workspace's, in order: a ticket per
+// pass, the wait error, the passes in which a wait gave up (a bit each), and
+// the grid barrier's two.
+constexpr int kWordErr = kMaxPasses, kWordFailed = kWordErr + 1, kWordBarrier = kWordFailed + 1;
+template <typename K, typename P, typename Id>
+struct SortJob {
+    PairList<K, P> first;
+    const K* plain;   // the list where it is what the passes move already, else null
+    K* buf[2];
+    uint64_t M, N, n_status16, n_rows;
+    unsigned long long *status, *tot;
+    uint32_t* words;
+    const uint32_t* sort_needed;   // null: always
+    Id* col;                       // null: the last pass writes pairs, too
+    uint64_t* row_ptr;
+    CsrWaitHook hook;
+    PassList pl;
+};
+
 // One LSD pass over a tile: load once, rank stably (per warp by match, then
 // across warps), reorder the tile by digit in shared memory, and write each
 // digit's run to its place in the output with consecutive threads on
@@ -226,40 +275,32 @@ CsrWaitHook csr_wait_hook() { return CsrWaitHook{g_hook_spin.load(), g_hook_with
 // goes on with the partial sum, which can only be too small, so every write
 // stays inside the output.
 template <typename K, typename In, typename Id, bool kShort>
-__global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
-    const In in, K* __restrict__ out, uint64_t M, const Digit dg,
-    unsigned long long* __restrict__ status,
-    uint32_t pass, const uint64_t* __restrict__ dstart, uint32_t* __restrict__ ticket,
-    uint32_t* __restrict__ err, const uint32_t* __restrict__ sort_needed, uint32_t spin_limit,
-    uint32_t withhold, Id* __restrict__ col_out, uint64_t* __restrict__ row_ptr, uint64_t N)
+__device__ __forceinline__ void scatter_pass(
+    const In in, K* __restrict__ out, Id* __restrict__ col_out, uint64_t* __restrict__ row_ptr,
+    const uint64_t M, const uint64_t N, const Digit dg, const uint32_t pass,
+    const uint64_t* __restrict__ dstart, unsigned long long* __restrict__ status,
+    uint32_t* __restrict__ words, const uint32_t spin_limit, const uint32_t withhold)
 {
+    extern __shared__ __align__(16) unsigned char smem[];
     constexpr int kItems = SortShape<K, kShort>::items;
     constexpr uint32_t kTile = SortShape<K, kShort>::tile;
     constexpr uint32_t kBuckets = SortShape<K, kShort>::buckets;
     constexpr int kBits = kBuckets == 512 ? 9 : 8;
-    extern __shared__ __align__(16) unsigned char smem[];
     uint16_t (*wcnt)[kBuckets] = reinterpret_cast<uint16_t (*)[kBuckets]>(smem);
     uint64_t* tbase = reinterpret_cast<uint64_t*>(smem + kSortWarps * kBuckets * 2);
     uint32_t* loff = reinterpret_cast<uint32_t*>(tbase + kBuckets);
     K* buf = reinterpret_cast<K*>(loff + kBuckets);                                  // tile
     __shared__ uint32_t s_part[kSortWarps + 1];
     __shared__ uint32_t s_tile;
-    // after a wait that gave up in an earlier pass the list this pass reads
-    // no longer has the digit totals dstart was made from, so a scatter
-    // could leave the output: the remaining passes do nothing
-    if (*sort_needed == 0 || *(volatile const uint32_t*)err != 0) return;
     const uint32_t nb = dg.mask + 1;
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint32_t wbase = wid * (32 * kItems);
-    #ifndef KL
-#define KL std::is_pointer_v<In>
-#endif
     K e[kItems];
     auto zero_counters = [&] {   // the warp's own
         for (uint32_t t = lane; t < kBuckets / 8; t += 32)
             reinterpret_cast<uint4*>(wcnt[wid])[t] = make_uint4(0u, 0u, 0u, 0u);
     };
-    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+    if (threadIdx.x == 0) s_tile = atomicAdd(words + pass, 1u);
     zero_counters();
     __syncthreads();
     uint32_t tile = s_tile;
@@ -413,7 +454,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
                     next -= used;
                     if (!go) {
                         if (++polls > spin_limit) {
-                            atomicOr(err, 1u);
+                            atomicOr(words + kWordErr, 1u);
+                            atomicOr(words + kWordFailed, 1u << pass);
                             break;
                         }
                         __nanosleep(32);
@@ -456,9 +498,105 @@ __global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
         }
         // (a ticket taken before the tile's own work is done would hold up the
         // tiles after it: 0.52 -> 0.59 ms at k = 20)
-        if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+        if (threadIdx.x == 0) s_tile = atomicAdd(words + pass, 1u);
         __syncthreads();   // the next tile reuses the tables
         tile = s_tile;
+    }
+}
+
+// What comes before the passes: the digits are counted, the status words start
+// at zero, and the row ends that the grouped pass wrote before it gave up go.
+template <uint32_t kCopies, typename K, typename P, typename Id, typename In>
+__device__ __forceinline__ void prepare_passes(const In in, const SortJob<K, P, Id>& job)
+{
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    count_digits<K, kCopies>(in, job.M, job.pl, job.tot);
+    for (uint64_t i = t; i < job.n_status16; i += stride)
+        reinterpret_cast<uint4*>(job.status)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint64_t i = t; i < job.n_rows; i += stride) job.row_ptr[i] = 0;
+}
+
+// After a wait that gave up in a pass the list the next ones read no longer
+// has the digit totals the starts are made from, so a scatter could leave the
+// output: the remaining passes do nothing.
+__device__ __forceinline__ bool pass_can_run(const uint32_t* words, uint32_t pass)
+{
+    return (*(volatile const uint32_t*)(words + kWordFailed) & ((1u << pass) - 1)) == 0;
+}
+
+// A long list: a launch for the digits, then one per pass. (One cooperative
+// launch, as below, spills 264 bytes per thread in this shape.)
+template <typename K, typename In, typename P, typename Id>
+__global__ void __launch_bounds__(256)
+    radix_hist_kernel(const In in, const __grid_constant__ SortJob<K, P, Id> job)
+{
+    if (job.sort_needed && *job.sort_needed == 0) return;
+    prepare_passes<kHistCopies>(in, job);
+}
+// Where each digit's run starts in pass k's output: the exclusive scan of
+// that pass's digit totals. grid = passes, block = pl.buckets threads.
+__global__ void __launch_bounds__(kMaxBuckets) radix_dstart_kernel(
+    const unsigned long long* __restrict__ tot, const __grid_constant__ PassList pl,
+    uint64_t* __restrict__ dstart, const uint32_t* __restrict__ sort_needed)
+{
+    __shared__ uint64_t s_warp[32];
+    if (sort_needed && *sort_needed == 0) return;
+    const uint32_t k = blockIdx.x, nb = 1u << pl.bits[k], d = threadIdx.x;
+    const uint64_t c = d < nb ? tot[(size_t)k * pl.buckets + d] : 0;
+    uint64_t total;
+    const uint64_t ex = block_exclusive_scan(c, s_warp, total);
+    if (d < nb) dstart[(size_t)k * pl.buckets + d] = ex;
+}
+template <typename K, typename In, typename Id>
+__global__ void __launch_bounds__(kSortThreads, 2) radix_scatter_kernel(
+    const In in, K* __restrict__ out, Id* __restrict__ col_out, uint64_t* __restrict__ row_ptr,
+    const uint64_t M, const uint64_t N, const Digit dg, const uint32_t pass,
+    const uint64_t* __restrict__ dstart, unsigned long long* __restrict__ status,
+    uint32_t* __restrict__ words, const uint32_t* __restrict__ sort_needed,
+    const uint32_t spin_limit, const uint32_t withhold)
+{
+    if (sort_needed && *sort_needed == 0) return;
+    if (!pass_can_run(words, pass)) return;
+    scatter_pass<K, In, Id, false>(in, out, col_out, row_ptr, M, N, dg, pass, dstart, status, words, spin_limit,
+                                   withhold);
+}
+
+// A short list in one cooperative launch, a grid barrier between its parts: a
+// launch per part costs more than most parts' work (CSR of 100,003 pairs,
+// k = 13: 0.067 -> 0.051 ms, 2^19 pairs: 0.098 -> 0.073), and a list that turned
+// out grouped pays one launch (160,000 vertices, m = 4: 0.057 -> 0.034).
+template <typename K, typename P, typename Id>
+__global__ void __launch_bounds__(kSortThreads, 2)
+    radix_sort_kernel(const __grid_constant__ SortJob<K, P, Id> job)
+{
+    if (job.sort_needed && *job.sort_needed == 0) return;
+    if (job.plain) prepare_passes<kHistCopies / 2>((const K*)job.plain, job);
+    else prepare_passes<kHistCopies / 2>(job.first, job);
+    __shared__ uint64_t s_dstart[kMaxBuckets], s_warp[32];
+    uint32_t epoch = 0;
+    for (uint32_t pass = 0; pass < job.pl.n; ++pass) {
+        if (!grid_barrier(job.words + kWordBarrier, job.words + kWordBarrier + 1, epoch)) {
+            if (threadIdx.x == 0) atomicOr(job.words + kWordErr, 1u);
+            return;
+        }
+        if (!pass_can_run(job.words, pass)) continue;   // the same in every CTA
+        {
+            const uint32_t d = threadIdx.x;
+            uint64_t total;
+            const uint64_t c = d < job.pl.buckets ? __ldcg(job.tot + pass * job.pl.buckets + d) : 0;
+            const uint64_t ex = block_exclusive_scan(c, s_warp, total);
+            if (d < job.pl.buckets) s_dstart[d] = ex;
+            __syncthreads();
+        }
+        auto run = [&](auto in) {
+            scatter_pass<K, decltype(in), Id, true>(
+                in, job.buf[pass & 1], pass + 1 == job.pl.n ? job.col : nullptr, job.row_ptr, job.M,
+                job.N, job.pl.digit(pass), pass, s_dstart, job.status, job.words,
+                job.hook.spin_limit, job.hook.withhold);
+        };
+        if (pass > 0 || job.plain) run((const K*)(pass ? job.buf[(pass - 1) & 1] : job.plain));
+        else run(job.first);
     }
 }
 
@@ -468,7 +606,7 @@ static_assert(SortShape<uint2, true>::items % kFly == 0 &&
               "whole groups of items");
 
 template <typename K, bool kShort>
-size_t scatter_smem_bytes()
+constexpr size_t sort_smem_bytes()
 {
     using Shape = SortShape<K, kShort>;
     // the reorder buffer, in which the digit words of the items in flight lie too
@@ -478,71 +616,12 @@ size_t scatter_smem_bytes()
            (tile > words ? tile : words);
 }
 
-// ---- exclusive scan of uint32 counts into uint64 offsets ------------------
-__device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t v, uint64_t* s_warp,
-                                                         uint64_t& total)
-{
-    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint32_t nw = blockDim.x >> 5;
-    uint64_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-        if (lane >= (uint32_t)o) x += y;
-    }
-    if (lane == 31) s_warp[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        uint64_t w = lane < nw ? s_warp[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, w, o);
-            if (lane >= (uint32_t)o) w += y;
-        }
-        if (lane < nw) s_warp[lane] = w;   // inclusive warp totals
-    }
-    __syncthreads();
-    total = s_warp[nw - 1];
-    const uint64_t before = wid ? s_warp[wid - 1] : 0;
-    __syncthreads();
-    return before + x - v;
-}
-
-// Zeroes the tile status words, and the row pointers a grouped list's tiles may
-// have written (n_rows of them), before a sort (nothing when no sort runs).
-__global__ void __launch_bounds__(256) sort_init_kernel(uint4* __restrict__ p, uint64_t n16,
-                                                        uint64_t* __restrict__ row_ptr, uint64_t n_rows,
-                                                        const uint32_t* __restrict__ sort_needed)
-{
-    if (*sort_needed == 0) return;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (uint64_t i = t; i < n16; i += stride) p[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (uint64_t i = t; i < n_rows; i += stride) row_ptr[i] = 0;
-}
-// Where each digit's run starts in pass k's output: the exclusive scan of
-// that pass's digit totals. grid = passes, block = pl.buckets threads.
-__global__ void __launch_bounds__(kMaxBuckets) radix_dstart_kernel(
-    const unsigned long long* __restrict__ tot, const __grid_constant__ PassList pl,
-    uint64_t* __restrict__ dstart, const uint32_t* __restrict__ sort_needed)
-{
-    __shared__ uint64_t s_warp[32];
-    if (*sort_needed == 0) return;
-    const uint32_t k = blockIdx.x, nb = 1u << pl.bits[k], d = threadIdx.x;
-    const uint64_t c = d < nb ? tot[(size_t)k * pl.buckets + d] : 0;
-    uint64_t total;
-    const uint64_t ex = block_exclusive_scan(c, s_warp, total);
-    if (d < nb) dstart[(size_t)k * pl.buckets + d] = ex;
-}
-
 // exclusive scan of n_parts sums in place, one CTA looping over chunks of
 // eight neighbouring sums per thread
 __global__ void __launch_bounds__(1024) scan_parts_kernel(uint64_t* __restrict__ part,
-                                                          uint64_t n_parts,
-                                                          const uint32_t* __restrict__ sort_needed)
+                                                          uint64_t n_parts)
 {
     __shared__ uint64_t s_warp[32];
-    if (*sort_needed == 0) return;
     constexpr int kPer = 8;
     uint64_t carry = 0;
     for (uint64_t base = 0; base < n_parts; base += kPer * blockDim.x) {
@@ -1097,7 +1176,7 @@ CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst =
     o += a256(M * pair_bytes);
     L.off_status = o;   // tile status words of the pass being sorted
     o += a256(L.n_status * 8);
-    L.off_flag = o;     // +0: sort-needed flag, +64: one ticket per pass, +128: look-back error
+    L.off_flag = o;     // +0: sort-needed flag, +64: SortJob's words (+128: wait error)
     o += 256;
     L.off_dig = o;      // digit totals, then digit starts, of every pass
     o += a256(2 * (size_t)kMaxPasses * kMaxBuckets * 8);
@@ -1111,121 +1190,122 @@ CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst =
 // The opt-in shared-memory sizes of the sort kernels, set once per device
 // for each id width.
 PerDeviceOnce g_csr_attrs[2];
-template <typename K, typename In, typename Id, bool kShort>
-cudaError_t scatter_attribute()
+template <typename F>
+cudaError_t allow_smem(F* kernel, size_t bytes)
 {
-    return cudaFuncSetAttribute(radix_scatter_kernel<K, In, Id, kShort>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)scatter_smem_bytes<K, kShort>());
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
-template <typename K, typename In>
-cudaError_t hist_attribute()
+template <typename K, typename P, typename Id>
+cudaError_t long_sort_attributes()
 {
-    return cudaFuncSetAttribute(radix_hist_all_kernel<K, In>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(kMaxPasses * 4 * 256 * kHistCopies));   // of 256, or 8 of 512
+    constexpr size_t smem = sort_smem_bytes<K, false>();
+    static_assert(smem <= 113 * 1024, "two CTAs per SM");
+    constexpr size_t counters = kMaxPasses * 256 * 4 * kHistCopies;
+    return first_error({allow_smem(radix_hist_kernel<K, const K*, P, Id>, counters),
+                        allow_smem(radix_hist_kernel<K, PairList<K, P>, P, Id>, counters),
+                        allow_smem(radix_scatter_kernel<K, const K*, Id>, smem),
+                        allow_smem(radix_scatter_kernel<K, PairList<K, P>, Id>, smem)});
 }
 template <typename Id>
 cudaError_t set_csr_attributes()
 {
     using P = typename PairOf<Id>::T;
     return g_csr_attrs[sizeof(Id) == 8].run_current([] {
-        cudaError_t e = first_error({scatter_attribute<uint2, PairList<uint2, P>, Id, false>(),
-                                     scatter_attribute<uint2, const uint2*, Id, false>(),
-                                     scatter_attribute<uint2, PairList<uint2, P>, Id, true>(),
-                                     scatter_attribute<uint2, const uint2*, Id, true>(),
-                                     hist_attribute<uint2, PairList<uint2, P>>(),
-                                     hist_attribute<uint2, const uint2*>()});
+        constexpr size_t smem = sort_smem_bytes<uint2, true>();
+        static_assert(smem <= 113 * 1024, "two CTAs per SM");
+        static_assert(8 * 512 * 4 * (kHistCopies / 2) <= smem, "the counters of 64 key bits");
+        cudaError_t e = first_error({long_sort_attributes<uint2, P, Id>(),
+                                     allow_smem(radix_sort_kernel<uint2, P, Id>, smem)});
         if constexpr (sizeof(Id) == 8)
-            if (e == cudaSuccess)
-                e = first_error({scatter_attribute<P, PairList<P, P>, Id, false>(),
-                                 scatter_attribute<P, const P*, Id, false>(),
-                                 hist_attribute<P, PairList<P, P>>(),
-                                 hist_attribute<P, const P*>()});
+            if (e == cudaSuccess) e = long_sort_attributes<P, P, Id>();
         return e;
     });
 }
 
-// LSD radix passes over the M pairs of `first` (the digits of the key
-// (src << nd) | dst from its low end); K is what the passes move. *sorted
-// receives the sorted list (unset when there is no digit to sort). With
-// col_final set, the last pass writes the CSR directly instead: destinations
-// to col_final, row ends raised into row_ptr (zeroed by the caller).
 int sort_grid(uint64_t work);
 
-template <typename K, typename P, typename Id>
-cudaError_t radix_passes(const PairList<K, P> first, uint64_t M, uint64_t N, const PassList& pl,
-                         const CsrLayout& L, unsigned char* ws, const uint32_t* sort_needed,
-                         cudaStream_t s, const K** sorted, Id* col_final, uint64_t* row_ptr)
+// The sort's words and digit totals start at zero on every call that has
+// edges; a call without edges has nothing to sort and no wait.
+cudaError_t clear_sort_words(unsigned char* ws, const CsrLayout& L, const PassList& pl, uint64_t M,
+                             cudaStream_t s)
 {
-    K* buf[2] = {(K*)(ws + L.off_a), (K*)(ws + L.off_b)};
-    unsigned long long* status = (unsigned long long*)(ws + L.off_status);
-    unsigned long long* tot = (unsigned long long*)(ws + L.off_dig);
-    uint64_t* dstart = (uint64_t*)(ws + L.off_dig) + (size_t)kMaxPasses * kMaxBuckets;
-    uint32_t* tickets = (uint32_t*)(ws + L.off_flag + 64);
-    uint32_t* err = (uint32_t*)(ws + L.off_flag + 128);
-    // a list that is what the passes move already is read as it is
-    const K* plain = nullptr;
+    const size_t bytes = M > 0 ? L.off_dig - L.off_flag + (size_t)pl.n * pl.buckets * 8 : 4;
+    return cudaMemsetAsync(ws + L.off_flag, 0, bytes, s);
+}
+
+// LSD radix sort of the M pairs of `first` (the digits of the key
+// (src << nd) | dst from its low end), unless *sort_needed is 0; K is what the
+// passes move. *sorted receives the sorted list (unset when there is no digit
+// to sort). With col_final set, the last pass writes the CSR directly instead:
+// destinations to col_final, row ends raised into row_ptr.
+template <typename K, typename P, typename Id>
+cudaError_t radix_sort(const PairList<K, P> first, uint64_t M, uint64_t N, const PassList& pl,
+                       const CsrLayout& L, unsigned char* ws, const uint32_t* sort_needed,
+                       cudaStream_t s, const K** sorted, Id* col_final, uint64_t* row_ptr)
+{
+    SortJob<K, P, Id> job;
+    job.first = first;
+    job.plain = nullptr;
     if constexpr (std::is_same<K, P>::value)
-        if (!first.sym) plain = first.p;
-    const K* cur = plain;
-    const CsrWaitHook hk = csr_wait_hook();
-    // the tickets and the wait error word start at zero on every call that
-    // has edges (a call without edges has nothing to sort and no wait)
-    if (M > 0 && cudaMemsetAsync(ws + L.off_flag + 64, 0, 128, s) != cudaSuccess)
-        return cudaErrorUnknown;
-    if (M > 0 && pl.n > 0) {
-        if (cudaMemsetAsync(tot, 0, (size_t)pl.n * pl.buckets * 8, s) != cudaSuccess)
-            return cudaErrorUnknown;
-        {
-            TraceScope trace("csr_radix_hist", s);
-            const uint64_t n_rows = col_final ? N + 1 : 0;   // else no grouped pass ran
-            const uint64_t work = L.n_status / 2 > n_rows ? L.n_status / 2 : n_rows;
-            { sort_init_kernel<<<sort_grid(work + 1), 256, 0, s>>>(
-                (uint4*)status, (L.n_status * 8 + 15) / 16, row_ptr, n_rows, sort_needed); note_launch(); }
-            const size_t smem = (size_t)pl.n * pl.buckets * 4 * kHistCopies;
-            if (plain)
-                { radix_hist_all_kernel<K, const K*><<<sort_grid(M), 256, smem, s>>>(
-                    plain, M, pl, tot, sort_needed); note_launch(); }
-            else
-                { radix_hist_all_kernel<K, PairList<K, P>><<<sort_grid(M), 256, smem, s>>>(
-                    first, M, pl, tot, sort_needed); note_launch(); }
-        }
-        {
-            TraceScope trace("csr_scan", s);
-            { radix_dstart_kernel<<<pl.n, pl.buckets, 0, s>>>(tot, pl, dstart, sort_needed); note_launch(); }
-        }
-        for (uint32_t k = 0; k < pl.n; ++k) {
-            TraceScope trace("csr_radix_scatter", s);
-            Id* col = k + 1 == pl.n ? col_final : nullptr;
-            const uint64_t* ds = dstart + (size_t)k * pl.buckets;
-            // Two CTAs per SM, what its registers hold, take tiles until none is
-            // left; a list that turned out grouped pays a launch per pass and not
-            // a CTA per tile (five passes over 2^24 x 5 edges: 0.089 -> 0.039 ms)
-            const unsigned places = 2 * (unsigned)device_sm_count();
-            const unsigned grid = L.n_tiles < places ? L.n_tiles : places;
-            auto launch = [&](auto in, auto is_short) {
-                constexpr bool kShort = decltype(is_short)::value;
-                { radix_scatter_kernel<K, decltype(in), Id, kShort>
-                    <<<grid, kSortThreads, scatter_smem_bytes<K, kShort>(), s>>>(
-                        in, buf[k & 1], M, pl.digit(k), status, k, ds, tickets + k, err, sort_needed,
-                        hk.spin_limit, hk.withhold, col, row_ptr, N); note_launch(); }
-            };
-            auto shaped = [&](auto in) {
-                if constexpr (sizeof(K) == 8)
-                    if (pl.buckets == SortShape<K, true>::buckets)
-                        return launch(in, std::true_type());
-                launch(in, std::false_type());
-            };
-            if (k == 0 && !plain) shaped(first);
-            else shaped(cur);
-            const cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            cur = buf[k & 1];
+        if (!first.sym) job.plain = first.p;
+    job.buf[0] = (K*)(ws + L.off_a);
+    job.buf[1] = (K*)(ws + L.off_b);
+    *sorted = pl.n ? job.buf[(pl.n - 1) & 1] : job.plain;
+    if (M == 0 || pl.n == 0) return cudaSuccess;
+    job.M = M;
+    job.N = N;
+    job.n_status16 = (L.n_status * 8 + 15) / 16;
+    job.n_rows = col_final ? N + 1 : 0;   // else no grouped pass ran
+    job.status = (unsigned long long*)(ws + L.off_status);
+    job.tot = (unsigned long long*)(ws + L.off_dig);
+    job.words = (uint32_t*)(ws + L.off_flag + 64);
+    job.sort_needed = sort_needed;
+    job.col = col_final;
+    job.row_ptr = row_ptr;
+    job.hook = csr_wait_hook();
+    job.pl = pl;
+    // Two CTAs per SM, what its registers hold, take tiles until none is left;
+    // a long list that turned out grouped pays a launch per pass and not a CTA
+    // per tile (five passes over 2^24 x 5 edges: 0.089 -> 0.039 ms)
+    const unsigned places = 2 * (unsigned)device_sm_count();
+    const unsigned grid = L.n_tiles < places ? L.n_tiles : places;
+    if constexpr (sizeof(K) == 8) {
+        if (pl.buckets == SortShape<K, true>::buckets) {
+            TraceScope trace("csr_sort", s);
+            constexpr size_t smem = sort_smem_bytes<K, true>();
+            void* args[] = {&job};
+            const cudaError_t e = cudaLaunchCooperativeKernel(
+                (const void*)radix_sort_kernel<K, P, Id>, dim3(grid), dim3(kSortThreads), args, smem, s);
+            note_launch();
+            return e;
         }
     }
-    *sorted = cur;
-    return cudaSuccess;
+    {
+        TraceScope trace("csr_radix_hist", s);
+        const size_t smem = (size_t)pl.n * pl.buckets * 4 * kHistCopies;
+        if (job.plain)
+            { radix_hist_kernel<K, const K*, P, Id><<<sort_grid(M), 256, smem, s>>>(job.plain, job); note_launch(); }
+        else
+            { radix_hist_kernel<K, PairList<K, P>, P, Id><<<sort_grid(M), 256, smem, s>>>(first, job); note_launch(); }
+    }
+    uint64_t* dstart = (uint64_t*)(ws + L.off_dig) + (size_t)kMaxPasses * kMaxBuckets;
+    {
+        TraceScope trace("csr_scan", s);
+        { radix_dstart_kernel<<<pl.n, pl.buckets, 0, s>>>(job.tot, pl, dstart, sort_needed); note_launch(); }
+    }
+    constexpr size_t smem = sort_smem_bytes<K, false>();
+    for (uint32_t k = 0; k < pl.n; ++k) {
+        TraceScope trace("csr_radix_scatter", s);
+        auto launch = [&](auto in) {
+            { radix_scatter_kernel<K, decltype(in), Id><<<grid, kSortThreads, smem, s>>>(
+                in, job.buf[k & 1], k + 1 == pl.n ? col_final : nullptr, row_ptr, M, N, pl.digit(k), k,
+                dstart + (size_t)k * pl.buckets, job.status, job.words, sort_needed,
+                job.hook.spin_limit, job.hook.withhold); note_launch(); }
+        };
+        if (k > 0 || job.plain) launch((const K*)(k ? job.buf[(k - 1) & 1] : job.plain));
+        else launch(first);
+    }
+    return cudaGetLastError();
 }
 
 // In-place prefix maximum over the n row pointers, whose values are at most M:
@@ -1271,7 +1351,8 @@ cudaError_t csr_impl(const void* d_edges, uint64_t M, uint64_t N, uint64_t N_dst
     unsigned char* ws = (unsigned char*)d_ws;
     uint32_t* sort_needed = (uint32_t*)(ws + L.off_flag);
     const int grid = sort_grid(M + 1);
-    if (cudaMemsetAsync(sort_needed, 0, 4, s) != cudaSuccess) return cudaErrorUnknown;
+    const PassList pl = make_passes(N, N_dst, M);
+    if ((err = clear_sort_words(ws, L, pl, M, s)) != cudaSuccess) return err;
     if (cudaMemsetAsync(d_row_ptr, 0, (N + 1) * 8, s) != cudaSuccess) return cudaErrorUnknown;
     {
         TraceScope trace("csr_grouped", s);
@@ -1284,16 +1365,15 @@ cudaError_t csr_impl(const void* d_edges, uint64_t M, uint64_t N, uint64_t N_dst
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     // with at least one digit to sort, the last pass writes col and the row
     // ends itself; a key without digits (one vertex) leaves the list as it is
-    const PassList pl = make_passes(N, N_dst, M);
     const bool in_sort = M > 0 && pl.n > 0;
     Id* col = in_sort ? (Id*)d_col : nullptr;
     if (ids_narrow(N, N_dst)) {
         const uint2* sorted;
-        err = radix_passes<uint2, P, Id>({(const P*)d_edges, 0}, M, N, pl, L, ws, sort_needed, s,
+        err = radix_sort<uint2, P, Id>({(const P*)d_edges, 0}, M, N, pl, L, ws, sort_needed, s,
                                          &sorted, col, d_row_ptr);
     } else if constexpr (sizeof(Id) == 8) {   // 32-bit ids are always narrow
         const P* sorted;
-        err = radix_passes<P, P, Id>({(const P*)d_edges, 0}, M, N, pl, L, ws, sort_needed, s, &sorted,
+        err = radix_sort<P, P, Id>({(const P*)d_edges, 0}, M, N, pl, L, ws, sort_needed, s, &sorted,
                                      col, d_row_ptr);
     }
     if (err != cudaSuccess) return err;
@@ -1331,8 +1411,7 @@ OptsLayout opts_layout(uint64_t M, uint64_t N, uint32_t flags, size_t pair_bytes
 // The wanted positions of the sorted list into col, and the row pointers.
 template <typename Id, typename List>
 cudaError_t csr_compact(const List& list, uint64_t M2, uint64_t N, uint32_t flags,
-                        const OptsLayout& O, unsigned char* ws, const uint32_t* sort_needed,
-                        uint64_t* d_row_ptr, Id* d_col, cudaStream_t s)
+                        const OptsLayout& O, unsigned char* ws, uint64_t* d_row_ptr, Id* d_col, cudaStream_t s)
 {
     cudaError_t err;
     TraceScope trace("csr_compact", s);
@@ -1340,7 +1419,7 @@ cudaError_t csr_compact(const List& list, uint64_t M2, uint64_t N, uint32_t flag
         uint64_t* cpart = (uint64_t*)(ws + O.off_cpart);
         uint32_t* keep = (uint32_t*)(ws + O.off_keep);
         { csr_keep_mask_kernel<List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, flags, keep, cpart); note_launch(); }
-        { scan_parts_kernel<<<1, 1024, 0, s>>>(cpart, O.n_cparts, sort_needed); note_launch(); }
+        { scan_parts_kernel<<<1, 1024, 0, s>>>(cpart, O.n_cparts); note_launch(); }
         { csr_keep_apply_kernel<Id, List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, N, keep, cpart,
                                                                               d_col, d_row_ptr); note_launch(); }
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
@@ -1357,35 +1436,29 @@ cudaError_t csr_opts_impl(const void* d_edges, uint64_t M, uint64_t N, uint32_t 
     cudaError_t err;
     if ((err = set_csr_attributes<Id>()) != cudaSuccess) return err;
     unsigned char* ws = (unsigned char*)d_ws;
-    uint32_t* sort_needed = (uint32_t*)(ws + O.L.off_flag);
     const uint64_t M2 = O.M2;
-    // every option needs the sorted list: the sort kernels run unconditionally
-    if (cudaMemsetAsync(sort_needed, 1, 4, s) != cudaSuccess) return cudaErrorUnknown;
     if (cudaMemsetAsync(d_row_ptr, 0, (N + 1) * 8, s) != cudaSuccess) return cudaErrorUnknown;
     const P* in = (const P*)d_edges;
     const uint32_t sym = (flags & kOptSym) ? 1 : 0;
     const PassList pl = make_passes(N, N, M2);
-    if (pl.n == 0) {
-        // one vertex: the list is sorted as it is (its reverse is the same
-        // again), and there is no sort to clear the wait word
-        if (M2 > 0 && cudaMemsetAsync(ws + O.L.off_flag + 64, 0, 128, s) != cudaSuccess)
-            return cudaErrorUnknown;
-        return csr_compact<Id>(PairList<P, P>{in, sym}, M2, N, flags, O, ws, sort_needed, d_row_ptr,
-                               (Id*)d_col, s);
-    }
+    if ((err = clear_sort_words(ws, O.L, pl, M2, s)) != cudaSuccess) return err;
+    // one vertex: the list is sorted as it is (its reverse is the same again)
+    if (pl.n == 0)
+        return csr_compact<Id>(PairList<P, P>{in, sym}, M2, N, flags, O, ws, d_row_ptr, (Id*)d_col, s);
+    // every option needs the sorted list: the sort runs unconditionally
     if (ids_narrow(N, N)) {
         const uint2* sorted;
-        if ((err = radix_passes<uint2, P, Id>({in, sym}, M2, N, pl, O.L, ws, sort_needed, s, &sorted,
+        if ((err = radix_sort<uint2, P, Id>({in, sym}, M2, N, pl, O.L, ws, nullptr, s, &sorted,
                                               nullptr, nullptr)) != cudaSuccess)
             return err;
-        return csr_compact<Id>(sorted, M2, N, flags, O, ws, sort_needed, d_row_ptr, (Id*)d_col, s);
+        return csr_compact<Id>(sorted, M2, N, flags, O, ws, d_row_ptr, (Id*)d_col, s);
     }
     if constexpr (sizeof(Id) == 8) {
         const P* sorted;
-        if ((err = radix_passes<P, P, Id>({in, sym}, M2, N, pl, O.L, ws, sort_needed, s, &sorted,
+        if ((err = radix_sort<P, P, Id>({in, sym}, M2, N, pl, O.L, ws, nullptr, s, &sorted,
                                           nullptr, nullptr)) != cudaSuccess)
             return err;
-        return csr_compact<Id>(sorted, M2, N, flags, O, ws, sort_needed, d_row_ptr, (Id*)d_col, s);
+        return csr_compact<Id>(sorted, M2, N, flags, O, ws, d_row_ptr, (Id*)d_col, s);
     }
     return cudaErrorInvalidValue;   // 32-bit ids are always narrow
 }

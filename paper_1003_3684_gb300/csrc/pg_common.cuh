@@ -199,4 +199,34 @@ __device__ __forceinline__ uint32_t seed_endpoint(uint64_t e, uint32_t side, uin
     return side ? a + 1 + (uint32_t)e : a;
 }
 
+// Barrier over a cooperative grid; both words start at zero. Each wait is
+// bounded; one that gives up sets the error word and its CTA leaves the
+// kernel, so the others give up too.
+constexpr uint32_t kBarrierPolls = 1u << 24;   // some ten seconds
+__device__ __forceinline__ bool grid_barrier(uint32_t* arrived, uint32_t* error, uint32_t& epoch)
+{
+    __shared__ uint32_t s_ok;
+    __syncthreads();
+    ++epoch;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(arrived, 1u);
+        const uint32_t want = epoch * gridDim.x;
+        uint32_t polls = 0, ok = 1;
+        // (the count may wrap; it is never far from what is waited for)
+        while ((int32_t)(*(volatile uint32_t*)arrived - want) < 0) {
+            if (++polls > kBarrierPolls || *(volatile uint32_t*)error) {
+                atomicOr(error, 1u);
+                ok = 0;
+                break;
+            }
+            __nanosleep(32);
+        }
+        __threadfence();
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
 }  // namespace pgen

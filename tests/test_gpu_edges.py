@@ -300,3 +300,22 @@ def test_csr_sort_of_long_lists(M, N, spread, id64):
     ref_rp, ref_col = o.csr(e.astype(np.uint64), N)
     np.testing.assert_array_equal(host(rp), ref_rp)
     np.testing.assert_array_equal(host(col), ref_col)
+
+
+@pytest.mark.parametrize("M", [2, 4095, 4096, 4097, 9 * 4096 + 1, 786_431, 786_432])
+@pytest.mark.parametrize("N", [2, 2**9, 2**13 + 1, 2**20])
+@pytest.mark.parametrize("flags,id64", [(0, False), (0, True), (pg.CSR_SYMMETRIZE, False),
+                                        (pg.CSR_ODD, True)])
+def test_csr_sort_of_short_lists(M, N, flags, id64):
+    """Digits of up to 9 bits, full and ragged tiles, both sides of the longest
+    short list (a symmetrised list has twice the pairs); few pairs take most
+    of the edges, so that every option has something to drop."""
+    rng = np.random.default_rng(M * 7 + flags)
+    e = rng.integers(0, N, (M, 2), dtype=np.int64)
+    e[::3] = e[0]
+    t = torch.from_numpy(e if id64 else e.astype(np.uint32).view(np.int32)).cuda()
+    rp, col = pg.edges_to_csr_opts(t, N, flags) if flags else pg.edges_to_csr(t, N, check=True)
+    ref_rp, ref_col = (o.csr_opts(e.astype(np.uint64), N, flags) if flags else
+                       o.csr(e.astype(np.uint64), N))
+    np.testing.assert_array_equal(host(rp), ref_rp)
+    np.testing.assert_array_equal(host(col)[:int(ref_rp[-1])], ref_col)
