@@ -759,12 +759,6 @@ __global__ void __launch_bounds__(256, kGroupPlaces<Id>)
     }
 }
 
-// In-place inclusive prefix maximum over the row pointers. A warp takes
-// kScanTile / 8 neighbouring entries, 32 at a time, so that every access is
-// coalesced (row_ptr is aligned to 8 bytes only); V is uint32_t when the
-// values, which are positions in the list, fit it. Bound by memory: an entry
-// is read twice and written once. 2^26 rows: 0.601 -> 0.259 ms with the
-// zeroing; 2^20: 0.025 -> 0.017 (a thread read 16 neighbouring entries before).
 template <typename V>
 __device__ __forceinline__ V warp_inclusive_max(V x, uint32_t lane)
 {
@@ -776,66 +770,66 @@ __device__ __forceinline__ V warp_inclusive_max(V x, uint32_t lane)
     return x;
 }
 
+// In-place inclusive prefix maximum over the n row pointers, in one cooperative
+// launch: a CTA takes neighbouring tiles of kScanTile entries, publishes their
+// maximum in part[], and after a grid barrier applies what came before to each.
+// A CTA with one tile (up to 2.4 million rows) keeps it in registers, one with
+// more reads them again. A warp takes kScanTile / 8 neighbouring entries, 32 at
+// a time, so that every access is coalesced (row_ptr is aligned to 8 bytes
+// only); V is uint32_t when the values, which are positions in the list, fit
+// it. Bound by its launch and barrier, then by memory: 160,000 rows 14 -> 8 us,
+// 2^20 16.7 -> 10.2, 2^24 75 -> 67, 2^26 259 -> 258 (three launches before).
+constexpr int kRowPlaces = 4;   // CTAs per SM
 template <typename V>
-__global__ void __launch_bounds__(256) max_reduce_kernel(const uint64_t* __restrict__ in, uint64_t n,
-                                                         uint64_t* __restrict__ part)
-{
-    __shared__ V s_warp[8];
-    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint64_t base = (uint64_t)blockIdx.x * kScanTile + threadIdx.x;
-    V m = 0;
-#pragma unroll
-    for (uint32_t t = 0; t < kScanTile; t += 256) {
-        const V a = base + t < n ? (V)in[base + t] : 0;
-        if (a > m) m = a;
-    }
-    m = warp_inclusive_max(m, lane);
-    if (lane == 31) s_warp[wid] = m;
-    __syncthreads();
-    if (wid == 0) {
-        m = warp_inclusive_max<V>(lane < 8 ? s_warp[lane] : 0, lane);
-        if (lane == 31) part[blockIdx.x] = m;
-    }
-}
-
-// exclusive prefix maximum of the tile maxima, one CTA looping over chunks
-__global__ void __launch_bounds__(1024) max_parts_kernel(uint64_t* __restrict__ part, uint64_t n_parts)
-{
-    __shared__ uint64_t s_warp[32];
-    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint64_t carry = 0;
-    for (uint64_t base = 0; base < n_parts; base += blockDim.x) {
-        const uint64_t i = base + threadIdx.x;
-        const uint64_t x = warp_inclusive_max<uint64_t>(i < n_parts ? part[i] : 0, lane);
-        uint64_t ex = __shfl_up_sync(0xFFFFFFFFu, x, 1);
-        if (lane == 0) ex = 0;
-        if (lane == 31) s_warp[wid] = x;
-        __syncthreads();
-        const uint64_t w = warp_inclusive_max<uint64_t>(s_warp[lane], lane);
-        const uint64_t before = wid ? __shfl_sync(0xFFFFFFFFu, w, (wid - 1) & 31) : 0;
-        if (before > ex) ex = before;
-        if (carry > ex) ex = carry;
-        if (i < n_parts) part[i] = ex;
-        const uint64_t total = __shfl_sync(0xFFFFFFFFu, w, 31);
-        if (total > carry) carry = total;
-        __syncthreads();
-    }
-}
-
-// part == null: one CTA scans all n entries, a tile after another.
-template <typename V>
-__global__ void __launch_bounds__(256) max_apply_kernel(uint64_t* __restrict__ data, uint64_t n,
-                                                        const uint64_t* __restrict__ part)
+__global__ void __launch_bounds__(256, kRowPlaces)
+    row_max_kernel(uint64_t* data, uint64_t n, uint64_t* part, uint32_t per, uint32_t* words,
+                   uint32_t* err)
 {
     __shared__ V s_warp[8];
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     constexpr int kRounds = kScanTile / 256;
-    V carry = part ? (V)part[blockIdx.x] : 0;
-    for (uint64_t tile = blockIdx.x; tile * kScanTile < n; tile += gridDim.x) {
+    const uint64_t first = (uint64_t)blockIdx.x * per;
+    V a[kRounds];
+    auto load = [&](uint64_t tile) {
         const uint64_t base = tile * kScanTile + wid * (32 * kRounds) + lane;
-        V a[kRounds];
 #pragma unroll
         for (int r = 0; r < kRounds; ++r) a[r] = base + 32 * r < n ? (V)data[base + 32 * r] : 0;
+    };
+    // the CTA's maximum of x, in every thread
+    auto reduce = [&](V x) {
+        x = warp_inclusive_max(x, lane);
+        if (lane == 31) s_warp[wid] = x;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < 8; ++w)
+            if (s_warp[w] > x) x = s_warp[w];
+        __syncthreads();
+        return x;
+    };
+    V carry = 0;
+    if (gridDim.x > 1) {
+        V m = 0;
+        for (uint32_t t = 0; t < per; ++t) {
+            load(first + t);
+#pragma unroll
+            for (int r = 0; r < kRounds; ++r)
+                if (a[r] > m) m = a[r];
+        }
+        m = reduce(m);
+        if (threadIdx.x == 0) part[blockIdx.x] = m;
+        uint32_t epoch = 0;
+        if (!grid_barrier(words, words + 1, epoch)) {
+            if (threadIdx.x == 0) atomicOr(err, 1u);
+            return;
+        }
+        for (uint32_t c = threadIdx.x; c < blockIdx.x; c += blockDim.x) {
+            const V x = (V)__ldcg(part + c);
+            if (x > carry) carry = x;
+        }
+        carry = reduce(carry);
+    }
+    for (uint32_t t = 0; t < per; ++t) {
+        if (per > 1 || gridDim.x == 1) load(first + t);
         V run = 0;   // the warp's maximum up to and including round r
 #pragma unroll
         for (int r = 0; r < kRounds; ++r) {
@@ -845,18 +839,17 @@ __global__ void __launch_bounds__(256) max_apply_kernel(uint64_t* __restrict__ d
         }
         if (lane == 0) s_warp[wid] = run;
         __syncthreads();
-        V before = carry, all = carry;
+        V before = carry;
 #pragma unroll
         for (uint32_t w = 0; w < 8; ++w) {
             const V x = s_warp[w];
             if (w < wid && x > before) before = x;
-            if (x > all) all = x;
+            if (x > carry) carry = x;
         }
+        const uint64_t base = (first + t) * kScanTile + wid * (32 * kRounds) + lane;
 #pragma unroll
         for (int r = 0; r < kRounds; ++r)
             if (base + 32 * r < n) data[base + 32 * r] = before > a[r] ? before : a[r];
-        if (part) return;
-        carry = all;
         __syncthreads();
     }
 }
@@ -1176,7 +1169,8 @@ CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst =
     o += a256(M * pair_bytes);
     L.off_status = o;   // tile status words of the pass being sorted
     o += a256(L.n_status * 8);
-    L.off_flag = o;     // +0: sort-needed flag, +64: SortJob's words (+128: wait error)
+    L.off_flag = o;     // +0: sort-needed flag, +64: SortJob's words (+128: wait error),
+                        // +192: the row kernel's barrier
     o += 256;
     L.off_dig = o;      // digit totals, then digit starts, of every pass
     o += a256(2 * (size_t)kMaxPasses * kMaxBuckets * 8);
@@ -1308,28 +1302,32 @@ cudaError_t radix_sort(const PairList<K, P> first, uint64_t M, uint64_t N, const
     return cudaGetLastError();
 }
 
-// In-place prefix maximum over the n row pointers, whose values are at most M:
-// three kernels, or one CTA alone where the launches would cost more than its
-// pass over a few tiles.
-constexpr uint64_t kMaxAlone = 8;
+// In-place prefix maximum over the N + 1 row pointers of a list of M > 0 pairs.
 template <typename V>
-cudaError_t prefix_max_as(uint64_t* data, uint64_t n, uint64_t* parts, cudaStream_t s)
+cudaError_t row_max_as(uint64_t* d_row_ptr, uint64_t N, const CsrLayout& L, unsigned char* ws,
+                       cudaStream_t s)
 {
-    const uint64_t n_parts = (n + kScanTile - 1) / kScanTile;
-    if (n_parts == 0) return cudaSuccess;
-    if (n_parts <= kMaxAlone) {
-        { max_apply_kernel<V><<<1, 256, 0, s>>>(data, n, nullptr); note_launch(); }
+    const uint64_t places = (uint64_t)kRowPlaces * device_sm_count();
+    uint32_t per = (uint32_t)((L.n_rparts + places - 1) / places);
+    const unsigned grid = (unsigned)((L.n_rparts + per - 1) / per);
+    uint64_t n = N + 1, *part = (uint64_t*)(ws + L.off_rpart);
+    uint32_t* words = (uint32_t*)(ws + L.off_flag + 192);
+    uint32_t* err = (uint32_t*)(ws + L.off_flag + 64) + kWordErr;
+    if (grid == 1) {   // nothing to wait for
+        { row_max_kernel<V><<<1, 256, 0, s>>>(d_row_ptr, n, part, per, words, err); note_launch(); }
         return cudaGetLastError();
     }
-    { max_reduce_kernel<V><<<(unsigned)n_parts, 256, 0, s>>>(data, n, parts); note_launch(); }
-    { max_parts_kernel<<<1, 1024, 0, s>>>(parts, n_parts); note_launch(); }
-    { max_apply_kernel<V><<<(unsigned)n_parts, 256, 0, s>>>(data, n, parts); note_launch(); }
-    return cudaGetLastError();
+    void* args[] = {&d_row_ptr, &n, &part, &per, &words, &err};
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)row_max_kernel<V>, dim3(grid),
+                                                      dim3(256), args, 0, s);
+    note_launch();
+    return e;
 }
-cudaError_t prefix_max(uint64_t* data, uint64_t n, uint64_t M, uint64_t* parts, cudaStream_t s)
+cudaError_t row_max(uint64_t* d_row_ptr, uint64_t N, uint64_t M, const CsrLayout& L,
+                    unsigned char* ws, cudaStream_t s)
 {
-    return M < ((uint64_t)1 << 32) ? prefix_max_as<uint32_t>(data, n, parts, s)
-                                   : prefix_max_as<uint64_t>(data, n, parts, s);
+    return M < ((uint64_t)1 << 32) ? row_max_as<uint32_t>(d_row_ptr, N, L, ws, s)
+                                   : row_max_as<uint64_t>(d_row_ptr, N, L, ws, s);
 }
 
 int sort_grid(uint64_t work)
@@ -1381,8 +1379,9 @@ cudaError_t csr_impl(const void* d_edges, uint64_t M, uint64_t N, uint64_t N_dst
         TraceScope trace("csr_finish", s);
         { csr_finish_kernel<Id><<<grid, 256, 0, s>>>((const P*)d_edges, M, N, d_row_ptr, (Id*)d_col, sort_needed); note_launch(); }
     }
+    if (M == 0) return cudaSuccess;    // every row is empty, row_ptr all zero
     TraceScope trace("csr_rows", s);   // rows without edges take the previous row's end
-    return prefix_max(d_row_ptr, N + 1, M, (uint64_t*)(ws + L.off_rpart), s);
+    return row_max(d_row_ptr, N, M, L, ws, s);
 }
 
 // Workspace of the options path: the sort's layout for the (possibly
@@ -1413,18 +1412,17 @@ template <typename Id, typename List>
 cudaError_t csr_compact(const List& list, uint64_t M2, uint64_t N, uint32_t flags,
                         const OptsLayout& O, unsigned char* ws, uint64_t* d_row_ptr, Id* d_col, cudaStream_t s)
 {
+    if (M2 == 0) return cudaSuccess;   // every row is empty, row_ptr all zero
     cudaError_t err;
     TraceScope trace("csr_compact", s);
-    if (M2 > 0) {
-        uint64_t* cpart = (uint64_t*)(ws + O.off_cpart);
-        uint32_t* keep = (uint32_t*)(ws + O.off_keep);
-        { csr_keep_mask_kernel<List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, flags, keep, cpart); note_launch(); }
-        { scan_parts_kernel<<<1, 1024, 0, s>>>(cpart, O.n_cparts); note_launch(); }
-        { csr_keep_apply_kernel<Id, List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, N, keep, cpart,
-                                                                              d_col, d_row_ptr); note_launch(); }
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    }
-    return prefix_max(d_row_ptr, N + 1, M2, (uint64_t*)(ws + O.L.off_rpart), s);
+    uint64_t* cpart = (uint64_t*)(ws + O.off_cpart);
+    uint32_t* keep = (uint32_t*)(ws + O.off_keep);
+    { csr_keep_mask_kernel<List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, flags, keep, cpart); note_launch(); }
+    { scan_parts_kernel<<<1, 1024, 0, s>>>(cpart, O.n_cparts); note_launch(); }
+    { csr_keep_apply_kernel<Id, List><<<(unsigned)O.n_cparts, 256, 0, s>>>(list, M2, N, keep, cpart,
+                                                                          d_col, d_row_ptr); note_launch(); }
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    return row_max(d_row_ptr, N, M2, O.L, ws, s);
 }
 
 template <typename Id>

@@ -319,3 +319,17 @@ def test_csr_sort_of_short_lists(M, N, flags, id64):
                        o.csr(e.astype(np.uint64), N))
     np.testing.assert_array_equal(host(rp), ref_rp)
     np.testing.assert_array_equal(host(col)[:int(ref_rp[-1])], ref_col)
+
+
+@pytest.mark.parametrize("N", [608 * 4096 - 2, 608 * 4096 - 1, 608 * 4096, 2 * 608 * 4096 + 5])
+@pytest.mark.parametrize("flags", [0, pg.CSR_DEDUP])
+def test_csr_rows_of_more_tiles_than_ctas(N, flags):
+    """Where a CTA of the row kernel goes from one tile to several."""
+    rng = np.random.default_rng(N)
+    e = rng.integers(0, N, size=(999, 2), dtype=np.uint32)
+    t = torch.from_numpy(e.view(np.int32)).cuda()
+    rp, col = pg.edges_to_csr_opts(t, N, flags) if flags else pg.edges_to_csr(t, N, check=True)
+    ref_rp, ref_col = (o.csr_opts(e.astype(np.uint64), N, flags) if flags else
+                       o.csr(e.astype(np.uint64), N))
+    np.testing.assert_array_equal(host(rp), ref_rp)
+    np.testing.assert_array_equal(host(col)[:int(ref_rp[-1])], ref_col)
