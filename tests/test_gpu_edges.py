@@ -333,3 +333,19 @@ def test_csr_rows_of_more_tiles_than_ctas(N, flags):
                        o.csr(e.astype(np.uint64), N))
     np.testing.assert_array_equal(host(rp), ref_rp)
     np.testing.assert_array_equal(host(col)[:int(ref_rp[-1])], ref_col)
+
+
+@pytest.mark.parametrize("N", [13 * 2**20 - 1, 13 * 2**20, 13 * 2**20 + 1, 2**24 + 384])
+@pytest.mark.parametrize("id64", [False, True])
+def test_degrees_counted_in_32_bits_and_widened(N, id64):
+    """Both sides of the size where counts move to 32 bits in the result's own
+    memory: every vertex's count, the first and last ones with long runs."""
+    rng = np.random.default_rng(N)
+    e = rng.integers(0, N, size=(2_000_003, 2), dtype=np.int64)
+    e[::5] = (N - 1, 0)
+    e[1::5, 1] = rng.integers(0, 64, e[1::5].shape[0])
+    t = torch.from_numpy(e if id64 else e.astype(np.uint32).view(np.int32)).cuda()
+    deg = torch.full((N + 2,), -7, dtype=torch.int64, device="cuda")
+    pg.degrees(t, N, pg.DEG_TOTAL, out=deg[1:N + 1])
+    np.testing.assert_array_equal(host(deg[1:N + 1]), o.degrees(e.astype(np.uint64), N, o.DEG_TOTAL))
+    assert int(deg[0]) == -7 and int(deg[N + 1]) == -7
