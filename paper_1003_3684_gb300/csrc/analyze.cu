@@ -7,7 +7,6 @@
 // the order in which a level's vertices are found depends on the schedule.
 #include <cstddef>
 #include <cstring>
-#include <utility>
 
 #include "../../include/pgen.h"
 #include "pg_internal.h"
@@ -345,7 +344,7 @@ __device__ __forceinline__ void bfs_long_rows(const uint64_t* __restrict__ row_p
     }
 }
 
-// Top-down levels from (level, fsize) on, in one cooperative launch with a
+// Top-down levels from the state's on, in one cooperative launch with a
 // grid barrier between levels instead of a launch and a host round trip (a
 // level of a small frontier is a few microseconds of latency): until the
 // frontier is empty, or until bottom-up would be chosen on an undirected
@@ -353,15 +352,15 @@ __device__ __forceinline__ void bfs_long_rows(const uint64_t* __restrict__ row_p
 template <typename Id>
 __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_top_down_kernel(
     const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, uint32_t* f0, uint32_t* f1,
-    uint32_t cur, uint32_t fsize, uint64_t visited, uint32_t level, uint32_t undirected,
-    uint32_t* dist, uint32_t* vis, uint64_t N, uint32_t* long_v, uint32_t* long_base,
-    BfsState* state)
+    uint32_t undirected, uint32_t* dist, uint32_t* vis, uint64_t N, uint32_t* long_v,
+    uint32_t* long_base, BfsState* state)
 {
     __shared__ uint32_t wbuf[kBfsWarps][64];
     __shared__ uint64_t wstart[kBfsWarps][32];   // the rows' starts in the concatenation
     __shared__ uint64_t wrow[kBfsWarps][32];     // and in col
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t epoch = 0;
+    uint32_t epoch = 0, cur = state->cur, fsize = state->fsize, level = state->level;
+    uint64_t visited = state->visited;
     for (bool first = true; fsize > 0; first = false) {
         if (visited >= N) {   // nothing left to find: the last level is empty
             fsize = 0;
@@ -402,9 +401,8 @@ __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_top_down_kernel(
 }
 
 // The frontier of `level` as a bitmap, from the distances.
-__global__ void __launch_bounds__(256) bfs_bitmap_kernel(const uint32_t* __restrict__ dist,
-                                                         uint32_t level, uint64_t N,
-                                                         uint32_t* __restrict__ bits)
+__device__ __forceinline__ void bfs_bitmap(const uint32_t* dist, uint32_t level, uint64_t N,
+                                           uint32_t* bits)
 {
     constexpr int kU = 8;   // words in flight per warp
     const uint32_t lane = threadIdx.x & 31;
@@ -427,9 +425,8 @@ __global__ void __launch_bounds__(256) bfs_bitmap_kernel(const uint32_t* __restr
 }
 
 // The vertices of a bitmap as a list (in any order), *count of them.
-__global__ void __launch_bounds__(256) bfs_list_kernel(const uint32_t* __restrict__ bits, uint64_t N,
-                                                       uint32_t* __restrict__ list,
-                                                       uint32_t* __restrict__ count)
+__device__ __forceinline__ void bfs_list(const uint32_t* bits, uint64_t N, uint32_t* list,
+                                         uint32_t* count)
 {
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t words = (N + 31) / 32, stride = (uint64_t)gridDim.x * blockDim.x;
@@ -451,7 +448,7 @@ __global__ void __launch_bounds__(256) bfs_list_kernel(const uint32_t* __restric
     }
 }
 
-// One BFS level bottom-up (Beamer, Asanovic and Patterson, "Direction-
+// One level bottom-up (Beamer, Asanovic and Patterson, "Direction-
 // Optimizing Breadth-First Search", SC'12), for a symmetric CSR: every vertex
 // not yet visited looks through its row for a neighbour in the frontier and,
 // at the first one, takes distance level + 1. The frontier is a bitmap (2 MB
@@ -464,10 +461,9 @@ __global__ void __launch_bounds__(256) bfs_list_kernel(const uint32_t* __restric
 // a grid stride apart, since neighbouring ids share hubs (eight neighbouring
 // words: 0.95 ms).
 template <typename Id>
-__global__ void __launch_bounds__(kBfsWarps * 32) bfs_bottom_up_kernel(
-    const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col,
-    const uint32_t* __restrict__ front, uint32_t* __restrict__ next, uint32_t* __restrict__ nsize,
-    uint32_t* __restrict__ dist, uint32_t* __restrict__ vis, uint32_t level, uint64_t N)
+__device__ __forceinline__ void bfs_bottom_up_level(
+    const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, const uint32_t* front,
+    uint32_t* next, uint32_t* nsize, uint32_t* dist, uint32_t* vis, uint32_t level, uint64_t N)
 {
     constexpr uint32_t kWords = 8;
     const uint32_t lane = threadIdx.x & 31;
@@ -516,13 +512,52 @@ __global__ void __launch_bounds__(kBfsWarps * 32) bfs_bottom_up_kernel(
     if (lane == 0 && found_all) atomicAdd(nsize, found_all);
 }
 
+// Bottom-up levels from the state's on, as the top-down kernel runs its: from
+// the frontier's bitmap until the frontier is empty, or until it is under 1/24
+// of all vertices; then its vertices go back to a list.
+template <typename Id>
+__global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_bottom_up_kernel(
+    const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, uint32_t* front, uint32_t* next,
+    uint32_t* list, uint32_t* dist, uint32_t* vis, uint64_t N, BfsState* state)
+{
+    uint32_t epoch = 0, fsize = state->fsize, level = state->level;
+    uint64_t visited = state->visited;
+    if (fsize == 0) return;   // the search is over
+    bfs_bitmap(dist, level, N, front);
+    if (!grid_barrier(&state->arrived, &state->error, epoch)) return;
+    do {
+        uint32_t* nsize = &state->size[level & 3];
+        if (blockIdx.x == 0 && threadIdx.x == 0) state->size[(level + 1) & 3] = 0;
+        bfs_bottom_up_level(row_ptr, col, front, next, nsize, dist, vis, level, N);
+        if (!grid_barrier(&state->arrived, &state->error, epoch)) return;
+        fsize = __ldcg(nsize);
+        visited += fsize;
+        ++level;
+        uint32_t* f = front;
+        front = next;
+        next = f;
+        if (fsize > 0 && visited >= N) {   // the last level finds nothing
+            fsize = 0;
+            ++level;
+        }
+    } while (fsize > 0 && (uint64_t)fsize * 24 >= N);
+    if (fsize > 0) bfs_list(front, N, list, &state->size[level & 3]);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        state->level = level;
+        state->fsize = fsize;
+        state->cur = 0;
+        state->visited = visited;
+    }
+}
+
 // scanned = the sum of the reached vertices' row lengths (what a top-down
-// search reads, whichever direction each level ran).
+// search reads, whichever direction each level ran), once the search is over.
 __global__ void __launch_bounds__(256) bfs_reach_kernel(const uint64_t* __restrict__ row_ptr,
                                                         const uint32_t* __restrict__ dist,
-                                                        uint64_t N,
-                                                        unsigned long long* __restrict__ scanned)
+                                                        uint64_t N, BfsState* __restrict__ state)
 {
+    if (state->fsize > 0) return;
+    unsigned long long* scanned = &state->scanned;
     constexpr int kU = 4;   // vertices in flight per thread
     unsigned long long sum = 0;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -545,11 +580,14 @@ __global__ void __launch_bounds__(256) bfs_reach_kernel(const uint64_t* __restri
     if ((threadIdx.x & 31) == 0 && sum) atomicAdd(scanned, sum);
 }
 
-__global__ void bfs_seed_kernel(uint32_t* dist, uint32_t* vis, uint32_t* frontier, uint32_t source)
+__global__ void bfs_seed_kernel(uint32_t* dist, uint32_t* vis, uint32_t* frontier, BfsState* state,
+                                uint32_t source)
 {
     dist[source] = 0;
     vis[source >> 5] = 1u << (source & 31);
     frontier[0] = source;
+    state->fsize = 1;   // of zeroed counters
+    state->visited = 1;
 }
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p & (a - 1)) == 0; }
@@ -561,37 +599,84 @@ int grid_cap(uint64_t items)
     return (int)(need < 1 ? 1 : (need < full ? need : full));
 }
 
-// Top-down levels from the host's state h on, in one cooperative launch: every
-// CTA resident, and no more of them than the graph can use.
-template <typename Id>
-cudaError_t launch_top_down(const uint64_t* row_ptr, const Id* col, uint32_t* const* fr,
-                            const BfsState& h, uint32_t undirected, uint32_t* dist, uint32_t* vis,
-                            uint64_t N, uint32_t* long_v, uint32_t* long_base, BfsState* state,
-                            cudaStream_t s)
+// Every CTA of a cooperative launch resident, and no more of them than the
+// graph can use. The counters and the barrier start at zero.
+template <typename F>
+cudaError_t launch_levels(F* kernel, uint64_t N, uint32_t per_cta, int most, void** args,
+                          BfsState* state, cudaStream_t s)
 {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bfs_top_down_kernel<Id>,
-                                                                  kBfsWarps * 32, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBfsWarps * 32, 0);
     if (e != cudaSuccess) return e;
-    // four CTAs per SM where levels are short (a barrier of 608 CTAs instead of
-    // 1216: 2^20 vertices 0.350 -> 0.237 ms per search); all that fit where wide
-    // levels run top-down (2^24 vertices, directed: 3.26 -> 3.08 ms)
-    if (per_sm > 4 && (undirected || N <= (1u << 22))) per_sm = 4;
+    if (per_sm > most) per_sm = most;
     const uint64_t full = (uint64_t)device_sm_count() * (per_sm > 0 ? per_sm : 1);
-    const uint64_t want = (N + 63) / 64;
+    const uint64_t want = (N + per_cta - 1) / per_cta;
     const unsigned grid = (unsigned)(want < full ? want : full);
-    // the counters and the barrier start at zero; scanned and error are kept
+    // scanned, error and where the search stands are kept
     e = cudaMemsetAsync(state, 0, offsetof(BfsState, scanned), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(&state->arrived, 0, 4, s);
     if (e != cudaSuccess) return e;
-    uint32_t *f0 = fr[0], *f1 = fr[1], cur = h.cur, fsize = h.fsize, level = h.level;
-    unsigned long long visited = h.visited;
-    void* args[] = {&row_ptr, &col,  &f0,  &f1, &cur,    &fsize,     &visited, &level,
-                    &undirected, &dist, &vis, &N,  &long_v, &long_base, &state};
-    e = cudaLaunchCooperativeKernel((const void*)bfs_top_down_kernel<Id>, dim3(grid),
-                                    dim3(kBfsWarps * 32), args, 0, s);
+    e = cudaLaunchCooperativeKernel((const void*)kernel, dim3(grid), dim3(kBfsWarps * 32), args, 0, s);
     note_launch();
     return e;
+}
+
+// The buffers of a search; bottom-up levels keep their bitmaps in the place of
+// the long-row list of top-down ones.
+struct BfsBuffers {
+    uint32_t *fr[2], *dist, *vis, *long_v, *long_base;
+    BfsState* state;
+};
+
+template <typename Id>
+cudaError_t launch_top_down(const uint64_t* row_ptr, const Id* col, BfsBuffers W, uint32_t undirected,
+                            uint64_t N, cudaStream_t s)
+{
+    void* args[] = {&row_ptr, &col, &W.fr[0], &W.fr[1], &undirected, &W.dist,
+                    &W.vis,   &N,   &W.long_v, &W.long_base, &W.state};
+    // four CTAs per SM where levels are short (a barrier of 608 CTAs instead of
+    // 1216: 2^20 vertices 0.350 -> 0.237 ms per search); all that fit where wide
+    // levels run top-down (2^24 vertices, directed: 3.26 -> 3.08 ms)
+    return launch_levels(bfs_top_down_kernel<Id>, N, 64, undirected || N <= (1u << 22) ? 4 : 8, args,
+                         W.state, s);
+}
+
+template <typename Id>
+cudaError_t launch_bottom_up(const uint64_t* row_ptr, const Id* col, BfsBuffers W, uint64_t N,
+                             cudaStream_t s)
+{
+    TraceScope trace("bfs_bottom_up", s);
+    void* args[] = {&row_ptr, &col, &W.long_v, &W.long_base, &W.fr[0], &W.dist, &W.vis, &N, &W.state};
+    return launch_levels(bfs_bottom_up_kernel<Id>, N, 256, 8, args, W.state, s);
+}
+
+// The search from the seeded state on. A round is a run of top-down levels, on
+// an undirected graph a run of bottom-up ones, and the count of what was
+// scanned, which each find from the state what is left to do, and one read of
+// the state by the host; most searches take one round (a read per run and per
+// bottom-up level before; 2^24 vertices, undirected, per search: 0.933 -> 0.900 ms,
+// 160,000: 0.195 -> 0.142, 8000: 0.161 -> 0.099).
+// Direction of a level (Beamer et al.'s rule with vertex counts standing in for
+// edge counts): bottom-up once the frontier is more than 1/30 of the vertices
+// not yet visited, top-down again once it is under 1/24 of all.
+template <typename Id>
+pg_status search(const uint64_t* row_ptr, const Id* col, const BfsBuffers& W, uint32_t undirected,
+                 uint64_t N, BfsState& h, cudaStream_t s)
+{
+    TraceScope trace("bfs", s);
+    bool bottom_up = undirected && 30 > N - 1;
+    do {
+        if (!bottom_up && launch_top_down(row_ptr, col, W, undirected, N, s) != cudaSuccess)
+            return PG_ECUDA;
+        if (undirected && launch_bottom_up(row_ptr, col, W, N, s) != cudaSuccess) return PG_ECUDA;
+        bottom_up = false;
+        { bfs_reach_kernel<<<grid_cap(N), 256, 0, s>>>(row_ptr, W.dist, N, W.state); note_launch(); }
+        if (cudaMemcpyAsync(&h, W.state, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess)
+            return PG_ECUDA;
+        if (h.error) return PG_ETIMEOUT;
+    } while (h.fsize > 0);
+    return PG_OK;
 }
 
 }  // namespace
@@ -694,78 +779,16 @@ pg_status pg_bfs(const uint64_t* d_row_ptr, const void* d_col, uint64_t n_vertic
     if (cudaMemsetAsync(d_dist, 0xFF, n_vertices * 4, s) != cudaSuccess) return PG_ECUDA;
     if (cudaMemsetAsync(ws + 2 * fbytes, 0, 256, s) != cudaSuccess) return PG_ECUDA;
     if (cudaMemsetAsync(vis, 0, vbytes, s) != cudaSuccess) return PG_ECUDA;
-    { bfs_seed_kernel<<<1, 1, 0, s>>>(d_dist, vis, fr[0], (uint32_t)source); note_launch(); }
-    TraceScope trace("bfs", s);
+    { bfs_seed_kernel<<<1, 1, 0, s>>>(d_dist, vis, fr[0], state, (uint32_t)source); note_launch(); }
     const uint32_t undirected = (flags & PG_BFS_UNDIRECTED) ? 1 : 0;
-    BfsState h;   // the search's state on the host
-    std::memset(&h, 0, sizeof(h));
-    h.fsize = 1;
-    h.visited = 1;
-    auto fetch = [&] {
-        return cudaMemcpyAsync(&h, state, sizeof(h), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-               cudaStreamSynchronize(s) == cudaSuccess;
-    };
-    // direction of a level (Beamer et al.'s rule with vertex counts standing in
-    // for edge counts): bottom-up once the frontier is more than 1/30 of the
-    // vertices not yet visited, top-down again once it is under 1/24 of all
-    bool bottom_up = undirected && (uint64_t)h.fsize * 30 > n_vertices - h.visited;
-    const uint32_t grid_all = (uint32_t)grid_cap(n_vertices);
-    while (h.fsize > 0) {
-        if (!bottom_up) {
-            const cudaError_t e =
-                w == PG_ID64
-                    ? launch_top_down(d_row_ptr, (const uint64_t*)d_col, fr, h, undirected, d_dist, vis,
-                                      n_vertices, long_v, long_base, state, s)
-                    : launch_top_down(d_row_ptr, (const uint32_t*)d_col, fr, h, undirected, d_dist, vis,
-                                      n_vertices, long_v, long_base, state, s);
-            if (e != cudaSuccess || !fetch()) return PG_ECUDA;
-            if (h.error) return PG_ETIMEOUT;
-            bottom_up = true;   // or the search is over
-            continue;
-        }
-        TraceScope bu_trace("bfs_bottom_up", s);
-        uint32_t *front = long_v, *next = long_base;
-        { bfs_bitmap_kernel<<<grid_all, 256, 0, s>>>(d_dist, h.level, n_vertices, front); note_launch(); }
-        do {
-            if (cudaMemsetAsync(&state->size[0], 0, 4, s) != cudaSuccess) return PG_ECUDA;
-            if (w == PG_ID64)
-                { bfs_bottom_up_kernel<uint64_t><<<grid_all, kBfsWarps * 32, 0, s>>>(
-                    d_row_ptr, (const uint64_t*)d_col, front, next, &state->size[0], d_dist, vis, h.level,
-                    n_vertices); note_launch(); }
-            else
-                { bfs_bottom_up_kernel<uint32_t><<<grid_all, kBfsWarps * 32, 0, s>>>(
-                    d_row_ptr, (const uint32_t*)d_col, front, next, &state->size[0], d_dist, vis, h.level,
-                    n_vertices); note_launch(); }
-            if (cudaGetLastError() != cudaSuccess) return PG_ECUDA;
-            // the next frontier's size decides whether and how another level runs
-            if (cudaMemcpyAsync(&h.fsize, &state->size[0], 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-                cudaStreamSynchronize(s) != cudaSuccess)
-                return PG_ECUDA;
-            h.visited += h.fsize;
-            ++h.level;
-            std::swap(front, next);
-            if (h.fsize > 0 && h.visited >= n_vertices) {   // the last level finds nothing
-                h.fsize = 0;
-                ++h.level;
-            }
-        } while (h.fsize > 0 && (uint64_t)h.fsize * 24 >= n_vertices);
-        bottom_up = false;
-        if (h.fsize > 0) {
-            // top-down again: the bitmap's vertices as a list
-            if (cudaMemsetAsync(&state->size[0], 0, 4, s) != cudaSuccess) return PG_ECUDA;
-            { bfs_list_kernel<<<grid_cap((n_vertices + 31) / 32), 256, 0, s>>>(front, n_vertices, fr[0],
-                                                                              &state->size[0]); note_launch(); }
-            h.cur = 0;
-        }
-    }
-    { bfs_reach_kernel<<<grid_all, 256, 0, s>>>(d_row_ptr, d_dist, n_vertices, &state->scanned); note_launch(); }
-    uint64_t sc = 0;
-    if (cudaMemcpyAsync(&sc, &state->scanned, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return PG_ECUDA;
-    const uint32_t level = h.level;
-    if (levels_out) *levels_out = level;
-    if (scanned_out) *scanned_out = sc;
+    const BfsBuffers W{{fr[0], fr[1]}, d_dist, vis, long_v, long_base, state};
+    BfsState h;
+    const pg_status st =
+        w == PG_ID64 ? search(d_row_ptr, (const uint64_t*)d_col, W, undirected, n_vertices, h, s)
+                     : search(d_row_ptr, (const uint32_t*)d_col, W, undirected, n_vertices, h, s);
+    if (st != PG_OK) return st;
+    if (levels_out) *levels_out = h.level;
+    if (scanned_out) *scanned_out = h.scanned;
     return PG_OK;
 }
 

@@ -349,3 +349,32 @@ def test_degrees_counted_in_32_bits_and_widened(N, id64):
     pg.degrees(t, N, pg.DEG_TOTAL, out=deg[1:N + 1])
     np.testing.assert_array_equal(host(deg[1:N + 1]), o.degrees(e.astype(np.uint64), N, o.DEG_TOTAL))
     assert int(deg[0]) == -7 and int(deg[N + 1]) == -7
+
+
+@pytest.mark.parametrize("N", [1, 2, 30, 31, 32, 60, 1000, 4097])
+@pytest.mark.parametrize("shape", ["path", "star", "two_stars", "complete"])
+def test_bfs_of_graphs_that_change_direction(N, shape):
+    """Searches that start bottom-up, end in either direction, or go back to
+    top-down: a path's frontier is always one vertex, a star's whole graph."""
+    v = np.arange(N, dtype=np.int64)
+    if shape == "path":
+        e = np.stack([v[:-1], v[1:]], 1)
+    elif shape == "star":
+        e = np.stack([np.zeros(N, np.int64), v], 1)
+    elif shape == "two_stars":   # joined by a path of a quarter of the vertices
+        q = N // 4
+        a, b = v[:q + 1], v[2 * q:]
+        e = np.concatenate([np.stack([np.zeros_like(a), a], 1), np.stack([v[q:2 * q], v[q + 1:2 * q + 1]], 1),
+                            np.stack([np.full_like(b, 2 * q), b], 1)])
+    else:
+        k = v[:40]
+        e = np.stack(np.meshgrid(k, k), -1).reshape(-1, 2)
+    rp_h, col_h = o.csr_opts(e.astype(np.uint64), N, pg.CSR_SYMMETRIZE)
+    rp = torch.from_numpy(rp_h.astype(np.int64)).cuda()
+    col = torch.from_numpy(np.append(col_h, 0).astype(np.uint32).view(np.int32)).cuda()
+    for source in {0, N // 3, N - 1}:
+        ref = o.bfs(rp_h, col_h, source)
+        for undirected in (False, True):
+            dist, levels, scanned = pg.bfs(rp, col, source, undirected=undirected)
+            assert np.array_equal(dist.cpu().numpy().view(np.uint32), ref[0]), (source, undirected)
+            assert (levels, scanned) == tuple(ref[1:3]), (source, undirected)
