@@ -1153,6 +1153,9 @@ CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst =
     CsrLayout L;
     const uint64_t nd = N_dst ? N_dst : N;
     const PassList pl = make_passes(N, nd, M);
+    // two copies of the list in the width its caller names, though a list of
+    // narrow ids takes half of that
+    const size_t lists = 2 * a256(M * pair_bytes);
     if (ids_narrow(N, nd)) pair_bytes = 8;
     int dbits = 0;
     for (uint32_t k = 0; k < pl.n; ++k) dbits = pl.bits[k] > dbits ? pl.bits[k] : dbits;
@@ -1166,7 +1169,7 @@ CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst =
     L.off_a = o;
     o += a256(M * pair_bytes);
     L.off_b = o;
-    o += a256(M * pair_bytes);
+    o = lists;
     L.off_status = o;   // tile status words of the pass being sorted
     o += a256(L.n_status * 8);
     L.off_flag = o;     // +0: sort-needed flag, +64: SortJob's words (+128: wait error),
