@@ -121,6 +121,7 @@ struct SortShape {
 };
 constexpr uint32_t kMaxBuckets = 512;
 constexpr uint64_t kShortList = 3u << 18;
+constexpr uint32_t kShortPasses = 8;   // 64 key bits in digits of 9
 
 // The digits of every LSD pass, from the host: pass k sorts by `bits[k]`
 // bits of the destination (field 0) or source (field 1) at `shift[k]`, or
@@ -274,11 +275,11 @@ struct SortJob {
 // one word (kSpinLimit unless a test hook shortened it) it sets *err and
 // goes on with the partial sum, which can only be too small, so every write
 // stays inside the output.
-template <typename K, typename In, typename Id, bool kShort>
+template <typename K, typename In, typename Id, bool kShort, typename D>
 __device__ __forceinline__ void scatter_pass(
     const In in, K* __restrict__ out, Id* __restrict__ col_out, uint64_t* __restrict__ row_ptr,
     const uint64_t M, const uint64_t N, const Digit dg, const uint32_t pass,
-    const uint64_t* __restrict__ dstart, unsigned long long* __restrict__ status,
+    const D* __restrict__ dstart, unsigned long long* __restrict__ status,
     uint32_t* __restrict__ words, const uint32_t spin_limit, const uint32_t withhold)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -300,10 +301,11 @@ __device__ __forceinline__ void scatter_pass(
         for (uint32_t t = lane; t < kBuckets / 8; t += 32)
             reinterpret_cast<uint4*>(wcnt[wid])[t] = make_uint4(0u, 0u, 0u, 0u);
     };
-    if (threadIdx.x == 0) s_tile = atomicAdd(words + pass, 1u);
+    if (!kShort && threadIdx.x == 0) s_tile = atomicAdd(words + pass, 1u);
     zero_counters();
     __syncthreads();
-    uint32_t tile = s_tile;
+    // (a short list's CTAs are all resident and need no ticket)
+    uint32_t tile = kShort ? blockIdx.x : s_tile;
     while ((uint64_t)tile * kTile < M) {   // uniform
         const uint32_t n = (uint32_t)(M - (uint64_t)tile * kTile < kTile ? M - (uint64_t)tile * kTile
                                                                         : kTile);
@@ -498,9 +500,9 @@ __device__ __forceinline__ void scatter_pass(
         }
         // (a ticket taken before the tile's own work is done would hold up the
         // tiles after it: 0.52 -> 0.59 ms at k = 20)
-        if (threadIdx.x == 0) s_tile = atomicAdd(words + pass, 1u);
+        if (!kShort && threadIdx.x == 0) s_tile = atomicAdd(words + pass, 1u);
         __syncthreads();   // the next tile reuses the tables
-        tile = s_tile;
+        tile = kShort ? tile + gridDim.x : s_tile;
     }
 }
 
@@ -573,7 +575,7 @@ __global__ void __launch_bounds__(kSortThreads, 2)
     if (job.sort_needed && *job.sort_needed == 0) return;
     if (job.plain) prepare_passes<kHistCopies / 2>((const K*)job.plain, job);
     else prepare_passes<kHistCopies / 2>(job.first, job);
-    __shared__ uint64_t s_dstart[kMaxBuckets], s_warp[32];
+    __shared__ uint32_t s_dstart[kShortPasses][kMaxBuckets];   // a short list's totals fit
     uint32_t epoch = 0;
     for (uint32_t pass = 0; pass < job.pl.n; ++pass) {
         if (!grid_barrier(job.words + kWordBarrier, job.words + kWordBarrier + 1, epoch)) {
@@ -581,18 +583,35 @@ __global__ void __launch_bounds__(kSortThreads, 2)
             return;
         }
         if (!pass_can_run(job.words, pass)) continue;   // the same in every CTA
-        {
-            const uint32_t d = threadIdx.x;
-            uint64_t total;
-            const uint64_t c = d < job.pl.buckets ? __ldcg(job.tot + pass * job.pl.buckets + d) : 0;
-            const uint64_t ex = block_exclusive_scan(c, s_warp, total);
-            if (d < job.pl.buckets) s_dstart[d] = ex;
+        if (pass == 0) {   // where each digit's run starts, a warp for every pass
+            const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+            if (wid < job.pl.n) {
+                constexpr uint32_t kPer = kMaxBuckets / 32;
+                const unsigned long long* tot = job.tot + wid * kMaxBuckets + lane * kPer;
+                uint32_t c[kPer], sum = 0;
+#pragma unroll
+                for (uint32_t t = 0; t < kPer; ++t) c[t] = (uint32_t)__ldcg(tot + t);
+#pragma unroll
+                for (uint32_t t = 0; t < kPer; ++t) sum += c[t];
+                uint32_t at = sum;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, at, o);
+                    if (lane >= (uint32_t)o) at += y;
+                }
+                at -= sum;
+#pragma unroll
+                for (uint32_t t = 0; t < kPer; ++t) {
+                    s_dstart[wid][lane * kPer + t] = at;
+                    at += c[t];
+                }
+            }
             __syncthreads();
         }
         auto run = [&](auto in) {
             scatter_pass<K, decltype(in), Id, true>(
                 in, job.buf[pass & 1], pass + 1 == job.pl.n ? job.col : nullptr, job.row_ptr, job.M,
-                job.N, job.pl.digit(pass), pass, s_dstart, job.status, job.words,
+                job.N, job.pl.digit(pass), pass, s_dstart[pass], job.status, job.words,
                 job.hook.spin_limit, job.hook.withhold);
         };
         if (pass > 0 || job.plain) run((const K*)(pass ? job.buf[(pass - 1) & 1] : job.plain));
@@ -1209,8 +1228,10 @@ cudaError_t set_csr_attributes()
     using P = typename PairOf<Id>::T;
     return g_csr_attrs[sizeof(Id) == 8].run_current([] {
         constexpr size_t smem = sort_smem_bytes<uint2, true>();
-        static_assert(smem <= 113 * 1024, "two CTAs per SM");
-        static_assert(8 * 512 * 4 * (kHistCopies / 2) <= smem, "the counters of 64 key bits");
+        static_assert(smem + kShortPasses * kMaxBuckets * 4 <= 113 * 1024, "two CTAs per SM");
+        static_assert(kShortPasses * kMaxBuckets * 4 * (kHistCopies / 2) <= smem, "the counters");
+        static_assert(kShortPasses <= kSortWarps && SortShape<uint2, true>::buckets == kMaxBuckets,
+                      "a warp for every pass");
         cudaError_t e = first_error({long_sort_attributes<uint2, P, Id>(),
                                      allow_smem(radix_sort_kernel<uint2, P, Id>, smem)});
         if constexpr (sizeof(Id) == 8)
