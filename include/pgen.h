@@ -428,8 +428,9 @@ pg_status gen_random_cells(uint64_t n_vertices, uint64_t n_edges, uint64_t seed,
  *   d_dist[v] (n_vertices uint32) = hops from source, 0xFFFFFFFF where
  *   unreached. n_vertices < 2^32 - 1. Workspace: pg_bfs_workspace_size()
  *   bytes, 256-byte aligned. Unlike the generators, this call waits for the
- *   stream: after each stretch of top-down levels (one cooperative launch)
- *   and after each bottom-up level, to read the next frontier's size.
+ *   stream: after a run of top-down levels and, with PG_BFS_UNDIRECTED, the
+ *   run of bottom-up levels that follows it (a cooperative launch each), to
+ *   read whether the search is over; most searches are by then.
  *   PG_ETIMEOUT: a bounded wait between levels gave up (d_dist unspecified);
  *   *levels_out (host) = number of levels run (the source's eccentricity + 1
  *   within its component), *scanned_out (host) = the sum of the reached
