@@ -647,7 +647,11 @@ cudaError_t launch_bottom_up(const uint64_t* row_ptr, const Id* col, BfsBuffers 
 {
     TraceScope trace("bfs_bottom_up", s);
     void* args[] = {&row_ptr, &col, &W.long_v, &W.long_base, &W.fr[0], &W.dist, &W.vis, &N, &W.state};
-    return launch_levels(bfs_bottom_up_kernel<Id>, N, 256, 8, args, W.state, s);
+    // six CTAs per SM up to five million vertices (2^20: 0.219 -> 0.191 ms per
+    // search, 2^21 0.252 -> 0.234, 2^22 0.365 -> 0.357), where a barrier and the
+    // slowest CTA weigh more than the loads in flight; eight above (2^23: 0.551
+    // against 0.567)
+    return launch_levels(bfs_bottom_up_kernel<Id>, N, 256, N <= (5u << 20) ? 6 : 8, args, W.state, s);
 }
 
 // The search from the seeded state on. A round is a run of top-down levels, on
