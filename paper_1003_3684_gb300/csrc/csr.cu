@@ -28,8 +28,8 @@
 // kernels read the flag that csr_grouped sets and return at once when the
 // grouped path applied, so no host round trip decides the path.
 //
-// Ids at or above n_vertices are never used as an index (such edges are
-// dropped), so a bad list cannot make a kernel write out of bounds.
+// Ids at or above n_vertices are never used as an index, so a bad list cannot
+// make a kernel write out of bounds, and such a source ends no row.
 #include <atomic>
 #include <cstring>
 #include <type_traits>
@@ -85,7 +85,13 @@ __device__ __forceinline__ uint32_t digit_of(const K& e, const Digit& g)
 }
 
 // The list of a call: its pairs, each twice when sym (the second time
-// reversed), in the width the sort moves.
+// reversed), in the width the sort moves. Where that is the narrower one, an id
+// it cannot hold becomes ~0, which is no vertex of such a call: its low word
+// may name one. A source like that takes its destination along, so that the
+// pair goes behind every row. Such ids are rare, so the readers take low words
+// and collect the high ones in `far`, and read again what that shows to be
+// wide (simple CSR of 2 * 10^7 pairs of 64-bit ids: 1.63 ms, with a test and a
+// choice per id 1.65).
 template <typename K, typename P>
 struct PairList {
     const P* p;
@@ -96,16 +102,43 @@ struct PairList {
         return PairList{p + (i >> sym), sym};
     }
     template <typename I>
-    __device__ __forceinline__ K operator[](I i) const
+    __device__ __forceinline__ K operator[](I i) const { return again(i); }
+    template <typename I>
+    __device__ __forceinline__ K read(I i, uint32_t& far) const
     {
         const P e = p[i >> sym];
         const bool back = (uint32_t)i & sym;
         K k;
         k.x = (decltype(k.x))(back ? e.y : e.x);
         k.y = (decltype(k.y))(back ? e.x : e.y);
+        if constexpr (sizeof(K) < sizeof(P)) far |= (uint32_t)(e.x >> 32) | (uint32_t)(e.y >> 32);
+        return k;
+    }
+    template <typename I>
+    __device__ __forceinline__ K again(I i) const
+    {
+        uint32_t wide = 0;
+        K k = read(i, wide);
+        if constexpr (sizeof(K) < sizeof(P)) {
+            const P e = p[i >> sym];
+            const bool back = (uint32_t)i & sym;
+            if ((back ? e.y : e.x) >> 32) k.x = k.y = ~0u;
+            if ((back ? e.x : e.y) >> 32) k.y = ~0u;
+        }
         return k;
     }
 };
+template <typename K, typename I>
+__device__ __forceinline__ K read_pair(const K* list, I i, uint32_t&) { return list[i]; }
+template <typename K, typename P, typename I>
+__device__ __forceinline__ K read_pair(const PairList<K, P>& list, I i, uint32_t& far)
+{
+    return list.read(i, far);
+}
+template <typename K, typename I>
+__device__ __forceinline__ K read_again(const K* list, I i) { return list[i]; }
+template <typename K, typename P, typename I>
+__device__ __forceinline__ K read_again(const PairList<K, P>& list, I i) { return list.again(i); }
 
 // A sort tile and the widest digit. Long lists: 16 pairs of 32-bit ids (8 of
 // 64-bit) per thread and digits of at most 8 bits. Short lists, up to
@@ -160,9 +193,14 @@ __device__ __forceinline__ void count_digits(const In in, uint64_t M, const Pass
     constexpr int kU = 4;
     for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < M; i0 += kU * stride) {
         K e[kU];
+        uint32_t far = 0;
 #pragma unroll
         for (int u = 0; u < kU; ++u)
-            if (i0 + u * stride < M) e[u] = in[i0 + u * stride];
+            if (i0 + u * stride < M) e[u] = read_pair(in, i0 + u * stride, far);
+        if (far)
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                if (i0 + u * stride < M) e[u] = read_again(in, i0 + u * stride);
         // pass by pass, so that each pass's digit rule is read once for the
         // kU elements
 #pragma unroll 2
@@ -310,11 +348,18 @@ __device__ __forceinline__ void scatter_pass(
         const uint32_t n = (uint32_t)(M - (uint64_t)tile * kTile < kTile ? M - (uint64_t)tile * kTile
                                                                         : kTile);
         const auto tile_in = in + (uint64_t)tile * kTile;
+        uint32_t far = 0;
 #pragma unroll
         for (int r = 0; r < kItems; ++r) {
             const uint32_t t = wbase + r * 32 + lane;
-            if (t < n) e[r] = tile_in[t];
+            if (t < n) e[r] = read_pair(tile_in, t, far);
         }
+        if (far)
+#pragma unroll
+            for (int r = 0; r < kItems; ++r) {
+                const uint32_t t = wbase + r * 32 + lane;
+                if (t < n) e[r] = read_again(tile_in, t);
+            }
         // ranks within the warp (< 32 * kItems <= 512), two per register; the
         // digits are recomputed from e[] where needed, so no array holds them
         uint32_t rk[kItems / 2];
@@ -1119,16 +1164,18 @@ struct CsrLayout {
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Whether the sort moves pairs of 32-bit ids.
-bool ids_narrow(uint64_t n_src, uint64_t n_dst)
+// Whether the sort moves pairs of 32-bit ids: any list of those, and one of
+// 64-bit ids whose vertices leave ~0 free for the ids that don't fit.
+bool ids_narrow(uint64_t n_src, uint64_t n_dst, bool id64)
 {
-    return n_src <= ((uint64_t)1 << 32) && n_dst <= ((uint64_t)1 << 32);
+    const uint64_t most = ((uint64_t)1 << 32) - (id64 ? 1 : 0);
+    return n_src <= most && n_dst <= most;
 }
 
 // Whether the sort of M pairs takes the short-list shape.
-bool short_list(uint64_t M, uint64_t n_src, uint64_t n_dst)
+bool short_list(uint64_t M, uint64_t n_src, uint64_t n_dst, bool id64)
 {
-    return M <= kShortList && ids_narrow(n_src, n_dst);
+    return M <= kShortList && ids_narrow(n_src, n_dst, id64);
 }
 
 // The LSD passes that sort pairs by (src, dst): the key (src << nd) | dst,
@@ -1136,14 +1183,14 @@ bool short_list(uint64_t M, uint64_t n_src, uint64_t n_dst)
 // into ceil((nd + ns) / digit_bits) digits whose widths differ by at most
 // one (the wider ones first). A digit inside one id reads that id alone; the
 // one that contains the boundary reads both.
-PassList make_passes(uint64_t n_src, uint64_t n_dst, uint64_t M)
+PassList make_passes(uint64_t n_src, uint64_t n_dst, uint64_t M, bool id64)
 {
     PassList pl;
     std::memset(&pl, 0, sizeof(pl));
     const int nd = bit_length(n_dst > 0 ? n_dst - 1 : 0);
     const int ns = bit_length(n_src > 0 ? n_src - 1 : 0);
     const int total = nd + ns;
-    const int digit_bits = short_list(M, n_src, n_dst) ? 9 : 8;
+    const int digit_bits = short_list(M, n_src, n_dst, id64) ? 9 : 8;
     const int n = (total + digit_bits - 1) / digit_bits;
     pl.buckets = 1u << digit_bits;
     pl.nd = nd;
@@ -1171,15 +1218,16 @@ CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst =
 {
     CsrLayout L;
     const uint64_t nd = N_dst ? N_dst : N;
-    const PassList pl = make_passes(N, nd, M);
+    const bool id64 = pair_bytes == 16;
+    const PassList pl = make_passes(N, nd, M, id64);
     // two copies of the list in the width its caller names, though a list of
     // narrow ids takes half of that
     const size_t lists = 2 * a256(M * pair_bytes);
-    if (ids_narrow(N, nd)) pair_bytes = 8;
+    if (ids_narrow(N, nd, id64)) pair_bytes = 8;
     int dbits = 0;
     for (uint32_t k = 0; k < pl.n; ++k) dbits = pl.bits[k] > dbits ? pl.bits[k] : dbits;
     const uint32_t tile = pair_bytes != 8 ? SortShape<ulonglong2, false>::tile
-                          : short_list(M, N, nd) ? SortShape<uint2, true>::tile
+                          : short_list(M, N, nd, id64) ? SortShape<uint2, true>::tile
                                                  : SortShape<uint2, false>::tile;
     L.max_nb = 1u << dbits;
     L.n_tiles = (uint32_t)((M + tile - 1) / tile);
@@ -1373,7 +1421,7 @@ cudaError_t csr_impl(const void* d_edges, uint64_t M, uint64_t N, uint64_t N_dst
     unsigned char* ws = (unsigned char*)d_ws;
     uint32_t* sort_needed = (uint32_t*)(ws + L.off_flag);
     const int grid = sort_grid(M + 1);
-    const PassList pl = make_passes(N, N_dst, M);
+    const PassList pl = make_passes(N, N_dst, M, sizeof(Id) == 8);
     if ((err = clear_sort_words(ws, L, pl, M, s)) != cudaSuccess) return err;
     if (cudaMemsetAsync(d_row_ptr, 0, (N + 1) * 8, s) != cudaSuccess) return cudaErrorUnknown;
     {
@@ -1389,7 +1437,7 @@ cudaError_t csr_impl(const void* d_edges, uint64_t M, uint64_t N, uint64_t N_dst
     // ends itself; a key without digits (one vertex) leaves the list as it is
     const bool in_sort = M > 0 && pl.n > 0;
     Id* col = in_sort ? (Id*)d_col : nullptr;
-    if (ids_narrow(N, N_dst)) {
+    if (ids_narrow(N, N_dst, sizeof(Id) == 8)) {
         const uint2* sorted;
         err = radix_sort<uint2, P, Id>({(const P*)d_edges, 0}, M, N, pl, L, ws, sort_needed, s,
                                          &sorted, col, d_row_ptr);
@@ -1462,13 +1510,13 @@ cudaError_t csr_opts_impl(const void* d_edges, uint64_t M, uint64_t N, uint32_t 
     if (cudaMemsetAsync(d_row_ptr, 0, (N + 1) * 8, s) != cudaSuccess) return cudaErrorUnknown;
     const P* in = (const P*)d_edges;
     const uint32_t sym = (flags & kOptSym) ? 1 : 0;
-    const PassList pl = make_passes(N, N, M2);
+    const PassList pl = make_passes(N, N, M2, sizeof(Id) == 8);
     if ((err = clear_sort_words(ws, O.L, pl, M2, s)) != cudaSuccess) return err;
     // one vertex: the list is sorted as it is (its reverse is the same again)
     if (pl.n == 0)
         return csr_compact<Id>(PairList<P, P>{in, sym}, M2, N, flags, O, ws, d_row_ptr, (Id*)d_col, s);
     // every option needs the sorted list: the sort runs unconditionally
-    if (ids_narrow(N, N)) {
+    if (ids_narrow(N, N, sizeof(Id) == 8)) {
         const uint2* sorted;
         if ((err = radix_sort<uint2, P, Id>({in, sym}, M2, N, pl, O.L, ws, nullptr, s, &sorted,
                                               nullptr, nullptr)) != cudaSuccess)

@@ -378,3 +378,23 @@ def test_bfs_of_graphs_that_change_direction(N, shape):
             dist, levels, scanned = pg.bfs(rp, col, source, undirected=undirected)
             assert np.array_equal(dist.cpu().numpy().view(np.uint32), ref[0]), (source, undirected)
             assert (levels, scanned) == tuple(ref[1:3]), (source, undirected)
+
+
+@pytest.mark.parametrize("M", [20_011, 900_001])                 # a short sort and a long one
+@pytest.mark.parametrize("N", [5000, 2**13])
+@pytest.mark.parametrize("flags", [0, pg.CSR_DEDUP, pg.CSR_ODD, pg.CSR_NO_LOOPS])
+def test_csr_drops_sources_whose_low_word_names_a_vertex(M, N, flags):
+    """64-bit sources above 2^32, whose low 32 bits are a vertex, some of them
+    in a copy of a valid pair: no row may hold them, and no option may take
+    them for that pair."""
+    rng = np.random.default_rng(M + N + flags)
+    e = rng.integers(0, N - 1, (M, 2), dtype=np.int64)           # (N - 1, N - 1) does not occur
+    e[2::9] = e[1::9][:e[2::9].shape[0]]
+    e[2::9, 0] += 2**32
+    e[3::9, 0] += rng.integers(1, 2**31, e[3::9].shape[0]) << 32
+    t = torch.from_numpy(e).cuda()
+    rp, col = pg.edges_to_csr_opts(t, N, flags) if flags else pg.edges_to_csr(t, N, check=True)
+    kept = e[e[:, 0] < N].astype(np.uint64)
+    ref_rp, ref_col = o.csr_opts(kept, N, flags) if flags else o.csr(kept, N)
+    np.testing.assert_array_equal(host(rp), ref_rp)
+    np.testing.assert_array_equal(host(col)[:ref_col.shape[0]], ref_col)
