@@ -398,3 +398,45 @@ def test_csr_drops_sources_whose_low_word_names_a_vertex(M, N, flags):
     ref_rp, ref_col = o.csr_opts(kept, N, flags) if flags else o.csr(kept, N)
     np.testing.assert_array_equal(host(rp), ref_rp)
     np.testing.assert_array_equal(host(col)[:ref_col.shape[0]], ref_col)
+
+
+@pytest.mark.parametrize("M", [3, 2049, 70_000, 800_000])
+@pytest.mark.parametrize("more", [-2, -1, 0, 1])
+@pytest.mark.parametrize("id64", [False, True])
+def test_csr_of_more_rows_than_edges_after_a_grouped_start(M, more, id64):
+    """The list is grouped but for its last edge, so most row ends are written
+    and must go again: on both sides of the vertex count from which the
+    list's rows alone are cleared, and well above it."""
+    N = 12 * M + more if more < 1 else 50 * M
+    src = np.sort(np.random.default_rng(M).integers(0, N, M))
+    src[-1] = 0
+    e = np.stack([src, np.arange(M)[::-1] % N], 1).astype(np.int64)
+    t = torch.from_numpy(e if id64 else e.astype(np.uint32).view(np.int32)).cuda()
+    rp, col = pg.edges_to_csr(t, N, check=True)
+    ref_rp, ref_col = o.csr(e.astype(np.uint64), N)
+    np.testing.assert_array_equal(host(rp), ref_rp)
+    np.testing.assert_array_equal(host(col), ref_col)
+
+
+def _median_ms(call):
+    call()
+    times = []
+    for _ in range(7):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        call()
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b))
+    return sorted(times)[3]
+
+
+def test_csr_of_few_edges_on_many_vertices_takes_no_longer_than_with_options():
+    """Both calls clear and scan the same rows, and sort a list that is nothing
+    beside them; with options there is no grouped pass to undo."""
+    M, N = 1000, 2**26
+    t = torch.randint(0, N, (M, 2), dtype=torch.int32, device="cuda")
+    rp = torch.empty(N + 1, dtype=torch.int64, device="cuda")
+    plain = _median_ms(lambda: pg.edges_to_csr(t, N, row_ptr=rp))
+    dedup = _median_ms(lambda: pg.edges_to_csr_opts(t, N, pg.CSR_DEDUP, row_ptr=rp))
+    assert plain < 2 * dedup, (plain, dedup)
