@@ -706,9 +706,12 @@ pg_status pg_degrees(const void* d_edges, uint64_t n_edges, uint64_t n_vertices,
     // cells: 15 million vertices 0.74 -> 0.62, 3.05 -> 2.60 and 3.29 -> 1.34 ms, 2^24
     // vertices 0.88 -> 0.70, 3.82 -> 3.71 and 4.28 -> 1.52; 11 million 0.47 -> 0.48, 2.17
     // -> 2.05 and 1.48 -> 1.00; fewer lose). One end alone gains less, and the sources
-    // of a grouped list lose.
-    const bool narrow = n_vertices >= kNarrowVertices && which == PG_DEG_TOTAL && n_edges > 0 &&
-                        n_edges < (1ull << 31);
+    // of a grouped list lose. Few edges don't pay for the widening: half an edge
+    // per vertex gains on 2^24 vertices (uniform and grouped: 0.31 -> 0.20 and 0.22
+    // -> 0.17 ms) but not in a grouped list on 2^28 (6.73 -> 6.83), and 1000 edges
+    // on 2^24 took 0.114 ms instead of 0.035.
+    const bool narrow = n_vertices >= kNarrowVertices && which == PG_DEG_TOTAL &&
+                        n_edges >= n_vertices - n_vertices / 4 && n_edges < (1ull << 31);
     uint32_t* cnt = reinterpret_cast<uint32_t*>(d_deg) + n_vertices;
     if (n_vertices > 0 && (narrow ? cudaMemsetAsync(cnt, 0, n_vertices * 4, s)
                                   : cudaMemsetAsync(d_deg, 0, n_vertices * 8, s)) != cudaSuccess)

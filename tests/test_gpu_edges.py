@@ -440,3 +440,30 @@ def test_csr_of_few_edges_on_many_vertices_takes_no_longer_than_with_options():
     plain = _median_ms(lambda: pg.edges_to_csr(t, N, row_ptr=rp))
     dedup = _median_ms(lambda: pg.edges_to_csr_opts(t, N, pg.CSR_DEDUP, row_ptr=rp))
     assert plain < 2 * dedup, (plain, dedup)
+
+
+@pytest.mark.parametrize("N", [13 * 2**20 - 1, 13 * 2**20 + 1, 2**24])
+@pytest.mark.parametrize("more", [-1, 0, 1])
+def test_degrees_of_three_edges_per_four_vertices(N, more):
+    """Both sides of the edge count from which many vertices' counts are taken
+    in 32 bits; the first and last vertices with long runs."""
+    M = N - N // 4 + more
+    rng = np.random.default_rng(M)
+    e = rng.integers(0, N, size=(M, 2), dtype=np.int64)
+    e[::5] = (N - 1, 0)
+    e[1::5, 1] = rng.integers(0, 64, e[1::5].shape[0])
+    deg = torch.full((N + 2,), -7, dtype=torch.int64, device="cuda")
+    pg.degrees(torch.from_numpy(e.astype(np.uint32).view(np.int32)).cuda(), N, pg.DEG_TOTAL,
+               out=deg[1:N + 1])
+    np.testing.assert_array_equal(host(deg[1:N + 1]), o.degrees(e.astype(np.uint64), N, o.DEG_TOTAL))
+    assert int(deg[0]) == -7 and int(deg[N + 1]) == -7
+
+
+def test_degrees_of_few_edges_on_many_vertices_take_as_long_for_both_ends_as_for_one():
+    """Either call is the clearing of the counts and little else."""
+    N = 2**24
+    t = torch.randint(0, N, (1000, 2), dtype=torch.int32, device="cuda")
+    deg = torch.empty(N, dtype=torch.int64, device="cuda")
+    both = _median_ms(lambda: pg.degrees(t, N, pg.DEG_TOTAL, out=deg))
+    one = _median_ms(lambda: pg.degrees(t, N, pg.DEG_OUT, out=deg))
+    assert both < 2 * one, (both, one)
