@@ -369,6 +369,13 @@ pg_status pg_csr_check(const void* d_ws, uint64_t n_edges, uint64_t n_vertices, 
  * Process-wide, read at each call; cannot fail. */
 void pg_csr_test_wait_hook(uint32_t spin_limit, uint32_t withhold_tile);
 
+/* The same hook for the barriers inside cooperative launches (a short list's
+ * sort, the row pointers, the levels of pg_bfs): polls (0 = the default, 2^24)
+ * is the number after which a wait gives up, and CTA withhold_cta (0xffffffff
+ * = none) of every such launch never arrives. Process-wide, read at each
+ * launch; cannot fail. */
+void pg_barrier_test_wait_hook(uint32_t polls, uint32_t withhold_cta);
+
 /* ------------------------------------------------------------------------
  * Checked build (a debugging aid, not part of the method). The same sources
  * compiled with -DPGEN_CHECKED give libpgen_checked.so, with the same entry

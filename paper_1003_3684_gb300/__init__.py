@@ -38,6 +38,7 @@ __all__ = [
     "pg_kron_edge_count", "gen_kronecker",
     "pg_csr_workspace_size", "edges_to_csr", "pg_trace_enable", "pg_trace_dump", "pg_launch_count",
     "pg_csr_wait_error_offset", "csr_wait_error", "pg_csr_check", "pg_csr_test_wait_hook",
+    "pg_barrier_test_wait_hook",
     "pg_checked_build", "pg_check_read", "pg_check_test_out_shift", "CheckReport",
     "empty_device", "set_fail_alloc_at", "BatchPlan", "gen_batch", "pg_batch_workspace_size",
     "gen_batch_csr", "pg_batch_csr_workspace_size", "pg_batch_csr_wait_error_offset",
@@ -615,6 +616,16 @@ def pg_csr_test_wait_hook(spin_limit: int = 0, withhold_tile: int = 0xFFFFFFFF) 
     L.pg_csr_test_wait_hook.argtypes = [u32, u32]
     L.pg_csr_test_wait_hook.restype = None
     L.pg_csr_test_wait_hook(spin_limit, withhold_tile)
+
+
+def pg_barrier_test_wait_hook(polls: int = 0, withhold_cta: int = 0xFFFFFFFF) -> None:
+    """Test hook: barrier waits of cooperative launches give up after `polls`
+    polls (0: the default) and CTA withhold_cta of every such launch never
+    arrives."""
+    L = lib()
+    L.pg_barrier_test_wait_hook.argtypes = [u32, u32]
+    L.pg_barrier_test_wait_hook.restype = None
+    L.pg_barrier_test_wait_hook(polls, withhold_cta)
 
 
 class CheckReport(NamedTuple):

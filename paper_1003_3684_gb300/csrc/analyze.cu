@@ -353,7 +353,7 @@ template <typename Id>
 __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_top_down_kernel(
     const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, uint32_t* f0, uint32_t* f1,
     uint32_t undirected, uint32_t* dist, uint32_t* vis, uint64_t N, uint32_t* long_v,
-    uint32_t* long_base, BfsState* state)
+    uint32_t* long_base, BfsState* state, BarrierLimits barrier)
 {
     __shared__ uint32_t wbuf[kBfsWarps][64];
     __shared__ uint64_t wstart[kBfsWarps][32];   // the rows' starts in the concatenation
@@ -379,13 +379,13 @@ __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_top_down_kernel(
         bfs_short_rows(row_ptr, col, frontier, fsize, Q, wstart[wid], wrow[wid],
                        &state->longs[slot], long_v, long_base);
         Q.flush(lane);
-        if (!grid_barrier(&state->arrived, &state->error, epoch)) return;
+        if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
         const unsigned long long ctr = __ldcg(&state->longs[slot]);
         if (ctr) {   // the same in every CTA
             Q.held = 0;
             bfs_long_rows(row_ptr, col, Q, ctr, slice_of(fsize), long_v, long_base);
             Q.flush(lane);
-            if (!grid_barrier(&state->arrived, &state->error, epoch)) return;
+            if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
         }
         fsize = __ldcg(&state->size[slot]);
         visited += fsize;
@@ -518,18 +518,18 @@ __device__ __forceinline__ void bfs_bottom_up_level(
 template <typename Id>
 __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_bottom_up_kernel(
     const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, uint32_t* front, uint32_t* next,
-    uint32_t* list, uint32_t* dist, uint32_t* vis, uint64_t N, BfsState* state)
+    uint32_t* list, uint32_t* dist, uint32_t* vis, uint64_t N, BfsState* state, BarrierLimits barrier)
 {
     uint32_t epoch = 0, fsize = state->fsize, level = state->level;
     uint64_t visited = state->visited;
     if (fsize == 0) return;   // the search is over
     bfs_bitmap(dist, level, N, front);
-    if (!grid_barrier(&state->arrived, &state->error, epoch)) return;
+    if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
     do {
         uint32_t* nsize = &state->size[level & 3];
         if (blockIdx.x == 0 && threadIdx.x == 0) state->size[(level + 1) & 3] = 0;
         bfs_bottom_up_level(row_ptr, col, front, next, nsize, dist, vis, level, N);
-        if (!grid_barrier(&state->arrived, &state->error, epoch)) return;
+        if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
         fsize = __ldcg(nsize);
         visited += fsize;
         ++level;
@@ -632,8 +632,9 @@ template <typename Id>
 cudaError_t launch_top_down(const uint64_t* row_ptr, const Id* col, BfsBuffers W, uint32_t undirected,
                             uint64_t N, cudaStream_t s)
 {
-    void* args[] = {&row_ptr, &col, &W.fr[0], &W.fr[1], &undirected, &W.dist,
-                    &W.vis,   &N,   &W.long_v, &W.long_base, &W.state};
+    BarrierLimits barrier = barrier_limits();
+    void* args[] = {&row_ptr, &col, &W.fr[0],  &W.fr[1],     &undirected, &W.dist,
+                    &W.vis,   &N,   &W.long_v, &W.long_base, &W.state,    &barrier};
     // four CTAs per SM where levels are short (a barrier of 608 CTAs instead of
     // 1216: 2^20 vertices 0.350 -> 0.237 ms per search); all that fit where wide
     // levels run top-down (2^24 vertices, directed: 3.26 -> 3.08 ms)
@@ -646,7 +647,9 @@ cudaError_t launch_bottom_up(const uint64_t* row_ptr, const Id* col, BfsBuffers 
                              cudaStream_t s)
 {
     TraceScope trace("bfs_bottom_up", s);
-    void* args[] = {&row_ptr, &col, &W.long_v, &W.long_base, &W.fr[0], &W.dist, &W.vis, &N, &W.state};
+    BarrierLimits barrier = barrier_limits();
+    void* args[] = {&row_ptr, &col,   &W.long_v, &W.long_base, &W.fr[0],
+                    &W.dist,  &W.vis, &N,        &W.state,     &barrier};
     // six CTAs per SM up to five million vertices (2^20: 0.219 -> 0.191 ms per
     // search, 2^21 0.252 -> 0.234, 2^22 0.365 -> 0.357), where a barrier and the
     // slowest CTA weigh more than the loads in flight; eight above (2^23: 0.551

@@ -612,6 +612,11 @@ void pg_csr_test_wait_hook(uint32_t spin_limit, uint32_t withhold_tile)
     set_csr_wait_hook(spin_limit, withhold_tile);
 }
 
+void pg_barrier_test_wait_hook(uint32_t polls, uint32_t withhold_cta)
+{
+    set_barrier_hook(polls, withhold_cta);
+}
+
 int pg_checked_build(void) { return kChecked ? 1 : 0; }
 
 #ifdef PGEN_CHECKED

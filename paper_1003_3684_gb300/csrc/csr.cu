@@ -241,6 +241,9 @@ struct CsrWaitHook {
 std::atomic<uint32_t> g_hook_spin{kSpinLimit};
 std::atomic<uint32_t> g_hook_withhold{0xFFFFFFFFu};
 CsrWaitHook csr_wait_hook() { return CsrWaitHook{g_hook_spin.load(), g_hook_withhold.load()}; }
+// The same for the barriers of cooperative launches: one CTA never arrives.
+std::atomic<uint32_t> g_barrier_polls{kBarrierPolls};
+std::atomic<uint32_t> g_barrier_withhold{0xFFFFFFFFu};
 
 // Exclusive scan of the CTA's values, and their sum.
 __device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t v, uint64_t* s_warp,
@@ -288,6 +291,7 @@ struct SortJob {
     Id* col;                       // null: the last pass writes pairs, too
     uint64_t* row_ptr;
     CsrWaitHook hook;
+    BarrierLimits barrier;
     PassList pl;
 };
 
@@ -634,7 +638,7 @@ __global__ void __launch_bounds__(kSortThreads, 2)
     __shared__ uint32_t s_dstart[kShortPasses][kMaxBuckets];   // a short list's totals fit
     uint32_t epoch = 0;
     for (uint32_t pass = 0; pass < job.pl.n; ++pass) {
-        if (!grid_barrier(job.words + kWordBarrier, job.words + kWordBarrier + 1, epoch)) {
+        if (!grid_barrier(job.words + kWordBarrier, job.words + kWordBarrier + 1, job.barrier, epoch)) {
             if (threadIdx.x == 0) atomicOr(job.words + kWordErr, 1u);
             return;
         }
@@ -858,7 +862,7 @@ constexpr int kRowPlaces = 4;   // CTAs per SM
 template <typename V>
 __global__ void __launch_bounds__(256, kRowPlaces)
     row_max_kernel(uint64_t* data, uint64_t n, uint64_t* part, uint32_t per, uint32_t* words,
-                   uint32_t* err)
+                   uint32_t* err, BarrierLimits barrier)
 {
     __shared__ V s_warp[8];
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -893,7 +897,7 @@ __global__ void __launch_bounds__(256, kRowPlaces)
         m = reduce(m);
         if (threadIdx.x == 0) part[blockIdx.x] = m;
         uint32_t epoch = 0;
-        if (!grid_barrier(words, words + 1, epoch)) {
+        if (!grid_barrier(words, words + 1, barrier, epoch)) {
             if (threadIdx.x == 0) atomicOr(err, 1u);
             return;
         }
@@ -1340,6 +1344,7 @@ cudaError_t radix_sort(const PairList<K, P> first, uint64_t M, uint64_t N, const
     job.col = col_final;
     job.row_ptr = row_ptr;
     job.hook = csr_wait_hook();
+    job.barrier = barrier_limits();
     job.pl = pl;
     // Two CTAs per SM, what its registers hold, take tiles until none is left;
     // a long list that turned out grouped pays a launch per pass and not a CTA
@@ -1396,11 +1401,12 @@ cudaError_t row_max_as(uint64_t* d_row_ptr, uint64_t N, const CsrLayout& L, unsi
     uint64_t n = N + 1, *part = (uint64_t*)(ws + L.off_rpart);
     uint32_t* words = (uint32_t*)(ws + L.off_flag + 192);
     uint32_t* err = (uint32_t*)(ws + L.off_flag + 64) + kWordErr;
+    BarrierLimits barrier = barrier_limits();
     if (grid == 1) {   // nothing to wait for
-        { row_max_kernel<V><<<1, 256, 0, s>>>(d_row_ptr, n, part, per, words, err); note_launch(); }
+        { row_max_kernel<V><<<1, 256, 0, s>>>(d_row_ptr, n, part, per, words, err, barrier); note_launch(); }
         return cudaGetLastError();
     }
-    void* args[] = {&d_row_ptr, &n, &part, &per, &words, &err};
+    void* args[] = {&d_row_ptr, &n, &part, &per, &words, &err, &barrier};
     const cudaError_t e = cudaLaunchCooperativeKernel((const void*)row_max_kernel<V>, dim3(grid),
                                                       dim3(256), args, 0, s);
     note_launch();
@@ -1550,6 +1556,16 @@ void set_csr_wait_hook(uint32_t spin_limit, uint32_t withhold_tile)
 {
     g_hook_spin.store(spin_limit ? spin_limit : kSpinLimit);
     g_hook_withhold.store(withhold_tile);
+}
+
+void set_barrier_hook(uint32_t polls, uint32_t withhold_cta)
+{
+    g_barrier_polls.store(polls ? polls : kBarrierPolls);
+    g_barrier_withhold.store(withhold_cta);
+}
+BarrierLimits barrier_limits()
+{
+    return BarrierLimits{g_barrier_polls.load(), g_barrier_withhold.load()};
 }
 
 size_t csr_workspace_bytes(uint64_t n_edges, uint64_t n_vertices, uint64_t n_dst)

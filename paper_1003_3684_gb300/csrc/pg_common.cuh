@@ -200,22 +200,27 @@ __device__ __forceinline__ uint32_t seed_endpoint(uint64_t e, uint32_t side, uin
 }
 
 // Barrier over a cooperative grid; both words start at zero. Each wait is
-// bounded; one that gives up sets the error word and its CTA leaves the
-// kernel, so the others give up too.
+// bounded (`polls`); one that gives up sets the error word and its CTA leaves
+// the kernel, so the others give up too. CTA `withhold` never arrives (test
+// hook; else no CTA's index).
 constexpr uint32_t kBarrierPolls = 1u << 24;   // some ten seconds
-__device__ __forceinline__ bool grid_barrier(uint32_t* arrived, uint32_t* error, uint32_t& epoch)
+struct BarrierLimits {
+    uint32_t polls, withhold;
+};
+__device__ __forceinline__ bool grid_barrier(uint32_t* arrived, uint32_t* error,
+                                             const BarrierLimits& lim, uint32_t& epoch)
 {
     __shared__ uint32_t s_ok;
     __syncthreads();
     ++epoch;
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(arrived, 1u);
+        if (blockIdx.x != lim.withhold) atomicAdd(arrived, 1u);
         const uint32_t want = epoch * gridDim.x;
         uint32_t polls = 0, ok = 1;
         // (the count may wrap; it is never far from what is waited for)
         while ((int32_t)(*(volatile uint32_t*)arrived - want) < 0) {
-            if (++polls > kBarrierPolls || *(volatile uint32_t*)error) {
+            if (++polls > lim.polls || *(volatile uint32_t*)error) {
                 atomicOr(error, 1u);
                 ok = 0;
                 break;

@@ -175,6 +175,8 @@ size_t csr_workspace_bytes(uint64_t n_edges, uint64_t n_vertices, uint64_t n_dst
 size_t csr_wait_error_offset(uint64_t n_edges, uint64_t n_vertices, uint32_t flags, int id64,
                              uint64_t n_dst = 0);
 void set_csr_wait_hook(uint32_t spin_limit, uint32_t withhold_tile);
+void set_barrier_hook(uint32_t polls, uint32_t withhold_cta);
+BarrierLimits barrier_limits();   // of a launch made now
 cudaError_t launch_csr(const void* d_edges, uint64_t n_edges, uint64_t n_vertices, int id64,
                        uint64_t* d_row_ptr, void* d_col, void* d_ws, size_t ws_bytes,
                        cudaStream_t s, uint64_t n_dst = 0);

@@ -164,3 +164,86 @@ def test_csr_leaves_output_past_its_rows_untouched(id64):
     torch.cuda.synchronize()
     assert bool((rp_buf[N + 1:] == C64).all())
     assert _untouched(col_buf[M:], id64)
+
+
+@pytest.fixture
+def no_arrival():
+    """CTA 1 (or another) of every cooperative launch never arrives at its
+    barriers; the waits give up after 64 polls."""
+    pg.pg_barrier_test_wait_hook(64, 1)
+    yield pg.pg_barrier_test_wait_hook
+    pg.pg_barrier_test_wait_hook(0, 0xFFFFFFFF)
+
+
+@pytest.mark.parametrize("flags,id64", [(0, False), (0, True), (pg.CSR_DEDUP, False),
+                                        (pg.CSR_ODD, True)])
+@pytest.mark.parametrize("grouped", [False, True])
+def test_csr_barrier_that_gives_up_is_reported_and_stays_in_bounds(no_arrival, flags, id64, grouped):
+    """A list that is not grouped waits in its sort, a grouped one only in the
+    row pointers."""
+    M, N = 100_001, 20_000
+    e = _multigraph(31 + flags, M, N, id64)
+    if grouped:
+        e[:, 0] = np.arange(M) // 6
+    t = torch.from_numpy(e.view(np.int64 if id64 else np.int32)).cuda()
+    size = (pg.pg_csr_workspace_size(M, N) if flags == 0 else
+            int(pg._opts_lib().pg_csr_opts_workspace_size(M, N, flags)))
+    ws_buf = torch.full((size + 64,), 0x5A, dtype=torch.uint8, device="cuda")
+    rp_buf = torch.full((N + 1 + 64,), C64, dtype=torch.int64, device="cuda")
+    col_buf = _canary((M + 64,), id64)
+    row_ptr, col, ws = rp_buf[:N + 1], col_buf[:M], ws_buf[:size]
+    _csr(t, N, flags, row_ptr, col, ws)
+    with pytest.raises(pg.PgenError) as err:
+        pg.pg_csr_check(ws, M, N, id64=id64, flags=flags)
+    assert err.value.status == pg.PG_ETIMEOUT
+    torch.cuda.synchronize()
+    assert bool((rp_buf[N + 1:] == C64).all()) and _untouched(col_buf[M:], id64)
+    assert bool((ws_buf[size:] == 0x5A).all())
+    no_arrival(0, 0xFFFFFFFF)                  # hook off: the same call again is right
+    _csr(t, N, flags, row_ptr, col, ws)
+    pg.pg_csr_check(ws, M, N, id64=id64, flags=flags)
+    ref_rp, ref_col = (o.csr(e.astype(np.uint64), N) if flags == 0 else
+                       o.csr_opts(e.astype(np.uint64), N, flags))
+    got_rp = row_ptr.cpu().numpy().view(np.uint64)
+    assert np.array_equal(got_rp, ref_rp)
+    got_col = col.cpu().numpy().view(np.uint64 if id64 else np.uint32).astype(np.uint64)
+    assert np.array_equal(got_col[:int(got_rp[-1])], ref_col)
+
+
+def test_batch_csr_barrier_that_gives_up_is_reported(no_arrival):
+    jobs = [dict(kind="kron", initiator=W.KRON_INITIATOR, k=12, n_edges=30_000 + i, seed=i,
+                 want_csr=True) for i in range(3)]
+    plan = pg.BatchPlan(jobs, tile_edges=2048)
+    arena = pg.gen_batch(plan)
+    with pytest.raises(pg.PgenError) as err:
+        pg.gen_batch_csr(plan, arena, check=True)
+    assert err.value.status == pg.PG_ETIMEOUT
+    no_arrival(0, 0xFFFFFFFF)
+    rp, col = pg.gen_batch_csr(plan, arena, check=True)
+    for i, j in enumerate(jobs):
+        ref = o.csr(np.asarray(o.kron(j["initiator"], 12, j["n_edges"], i)).astype(np.uint64), 2**12)
+        for got, want in zip(plan.csr_of(rp, col, i), ref):
+            assert np.array_equal(got.cpu().numpy().astype(np.uint64), want)
+
+
+@pytest.mark.parametrize("N,undirected,cta", [(20_000, False, 1), (20_000, True, 1), (20, True, 0)])
+def test_search_barrier_that_gives_up_is_reported_and_stays_in_bounds(no_arrival, N, undirected, cta):
+    """The first level's barrier, of a run of top-down levels (a bottom-up run is
+    queued behind it) and, for 20 vertices, of a bottom-up one."""
+    no_arrival(64, cta)
+    e = _multigraph(7, 3 * N, N, False).astype(np.uint64)
+    rp_h, col_h = o.csr_opts(e, N, pg.CSR_SYMMETRIZE)
+    rp = torch.from_numpy(rp_h.view(np.int64)).cuda()
+    col = torch.from_numpy(col_h.astype(np.uint32).view(np.int32)).cuda()
+    size = int(pg._analysis_lib().pg_bfs_workspace_size(N))
+    ws = torch.full((size + 64,), 0x5A, dtype=torch.uint8, device="cuda")
+    dist = _canary((N + 64,), False)
+    with pytest.raises(pg.PgenError) as err:
+        pg.bfs(rp, col, 3, dist=dist[:N], workspace=ws[:size], undirected=undirected)
+    assert err.value.status == pg.PG_ETIMEOUT
+    torch.cuda.synchronize()
+    assert _untouched(dist[N:], False) and bool((ws[size:] == 0x5A).all())
+    no_arrival(0, 0xFFFFFFFF)
+    got, levels, scanned = pg.bfs(rp, col, 3, dist=dist[:N], workspace=ws[:size], undirected=undirected)
+    ref = o.bfs(rp_h, col_h, 3)
+    assert np.array_equal(got.cpu().numpy().view(np.uint32), ref[0]) and (levels, scanned) == ref[1:]
