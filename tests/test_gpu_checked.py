@@ -144,3 +144,22 @@ def test_batch_stores_past_the_shortened_bound_are_skipped_and_reported():
     plan = pg.BatchPlan(jobs, tile_edges=1024)
     E = plan.total_edges               # 39,568: the halved bound is even
     _hooked(lambda out: pg.gen_batch(plan, arena=out), E, UNIT_BATCH)
+
+
+@in_child
+@pytest.mark.check_violations
+@pytest.mark.parametrize("id64", [False, True])
+def test_csr_col_stores_of_a_long_sort_past_the_shortened_bound_are_skipped(id64):
+    """The same for a list that takes a launch per pass (the canaries of 64-bit
+    ids are 32-bit ones, widened)."""
+    M, N = 900_000, 2_000
+    e = np.random.default_rng(12).integers(0, N, size=(M, 2), dtype=np.int64)
+    t = torch.from_numpy(e if id64 else e.astype(np.uint32).view(np.int32)).cuda()
+
+    def call(col):
+        out = col.to(torch.int64) if id64 else col
+        pg.edges_to_csr(t, N, col=out, check=True)
+        if id64:
+            col.copy_(out)
+
+    _hooked(call, M, UNIT_CSR, cols=0)

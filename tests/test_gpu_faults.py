@@ -247,3 +247,53 @@ def test_search_barrier_that_gives_up_is_reported_and_stays_in_bounds(no_arrival
     got, levels, scanned = pg.bfs(rp, col, 3, dist=dist[:N], workspace=ws[:size], undirected=undirected)
     ref = o.bfs(rp_h, col_h, 3)
     assert np.array_equal(got.cpu().numpy().view(np.uint32), ref[0]) and (levels, scanned) == ref[1:]
+
+
+@pytest.mark.parametrize("M,N,flags,id64", [
+    (1_000_003, 5_000, 0, False), (1_000_003, 5_000, 0, True),     # 123 tiles of 32-bit pairs
+    (1_000_003, 5_000, pg.CSR_ODD, True),
+    (1_000_003, 5_000, pg.CSR_SYMMETRIZE | pg.CSR_DEDUP, False),   # 245
+    (300_001, 2**32 + 1, 0, True), (300_001, 2**32 + 1, pg.CSR_DEDUP, True),   # 74 of 64-bit pairs
+])
+def test_long_sort_wait_that_gives_up_is_reported_and_stays_in_bounds(M, N, flags, id64):
+    """The sorts with a launch per pass: tile 1 never publishes its counts."""
+    e = _multigraph(43 + flags, M, N, id64)
+    t = torch.from_numpy(e.view(np.int64 if id64 else np.int32)).cuda()
+    listed = 2 * M if flags & pg.CSR_SYMMETRIZE else M
+    size = (pg.pg_csr_workspace_size(M, N) if flags == 0 else
+            int(pg._opts_lib().pg_csr_opts_workspace_size(M, N, flags)))
+    ws_buf = torch.empty(size + 64, dtype=torch.uint8, device="cuda")
+    ws_buf[size:] = 0x5A
+    rp_buf = torch.empty(N + 1 + 64, dtype=torch.int64, device="cuda")   # 34 GB for 2^32 rows
+    rp_buf[N + 1:] = C64
+    col_buf = _canary((listed + 64,), id64)
+    row_ptr, col, ws = rp_buf[:N + 1], col_buf[:listed], ws_buf[:size]
+    pg.pg_csr_test_wait_hook(256, 1)
+    try:
+        _csr(t, N, flags, row_ptr, col, ws)
+        with pytest.raises(pg.PgenError) as err:
+            pg.pg_csr_check(ws, M, N, id64=id64, flags=flags)
+        assert err.value.status == pg.PG_ETIMEOUT
+    finally:
+        pg.pg_csr_test_wait_hook(0, 0xFFFFFFFF)
+    assert bool((rp_buf[N + 1:] == C64).all()) and _untouched(col_buf[listed:], id64)
+    assert bool((ws_buf[size:] == 0x5A).all())
+    # the next call is right: rows with edges and what follows them, and col
+    _csr(t, N, flags, row_ptr, col, ws)
+    pg.pg_csr_check(ws, M, N, id64=id64, flags=flags)
+    pairs = e.astype(np.uint64)
+    if flags & pg.CSR_SYMMETRIZE:
+        pairs = np.concatenate([pairs, pairs[:, ::-1]])
+    if flags & pg.CSR_DEDUP:
+        pairs = np.unique(pairs, axis=0)
+    elif flags & pg.CSR_ODD:
+        pairs, times = np.unique(pairs, axis=0, return_counts=True)
+        pairs = pairs[times % 2 == 1]
+    pairs = pairs[np.lexsort((pairs[:, 1], pairs[:, 0]))]
+    rows, first, counts = np.unique(pairs[:, 0], return_index=True, return_counts=True)
+    at = torch.from_numpy(rows.view(np.int64)).cuda()
+    assert np.array_equal(row_ptr[at].cpu().numpy(), first)
+    assert np.array_equal(row_ptr[at + 1].cpu().numpy(), first + counts)
+    assert int(row_ptr[-1]) == len(pairs)
+    got_col = col.cpu().numpy().view(np.uint64 if id64 else np.uint32).astype(np.uint64)
+    assert np.array_equal(got_col[:len(pairs)], pairs[:, 1])
