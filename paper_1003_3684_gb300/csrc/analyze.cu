@@ -200,12 +200,25 @@ __device__ __forceinline__ uint32_t slice_of(uint32_t fsize)
     return fsize < kWideFrontier ? 64u : 512u;
 }
 
-// Counters of a search, in its workspace. Sizes and long-row counts have a
-// slot per level mod 4: a slot is cleared a level before its use, three levels
-// after its last reader passed a barrier.
+// What the levels count: the next frontier's vertices, and long rows << 32 |
+// their slices. Every warp reads both at a level's end, in one request, as
+// thousands of them queue at one place of the L2 (2^20 vertices: 8 us of a
+// search's 0.2 ms when bottom-up levels read them one by one).
+struct __align__(16) BfsCounts {
+    unsigned long long longs;
+    uint32_t size, pad;
+    __device__ __forceinline__ BfsCounts now() const
+    {
+        const uint4 x = __ldcg(reinterpret_cast<const uint4*>(this));
+        return BfsCounts{(unsigned long long)x.y << 32 | x.x, x.z, 0};
+    }
+};
+
+// Counters of a search, in its workspace. The counts have a slot per level mod
+// 4: a slot is cleared a level before its use, three levels after its last
+// reader passed a barrier.
 struct BfsState {
-    uint32_t size[4];              // next frontier's vertices
-    unsigned long long longs[4];   // long rows << 32 | their slices
+    BfsCounts counts[4];
     unsigned long long scanned;
     uint32_t arrived, error;       // grid barrier: arrivals so far, a wait that gave up
     uint32_t level, fsize, cur, pad;
@@ -298,11 +311,45 @@ __device__ __forceinline__ void bfs_short_rows(const uint64_t* __restrict__ row_
     }
 }
 
-// A top-down level's long rows: slice t of them is entries [t - long_base[r])
-// * slice, ...) of row r, the last row whose base is at or below t. Warps take
-// slices t = warp, warp + warps, ...; a warp finds r by a 32-way search (each
-// round the lanes test 32 evenly spaced bases and a ballot keeps the interval
-// below the first base above t), then walks the slice.
+// Slice t of a level's long rows: the `slice` entries from (t - long_base[r]) *
+// slice on of row r without its first `skip` ones, r the last row whose base is
+// at or below t. A warp finds r by a 32-way search (each round the lanes test
+// 32 evenly spaced bases and a ballot keeps the interval below the first base
+// above t).
+struct BfsSlice {
+    uint32_t v;
+    uint64_t e0, e1;
+};
+__device__ __forceinline__ BfsSlice bfs_slice(const uint64_t* __restrict__ row_ptr, uint64_t N,
+                                              uint32_t t, uint32_t rows, uint32_t skip,
+                                              uint32_t slice, const uint32_t* long_v,
+                                              const uint32_t* long_base)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t lo = 0, n = rows;   // r lies in [lo, lo + n); long_base[lo] <= t
+    while (n > 1) {
+        const uint32_t step = (n + 31) / 32;
+        const uint32_t off = lane * step;
+        const bool le = off < n && PG_CHECK(lo + off, rows) && __ldcg(long_base + lo + off) <= t;
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, le);   // lane 0 always set
+        const uint32_t k = 31 - __clz(m);
+        lo += k * step;
+        n = (n - k * step < step) ? n - k * step : step;
+    }
+    BfsSlice s{0, 0, 0};
+    if (PG_CHECK(lo, rows)) {
+        s.v = __ldcg(long_v + lo);
+        if (PG_CHECK(s.v, N)) {
+            const uint64_t a = row_ptr[s.v] + skip, end = row_ptr[s.v + 1];
+            s.e0 = a + (uint64_t)(t - __ldcg(long_base + lo)) * slice;
+            s.e1 = (s.e0 + slice < end) ? s.e0 + slice : end;
+            if (s.e0 > s.e1) s.e0 = s.e1;
+        }
+    }
+    return s;
+}
+
+// A top-down level's long rows. Warps take slices t = warp, warp + warps, ...
 template <typename Id>
 __device__ __forceinline__ void bfs_long_rows(const uint64_t* __restrict__ row_ptr,
                                               const Id* __restrict__ col, BfsQueue& Q,
@@ -315,29 +362,10 @@ __device__ __forceinline__ void bfs_long_rows(const uint64_t* __restrict__ row_p
     const uint32_t rows = (uint32_t)(ctr >> 32), slices = (uint32_t)ctr;
     const uint32_t warps = gridDim.x * kBfsWarps;
     for (uint32_t t = blockIdx.x * kBfsWarps + (threadIdx.x >> 5); t < slices; t += warps) {
-        uint32_t lo = 0, n = rows;   // r lies in [lo, lo + n); long_base[lo] <= t
-        while (n > 1) {
-            const uint32_t step = (n + 31) / 32;
-            const uint32_t off = lane * step;
-            const bool le = off < n && PG_CHECK(lo + off, rows) && __ldcg(long_base + lo + off) <= t;
-            const uint32_t m = __ballot_sync(0xFFFFFFFFu, le);   // lane 0 always set
-            const uint32_t k = 31 - __clz(m);
-            lo += k * step;
-            n = (n - k * step < step) ? n - k * step : step;
-        }
-        uint64_t e0 = 0, e1 = 0;
-        if (PG_CHECK(lo, rows)) {
-            const uint32_t v = __ldcg(long_v + lo);
-            if (PG_CHECK(v, N)) {
-                const uint64_t a = row_ptr[v], end = row_ptr[v + 1];
-                e0 = a + (uint64_t)(t - __ldcg(long_base + lo)) * slice;
-                e1 = (e0 + slice < end) ? e0 + slice : end;
-                if (e0 > e1) e0 = e1;
-            }
-        }
-        for (uint64_t e = e0; e < e1; e += 64)
+        const BfsSlice s = bfs_slice(row_ptr, N, t, rows, 0, slice, long_v, long_base);
+        for (uint64_t e = s.e0; e < s.e1; e += 64)
             bfs_claim_two(Q, N, lane, lt, [&](int k, uint64_t& u) {
-                if (e + 32 * k + lane >= e1) return false;
+                if (e + 32 * k + lane >= s.e1) return false;
                 u = load_streaming(col + e + 32 * k + lane);
                 return true;
             });
@@ -371,23 +399,22 @@ __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_top_down_kernel(
         uint32_t* frontier = cur ? f1 : f0;
         uint32_t* next = cur ? f0 : f1;
         const uint32_t slot = level & 3, after = (level + 1) & 3;
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            state->size[after] = 0;
-            state->longs[after] = 0;
-        }
-        BfsQueue Q{wbuf[wid], 0, next, &state->size[slot], dist, vis, level, N};
+        if (blockIdx.x == 0 && threadIdx.x == 0) state->counts[after] = BfsCounts{0, 0, 0};
+        BfsCounts* counts = &state->counts[slot];
+        BfsQueue Q{wbuf[wid], 0, next, &counts->size, dist, vis, level, N};
         bfs_short_rows(row_ptr, col, frontier, fsize, Q, wstart[wid], wrow[wid],
-                       &state->longs[slot], long_v, long_base);
+                       &counts->longs, long_v, long_base);
         Q.flush(lane);
         if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
-        const unsigned long long ctr = __ldcg(&state->longs[slot]);
-        if (ctr) {   // the same in every CTA
+        BfsCounts c = counts->now();
+        if (c.longs) {   // the same in every CTA
             Q.held = 0;
-            bfs_long_rows(row_ptr, col, Q, ctr, slice_of(fsize), long_v, long_base);
+            bfs_long_rows(row_ptr, col, Q, c.longs, slice_of(fsize), long_v, long_base);
             Q.flush(lane);
             if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
+            c = counts->now();
         }
-        fsize = __ldcg(&state->size[slot]);
+        fsize = c.size;
         visited += fsize;
         cur ^= 1;
         ++level;
@@ -459,11 +486,17 @@ __device__ __forceinline__ void bfs_list(const uint32_t* bits, uint64_t N, uint3
 // other warp writes them during the level. It looks at eight words at once, so
 // that late levels, whose words are full, cost no wait per word; the words are
 // a grid stride apart, since neighbouring ids share hubs (eight neighbouring
-// words: 0.95 ms).
+// words: 0.95 ms). A lane reads at most kWalk entries; most rows are shorter or
+// have their neighbour among those. The others go to a list, as long rows do
+// top-down, and are read in slices by all warps: a hub of another component, of
+// 2^22 entries, held its level up for 0.48 s, and larger ones would have let the
+// barrier's wait give up.
+constexpr uint32_t kWalk = 256, kWalkSlice = 2048;
 template <typename Id>
 __device__ __forceinline__ void bfs_bottom_up_level(
     const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, const uint32_t* front,
-    uint32_t* next, uint32_t* nsize, uint32_t* dist, uint32_t* vis, uint32_t level, uint64_t N)
+    uint32_t* next, BfsCounts* counts, uint32_t* dist, uint32_t* vis, uint32_t level, uint64_t N,
+    uint32_t* long_v, uint32_t* long_base)
 {
     constexpr uint32_t kWords = 8;
     const uint32_t lane = threadIdx.x & 31;
@@ -490,12 +523,24 @@ __device__ __forceinline__ void bfs_bottom_up_level(
             const uint64_t v = (w0 + t * warps) * 32 + lane;
             bool found = false;
             if (((word >> lane) & 1u) == 0) {
-                const uint64_t b = row_ptr[v + 1];
-                for (uint64_t e = row_ptr[v]; e < b; ++e) {
-                    const uint64_t u = __ldg(col + e);
+                const Id* at = col + row_ptr[v];
+                const uint64_t len = row_ptr[v + 1] - row_ptr[v];
+                const bool more = len > kWalk;
+                for (uint32_t left = more ? kWalk : (uint32_t)len; left > 0; --left, ++at) {
+                    const uint64_t u = __ldg(at);
                     if (u < N && ((front[u >> 5] >> (u & 31)) & 1u)) {
                         found = true;
                         break;
+                    }
+                }
+                if (!found && more) {
+                    const uint64_t rest = row_ptr[v + 1] - row_ptr[v] - kWalk;
+                    const uint64_t ns = (rest + kWalkSlice - 1) / kWalkSlice;
+                    const unsigned long long old = atomicAdd(&counts->longs, (1ull << 32) | ns);
+                    const uint32_t r = (uint32_t)(old >> 32);
+                    if (PG_CHECK(r, N)) {
+                        long_v[r] = (uint32_t)v;
+                        long_base[r] = (uint32_t)old;
                     }
                 }
             }
@@ -509,7 +554,42 @@ __device__ __forceinline__ void bfs_bottom_up_level(
             if (out) vis[my_w] = mine | out;
         }
     }
-    if (lane == 0 && found_all) atomicAdd(nsize, found_all);
+    if (lane == 0 && found_all) atomicAdd(&counts->size, found_all);
+}
+
+// The rest of the listed rows, a slice per warp at a time. The first neighbour
+// found in the frontier claims the vertex; slices of a claimed one are left out.
+template <typename Id>
+__device__ __forceinline__ void bfs_bottom_up_long(
+    const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, const uint32_t* front,
+    uint32_t* next, BfsCounts* counts, uint32_t* dist, uint32_t* vis, uint32_t level, uint64_t N,
+    unsigned long long ctr, const uint32_t* long_v, const uint32_t* long_base)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t rows = (uint32_t)(ctr >> 32), slices = (uint32_t)ctr;
+    const uint32_t warps = gridDim.x * kBfsWarps;
+    for (uint32_t t = blockIdx.x * kBfsWarps + (threadIdx.x >> 5); t < slices; t += warps) {
+        const BfsSlice s = bfs_slice(row_ptr, N, t, rows, kWalk, kWalkSlice, long_v, long_base);
+        const uint32_t word = s.v >> 5, bit = 1u << (s.v & 31);
+        // one lane's view, as another warp may claim it meanwhile
+        if (__shfl_sync(0xFFFFFFFFu, lane == 0 ? __ldcg(vis + word) : 0u, 0) & bit) continue;
+        for (uint64_t e = s.e0; e < s.e1; e += 64) {
+            bool hit = false;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const uint64_t at = e + 32 * k + lane;
+                const uint64_t u = at < s.e1 ? (uint64_t)load_streaming(col + at) : N;
+                hit |= u < N && ((front[u >> 5] >> (u & 31)) & 1u);
+            }
+            if (!__any_sync(0xFFFFFFFFu, hit)) continue;
+            if (lane == 0 && (atomicOr(&vis[word], bit) & bit) == 0) {
+                atomicOr(&next[word], bit);
+                dist[s.v] = level + 1;
+                atomicAdd(&counts->size, 1u);
+            }
+            break;
+        }
+    }
 }
 
 // Bottom-up levels from the state's on, as the top-down kernel runs its: from
@@ -518,7 +598,8 @@ __device__ __forceinline__ void bfs_bottom_up_level(
 template <typename Id>
 __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_bottom_up_kernel(
     const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, uint32_t* front, uint32_t* next,
-    uint32_t* list, uint32_t* dist, uint32_t* vis, uint64_t N, BfsState* state, BarrierLimits barrier)
+    uint32_t* list, uint32_t* long_base, uint32_t* dist, uint32_t* vis, uint64_t N, BfsState* state,
+    BarrierLimits barrier)
 {
     uint32_t epoch = 0, fsize = state->fsize, level = state->level;
     uint64_t visited = state->visited;
@@ -526,11 +607,18 @@ __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_bottom_up_kernel(
     bfs_bitmap(dist, level, N, front);
     if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
     do {
-        uint32_t* nsize = &state->size[level & 3];
-        if (blockIdx.x == 0 && threadIdx.x == 0) state->size[(level + 1) & 3] = 0;
-        bfs_bottom_up_level(row_ptr, col, front, next, nsize, dist, vis, level, N);
+        BfsCounts* counts = &state->counts[level & 3];
+        if (blockIdx.x == 0 && threadIdx.x == 0) state->counts[(level + 1) & 3] = BfsCounts{0, 0, 0};
+        bfs_bottom_up_level(row_ptr, col, front, next, counts, dist, vis, level, N, list, long_base);
         if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
-        fsize = __ldcg(nsize);
+        BfsCounts c = counts->now();
+        if (c.longs) {   // the same in every CTA
+            bfs_bottom_up_long(row_ptr, col, front, next, counts, dist, vis, level, N, c.longs, list,
+                               long_base);
+            if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
+            c = counts->now();
+        }
+        fsize = c.size;
         visited += fsize;
         ++level;
         uint32_t* f = front;
@@ -541,7 +629,7 @@ __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_bottom_up_kernel(
             ++level;
         }
     } while (fsize > 0 && (uint64_t)fsize * 24 >= N);
-    if (fsize > 0) bfs_list(front, N, list, &state->size[level & 3]);
+    if (fsize > 0) bfs_list(front, N, list, &state->counts[level & 3].size);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         state->level = level;
         state->fsize = fsize;
@@ -648,8 +736,9 @@ cudaError_t launch_bottom_up(const uint64_t* row_ptr, const Id* col, BfsBuffers 
 {
     TraceScope trace("bfs_bottom_up", s);
     BarrierLimits barrier = barrier_limits();
-    void* args[] = {&row_ptr, &col,   &W.long_v, &W.long_base, &W.fr[0],
-                    &W.dist,  &W.vis, &N,        &W.state,     &barrier};
+    // the frontier lists are free meanwhile: they take the level's long rows
+    void* args[] = {&row_ptr, &col,    &W.long_v, &W.long_base, &W.fr[0], &W.fr[1],
+                    &W.dist,  &W.vis,  &N,        &W.state,     &barrier};
     // six CTAs per SM up to five million vertices (2^20: 0.219 -> 0.191 ms per
     // search, 2^21 0.252 -> 0.234, 2^22 0.365 -> 0.357), where a barrier and the
     // slowest CTA weigh more than the loads in flight; eight above (2^23: 0.551

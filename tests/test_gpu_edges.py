@@ -467,3 +467,54 @@ def test_degrees_of_few_edges_on_many_vertices_take_as_long_for_both_ends_as_for
     both = _median_ms(lambda: pg.degrees(t, N, pg.DEG_TOTAL, out=deg))
     one = _median_ms(lambda: pg.degrees(t, N, pg.DEG_OUT, out=deg))
     assert both < 2 * one, (both, one)
+
+
+def _csr_on_gpu(e, N, id64=False):
+    rp_h, col_h = o.csr_opts(e.astype(np.uint64), N, pg.CSR_SYMMETRIZE)
+    col = col_h.astype(np.uint64 if id64 else np.uint32).view(np.int64 if id64 else np.int32)
+    return rp_h, col_h, torch.from_numpy(rp_h.view(np.int64)).cuda(), torch.from_numpy(col).cuda()
+
+
+@pytest.mark.parametrize("own", [254, 255, 256, 257, 256 + 2047, 256 + 2048, 256 + 2049, 20_000])
+@pytest.mark.parametrize("hubs", [1, 40])
+@pytest.mark.parametrize("id64", [False, True])
+def test_bfs_of_hubs_found_at_the_end_of_their_rows(own, hubs, id64):
+    """Hubs one bottom-up level away, the neighbour in the frontier the last of
+    their row, or the last but one, or missing: rows around what a lane walks
+    and around the slices of what is left of them."""
+    K = own * hubs // 4 + 100                       # the source's leaves: a wide frontier
+    hub = 1 + np.arange(hubs)
+    leaves = 1 + hubs + np.arange(hubs * own)
+    last = 1 + hubs + hubs * own + np.arange(K)
+    joined = hub[hub % 5 != 3]                      # the others are in components of their own
+    e = np.concatenate([
+        np.stack([np.zeros_like(last), last], 1),
+        np.stack([np.repeat(hub, own), leaves], 1),
+        np.stack([joined, last[joined]], 1),
+        np.stack([joined[::2], last[joined[::2]] + 1], 1)])
+    N = int(last[-1]) + 1
+    rp_h, col_h, rp, col = _csr_on_gpu(e, N, id64)
+    for source in (0, 1, int(last[0])):
+        ref = o.bfs(rp_h, col_h, source)
+        dist, levels, scanned = pg.bfs(rp, col, source, undirected=True)
+        assert np.array_equal(dist.cpu().numpy().view(np.uint32), ref[0]), source
+        assert (levels, scanned) == tuple(ref[1:3]), source
+
+
+def test_bfs_past_a_hub_that_no_level_reaches_keeps_its_barriers_short():
+    """A hub of 2^20 entries in another component: walked by one lane it holds a
+    bottom-up level up for 0.1 s, and the others' barrier waits, here of some ten
+    milliseconds, give up."""
+    H, K = 2**20, 2**18
+    e = np.concatenate([np.stack([np.full(H, 1), 2 + np.arange(H)], 1),
+                        np.stack([np.zeros(K, np.int64), 2 + H + np.arange(K)], 1)])
+    N = 2 + H + K
+    _, _, rp, col = _csr_on_gpu(e, N)
+    pg.pg_barrier_test_wait_hook(1 << 14, 0xFFFFFFFF)
+    try:
+        dist, levels, scanned = pg.bfs(rp, col, 0, undirected=True)
+    finally:
+        pg.pg_barrier_test_wait_hook(0, 0xFFFFFFFF)
+    want = np.full(N, -1, np.int32)
+    want[0], want[2 + H:] = 0, 1
+    assert np.array_equal(dist.cpu().numpy(), want) and (levels, scanned) == (2, 2 * K)
