@@ -134,11 +134,18 @@ pg_status pg_int_probe(int op, uint32_t iters, uint32_t* d_out, size_t out_words
  *
  * d_edges/cap_edges  output buffer and its capacity in edges.
  * n_edges_out        (host, may be NULL) receives the edge count.
- * d_ws/ws_bytes      device workspace of at least pg_pba_workspace_size()
- *                    bytes, 256-byte aligned (unused when blocks == 1).
+ * d_ws/ws_bytes      device workspace of pg_pba_workspace_size() bytes,
+ *                    256-byte aligned (unused when blocks == 1). Less, down
+ *                    to pg_pba_min_workspace_size() bytes, is taken, too: the
+ *                    graph then has fewer, longer segments (one warp's share
+ *                    of the emission), the same edges, and takes longer if it
+ *                    does not fill the GPU that way. The two sizes are the
+ *                    same from about 6 * 10^8 entries (B * n_b * m) on; below,
+ *                    the first is at most 4 times the second.
  * ---------------------------------------------------------------------- */
 uint64_t pg_pba_edge_count(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0);
 size_t pg_pba_workspace_size(uint64_t n, uint32_t m, uint32_t blocks);
+size_t pg_pba_min_workspace_size(uint64_t n, uint32_t m, uint32_t blocks);
 pg_status gen_pba(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0, uint32_t faction_width,
                   double inter_frac, uint64_t seed, pg_idwidth w, void* d_edges,
                   uint64_t cap_edges, uint64_t* n_edges_out, void* d_ws, size_t ws_bytes,
@@ -202,8 +209,8 @@ pg_status gen_pba_factions(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0,
  * may follow one prepare -- in any order, into buffers much smaller than
  * the whole graph (stream a graph to host or disk range by range, or
  * regenerate a lost range after a restart from the arguments alone). The
- * workspace must not change between the two calls; n, m, blocks, n0 and
- * seed must match. blocks = 1 (serial BA) needs no prepare: the only range
+ * workspace must not change between the two calls; n, m, blocks, n0, seed
+ * and ws_bytes (which decides the layout) must match. blocks = 1 (serial BA) needs no prepare: the only range
  * is [0, 1).
  * ---------------------------------------------------------------------- */
 pg_status pg_pba_prepare(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0,
@@ -227,9 +234,9 @@ pg_status gen_pba_blocks(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0, u
  *
  * Scratch: a fixed device array of pg_pba_noalloc_scratch_bytes() (32 MiB)
  * compiled into the library, held by every GPU that loads it until the
- * process exits. A graph whose workspace (pg_pba_workspace_size) exceeds it
- * is rejected with PG_ENOMEM before anything is launched; blocks = 1 needs
- * no scratch. The first call on each device looks up the array's device
+ * process exits. A graph whose smallest workspace (pg_pba_min_workspace_size)
+ * exceeds it is rejected with PG_ENOMEM before anything is launched; blocks =
+ * 1 needs no scratch. The first call on each device looks up the array's device
  * address (once per device, with that device current); make that first call
  * before any stream capture. All calls share the one array: calls whose work
  * overlaps on the GPU (other streams, or other host threads) race and give
@@ -495,7 +502,8 @@ pg_status pg_bfs(const uint64_t* d_row_ptr, const void* d_col, uint64_t n_vertic
  * kernels (phase 1, the count exchange, the emission) in d_ws after the
  * counter. h_plan is the host plan d_plan was copied from (its two-phase
  * geometry is read there). d_ws: pg_batch_workspace_size(h_plan) bytes,
- * 256-byte aligned. The call is stream-ordered with no host
+ * 256-byte aligned (or less, down to 256 bytes and the largest
+ * pg_pba_min_workspace_size of the two-phase jobs, as for gen_pba). The call is stream-ordered with no host
  * synchronisation and can be captured in a CUDA graph; a replay regenerates
  * the same edges.
  *

@@ -29,7 +29,8 @@ __all__ = [
     "PG_OK", "PG_EINVAL", "PG_ENOSPC", "PG_ECUDA", "PG_ETIMEOUT", "PG_ENOMEM",
     "PgenError", "lib", "library_path",
     "pg_status_string", "pg_device_sm_count", "pg_version",
-    "pg_pba_edge_count", "pg_force_wide_path", "pg_pba_workspace_size", "gen_pba", "gen_pba_to_host",
+    "pg_pba_edge_count", "pg_force_wide_path", "pg_pba_workspace_size",
+    "pg_pba_min_workspace_size", "gen_pba", "gen_pba_to_host",
     "pba_faction_table", "gen_pba_factions", "pg_pba_prepare", "gen_pba_blocks",
     "gen_kronecker_range", "philox_rate", "int_pipe_rates", "edges_to_csr_opts", "gen_random_cells",
     "kronecker_xor_random", "CSR_SYMMETRIZE", "CSR_DEDUP", "CSR_NO_LOOPS", "CSR_ODD",
@@ -95,6 +96,8 @@ def lib():
             L.pg_pba_edge_count.restype = u64
             L.pg_pba_workspace_size.argtypes = [u64, u32, u32]
             L.pg_pba_workspace_size.restype = sz
+            L.pg_pba_min_workspace_size.argtypes = [u64, u32, u32]
+            L.pg_pba_min_workspace_size.restype = sz
             L.gen_pba.argtypes = [u64, u32, u32, u32, u32, dbl, u64, i32, vp, u64,
                                   C.POINTER(u64), vp, sz, vp]
             L.gen_pba.restype = i32
@@ -203,6 +206,11 @@ def pg_pba_edge_count(n: int, m: int, blocks: int, n0: int) -> int:
 
 def pg_pba_workspace_size(n: int, m: int, blocks: int) -> int:
     return int(lib().pg_pba_workspace_size(n, m, blocks))
+
+
+def pg_pba_min_workspace_size(n: int, m: int, blocks: int) -> int:
+    """The smallest workspace the two-phase calls take (same edges; pgen.h)."""
+    return int(lib().pg_pba_min_workspace_size(n, m, blocks))
 
 
 def gen_pba(n: int, m: int, blocks: int = 1, n0: int | None = None, faction_width: int = 1,

@@ -113,6 +113,12 @@ PbaGeom make_geom(uint64_t n_b, uint64_t N_e, uint32_t m, uint32_t B, uint32_t n
     return g;
 }
 
+size_t pba_workspace_bytes(uint64_t N_e, uint32_t B, bool coarse)
+{
+    const uint32_t S = pba_segments(N_e, pba_segment_length(N_e, B, device_sm_count(), coarse));
+    return pba_workspace_layout((N_e + 7) & ~(uint64_t)7, B, S).total;
+}
+
 // Kronecker thresholds T_c, c < n0^2 - 1 (left-to-right double sums).
 bool kron_thresholds(const double* P, uint32_t n0, uint64_t* T)
 {
@@ -202,9 +208,14 @@ size_t pg_pba_workspace_size(uint64_t n, uint32_t m, uint32_t blocks)
     if (blocks <= 1) return 0;
     const PbaCheck c = check_pba(n, m, blocks, 2, blocks, 0.0, PG_ID64);
     if (c.st != PG_OK) return 0;
-    const uint32_t S =
-        pba_segments(c.N_e, pba_segment_length(c.N_e, blocks, device_sm_count(), false));
-    return pba_workspace_layout((c.N_e + 7) & ~(uint64_t)7, blocks, S).total;
+    return pba_workspace_bytes(c.N_e, blocks, false);
+}
+
+size_t pg_pba_min_workspace_size(uint64_t n, uint32_t m, uint32_t blocks)
+{
+    if (blocks <= 1) return 0;
+    const PbaCheck c = check_pba(n, m, blocks, 2, blocks, 0.0, PG_ID64);
+    return c.st == PG_OK ? pba_workspace_bytes(c.N_e, blocks, true) : 0;
 }
 
 pg_status gen_pba(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0, uint32_t faction_width,
@@ -217,11 +228,10 @@ pg_status gen_pba(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0, uint32_t
     if (n_edges_out) *n_edges_out = c.edges;
     if (cap_edges < c.edges) return PG_ENOSPC;
     if (c.edges > 0 && (!d_edges || !aligned(d_edges, 16))) return PG_EINVAL;
-    const PbaGeom g = make_geom(c.n_b, c.N_e, m, blocks, n0, faction_width, inter_frac, seed);
+    PbaGeom g = make_geom(c.n_b, c.N_e, m, blocks, n0, faction_width, inter_frac, seed);
     cudaStream_t s = (cudaStream_t)stream;
     if (blocks == 1) return from_cuda(launch_ba(g, w == PG_ID64, d_edges, s));
-    const size_t need = pba_workspace_layout(g.A_stride, blocks, g.S).total;
-    if (!d_ws || ws_bytes < need) return PG_ENOMEM;
+    if (!d_ws || !pba_fit_workspace(&g, ws_bytes)) return PG_ENOMEM;
     if (!aligned(d_ws, 256)) return PG_EINVAL;
     return from_cuda(launch_pba(g, w == PG_ID64, d_edges, d_ws, s));
 }
@@ -279,8 +289,7 @@ pg_status gen_pba_factions(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0,
     // one block: every list holds only block 0, so phase 1 is trivial
     if (blocks == 1) return from_cuda(launch_ba(g, w == PG_ID64, d_edges, s));
     g.ftab = (const uint16_t*)d_faction_table;
-    const size_t need = pba_workspace_layout(g.A_stride, blocks, g.S).total;
-    if (!d_ws || ws_bytes < need) return PG_ENOMEM;
+    if (!d_ws || !pba_fit_workspace(&g, ws_bytes)) return PG_ENOMEM;
     if (!aligned(d_ws, 256)) return PG_EINVAL;
     return from_cuda(launch_pba(g, w == PG_ID64, d_edges, d_ws, s));
 }
@@ -296,8 +305,7 @@ pg_status pg_pba_prepare(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0,
     if (d_faction_table && !aligned(d_faction_table, 16)) return PG_EINVAL;
     PbaGeom g = make_geom(c.n_b, c.N_e, m, blocks, n0, W, inter_frac, seed);
     g.ftab = (const uint16_t*)d_faction_table;
-    const size_t need = pba_workspace_layout(g.A_stride, blocks, g.S).total;
-    if (!d_ws || ws_bytes < need) return PG_ENOMEM;
+    if (!d_ws || !pba_fit_workspace(&g, ws_bytes)) return PG_ENOMEM;
     if (!aligned(d_ws, 256)) return PG_EINVAL;
     return from_cuda(launch_pba_phase1(g, d_ws, (cudaStream_t)stream));
 }
@@ -316,11 +324,10 @@ pg_status gen_pba_blocks(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0, u
     if (cap_edges < count) return PG_ENOSPC;
     if (count == 0) return PG_OK;
     if (!d_edges || !aligned(d_edges, 16)) return PG_EINVAL;
-    const PbaGeom g = make_geom(c.n_b, c.N_e, m, blocks, n0, 1, 0.0, seed);
+    PbaGeom g = make_geom(c.n_b, c.N_e, m, blocks, n0, 1, 0.0, seed);
     cudaStream_t s = (cudaStream_t)stream;
     if (blocks == 1) return from_cuda(launch_ba(g, w == PG_ID64, d_edges, s));
-    const size_t need = pba_workspace_layout(g.A_stride, blocks, g.S).total;
-    if (!d_ws || ws_bytes < need) return PG_ENOMEM;
+    if (!d_ws || !pba_fit_workspace(&g, ws_bytes)) return PG_ENOMEM;
     if (!aligned(d_ws, 256)) return PG_EINVAL;
     return from_cuda(launch_pba_emit(g, w == PG_ID64, d_edges, d_ws, b_begin, b_end, s));
 }
@@ -384,7 +391,7 @@ pg_status gen_pba_to_host(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0,
     if (n_edges_out) *n_edges_out = c.edges;
     if (cap_edges < c.edges) return PG_ENOSPC;
     if (c.edges > 0 && (!d_edges || !aligned(d_edges, 16))) return PG_EINVAL;
-    const PbaGeom g = make_geom(c.n_b, c.N_e, m, blocks, n0, faction_width, inter_frac, seed);
+    PbaGeom g = make_geom(c.n_b, c.N_e, m, blocks, n0, faction_width, inter_frac, seed);
     cudaStream_t s = (cudaStream_t)stream;
     const size_t bytes = c.edges * (w == PG_ID64 ? 16 : 8);
     if (blocks == 1) {
@@ -392,8 +399,7 @@ pg_status gen_pba_to_host(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0,
         return cudaMemcpyAsync(h_edges, d_edges, bytes, cudaMemcpyDeviceToHost, s) == cudaSuccess
                    ? PG_OK : PG_ECUDA;
     }
-    const size_t need = pba_workspace_layout(g.A_stride, blocks, g.S).total;
-    if (!d_ws || ws_bytes < need) return PG_ENOMEM;
+    if (!d_ws || !pba_fit_workspace(&g, ws_bytes)) return PG_ENOMEM;
     if (!aligned(d_ws, 256)) return PG_EINVAL;
     // one copy stream and its events per device, made on first use; a
     // set-up that fails destroys what it made, and its status is kept

@@ -657,8 +657,12 @@ pg_status gen_batch(const void* h_plan, const void* d_plan, uint32_t n_jobs, pg_
     if (!HP || HP->total_edges != total_edges) return PG_EINVAL;
     if (cap_edges < total_edges) return PG_ENOSPC;
     if (total_edges > 0 && (!d_arena || ((uintptr_t)d_arena & 15))) return PG_EINVAL;
-    if (!d_ws || ws_bytes < pg_batch_workspace_size(h_plan) || ((uintptr_t)d_ws & 255))
-        return PG_ENOMEM;
+    if (!d_ws || ws_bytes < 256 || ((uintptr_t)d_ws & 255)) return PG_ENOMEM;
+    const TwoPhaseJob* two = (const TwoPhaseJob*)((const unsigned char*)h_plan + HP->off_two);
+    for (uint32_t t = 0; t < HP->n_two; ++t) {
+        PbaGeom g = two[t].g;
+        if (!pba_fit_workspace(&g, ws_bytes - 256)) return PG_ENOMEM;
+    }
     cudaStream_t s = (cudaStream_t)stream;
     const size_t id_bytes = w == PG_ID64 ? 8 : 4;
     const size_t smem = kMaxTile * id_bytes + (size_t)(n_jobs + 1) * 4;
@@ -695,11 +699,12 @@ pg_status gen_batch(const void* h_plan, const void* d_plan, uint32_t n_jobs, pg_
     }
     // two-phase PBA jobs: phase 1, the count exchange and the emission of
     // each, in the shared workspace region after the counter
-    const TwoPhaseJob* two = (const TwoPhaseJob*)((const unsigned char*)h_plan + HP->off_two);
     const BatchJob* J = (const BatchJob*)((const unsigned char*)h_plan + HP->off_jobs);
     for (uint32_t t = 0; t < HP->n_two; ++t) {
         const uint64_t at = J[two[t].job].out_edge;
-        if (launch_pba(two[t].g, w == PG_ID64, (unsigned char*)d_arena + at * 2 * id_bytes,
+        PbaGeom g = two[t].g;
+        pba_fit_workspace(&g, ws_bytes - 256);
+        if (launch_pba(g, w == PG_ID64, (unsigned char*)d_arena + at * 2 * id_bytes,
                        (unsigned char*)d_ws + 256, s) != cudaSuccess)
             return PG_ECUDA;
     }

@@ -76,9 +76,7 @@ pg_status gen_pba_noalloc(uint64_t n, uint32_t m, uint32_t blocks, uint32_t n0,
     if (blocks == 1) return launch_ba(g, w == PG_ID64, d_edges, s) == cudaSuccess ? PG_OK : PG_ECUDA;
     // the graph must fit the fixed scratch (in its smallest layout, if need
     // be); nothing is launched otherwise
-    if (pba_workspace_layout(g.A_stride, g.B, g.S).total > kScratchBytes)
-        pba_set_segments(&g, pba_segment_length(g.N_e, g.B, device_sm_count(), true));
-    if (pba_workspace_layout(g.A_stride, g.B, g.S).total > kScratchBytes) return PG_ENOMEM;
+    if (!pba_fit_workspace(&g, kScratchBytes)) return PG_ENOMEM;
     pg_status st;
     void* scratch = scratch_on_current_device(&st);
     if (!scratch) return st;

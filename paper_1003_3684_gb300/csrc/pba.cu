@@ -350,14 +350,15 @@ __device__ __forceinline__ uint32_t sigma32(uint32_t x, const QRecip& c)
     return (uint32_t)(t1 >> 32) + x * c.C2;
 }
 
-// `in`: the counts themselves (off: another array), or chunk sums (in place).
+// `in`: the counts themselves, or the sums of chunks of rows, `step` rows apart
+// in the offsets (in place).
 template <typename In>
 __global__ void __launch_bounds__(1024) pba_scan_kernel(const In* in, uint64_t* off,
                                                         uint64_t* __restrict__ R,
                                                         FastDiv* __restrict__ divR,
                                                         QRecip* __restrict__ recip, uint32_t nb,
-                                                        uint32_t B, uint32_t rows, uint64_t e0,
-                                                        uint32_t force_wide,
+                                                        uint32_t B, uint32_t rows, uint32_t step,
+                                                        uint64_t e0, uint32_t force_wide,
                                                         uint32_t* __restrict__ wide_flag,
                                                         uint32_t n0, uint32_t* __restrict__ stab)
 {
@@ -374,10 +375,11 @@ __global__ void __launch_bounds__(1024) pba_scan_kernel(const In* in, uint64_t* 
     const uint32_t per = (rows + slabs - 1) / slabs;
     const uint32_t r0 = slab * per < rows ? slab * per : rows;
     const uint32_t r1 = (r0 + per < rows) ? r0 + per : rows;
+    const uint64_t stride = (uint64_t)step * B;
     uint64_t sum = 0;
     if (in_use) {
 #pragma unroll 8
-        for (uint32_t r = r0; r < r1; ++r) sum += in[(uint64_t)r * B + q];
+        for (uint32_t r = r0; r < r1; ++r) sum += in[r * stride + q];
     }
     part[threadIdx.x] = sum;
     __syncthreads();
@@ -400,8 +402,8 @@ __global__ void __launch_bounds__(1024) pba_scan_kernel(const In* in, uint64_t* 
     acc -= sum;
 #pragma unroll 8
     for (uint32_t r = r0; r < r1; ++r) {
-        const uint64_t c = in[(uint64_t)r * B + q];
-        off[(uint64_t)r * B + q] = acc;
+        const uint64_t c = in[r * stride + q];
+        off[r * stride + q] = acc;
         acc += c;
     }
 }
@@ -410,15 +412,15 @@ __global__ void __launch_bounds__(1024) pba_scan_kernel(const In* in, uint64_t* 
 // -> 0.174 ms): the column scan in three steps, over chunks of kChunkRows rows
 // or more. A CTA owns one chunk; its threads take (row group, target) places,
 // consecutive threads on consecutive targets. Step 1 (kApply false) writes the
-// chunk's column sums, the kernel above scans them, and step 2 (kApply true)
-// turns them into every row's offsets. Bound by memory: 4 bytes read twice
-// and 8 written per (row, target).
+// chunk's column sums to its first row of offsets, the kernel above scans them
+// there, and step 2 (kApply true) adds every row's own; the first row's offsets
+// are the scanned sums. Bound by memory: 4 bytes read twice and 8 written per
+// (row, target).
 constexpr uint32_t kScanThreads = 256;
 constexpr uint32_t kChunkRows = 32;
 constexpr uint32_t kOneStepRows = 64;    // rows per thread up to which one launch scans them all
 template <bool kApply>
 __global__ void __launch_bounds__(kScanThreads) pba_chunk_kernel(const uint32_t* __restrict__ cnt,
-                                                                 uint64_t* __restrict__ sums,
                                                                  uint64_t* __restrict__ off,
                                                                  uint32_t B, uint32_t rows,
                                                                  uint32_t chunk_rows)
@@ -437,6 +439,8 @@ __global__ void __launch_bounds__(kScanThreads) pba_chunk_kernel(const uint32_t*
     for (uint32_t q0 = 0; q0 < B; q0 += lanes) {
         const uint32_t q = q0 + threadIdx.x % lanes;
         const bool in = q < B;
+        uint64_t* chunk = off + (uint64_t)r0 * B + q;
+        const uint64_t before = in && kApply ? *chunk : 0;
         uint64_t sum = 0;
         if (in && (!kApply || groups > 1)) {
 #pragma unroll 8
@@ -454,9 +458,9 @@ __global__ void __launch_bounds__(kScanThreads) pba_chunk_kernel(const uint32_t*
         }
         if (!in) continue;
         if (!kApply) {
-            if (grp == 0) sums[(uint64_t)blockIdx.x * B + q] = sum;
+            if (grp == 0) *chunk = sum;
         } else {
-            uint64_t acc = sums[(uint64_t)blockIdx.x * B + q] + sum;
+            uint64_t acc = before + sum;
 #pragma unroll 8
             for (uint32_t r = a; r < b; ++r) {
                 const uint64_t c = cnt[(uint64_t)r * B + q];
@@ -1112,14 +1116,15 @@ PbaWorkspace pba_workspace_layout(uint64_t A_stride, uint32_t B, uint32_t S)
     o += 256;
     w.off_stab = o;
     o += align256(kSeedTab * 4);
-    w.off_sums = o;
-    const uint64_t rows = (uint64_t)B * S;
-    if (!scan_in_one_step(rows, B)) {
-        const uint32_t per = scan_chunk_rows(B);
-        o += align256((size_t)((rows + per - 1) / per) * B * 8);
-    }
     w.total = o;
     return w;
+}
+
+bool pba_fit_workspace(PbaGeom* g, size_t bytes)
+{
+    if (pba_workspace_layout(g->A_stride, g->B, g->S).total <= bytes) return true;
+    pba_set_segments(g, pba_segment_length(g->N_e, g->B, device_sm_count(), true));
+    return pba_workspace_layout(g->A_stride, g->B, g->S).total <= bytes;
 }
 
 // When set, the serial and two-phase kernels take their 64-bit-index
@@ -1173,7 +1178,6 @@ struct PbaBuffers {
     QRecip* recip;
     uint32_t* wide;
     uint32_t* stab;
-    uint64_t* sums;
 };
 
 PbaBuffers pba_buffers(const PbaGeom& g, void* d_ws)
@@ -1183,8 +1187,7 @@ PbaBuffers pba_buffers(const PbaGeom& g, void* d_ws)
     return PbaBuffers{(uint16_t*)(ws + L.off_A), (uint32_t*)(ws + L.off_cnt),
                       (uint64_t*)(ws + L.off_off), (uint64_t*)(ws + L.off_R),
                       (FastDiv*)(ws + L.off_magic), (QRecip*)(ws + L.off_recip),
-                      (uint32_t*)(ws + L.off_flag), (uint32_t*)(ws + L.off_stab),
-                      (uint64_t*)(ws + L.off_sums)};
+                      (uint32_t*)(ws + L.off_flag), (uint32_t*)(ws + L.off_stab)};
 }
 
 constexpr size_t kSmemFast = kEmitWarps * sizeof(EmitWarpSmem<uint32_t>);
@@ -1299,15 +1302,13 @@ cudaError_t launch_pba_phase1(const PbaGeom& g, void* d_ws, cudaStream_t s)
         const uint32_t qs = g.B < 32 ? 1 : (g.B + 31) / 32, nb = (uint32_t)g.n_b;
         if (scan_in_one_step(rows, g.B)) {
             { pba_scan_kernel<uint32_t><<<qs, 1024, 0, s>>>(W.cnt, W.off, W.R, W.divR, W.recip, nb, g.B,
-                                                           rows, g.e0, fw, W.wide, g.n0, W.stab); note_launch(); }
+                                                           rows, 1, g.e0, fw, W.wide, g.n0, W.stab); note_launch(); }
         } else {
             const uint32_t per = scan_chunk_rows(g.B), chunks = (rows + per - 1) / per;
-            { pba_chunk_kernel<false><<<chunks, kScanThreads, 0, s>>>(W.cnt, W.sums, W.off, g.B, rows,
-                                                                     per); note_launch(); }
-            { pba_scan_kernel<uint64_t><<<qs, 1024, 0, s>>>(W.sums, W.sums, W.R, W.divR, W.recip, nb, g.B,
-                                                           chunks, g.e0, fw, W.wide, g.n0, W.stab); note_launch(); }
-            { pba_chunk_kernel<true><<<chunks, kScanThreads, 0, s>>>(W.cnt, W.sums, W.off, g.B, rows,
-                                                                    per); note_launch(); }
+            { pba_chunk_kernel<false><<<chunks, kScanThreads, 0, s>>>(W.cnt, W.off, g.B, rows, per); note_launch(); }
+            { pba_scan_kernel<uint64_t><<<qs, 1024, 0, s>>>(W.off, W.off, W.R, W.divR, W.recip, nb, g.B,
+                                                           chunks, per, g.e0, fw, W.wide, g.n0, W.stab); note_launch(); }
+            { pba_chunk_kernel<true><<<chunks, kScanThreads, 0, s>>>(W.cnt, W.off, g.B, rows, per); note_launch(); }
         }
     }
     return cudaGetLastError();

@@ -130,13 +130,16 @@ constexpr uint32_t kFacStride = kFacHeader + 2 * kFacSlots;
 
 // Workspace layout for B > 1 (all offsets 256-byte aligned).
 struct PbaWorkspace {
-    size_t off_A, off_cnt, off_off, off_R, off_magic, off_recip, off_flag, off_stab, off_sums, total;
+    size_t off_A, off_cnt, off_off, off_R, off_magic, off_recip, off_flag, off_stab, total;
 };
 PbaWorkspace pba_workspace_layout(uint64_t A_stride, uint32_t B, uint32_t S);
 uint32_t pba_segments(uint64_t N_e, uint64_t seg_len);
 uint32_t pba_prefix_len(uint64_t N_e, uint32_t B, int sm_count);
 uint64_t pba_segment_length(uint64_t N_e, uint32_t B, int sm_count, bool coarse);
 void pba_set_segments(PbaGeom* g, uint64_t seg_len);
+// Whether the graph's workspace fits `bytes`; if only the smallest layout does,
+// the graph takes that.
+bool pba_fit_workspace(PbaGeom* g, size_t bytes);
 
 void set_wide_path_forced(bool on);
 bool wide_path_forced();

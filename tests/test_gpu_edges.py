@@ -518,3 +518,57 @@ def test_bfs_past_a_hub_that_no_level_reaches_keeps_its_barriers_short():
     want = np.full(N, -1, np.int32)
     want[0], want[2 + H:] = 0, 1
     assert np.array_equal(dist.cpu().numpy(), want) and (levels, scanned) == (2, 2 * K)
+
+
+@pytest.mark.parametrize("n,m,B,n0,most", [
+    (1_000_000, 8, 1000, 9, 28_041_728), (2**20, 2, 2, 3, 4_199_424),
+    (15 * 2**20, 4, 5, 5, 126_061_568), (256 * 3000, 5, 256, 6, None),
+    (2**26, 5, 1024, 6, 922_789_120),      # the column scan in three steps
+])
+@pytest.mark.parametrize("id64", [False, True])
+def test_pba_takes_the_smallest_workspace_and_none_below(n, m, B, n0, most, id64):
+    """Whole-granule segments, `most` bytes or less (what these graphs took
+    when they had no others): the same edges through every entry point."""
+    need = pg.pg_pba_min_workspace_size(n, m, B)
+    assert need <= pg.pg_pba_workspace_size(n, m, B) and (most is None or need <= most)
+    buf = torch.full((need + 64,), 0x5A, dtype=torch.uint8, device="cuda")
+    ws = buf[:need]
+    ref = pg.gen_pba(n, m, B, n0, 1, 0.1, 3, id64=id64)
+    assert torch.equal(pg.gen_pba(n, m, B, n0, 1, 0.1, 3, id64=id64, workspace=ws), ref)
+    out = torch.empty_like(ref)
+    host_out = torch.empty(ref.shape, dtype=ref.dtype, pin_memory=True)
+    pg.gen_pba_to_host(host_out, n, m, B, n0, 1, 0.1, 3, id64=id64, out=out, workspace=ws)
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref) and torch.equal(host_out.cuda(), ref)
+    alone = [[b] for b in range(B)]            # width-1 factions, as a table
+    got = pg.gen_pba_factions(n, m, alone, n0=n0, inter_frac=0.1, seed=3, id64=id64, out=out,
+                              workspace=ws)
+    assert torch.equal(got, ref)
+    pg.pg_pba_prepare(n, m, B, n0, seed=3, workspace=ws)
+    per = ref.shape[0] // B
+    part = pg.gen_pba_blocks(ws, n, m, B, B // 2, B, n0=n0, seed=3, id64=id64)
+    assert torch.equal(part, ref[B // 2 * per:])
+    assert bool((buf[need:] == 0x5A).all())
+    for call in (lambda w: pg.gen_pba(n, m, B, n0, 1, 0.1, 3, id64=id64, out=out, workspace=w),
+                 lambda w: pg.pg_pba_prepare(n, m, B, n0, seed=3, workspace=w)):
+        with pytest.raises(pg.PgenError) as err:
+            call(ws[:need - 1])
+        assert err.value.status == pg.PG_ENOMEM
+
+
+def test_batch_takes_the_smallest_workspace_of_its_two_phase_jobs():
+    jobs = [dict(kind="pba", n=256 * 3000, m=5, n0=6, seed=1, blocks=256, inter_frac=0.1),
+            dict(kind="pba", n=2**20, m=2, n0=3, seed=2, blocks=2, inter_frac=0.1),
+            dict(kind="kron", initiator=W.KRON_INITIATOR, k=12, n_edges=30_001, seed=3)]
+    plan = pg.BatchPlan(jobs, tile_edges=2048)
+    need = 256 + max(pg.pg_pba_min_workspace_size(j["n"], j["m"], j["blocks"]) for j in jobs[:2])
+    assert need < pg.pg_batch_workspace_size(plan)
+    ref = pg.gen_batch(plan)
+    buf = torch.full((need + 64,), 0x5A, dtype=torch.uint8, device="cuda")
+    got = pg.gen_batch(plan, workspace=buf[:need])
+    for i in range(len(jobs)):
+        assert torch.equal(plan.edges_of(got, i), plan.edges_of(ref, i)), i
+    assert bool((buf[need:] == 0x5A).all())
+    with pytest.raises(pg.PgenError) as err:
+        pg.gen_batch(plan, workspace=buf[:need - 1])
+    assert err.value.status == pg.PG_ENOMEM
