@@ -152,7 +152,7 @@ struct SortShape {
     static constexpr uint32_t tile = kSortThreads * items;
     static constexpr uint32_t buckets = kShort ? 512 : 256;
 };
-constexpr uint32_t kMaxBuckets = 512;
+constexpr uint32_t kMaxBuckets = 512, kLongBuckets = 256;
 constexpr uint64_t kShortList = 3u << 18;
 constexpr uint32_t kShortPasses = 8;   // 64 key bits in digits of 9
 
@@ -1235,15 +1235,15 @@ CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst =
     const uint64_t nd = N_dst ? N_dst : N;
     const bool id64 = pair_bytes == 16;
     const PassList pl = make_passes(N, nd, M, id64);
-    // two copies of the list in the width its caller names, though a list of
-    // narrow ids takes half of that
+    // a list of narrow ids takes half of two copies in the width its caller
+    // names; the status words lie in the rest, and what follows behind both
     const size_t lists = 2 * a256(M * pair_bytes);
     if (ids_narrow(N, nd, id64)) pair_bytes = 8;
     int dbits = 0;
     for (uint32_t k = 0; k < pl.n; ++k) dbits = pl.bits[k] > dbits ? pl.bits[k] : dbits;
+    const bool is_short = short_list(M, N, nd, id64);
     const uint32_t tile = pair_bytes != 8 ? SortShape<ulonglong2, false>::tile
-                          : short_list(M, N, nd, id64) ? SortShape<uint2, true>::tile
-                                                 : SortShape<uint2, false>::tile;
+                          : is_short ? SortShape<uint2, true>::tile : SortShape<uint2, false>::tile;
     L.max_nb = 1u << dbits;
     L.n_tiles = (uint32_t)((M + tile - 1) / tile);
     L.n_status = (uint64_t)L.max_nb * L.n_tiles;
@@ -1251,14 +1251,15 @@ CsrLayout csr_layout(uint64_t M, uint64_t N, size_t pair_bytes, uint64_t N_dst =
     L.off_a = o;
     o += a256(M * pair_bytes);
     L.off_b = o;
-    o = lists;
+    o += a256(M * pair_bytes);
     L.off_status = o;   // tile status words of the pass being sorted
     o += a256(L.n_status * 8);
+    if (o < lists) o = lists;
     L.off_flag = o;     // +0: sort-needed flag, +64: SortJob's words (+128: wait error),
                         // +192: the row kernel's barrier
     o += 256;
-    L.off_dig = o;      // digit totals, then digit starts, of every pass
-    o += a256(2 * (size_t)kMaxPasses * kMaxBuckets * 8);
+    L.off_dig = o;      // digit totals and, of a long list, digit starts of every pass
+    o += is_short ? (size_t)kShortPasses * kMaxBuckets * 8 : 2 * (size_t)kMaxPasses * kLongBuckets * 8;
     L.n_rparts = (N + 1 + kScanTile - 1) / kScanTile;
     L.off_rpart = o;
     o += a256((L.n_rparts + 1) * 8);
@@ -1370,7 +1371,7 @@ cudaError_t radix_sort(const PairList<K, P> first, uint64_t M, uint64_t N, const
         else
             { radix_hist_kernel<K, PairList<K, P>, P, Id><<<sort_grid(M), 256, smem, s>>>(first, job); note_launch(); }
     }
-    uint64_t* dstart = (uint64_t*)(ws + L.off_dig) + (size_t)kMaxPasses * kMaxBuckets;
+    uint64_t* dstart = (uint64_t*)(ws + L.off_dig) + (size_t)kMaxPasses * kLongBuckets;
     {
         TraceScope trace("csr_scan", s);
         { radix_dstart_kernel<<<pl.n, pl.buckets, 0, s>>>(job.tot, pl, dstart, sort_needed); note_launch(); }
@@ -1490,8 +1491,10 @@ OptsLayout opts_layout(uint64_t M, uint64_t N, uint32_t flags, size_t pair_bytes
     O.n_cparts = (O.M2 + kScanTile - 1) / kScanTile;
     O.off_cpart = o;
     o += a256((O.n_cparts + 1) * 8);
-    O.off_keep = o;
-    o += a256((O.M2 + 31) / 32 * 4);
+    // (nothing between the lists and the sort's words is needed after the sort)
+    const size_t keep = a256((O.M2 + 31) / 32 * 4);
+    O.off_keep = O.L.off_flag - O.L.off_status >= keep ? O.L.off_status : o;
+    if (O.off_keep == o) o += keep;
     O.total = o;
     return O;
 }

@@ -282,3 +282,29 @@ def test_binding_rejects_an_unknown_library_variant():
     r = subprocess.run([sys.executable, "-c", "import paper_1003_3684_gb300"], cwd=ROOT, env=env,
                        capture_output=True, text=True, timeout=300)
     assert r.returncode != 0 and "PGEN_LIBRARY" in r.stderr
+
+
+@pytest.mark.parametrize("M", [1, 100, 4096, 4097, 100_003, 786_432, 786_433, 2**24, 2**31 + 5])
+@pytest.mark.parametrize("N", [1, 2, 5, 2**9, 5_000, 2**20, 2**32, 2**33 + 5])
+@pytest.mark.parametrize("flags", [0, 1, 2, 8 | 1])
+def test_csr_workspace_is_what_64_bit_pairs_in_8_bit_digits_need(L, M, N, flags):
+    """Two copies of the list in 64-bit ids, a status word per digit and 4096
+    pairs, the digits' totals and starts of 16 passes, and the maxima of the row
+    pointers (and, with options, of the kept counts): no shape of the sort asks
+    for more."""
+    import paper_1003_3684_gb300 as pg
+
+    def up(x):
+        return (x + 255) // 256 * 256
+
+    listed = 2 * M if flags & 1 else M
+    bits = 2 * (N - 1).bit_length()
+    passes = -(-bits // 8)
+    digit = max((bits // passes + (k < bits % passes) for k in range(passes)), default=0)
+    want = (2 * up(16 * listed) + up(2**digit * -(-listed // 4096) * 8) + 256 + 2 * 16 * 256 * 8
+            + up((-(-(N + 1) // 4096) + 1) * 8))
+    if flags:
+        want += up((-(-listed // 4096) + 1) * 8)
+    size = (pg.pg_csr_workspace_size(M, N) if flags == 0 else
+            int(pg._opts_lib().pg_csr_opts_workspace_size(M, N, flags)))
+    assert size <= want
