@@ -131,7 +131,11 @@ def _stream(stream):
         # the handle alone: current_stream() makes an object around it, 3 us a
         # call (with plain addresses of host arrays, host time per small call:
         # gen_pba 18.5 -> 14.0 us, gen_kronecker 29.8 -> 20.4, edges_to_csr 26.2 -> 20.6)
-        return vp(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        # (torch names that function for its own use, so it need not stay)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            return vp(torch.cuda.current_stream().cuda_stream)
+        return vp(raw(torch.cuda.current_device()))
     return vp(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 

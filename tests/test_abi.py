@@ -308,3 +308,20 @@ def test_csr_workspace_is_what_64_bit_pairs_in_8_bit_digits_need(L, M, N, flags)
     size = (pg.pg_csr_workspace_size(M, N) if flags == 0 else
             int(pg._opts_lib().pg_csr_opts_workspace_size(M, N, flags)))
     assert size <= want
+
+
+@pytest.mark.parametrize("raw", [True, False])
+def test_current_stream_with_and_without_torchs_raw_handle(monkeypatch, raw):
+    import types
+
+    import paper_1003_3684_gb300 as pg
+    torch = pytest.importorskip("torch")
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0x1230))
+    if raw:
+        monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 0x4560 + device,
+                            raising=False)
+    else:
+        monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    assert pg._stream(None).value == (0x4563 if raw else 0x1230)
+    assert pg._stream(0x7890).value == 0x7890
