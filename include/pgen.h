@@ -307,7 +307,11 @@ pg_status gen_kronecker_range(const double* h_initiator, uint32_t n0, uint32_t k
  * Every id must be < n_vertices (the generators above always satisfy it).
  * The device does not report a violation, but it never indexes memory with
  * such an id: an edge whose src is out of range is dropped, and the rows
- * and col entries it would have touched are unspecified.
+ * and col entries it would have touched (those of the vertex its src's low
+ * bits name; of a 64-bit src that does not fit 32 bits, where n_vertices
+ * does, the last row at most) are unspecified. An edge whose dst alone is
+ * out of range stays in its row, under an id that is out of range, too (not
+ * always its own, and not always in order).
  * ---------------------------------------------------------------------- */
 size_t pg_csr_workspace_size(uint64_t n_edges, uint64_t n_vertices);
 pg_status edges_to_csr(const void* d_edges, uint64_t n_edges, uint64_t n_vertices,
@@ -342,10 +346,13 @@ pg_status edges_to_csr_opts(const void* d_edges, uint64_t n_edges, uint64_t n_ve
 
 /* The sort's wait status (not in the paper; host only, no device call). The
  * digit pass of the sort finds where each tile's run of a digit starts by
- * reading counts that earlier tiles publish. Tiles are handed out in order, so every count it
- * waits for is written by a CTA already running. Each wait still gives up
- * after a fixed number of polls and then sets a uint32 word of the
- * workspace to nonzero. That word is zeroed by every edges_to_csr or
+ * reading counts that earlier tiles publish. A long list's tiles are handed
+ * out in order, so every count it waits for is written by a CTA already
+ * running. A short list (up to 786,432 pairs) is sorted, and the row pointers
+ * of any list are filled, by cooperative launches, whose CTAs all run and wait
+ * for one another between their parts. Each wait still gives up after a fixed
+ * number of polls and then sets a uint32 word of the workspace to nonzero.
+ * That word is zeroed by every edges_to_csr or
  * edges_to_csr_opts call that sorts, which is any call with n_edges > 0 and
  * n_vertices > 1. When the word is nonzero after such a call, the CSR it
  * wrote is unspecified.

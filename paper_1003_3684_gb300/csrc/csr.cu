@@ -300,12 +300,14 @@ struct SortJob {
 // digit's run to its place in the output with consecutive threads on
 // consecutive elements. Where a tile's run of digit d starts is dstart[d]
 // (from the pass's digit totals) plus the count of d in earlier tiles, found
-// by decoupled look-back over the status words. A CTA takes its tile index
-// from a ticket, so every earlier tile belongs to a CTA already running or
-// done. It publishes its own counts before it waits on anything, and it sums
-// earlier tiles' counts, kLookWindow at a time, until it meets an inclusive
-// one (windows of 3, 6 and 8: 2 to 4 % slower at k = 20). The look-back runs
-// after the reorder, when the tile's pairs no longer occupy registers.
+// by decoupled look-back over the status words. A long list's CTA takes its
+// tile index from a ticket, so every earlier tile belongs to a CTA already
+// running or done; a short list's CTAs take theirs by block index and are all
+// resident, in one cooperative launch. A CTA publishes its own counts before it
+// waits on anything, and it sums earlier tiles' counts, kLookWindow at a time,
+// until it meets an inclusive one (windows of 3, 6 and 8: 2 to 4 % slower at k
+// = 20). The look-back runs after the reorder, when the tile's pairs no longer
+// occupy registers.
 //
 // Bound by the shared-memory pipe: 28 wavefronts per 32 pairs and 8 more for
 // global memory, 71 % of its rate, the vector ALU 53 %. So three of eight
