@@ -187,8 +187,6 @@ struct BfsQueue {
     }
 };
 
-// Rows of kLongRow or more entries are cut into slices spread over all warps.
-constexpr uint64_t kLongRow = 64;
 // Slices, and frontier vertices per warp, are short while the frontier is: a
 // level is a chain of dependent loads per step of a warp, and few vertices
 // must not become many steps of few warps. (2^24 vertices: levels of 7, 96 and
@@ -198,6 +196,15 @@ constexpr uint32_t kWideFrontier = 1u << 15;
 __device__ __forceinline__ uint32_t slice_of(uint32_t fsize)
 {
     return fsize < kWideFrontier ? 64u : 512u;
+}
+// Rows of this many entries or more are cut into slices spread over all warps:
+// few in a wide level, whose warps have work enough, and where a list of rows
+// that are one slice each costs a search per row (2^22 vertices with 64 neighbours on
+// average, a level of all: 4.1 -> 1.7 ms; two-phase graphs, whose narrow levels
+// hold the hubs, lose 2 to 4 % by 128 everywhere).
+__device__ __forceinline__ uint32_t long_row(uint32_t fsize)
+{
+    return fsize < (1u << 17) ? 64u : 128u;
 }
 
 // What the levels count: the next frontier's vertices, and long rows << 32 |
@@ -247,19 +254,19 @@ __device__ __forceinline__ void bfs_claim_two(BfsQueue& Q, uint64_t N, uint32_t 
 // lanes idle. A long row is appended to the long-row list instead: one 64-bit
 // atomic on long_ctr adds 1 to the row count (high word) and its slice count
 // to the slice total (low word), so the slice bases of the list ascend with
-// its index. Lists written in this launch are read past the L1 (ldcg).
+// its index.
 template <typename Id>
 __device__ __forceinline__ void bfs_short_rows(const uint64_t* __restrict__ row_ptr,
                                                const Id* __restrict__ col,
                                                const uint32_t* frontier, uint32_t fsize,
-                                               BfsQueue& Q, uint64_t* st, uint64_t* rw,
+                                               uint32_t ctas, BfsQueue& Q, uint64_t* st, uint64_t* rw,
                                                unsigned long long* long_ctr, uint32_t* long_v,
                                                uint32_t* long_base)
 {
     const uint64_t N = Q.N;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
-    const uint64_t warps = (uint64_t)gridDim.x * kBfsWarps;
+    const uint64_t warps = (uint64_t)ctas * kBfsWarps;
     const uint64_t warp = (uint64_t)blockIdx.x * kBfsWarps + (threadIdx.x >> 5);
     const uint32_t slice = slice_of(fsize);
     uint64_t chunk = (fsize + warps - 1) / warps;
@@ -271,7 +278,7 @@ __device__ __forceinline__ void bfs_short_rows(const uint64_t* __restrict__ row_
             if (PG_CHECK(v, N)) {
                 a = row_ptr[v];
                 d = row_ptr[v + 1] - a;
-                if (d >= kLongRow) {
+                if (d >= long_row(fsize)) {
                     const uint64_t ns = (d + slice - 1) / slice;
                     const unsigned long long old = atomicAdd(long_ctr, (1ull << 32) | ns);
                     const uint32_t r = (uint32_t)(old >> 32);
@@ -315,7 +322,9 @@ __device__ __forceinline__ void bfs_short_rows(const uint64_t* __restrict__ row_
 // slice on of row r without its first `skip` ones, r the last row whose base is
 // at or below t. A warp finds r by a 32-way search (each round the lanes test
 // 32 evenly spaced bases and a ballot keeps the interval below the first base
-// above t).
+// above t). The list's first search rounds are the same for all warps and are
+// served by the L1 (read past it, a graph of 2^20 vertices and 16 edges each: 0.46
+// -> 0.48 ms per search).
 struct BfsSlice {
     uint32_t v;
     uint64_t e0, e1;
@@ -330,7 +339,7 @@ __device__ __forceinline__ BfsSlice bfs_slice(const uint64_t* __restrict__ row_p
     while (n > 1) {
         const uint32_t step = (n + 31) / 32;
         const uint32_t off = lane * step;
-        const bool le = off < n && PG_CHECK(lo + off, rows) && __ldcg(long_base + lo + off) <= t;
+        const bool le = off < n && PG_CHECK(lo + off, rows) && long_base[lo + off] <= t;
         const uint32_t m = __ballot_sync(0xFFFFFFFFu, le);   // lane 0 always set
         const uint32_t k = 31 - __clz(m);
         lo += k * step;
@@ -338,10 +347,10 @@ __device__ __forceinline__ BfsSlice bfs_slice(const uint64_t* __restrict__ row_p
     }
     BfsSlice s{0, 0, 0};
     if (PG_CHECK(lo, rows)) {
-        s.v = __ldcg(long_v + lo);
+        s.v = long_v[lo];
         if (PG_CHECK(s.v, N)) {
             const uint64_t a = row_ptr[s.v] + skip, end = row_ptr[s.v + 1];
-            s.e0 = a + (uint64_t)(t - __ldcg(long_base + lo)) * slice;
+            s.e0 = a + (uint64_t)(t - long_base[lo]) * slice;
             s.e1 = (s.e0 + slice < end) ? s.e0 + slice : end;
             if (s.e0 > s.e1) s.e0 = s.e1;
         }
@@ -352,15 +361,15 @@ __device__ __forceinline__ BfsSlice bfs_slice(const uint64_t* __restrict__ row_p
 // A top-down level's long rows. Warps take slices t = warp, warp + warps, ...
 template <typename Id>
 __device__ __forceinline__ void bfs_long_rows(const uint64_t* __restrict__ row_ptr,
-                                              const Id* __restrict__ col, BfsQueue& Q,
-                                              unsigned long long ctr, uint32_t slice,
+                                              const Id* __restrict__ col, uint32_t ctas,
+                                              BfsQueue& Q, unsigned long long ctr, uint32_t slice,
                                               const uint32_t* long_v, const uint32_t* long_base)
 {
     const uint64_t N = Q.N;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     const uint32_t rows = (uint32_t)(ctr >> 32), slices = (uint32_t)ctr;
-    const uint32_t warps = gridDim.x * kBfsWarps;
+    const uint32_t warps = ctas * kBfsWarps;
     for (uint32_t t = blockIdx.x * kBfsWarps + (threadIdx.x >> 5); t < slices; t += warps) {
         const BfsSlice s = bfs_slice(row_ptr, N, t, rows, 0, slice, long_v, long_base);
         for (uint64_t e = s.e0; e < s.e1; e += 64)
@@ -376,13 +385,16 @@ __device__ __forceinline__ void bfs_long_rows(const uint64_t* __restrict__ row_p
 // grid barrier between levels instead of a launch and a host round trip (a
 // level of a small frontier is a few microseconds of latency): until the
 // frontier is empty, or until bottom-up would be chosen on an undirected
-// graph (never for the first level). Leaves where it stopped in the state.
+// graph (never for the first level). Leaves where it stopped in the state. The
+// first `few` CTAs do it all unless the rows have `dense` entries on average.
 template <typename Id>
 __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_top_down_kernel(
     const uint64_t* __restrict__ row_ptr, const Id* __restrict__ col, uint32_t* f0, uint32_t* f1,
     uint32_t undirected, uint32_t* dist, uint32_t* vis, uint64_t N, uint32_t* long_v,
-    uint32_t* long_base, BfsState* state, BarrierLimits barrier)
+    uint32_t* long_base, BfsState* state, uint32_t few, uint32_t dense, BarrierLimits barrier)
 {
+    const uint32_t ctas = few < gridDim.x && row_ptr[N] < dense * N ? few : gridDim.x;
+    if (blockIdx.x >= ctas) return;
     __shared__ uint32_t wbuf[kBfsWarps][64];
     __shared__ uint64_t wstart[kBfsWarps][32];   // the rows' starts in the concatenation
     __shared__ uint64_t wrow[kBfsWarps][32];     // and in col
@@ -402,16 +414,16 @@ __global__ void __launch_bounds__(kBfsWarps * 32, 8) bfs_top_down_kernel(
         if (blockIdx.x == 0 && threadIdx.x == 0) state->counts[after] = BfsCounts{0, 0, 0};
         BfsCounts* counts = &state->counts[slot];
         BfsQueue Q{wbuf[wid], 0, next, &counts->size, dist, vis, level, N};
-        bfs_short_rows(row_ptr, col, frontier, fsize, Q, wstart[wid], wrow[wid],
+        bfs_short_rows(row_ptr, col, frontier, fsize, ctas, Q, wstart[wid], wrow[wid],
                        &counts->longs, long_v, long_base);
         Q.flush(lane);
-        if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
+        if (!grid_barrier(&state->arrived, &state->error, barrier, epoch, ctas)) return;
         BfsCounts c = counts->now();
         if (c.longs) {   // the same in every CTA
             Q.held = 0;
-            bfs_long_rows(row_ptr, col, Q, c.longs, slice_of(fsize), long_v, long_base);
+            bfs_long_rows(row_ptr, col, ctas, Q, c.longs, slice_of(fsize), long_v, long_base);
             Q.flush(lane);
-            if (!grid_barrier(&state->arrived, &state->error, barrier, epoch)) return;
+            if (!grid_barrier(&state->arrived, &state->error, barrier, epoch, ctas)) return;
             c = counts->now();
         }
         fsize = c.size;
@@ -720,14 +732,21 @@ template <typename Id>
 cudaError_t launch_top_down(const uint64_t* row_ptr, const Id* col, BfsBuffers W, uint32_t undirected,
                             uint64_t N, cudaStream_t s)
 {
+    // CTAs per SM: few where levels are short, as a barrier of 608 costs less than
+    // one of 1216 (2^20 vertices 0.350 -> 0.237 ms per search), more where wide levels
+    // run top-down, and all that fit where those read many entries per vertex
+    // (Kronecker graphs of 16 edges per vertex, four / six / eight per SM, ms: 2^20
+    // vertices 0.46 / 0.42 / 0.44, 2^22 1.30 / 1.10 / 1.02, 2^23 - / 1.82 / 1.66;
+    // uniform ones of 2: 2^24 - / 2.38 / 2.51, 2^25 - / 4.69 / 4.88). Undirected
+    // searches leave the wide levels to the other kernel, most of them (2^23 vertices,
+    // four / six: Kronecker 0.82 / 0.74, two-phase 0.52 / 0.56).
+    const bool large = N > (5u << 20);
+    const int most = undirected ? (large ? 6 : 4) : N <= (5u << 18) ? 4 : large ? 8 : 6;
+    uint32_t few = (uint32_t)device_sm_count() * (undirected ? 4 : 6), dense = undirected ? 24 : 8;
     BarrierLimits barrier = barrier_limits();
-    void* args[] = {&row_ptr, &col, &W.fr[0],  &W.fr[1],     &undirected, &W.dist,
-                    &W.vis,   &N,   &W.long_v, &W.long_base, &W.state,    &barrier};
-    // four CTAs per SM where levels are short (a barrier of 608 CTAs instead of
-    // 1216: 2^20 vertices 0.350 -> 0.237 ms per search); all that fit where wide
-    // levels run top-down (2^24 vertices, directed: 3.26 -> 3.08 ms)
-    return launch_levels(bfs_top_down_kernel<Id>, N, 64, undirected || N <= (1u << 22) ? 4 : 8, args,
-                         W.state, s);
+    void* args[] = {&row_ptr,  &col,         &W.fr[0], &W.fr[1], &undirected, &W.dist, &W.vis, &N,
+                    &W.long_v, &W.long_base, &W.state, &few,     &dense,      &barrier};
+    return launch_levels(bfs_top_down_kernel<Id>, N, 64, most, args, W.state, s);
 }
 
 template <typename Id>

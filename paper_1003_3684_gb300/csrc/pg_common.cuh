@@ -199,7 +199,7 @@ __device__ __forceinline__ uint32_t seed_endpoint(uint64_t e, uint32_t side, uin
     return side ? a + 1 + (uint32_t)e : a;
 }
 
-// Barrier over a cooperative grid; both words start at zero. Each wait is
+// Barrier over a cooperative grid (its first `ctas` CTAs); both words start at zero. Each wait is
 // bounded (`polls`); one that gives up sets the error word and its CTA leaves
 // the kernel, so the others give up too. CTA `withhold` never arrives (test
 // hook; else no CTA's index).
@@ -208,7 +208,8 @@ struct BarrierLimits {
     uint32_t polls, withhold;
 };
 __device__ __forceinline__ bool grid_barrier(uint32_t* arrived, uint32_t* error,
-                                             const BarrierLimits& lim, uint32_t& epoch)
+                                             const BarrierLimits& lim, uint32_t& epoch,
+                                             uint32_t ctas = gridDim.x)
 {
     __shared__ uint32_t s_ok;
     __syncthreads();
@@ -216,7 +217,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* arrived, uint32_t* error,
     if (threadIdx.x == 0) {
         __threadfence();
         if (blockIdx.x != lim.withhold) atomicAdd(arrived, 1u);
-        const uint32_t want = epoch * gridDim.x;
+        const uint32_t want = epoch * ctas;
         uint32_t polls = 0, ok = 1;
         // (the count may wrap; it is never far from what is waited for)
         while ((int32_t)(*(volatile uint32_t*)arrived - want) < 0) {

@@ -572,3 +572,23 @@ def test_batch_takes_the_smallest_workspace_of_its_two_phase_jobs():
     with pytest.raises(pg.PgenError) as err:
         pg.gen_batch(plan, workspace=buf[:need - 1])
     assert err.value.status == pg.PG_ENOMEM
+
+
+@pytest.mark.parametrize("N,degree", [
+    (2**18, 32), (2**18, 64),                         # rows around 64 and 128 in a level of most vertices
+    ((5 << 18) + 1, 4), ((5 << 20) - 31, 3),          # more CTAs per SM, up to the last of them
+    ((5 << 20) + 1, 2), ((5 << 20) + 1, 4), ((5 << 20) + 1, 12)])   # all CTAs, or the first few
+def test_bfs_of_uniform_graphs_around_the_switches_of_wide_levels(N, degree):
+    """Symmetrised lists of `degree` edges per vertex: row lengths on both sides
+    of what is long in a narrow and in a wide level, and graphs on both sides
+    of the rules for the number of CTAs (8 and 24 entries per row)."""
+    rng = np.random.default_rng(N + degree)
+    e = rng.integers(0, N, size=(N * degree, 2), dtype=np.uint32)
+    rp, col = pg.edges_to_csr_opts(torch.from_numpy(e.view(np.int32)).cuda(), N, pg.CSR_SYMMETRIZE)
+    rp_h, col_h = host(rp), host(col)
+    for source in (0, N - 1):
+        ref = o.bfs(rp_h, col_h, source)
+        for undirected in (False, True):
+            dist, levels, scanned = pg.bfs(rp, col, source, undirected=undirected)
+            assert np.array_equal(dist.cpu().numpy().view(np.uint32), ref[0]), (source, undirected)
+            assert (levels, scanned) == tuple(ref[1:3]), (source, undirected)
