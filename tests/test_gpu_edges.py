@@ -592,3 +592,18 @@ def test_bfs_of_uniform_graphs_around_the_switches_of_wide_levels(N, degree):
             dist, levels, scanned = pg.bfs(rp, col, source, undirected=undirected)
             assert np.array_equal(dist.cpu().numpy().view(np.uint32), ref[0]), (source, undirected)
             assert (levels, scanned) == tuple(ref[1:3]), (source, undirected)
+
+
+@pytest.mark.parametrize("which", [pg.DEG_OUT, pg.DEG_IN, pg.DEG_TOTAL])
+@pytest.mark.parametrize("M", [1, 63, 64, 65, 511, 513, 152 * 6 * 512 - 1, 152 * 6 * 512 + 33])
+@pytest.mark.parametrize("id64", [False, True])
+def test_degrees_of_runs_across_a_warps_groups(which, M, id64):
+    """Runs of every length up to 70 over the two groups of 32 edges a warp
+    counts at once and over its trips; some ids past the vertex count."""
+    rng = np.random.default_rng(M)
+    src = np.repeat(rng.integers(0, 5000, M // 20 + 2), rng.integers(1, 71, M // 20 + 2))
+    src = np.resize(src, M)
+    e = np.stack([src, rng.integers(0, 5000, M)], 1).astype(np.int64)
+    t = torch.from_numpy(e if id64 else e.astype(np.uint32).view(np.int32)).cuda()
+    deg = pg.degrees(t, 4900, which)
+    assert np.array_equal(host(deg), o.degrees(e.astype(np.uint64), 4900, which))
